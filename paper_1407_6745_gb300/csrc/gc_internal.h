@@ -162,6 +162,11 @@ gc_status priorities_device(uint64_t seed, int64_t n, uint32_t* out, cudaStream_
 gc_status validate_device(const Graph& g, const int32_t* colors, gc_validation* out,
                           cudaStream_t s);
 
+// The check of a recoloring input: GC_ERR_BAD_GRAPH, GC_ERR_IMPROPER_INPUT
+// (a conflict, or a color outside [1, max_allowed]) or GC_OK and its max color.
+gc_status check_input_device(const Graph& g, const int32_t* colors, int32_t max_allowed, int32_t* max_color,
+                             cudaStream_t s);
+
 gc_status validate_noalloc_device(const Graph& g, const int32_t* colors, gc_validation* out,
                                   cudaStream_t s);
 

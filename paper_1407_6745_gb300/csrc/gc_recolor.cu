@@ -130,8 +130,7 @@ __device__ __forceinline__ int32_t add_acq_rel(int32_t* p) {
 __device__ __forceinline__ int32_t chunks_of(int32_t deg) { return (deg + kChunk - 1) / kChunk; }
 
 // ---------------------------------------------------------------------------
-// Per-call set-up: degree buckets (X = 1) and, for untrusted input, the
-// proper-coloring check of Sec. 1 plus the max color.
+// Per-call set-up: degree buckets (X = 1).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBlock) k_rc_bucket(RcArgs a) {
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kBlock;
@@ -149,31 +148,6 @@ __global__ void __launch_bounds__(kBlock) k_rc_bucket(RcArgs a) {
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) heavy += __shfl_xor_sync(kFull, heavy, d);
     if (lane_id() == 0 && heavy) atomicAdd(&a.ctrl->n_heavy, heavy);
-}
-
-__global__ void __launch_bounds__(kBlock) k_rc_validate(RcArgs a) {
-    const int w = (blockIdx.x * kBlock + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * kBlock) >> 5;
-    const int l = lane_id();
-    int32_t my_max = 0;
-    for (int64_t v = w; v < a.g.n; v += nw) {
-        const int32_t cv = a.old_c[v];
-        if (cv < 1 || cv > kMaxInputColor) {
-            if (l == 0) atomicOr(&a.ctrl->err, kErrImproper);
-            continue;
-        }
-        my_max = max(my_max, cv);
-        int64_t beg;
-        int32_t deg;
-        row_of(a.g, static_cast<int32_t>(v), beg, deg, &a.ctrl->err);
-        bool bad = false;
-        for (int32_t k = l; k < deg; k += 32) {
-            const int32_t u = load_nbr(a.g, beg + k, &a.ctrl->err);
-            if (u >= 0 && a.old_c[u] == cv) bad = true;
-        }
-        if (__any_sync(kFull, bad) && l == 0) atomicOr(&a.ctrl->err, kErrImproper);
-    }
-    warp_max(&a.ctrl->max_in, my_max);
 }
 
 // Max color of a coloring known to be proper (colors outside [1, max input
@@ -899,14 +873,18 @@ gc_status class_ranks_device(const Graph& g, const int32_t* colors, bool trusted
     a.ctrl = sc_ctrl.as<RcCtrl>();
     cudaMemsetAsync(a.ctrl, 0, sizeof(RcCtrl), s);
     GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
-    if (!trusted) GC_LAUNCH(KID_RC_VALIDATE, s, k_rc_validate<<<grid, kBlock, 0, s>>>(a));
+    int32_t max_checked = 0;
+    gc_status st = GC_OK;
+    if (!trusted) st = check_input_device(g, colors, kMaxInputColor, &max_checked, s);
     else GC_LAUNCH(KID_RC_VALIDATE, s, k_rc_maxin<<<vgrid, kBlock, 0, s>>>(a));
+    if (st != GC_OK && st != GC_ERR_IMPROPER_INPUT) return st;
     RcCtrl h;
     cudaError_t ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
     if (ce != cudaSuccess) return cuda_status(ce);
     if (h.err & kErrBadGraph) return GC_ERR_BAD_GRAPH;
-    if (h.err & kErrImproper) return GC_ERR_IMPROPER_INPUT;
+    if (st != GC_OK || (h.err & kErrImproper)) return GC_ERR_IMPROPER_INPUT;
+    if (!trusted) h.max_in = max_checked;
     *maxc_out = h.max_in;
     if (!rank_out) return GC_OK;
     const int32_t cap = std::max(h.max_in, 1);
@@ -1102,7 +1080,11 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     std::memset(&h, 0, sizeof(h));
     if (n > 0) {
         GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
-        if (!trusted) GC_LAUNCH(KID_RC_VALIDATE, s, k_rc_validate<<<grid, kBlock, 0, s>>>(a));
+    }
+    gc_status input = GC_OK;
+    if (!trusted) {
+        input = check_input_device(g, colors_in, kMaxInputColor, &maxc_in, s);
+        if (input != GC_OK && input != GC_ERR_IMPROPER_INPUT) return input;
     }
     // A trusted input (our own coloring) has a known max color; the split
     // rows are then sized by a bound (a bucket-0 row has more than
@@ -1117,9 +1099,8 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
         if (ce != cudaSuccess) return cuda_status(ce);
         if (h.err & kErrBadGraph) return GC_ERR_BAD_GRAPH;
-        if (h.err & kErrImproper) return GC_ERR_IMPROPER_INPUT;
+        if (input != GC_OK) return input;
         if (!trusted) {
-            maxc_in = h.max_in;
             if (n > 0 && chain_bound(maxc_in)) {  // the buckets again, with the chain-bound threshold
                 a.tune.g2_max_deg = std::min(kChainRcG2MaxDeg, a.tune.g4_max_deg);
                 cudaMemsetAsync(&a.ctrl->n_heavy, 0, sizeof(int32_t), s);
@@ -1325,14 +1306,19 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
     cudaMemsetAsync(a.ctrl, 0, sizeof(RcCtrl), s);
     if (n > 0) {
         GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
-        if (!trusted) GC_LAUNCH(KID_RC_VALIDATE, s, k_rc_validate<<<grid, kBlock, 0, s>>>(a));
+    }
+    gc_status input = GC_OK;
+    if (!trusted) {
+        int32_t max_checked = 0;
+        input = check_input_device(g, colors_in, kMaxInputColor, &max_checked, s);
+        if (input != GC_OK && input != GC_ERR_IMPROPER_INPUT) return input;
     }
     RcCtrl h;
     ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
     if (ce != cudaSuccess) return cuda_status(ce);
     if (h.err & kErrBadGraph) return GC_ERR_BAD_GRAPH;
-    if (h.err & kErrImproper) return GC_ERR_IMPROPER_INPUT;
+    if (input != GC_OK) return input;
     // each graph's max input color sizes its rows of the (graph, color) tables
     std::vector<int32_t> gmax(ng, 0);
     if (trusted && max_in) {

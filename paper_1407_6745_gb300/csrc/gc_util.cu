@@ -44,6 +44,8 @@ struct ValArgs {
     int32_t* heavy;    // n
     int2* pieces;      // gc_validate: (row, piece index) of the rows beyond kValWarpDeg
     int64_t piece_cap;
+    int32_t max_allowed;  // a recoloring input: the row of a vertex whose color is outside [1, max_allowed]
+                          // is not read; 0: a validation, which reads every row
 };
 
 // Count of neighbors with v's color in this lane's stripe.
@@ -89,7 +91,8 @@ __device__ __forceinline__ void flush_presence(const ValArgs& a, uint32_t* s_pre
 
 // Light rows: kValG lanes per vertex; longer rows are listed for the next
 // pass, from the front of `heavy` up to kValWarpDeg entries, from the back
-// beyond.
+// beyond.  kInput: a recoloring input, with max_allowed.
+template <bool kInput>
 __global__ void __launch_bounds__(kBlock) k_validate(ValArgs a) {
     __shared__ uint32_t s_pres[kPresWords];
     for (int i = threadIdx.x; i < kPresWords; i += kBlock) s_pres[i] = 0u;
@@ -107,6 +110,7 @@ __global__ void __launch_bounds__(kBlock) k_validate(ValArgs a) {
         if (valid) {
             row_of(a.g, static_cast<int32_t>(v), beg, deg, &a.c->err);
             cv = a.colors[v];
+            if (kInput && (cv < 1 || cv > a.max_allowed)) deg = 0;
             heavy = deg > kValLightDeg;
         }
         int32_t same = same_color<1>(a, beg, heavy ? 0 : deg, cv, gl, kValG);
@@ -197,28 +201,66 @@ __global__ void __launch_bounds__(kBlock) k_count_bits(int64_t words, const uint
     warp_add(&c->distinct, s);
 }
 
+// The scratch of one validation and its two passes over the rows.
+struct ValRun {
+    Scratch sc, sp, shv, spc;
+    ValArgs a{};
+    gc_status start(const Graph& g, const int32_t* colors, int32_t max_allowed, const Tuning& t, cudaStream_t s) {
+        // pieces: at most one per kValPiece entries, plus one per row beyond kValWarpDeg
+        const int64_t piece_cap = g.nnz / kValPiece + g.nnz / kValWarpDeg + 1;
+        if (!sc.alloc(sizeof(ValCtrl), s) || !sp.alloc(kPresWords * 4, s) ||
+            !shv.alloc(static_cast<int64_t>(g.n) * 4, s) || !spc.alloc(piece_cap * sizeof(int2), s))
+            return GC_ERR_OOM;
+        a = ValArgs{g, colors, sc.as<ValCtrl>(), sp.as<uint32_t>(), shv.as<int32_t>(), spc.as<int2>(), piece_cap,
+                    max_allowed};
+        ValCtrl h;
+        std::memset(&h, 0, sizeof(h));
+        h.first_bad = LLONG_MAX;
+        cudaMemcpyAsync(a.c, &h, sizeof(h), cudaMemcpyHostToDevice, s);
+        cudaMemsetAsync(a.pres, 0, kPresWords * 4, s);
+        const bool input = max_allowed != 0;
+        const auto light = input ? k_validate<true> : k_validate<false>;
+        GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE, s, light<<<resident_grid(light, t), kBlock, 0, s>>>(a));
+        GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE_HEAVY, s,
+                  k_validate_heavy<<<resident_grid(k_validate_heavy, t), kBlock, 0, s>>>(a));
+        return GC_OK;
+    }
+};
+
+// The input of a recoloring call: proper (Sec. 1), colors in [1,
+// max_allowed].  The validation's passes (4 lanes a light row, longer rows
+// listed and cut into pieces) instead of a warp per row, which left one warp
+// walking each hub row: R-MAT 18 742 -> 70 us (of 4.75 ms -> 3.98 ms for
+// the call with 5 iterations).
+gc_status check_input_device(const Graph& g, const int32_t* colors, int32_t max_allowed, int32_t* max_color,
+                             cudaStream_t s) {
+    *max_color = 0;
+    if (g.n == 0) return GC_OK;
+    ValRun run;
+    const gc_status st = run.start(g, colors, max_allowed, current_tuning(), s);
+    if (st != GC_OK) return st;
+    ValCtrl h;
+    cudaError_t ce = cudaMemcpyAsync(&h, run.a.c, sizeof(h), cudaMemcpyDeviceToHost, s);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+    if (ce != cudaSuccess) return cuda_status(ce);
+    if (h.err & kErrBadGraph) return GC_ERR_BAD_GRAPH;
+    if (h.conflicts || h.uncolored || h.max_color > max_allowed) return GC_ERR_IMPROPER_INPUT;
+    *max_color = h.max_color;
+    return GC_OK;
+}
+
 gc_status validate_device(const Graph& g, const int32_t* colors, gc_validation* out,
                           cudaStream_t s) {
     std::memset(out, 0, sizeof(*out));
     out->first_bad_vertex = -1;
     if (g.n == 0) return GC_OK;
-    Scratch sc, sp, shv, spc;
-    // pieces: at most one per kValPiece entries, plus one per row beyond kValWarpDeg
-    const int64_t piece_cap = g.nnz / kValPiece + g.nnz / kValWarpDeg + 1;
-    if (!sc.alloc(sizeof(ValCtrl), s) || !sp.alloc(kPresWords * 4, s) || !shv.alloc(static_cast<int64_t>(g.n) * 4, s) ||
-        !spc.alloc(piece_cap * sizeof(int2), s))
-        return GC_ERR_OOM;
-    ValArgs a{g, colors, sc.as<ValCtrl>(), sp.as<uint32_t>(), shv.as<int32_t>(), spc.as<int2>(), piece_cap};
-    ValCtrl h;
-    std::memset(&h, 0, sizeof(h));
-    h.first_bad = LLONG_MAX;
-    cudaMemcpyAsync(a.c, &h, sizeof(h), cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(a.pres, 0, kPresWords * 4, s);
     const Tuning t = current_tuning();
     const int grid = persistent_grid(t);
-    GC_LAUNCH(KID_VALIDATE, s, k_validate<<<resident_grid(k_validate, t), kBlock, 0, s>>>(a));
-    GC_LAUNCH(KID_VALIDATE_HEAVY, s,
-              k_validate_heavy<<<resident_grid(k_validate_heavy, t), kBlock, 0, s>>>(a));
+    ValRun run;
+    const gc_status st = run.start(g, colors, 0, t, s);
+    if (st != GC_OK) return st;
+    const ValArgs& a = run.a;
+    ValCtrl h;
     GC_LAUNCH(KID_COUNT_BITS, s, k_count_bits<<<8, kBlock, 0, s>>>(kPresWords, a.pres, a.c));
     cudaError_t ce = cudaMemcpyAsync(&h, a.c, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);

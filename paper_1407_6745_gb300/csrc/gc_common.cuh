@@ -40,10 +40,6 @@ constexpr uint32_t kErrRoundLimit = 8u;
 // default is lifted so that every heavy row is a warp row (see color_impl).
 constexpr int32_t kDefaultWarpMaxDeg = 1024;
 constexpr int32_t kPullAllMaxDeg = 12288;
-// Default 2-lane threshold of the recoloring phase, and the one a recoloring
-// launch bound by its class chain takes instead (see recolor_device).
-constexpr int32_t kDefaultRcG2MaxDeg = 16;
-constexpr int32_t kChainRcG2MaxDeg = 8;
 
 // Scheduling thresholds (runtime; tuned per workload).
 struct Tuning {
@@ -254,6 +250,10 @@ __device__ __forceinline__ int4 ld_stream4(const void* ptr) {
     return r;
 }
 
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 __device__ __forceinline__ int32_t load_nbr(const Graph& g, int64_t e, uint32_t* err) {
     const int32_t u = ld_stream(g.idx + e);
     if (static_cast<uint32_t>(u) >= static_cast<uint32_t>(g.n)) {
@@ -457,12 +457,6 @@ __device__ __forceinline__ int32_t choose_warp(const Graph& g, int64_t beg, int3
         __syncwarp();
     }
 }
-
-// Single ids per lane per batch in the recoloring scans, in units of 4, per
-// group size (32/16/8/4/2 lanes).  (2 lanes: 4 ids each, rows of at most 16
-// entries; 8 in flight were measured 1-3 % slower on R-MAT, where most of
-// those rows have 1 or 2 entries.)
-template <int G> struct LanesUnroll { static constexpr int U = (G == 4) ? 2 : 1; };
 
 // ---------------------------------------------------------------------------
 // Tiles: a list is cut into segments (one bucket each); segment s holds

@@ -26,7 +26,8 @@
 // earlier than v" and "what color did u take".  Rows longer than
 // rc_warp_max_deg are cut into chunks of 256 neighbors handled by different
 // warps; the chunks OR their forbidden colors into a per-row bitmap and the
-// warp that finishes the last chunk picks the color.
+// warp that finishes the last chunk waits for the row's nearest classes and
+// picks the color.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -40,17 +41,37 @@ constexpr int kOrderThreads = 1024;
 constexpr int kShuffleSmem = 4096;
 constexpr int32_t kChunk = 256;   // neighbors per chunk of a split (heavy) row (measured best on R-MAT)
 
+// A chunk of a split row leaves its in-flight neighbors of the kNearClasses
+// classes before its own to the row's last chunk, through a list of kRowPend
+// entries a row (see defer_near; both measured there).
+constexpr int32_t kNearClasses = 2;
+constexpr int32_t kRowPend = 256;
+static_assert(kRowPend == 256, "8 entries per lane of the warp that takes them");
+
 // An isolated vertex (no neighbor) takes color 1 in every iteration and no
 // vertex waits on it: it gets bucket kIsoBucket, no list entry and no tile;
 // the scatter writes its color and it is counted in iso_cnt (class sizes
 // only).  (R-MAT 24: 47 % of the vertices; the recoloring kernel went from
 // 5.07 to 4.91 ms per iteration.)
-constexpr int kIsoBucket = 7;
+constexpr int kIsoBucket = 8;
 
-// Vertices (or, bucket 0, row chunks) per warp tile.
-__host__ __device__ constexpr int warp_tile(int b) {
-    return b <= 2 ? 1 : b == 3 ? 2 : b == 4 ? 4 : b == 5 ? 8 : 16;
+// The recoloring phase's buckets: those of bucket_of, and 7: rows of up to
+// kOneLaneDeg entries, a lane each (its gathers are one batch), where the
+// 2-lane threshold allows it.  Such rows are most of a skewed graph's and all
+// of a 7-point mesh's; with 2 lanes a warp tile held 16 of them (recoloring
+// launch, 2 lanes -> 1: 7-point mesh of 1 M vertices 53 -> 40 us, a batch of
+// 512 graphs 0.74 -> 0.66 ms, RMAT-Bad 22 0.56 -> 0.53, R-MAT 24 within 3 %).
+constexpr int kRcNB = 8;
+constexpr int32_t kOneLaneDeg = 8;
+__device__ __forceinline__ int rc_bucket_of(int32_t deg, const Tuning& t) {
+    if (deg == 0) return kIsoBucket;
+    return deg <= min(kOneLaneDeg, t.g2_max_deg) ? 7 : bucket_of(deg, 1, t);
 }
+
+// Lanes per row (log2) of a bucket's warp tiles, and rows (bucket 0: row
+// chunks) per tile.
+__host__ __device__ constexpr int lanes_log2(int b) { return b < 2 ? 5 : 7 - b; }
+__host__ __device__ constexpr int warp_tile(int b) { return 32 >> lanes_log2(b); }
 
 struct RcCtrl {
     int32_t k;            // present classes this iteration
@@ -74,7 +95,7 @@ struct RcArgs {
     const int32_t* old_c;
     int32_t* new_c;
     uint8_t* bucket;
-    int32_t* cls_cnt;     // (cap + 1) * kNB vertices per (class, bucket)
+    int32_t* cls_cnt;     // (cap + 1) * kRcNB vertices per (class, bucket)
     int32_t* cls_units;   // cap + 1: row chunks of the bucket-0 vertices per class
     int32_t* nxt_cnt;     // the same two histograms of the new colors, filled by
     int32_t* nxt_units;   //   the recoloring kernel for the next iteration
@@ -85,9 +106,9 @@ struct RcArgs {
     int32_t* order;       // cap + 1 (class order, colors)
     int32_t* jtab;        // cap + 1 (shuffle indices)
     int32_t* rank_of;     // cap + 1
-    int32_t* seg_start;   // (cap + 1) * kNB + 1, in list entries
-    int32_t* tile_prefix; // (cap + 1) * kNB + 1, in warp tiles
-    int32_t* fill;        // (cap + 1) * kNB
+    int32_t* seg_start;   // (cap + 1) * kRcNB + 1, in list entries
+    int32_t* tile_prefix; // (cap + 1) * kRcNB + 1, in warp tiles
+    int32_t* fill;        // (cap + 1) * kRcNB
     WorkItem* list;       // list entries in class-major order
     int32_t* ncolors;     // iterations + 1
     int32_t* hub_v;       // split rows: vertex, chunk count, finished chunks,
@@ -95,6 +116,8 @@ struct RcArgs {
     int32_t* hub_done;
     uint32_t* hub_bm;
     int32_t hub_words;
+    int32_t* hub_pcnt;    // neighbors left to the row's last chunk: count, kRowPend entries
+    int32_t* hub_pend;
     RcCtrl* ctrl;
     // batches (nullptr for one graph): graph of every vertex, descriptors,
     // and the start of each graph's colors in the (graph, color) tables
@@ -104,6 +127,7 @@ struct RcArgs {
     const int64_t* cls_base;
     int32_t ngraphs;
     int32_t fuse_hist;    // 1: the recoloring kernel fills nxt_cnt (one graph only)
+    int32_t scatter_segs; // segments the scatter counts in shared memory
     int32_t hist_smem;    // entries of its dynamic shared-memory histogram (0: global)
     int32_t* gpresent;    // per (graph, color): present colors, sizes, order, shuffle
     int32_t* gpsize;
@@ -140,7 +164,7 @@ __global__ void __launch_bounds__(kBlock) k_rc_bucket(RcArgs a) {
         int32_t deg;
         row_of(a.g, static_cast<int32_t>(i), beg, deg, &a.ctrl->err);
         my_max = max(my_max, deg);
-        const int b = deg == 0 ? kIsoBucket : bucket_of(deg, 1, a.tune);
+        const int b = rc_bucket_of(deg, a.tune);
         a.bucket[i] = static_cast<uint8_t>(b);
         heavy += b == 0;
     }
@@ -173,7 +197,7 @@ constexpr int kIsoSmem = 1024;  // isolated vertices per class, colors below thi
 __global__ void __launch_bounds__(kBlock) k_rc_hist(RcArgs a) {
     __shared__ int32_t sh[kHistSmem];
     __shared__ int32_t s_iso[kIsoSmem];
-    const int32_t entries = (a.cap + 1) * kNB;
+    const int32_t entries = (a.cap + 1) * kRcNB;
     const bool local = entries <= kHistSmem;
     for (int i = threadIdx.x; i < kIsoSmem; i += kBlock) s_iso[i] = 0;
     if (local)
@@ -192,7 +216,7 @@ __global__ void __launch_bounds__(kBlock) k_rc_hist(RcArgs a) {
             else atomicAdd(&a.iso_cnt[c], 1);
             continue;
         }
-        const int32_t key = c * kNB + b;
+        const int32_t key = c * kRcNB + b;
         const unsigned act = __activemask();
         const unsigned peers = __match_any_sync(act, key);
         if (lane_id() == __ffs(peers) - 1) {
@@ -244,18 +268,18 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t x, OrderShared& 
 }
 
 // Segment starts (list entries) and tile prefix (warp tiles) of the k
-// ranks x kNB buckets, class-major; units(sg) gives a segment's entries.
+// ranks x kRcNB buckets, class-major; units(sg) gives a segment's entries.
 template <class Units>
 __device__ __forceinline__ void build_segments(const RcArgs& a, int32_t k, OrderShared& s, Units&& units) {
     const int t = threadIdx.x;
-    const int32_t nseg = k * kNB;
+    const int32_t nseg = k * kRcNB;
     int32_t vbase = 0, tbase = 0;
     unsigned long long best = 0;  // (entries << 32) | segment, over the single-entry buckets
     for (int32_t s0 = 0; s0 < nseg; s0 += kOrderThreads) {
         const int32_t sg = s0 + t;
         int32_t cnt = 0, tiles = 0;
         if (sg < nseg) {
-            const int b = sg % kNB;
+            const int b = sg % kRcNB;
             cnt = units(sg);
             tiles = (cnt + warp_tile(b) - 1) / warp_tile(b);
             a.fill[sg] = 0;
@@ -301,7 +325,7 @@ __global__ void __launch_bounds__(kOrderThreads) k_rc_order(RcArgs a) {
         const int32_t c = c0 + t;
         int32_t size = 0;
         if (c <= a.cap) {
-            for (int b = 0; b < kNB; ++b) size += a.cls_cnt[c * kNB + b];
+            for (int b = 0; b < kRcNB; ++b) size += a.cls_cnt[c * kRcNB + b];
             size += a.iso_cnt[c];
         }
         int32_t total;
@@ -360,9 +384,9 @@ __global__ void __launch_bounds__(kOrderThreads) k_rc_order(RcArgs a) {
     // list entries and in warp tiles
     for (int32_t p = t; p < k; p += kOrderThreads) a.rank_of[a.order[p]] = p;
     build_segments(a, k, s, [&](int32_t sg) {
-        const int b = sg % kNB;
-        const int32_t c = a.order[sg / kNB];
-        return b == 0 ? a.cls_units[c] : a.cls_cnt[c * kNB + b];
+        const int b = sg % kRcNB;
+        const int32_t c = a.order[sg / kRcNB];
+        return b == 0 ? a.cls_units[c] : a.cls_cnt[c * kRcNB + b];
     });
 }
 
@@ -374,7 +398,7 @@ __global__ void __launch_bounds__(kOrderThreads) k_rc_order(RcArgs a) {
 // a split-row slot.  (Order inside a segment is free: a class is an
 // independent set.)
 // ---------------------------------------------------------------------------
-constexpr int kScatterSegs = 4096;
+constexpr int kScatterSegs = 6144;  // segments counted in (dynamic) shared memory: 48 KB
 
 struct ScatterInfo {
     int32_t sg;
@@ -405,7 +429,7 @@ __device__ __forceinline__ ScatterInfo scatter_info(const RcArgs& a, int32_t v) 
         si.deg = 0;
         return si;
     }
-    si.sg = a.rank_of[key] * kNB + b;
+    si.sg = a.rank_of[key] * kRcNB + b;
     row_of(a.g, v, si.beg, si.deg, &a.ctrl->err);
     si.units = b == 0 ? chunks_of(si.deg) : 1;
     return si;
@@ -423,8 +447,10 @@ __device__ __forceinline__ void place_unlisted(const RcArgs& a, int32_t v, int32
 }
 
 // The isolated vertices placed by a block: counted in the next iteration's
-// class 1 (one graph), and the iteration's max color is at least 1.
-__device__ __forceinline__ void flush_isolated(const RcArgs& a, int32_t iso) {
+// class 1 (one graph), and the iteration's max color is at least 1.  The
+// entries of the others' rows are the ones this iteration examines.
+__device__ __forceinline__ void flush_placed(const RcArgs& a, int32_t iso, unsigned long long edges) {
+    warp_add(&a.ctrl->edges, edges);
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) iso += __shfl_xor_sync(kFull, iso, d);
     if (lane_id() == 0 && iso > 0) {
@@ -434,15 +460,16 @@ __device__ __forceinline__ void flush_isolated(const RcArgs& a, int32_t iso) {
 }
 
 __device__ __forceinline__ void place(const RcArgs& a, int32_t v, const ScatterInfo& si, int32_t pos) {
-    a.new_c[v] = -(si.sg / kNB + 1);
-    if (si.sg % kNB != 0) {
+    a.new_c[v] = -(si.sg / kRcNB + 1);
+    if (si.sg % kRcNB != 0) {
         store_item(a.list + pos, si.beg, v, si.deg);
         return;
     }
     const int32_t slot = atomicAdd(&a.ctrl->hub_next, 1);
     a.hub_v[slot] = v;
     a.hub_nch[slot] = si.units;
-    a.hub_done[slot] = 0;
+    a.hub_pcnt[slot] = 0;
+    a.hub_done[slot] = -si.units;  // counted up to 0 by the chunks
     for (int32_t w = 0; w < a.hub_words; ++w) a.hub_bm[static_cast<int64_t>(slot) * a.hub_words + w] = 0u;
     for (int32_t c = 0; c < si.units; ++c) {
         const int32_t len = min(kChunk, si.deg - c * kChunk);
@@ -479,17 +506,18 @@ __device__ __forceinline__ int32_t hot_or_own(int32_t* s_cnt, int32_t sg, int32_
 }
 
 __global__ void __launch_bounds__(kBlock) k_rc_scatter(RcArgs a) {
-    __shared__ int32_t s_cnt[kScatterSegs];
-    __shared__ int32_t s_base[kScatterSegs];
+    extern __shared__ int32_t s_cnt[];  // a.scatter_segs counts, then as many bases
+    int32_t* const s_base = s_cnt + a.scatter_segs;
     if (a.ctrl->err & (kErrImproper | kErrBadGraph)) return;
-    const int32_t nseg = a.ctrl->k * kNB;
+    const int32_t nseg = a.ctrl->k * kRcNB;
     const int64_t chunk = (static_cast<int64_t>(a.g.n) + gridDim.x - 1) / gridDim.x;
     const int64_t lo = blockIdx.x * chunk;
     const int64_t hi = a.g.n < lo + chunk ? a.g.n : lo + chunk;
-    if (nseg > kScatterSegs) {
+    if (nseg > a.scatter_segs) {
         // many classes: global atomics
         int32_t iso = 0;
-        for (int64_t i0 = lo; i0 < hi; i0 += kBlock) {  // whole warps: flush_isolated shuffles
+        unsigned long long edges = 0;
+        for (int64_t i0 = lo; i0 < hi; i0 += kBlock) {  // whole warps: flush_placed shuffles
             const int64_t i = i0 + threadIdx.x;
             if (i >= hi) continue;
             const int32_t v = static_cast<int32_t>(i);
@@ -498,10 +526,11 @@ __global__ void __launch_bounds__(kBlock) k_rc_scatter(RcArgs a) {
                 place_unlisted(a, v, si.sg, iso);
                 continue;
             }
+            edges += static_cast<unsigned long long>(si.deg);
             const int32_t off = reserve(a.fill, si);
             place(a, v, si, a.seg_start[si.sg] + off);
         }
-        flush_isolated(a, iso);
+        flush_placed(a, iso, edges);
         return;
     }
     for (int i = threadIdx.x; i < nseg; i += kBlock) s_cnt[i] = 0;
@@ -522,7 +551,7 @@ __global__ void __launch_bounds__(kBlock) k_rc_scatter(RcArgs a) {
             if (a.iteration >= a.desc[gi].iterations) continue;
             key += a.cls_base[gi];
         }
-        const int32_t sg = a.rank_of[key] * kNB + b;
+        const int32_t sg = a.rank_of[key] * kRcNB + b;
         int32_t units = 1;
         if (b == 0) {
             int64_t beg;
@@ -540,6 +569,7 @@ __global__ void __launch_bounds__(kBlock) k_rc_scatter(RcArgs a) {
     }
     __syncthreads();
     int32_t iso = 0;
+    unsigned long long edges = 0;
     for (int64_t i = lo + threadIdx.x; i < hi; i += kBlock) {
         const int32_t v = static_cast<int32_t>(i);
         const ScatterInfo si = scatter_info(a, v);
@@ -547,10 +577,11 @@ __global__ void __launch_bounds__(kBlock) k_rc_scatter(RcArgs a) {
             place_unlisted(a, v, si.sg, iso);
             continue;
         }
+        edges += static_cast<unsigned long long>(si.deg);
         const int32_t off = hot_or_own(s_cnt, si.sg, si.units, hot);
         place(a, v, si, s_base[si.sg] + off);
     }
-    flush_isolated(a, iso);
+    flush_placed(a, iso, edges);
 }
 
 // ---------------------------------------------------------------------------
@@ -612,7 +643,7 @@ struct RecolorFetch {
 // the same (color, bucket) are merged into one atomic (most vertices of a
 // skewed graph take the same few colors, and unmerged adds to one global
 // counter serialise in L2).
-constexpr int kRcHistSmem = 6144;
+constexpr int kRcHistSmem = 8192;
 
 struct NextHist {
     int32_t* sh;     // nullptr: count in global memory
@@ -621,7 +652,7 @@ struct NextHist {
     int32_t cap;
     __device__ __forceinline__ void add(int32_t c, int b, int32_t chunks) const {
         if (c < 1 || c > cap) return;
-        const int32_t key = c * kNB + b;
+        const int32_t key = c * kRcNB + b;
         if (sh) {
             atomicAdd(&sh[key], 1);
         } else {
@@ -633,138 +664,453 @@ struct NextHist {
     }
 };
 
-template <int G, bool kDataflow>
-__device__ __forceinline__ void recolor_group_tile(const RcArgs& a, const RecolorFetch<kDataflow>& f,
-                                                   const NextHist& nh, int b, int32_t first,
-                                                   int32_t last, int32_t& my_max,
-                                                   unsigned long long& edges) {
-    const int gi = lane_id() / G, gl = lane_id() % G;
-    const int32_t k = first + gi;
-    const bool valid = k < last;
-    WorkItem it{0, 0, 0};
-    if (valid) it = load_item(a.list + k);
-    const int32_t c = choose_reg<G, LanesUnroll<G>::U>(a.g, it.beg, it.deg, gl, 0u, f, &a.ctrl->err);
-    if (valid && gl == 0) {
-        st_relaxed(a.new_c + it.v, c);
-        my_max = max(my_max, c);
-        edges += static_cast<unsigned long long>(it.deg);
-        nh.add(c, b, 0);
+// A neighbor that is not there: later than every class.
+constexpr int32_t kNoNeighbor = -0x7fffffff;
+
+// A neighbor that was read as -(rank + 1), of a class rank below `horizon`:
+// earlier and still in flight.  (A color, 1 or more, gives a huge number.)
+__device__ __forceinline__ bool in_flight(int32_t x, int32_t horizon) {
+    return static_cast<uint32_t>(~x) < static_cast<uint32_t>(horizon);
+}
+
+// Colors of up to 8 neighbors per lane (u[i] < 0: none), all loads in flight
+// together.
+template <bool kDataflow>
+__device__ __forceinline__ void load8(const RecolorFetch<kDataflow>& f, const int32_t (&u)[8], int32_t (&x)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        x[i] = kNoNeighbor;
+        if (u[i] >= 0) x[i] = f.raw(u[i]);
     }
 }
 
-// One chunk of a split row: the chunk's forbidden colors are OR-ed into the
-// row's bitmap; the warp finishing the last chunk picks the First-Fit color.
-//
-// Ordering: the lanes' OR-s into the row's bitmap precede a warp barrier,
-// and lane 0 then counts the chunk with one acquire-release atomic.  Its
-// release covers the warp's OR-s (the barrier orders them before it); the
-// last chunk's acquire reads the end of the counter's chain of increments,
-// so it sees every chunk's OR-s, and the barrier after it orders the lanes'
-// bitmap reads after it.  (One atomic by one lane instead of a fence by all
-// 32: R-MAT 24 4.86 -> 4.37 ms per iteration, RXF-4 5.17 -> 4.62 ms.)
+// Waits until no neighbor of a class before `horizon` is in flight (bounded;
+// once any wait of the launch has run out, every other one gives up at once,
+// so a launch never spends more than about one spin_limit in waits).  Each
+// lane polls its pending neighbor of the latest class; when it is there, the
+// others mostly are too and all are read again.  A poll is one load and a
+// few instructions per lane, so it does not back off: with sleeps of up to
+// 256 ns the class chain (which every poll is a link of) was 10-20 % slower
+// (R-MAT 22 1.33 -> 1.27 ms per iteration, R-MAT 18 0.51 -> 0.48), and with
+// all of a lane's pending neighbors in every poll R-MAT 24 lost 4 %.  The
+// whole warp calls it.
 template <bool kDataflow>
-__device__ __forceinline__ void recolor_chunk(const RcArgs& a, const RecolorFetch<kDataflow>& f,
-                                              const NextHist& nh, const WorkItem& it, uint32_t* bm,
-                                              int32_t& my_max, unsigned long long& edges) {
+__device__ __forceinline__ void wait8(const RecolorFetch<kDataflow>& f, const int32_t (&u)[8], int32_t (&x)[8],
+                                      int32_t horizon) {
+    if (!kDataflow) return;
+    for (int32_t it = 0;;) {
+        int32_t q = -1, r = -1;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (in_flight(x[i], horizon) && ~x[i] > r) {
+                r = ~x[i];
+                q = u[i];
+            }
+        bool there = q < 0;
+        if (__all_sync(kFull, there)) return;
+        for (;; ++it) {
+            if (it >= f.spin_limit) {
+                if (!there) atomicOr(f.err, kErrTimeout);
+                return;
+            }
+            if (!there) there = ld_relaxed(f.new_c + q) > 0;
+            if (__all_sync(kFull, there)) break;
+            // (a vote: a lane that left alone would be missed by the others)
+            if ((it & 63) == 0 &&
+                __any_sync(kFull, ld_relaxed(reinterpret_cast<const int32_t*>(f.err)) & static_cast<int32_t>(kErrTimeout)))
+                return;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (in_flight(x[i], f.p)) x[i] = ld_relaxed(f.new_c + u[i]);
+    }
+}
+
+// 1 << d, 0 for d outside [0, 32) (the shift clamps).
+__device__ __forceinline__ uint32_t bit_or_none(int32_t d) {
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(d));
+    return r;
+}
+
+// What a warp keeps in shared memory: the work items of its current and next
+// tile, the ids of its next tile (kStageIds over the tile's rows), the two
+// tiles' segments and entry counts, and a bitmap of forbidden colors.
+constexpr int kStageIds = 384;
+struct __align__(16) WarpStage {
+    WorkItem item[2][32];
+    int32_t ids[kStageIds];
+    int4 meta[2];  // segment, entries
+    uint32_t bm[kWarpBitmapWords];
+    uint32_t have[kWarpBitmapWords];  // a chunk's row: its merged bits, as read with the chunk
+    int32_t win_t[32], win_s[32];     // tile prefix and start of the segments sought next
+};
+
+__device__ __forceinline__ void stage_copy16(void* smem, const void* gmem, int bytes) {
+    const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;" ::"r"(sa), "l"(gmem), "r"(bytes),
+                 "l"(policy_evict_first())
+                 : "memory");
+}
+
+__device__ __forceinline__ void stage_copy4(void* smem, const void* gmem) {
+    const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+// The ids that the tile's lanes take first (8 per lane: the whole row except
+// for 4-lane rows above 32 entries and warp rows above 256), as aligned
+// 16-byte pieces, into each row's part of the stage.
+__device__ __forceinline__ void stage_ids(const RcArgs& a, WarpStage& w, int slot) {
+    if (!a.g.vec) return;
+    const int4 m = w.meta[slot];
+    const int lg = lanes_log2(m.x % kRcNB), G = 1 << lg;
+    const int gi = lane_id() >> lg, gl = lane_id() & (G - 1);
+    if (gi >= m.y) return;
+    const WorkItem it = w.item[slot][gi];
+    int32_t* dst = w.ids + gi * (kStageIds >> (5 - lg));
+    const int64_t e0 = it.beg & ~static_cast<int64_t>(3);
+    const int32_t nch = (static_cast<int32_t>(it.beg & 3) + min(it.deg, 8 << lg) + 3) >> 2;
+    for (int32_t c = gl; c < nch; c += G) {
+        const int64_t e = e0 + 4 * static_cast<int64_t>(c);
+        stage_copy16(dst + 4 * c, a.g.idx + e, static_cast<int>(min(static_cast<int64_t>(16), 4 * (a.g.nnz - e))));
+    }
+}
+
+// Skewed graphs have hundreds of classes that hold hub rows only, and a
+// hub waits for hubs of the class just before its own: the launch is a chain
+// of as many links, each the time from one hub's color to the next one's.
+// Were every chunk to wait for its own neighbors, a link would be poll,
+// merge into the row's bitmap, counting atomic (with its fence), bitmap
+// read and pick, about 4 us.  Instead a chunk waits only for classes more
+// than kNearClasses before its own, merges and counts at once, and leaves the
+// nearer neighbors still in flight to the row's last chunk: that one holds the
+// merged bitmap while it polls them, so a link is poll, pick and store.  A
+// chunk that finds the row's list full waits for its own.  (ms per iteration,
+// no deferral / 1 / 2 / 4 classes: R-MAT 22 1.30 / 1.10 / 0.98 / 1.00, R-MAT 18
+// 0.50 / 0.40 / 0.34 / 0.33, RMAT-Bad 22 0.61 / 0.58 / 0.56 / 0.55, R-MAT 24
+// 3.43 / 3.30 / 3.21 / 3.27; a list of 128 entries overflowed: R-MAT 24 4.3.)
+//
+// Ends: the smallest-class unfinished row has all its tiles dealt before any
+// that waits for it, and their owners can only be waiting for rows of still
+// smaller classes.
+__device__ __forceinline__ void defer_near(const RcArgs& a, const RecolorFetch<true>& f, int32_t slot,
+                                           const int32_t (&u)[8], int32_t (&x)[8]) {
     const int l = lane_id();
-    const int32_t slot = -it.v - 1;
-    uint32_t* hb = a.hub_bm + static_cast<int64_t>(slot) * a.hub_words;
-    // written by the scatter (an earlier launch): read-only here, loaded early
-    const int32_t nch = l == 0 ? __ldg(a.hub_nch + slot) : 0;
-    const int32_t hv = l == 0 ? __ldg(a.hub_v + slot) : 0;
-    static_assert(kWarpBitmapWords == 64, "two bitmap words per lane");
-    for (int32_t w0 = 0; w0 < a.hub_words; w0 += kWarpBitmapWords) {
-        // The row's bits already merged (read before the scan, in the shadow
-        // of its loads): a word adding no new bit is not merged again.  Bits
-        // are only ever set during the launch, so skipping is exact; the
-        // chunks of one row otherwise all send atomics to the same few words
-        // (R-MAT 24: 4.91 -> 4.84 ms per iteration).
-        const uint32_t have0 = w0 + l < a.hub_words ? __ldcg(hb + w0 + l) : 0u;
-        const uint32_t have1 = w0 + l + 32 < a.hub_words ? __ldcg(hb + w0 + l + 32) : 0u;
-        bm[l] = 0u;
-        bm[l + 32] = 0u;
-        __syncwarp();
-        const int32_t base = w0 * 32 + 1;
-        scan_row<2>(a.g, it.beg, it.deg, l, 32, f,
-                    [&](int32_t c) {
-                        const uint32_t d = static_cast<uint32_t>(c - base);
-                        if (c > 0 && d < 32u * kWarpBitmapWords) atomicOr(&bm[d >> 5], 1u << (d & 31));
-                    },
-                    &a.ctrl->err);
-        __syncwarp();
-        if (w0 + l < a.hub_words && (bm[l] & ~have0)) atomicOr(&hb[w0 + l], bm[l]);
-        if (w0 + l + 32 < a.hub_words && (bm[l + 32] & ~have1)) atomicOr(&hb[w0 + l + 32], bm[l + 32]);
+    uint32_t mine = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mine += in_flight(x[i], f.p);
+    const uint32_t incl = warp_inclusive_scan(mine);
+    const int32_t total = static_cast<int32_t>(__shfl_sync(kFull, incl, 31));
+    if (total == 0) return;
+    int32_t base = 0;
+    if (l == 0) base = atomicAdd(a.hub_pcnt + slot, total);
+    base = __shfl_sync(kFull, base, 0);
+    int32_t* pend = a.hub_pend + static_cast<int64_t>(slot) * kRowPend;
+    int32_t pos = base + static_cast<int32_t>(incl - mine);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (in_flight(x[i], f.p)) {
+            if (pos < kRowPend) pend[pos] = u[i];
+            ++pos;
+        }
+    if (base + total > kRowPend) wait8<true>(f, u, x, f.p);
+}
+__device__ __forceinline__ void defer_near(const RcArgs&, const RecolorFetch<false>&, int32_t, const int32_t (&)[8],
+                                           int32_t (&)[8]) {}
+
+// One warp tile whose items and ids are staged: its rows' lanes gather the
+// neighbors' colors 8 at a time.  A row of the lane buckets (2..6) keeps its
+// forbidden colors in 64 register bits; a warp row or a chunk of a split row
+// keeps colors 1..32 in a register (most neighbors of a hub carry one of the
+// lowest colors, and as shared atomics they would all hit one word) and the
+// others in a shared bitmap.
+//
+// A chunk's forbidden colors are OR-ed into the row's bitmap; the warp
+// finishing the last chunk picks the First-Fit color.  Ordering: the lanes'
+// OR-s into the row's bitmap precede a warp barrier, and lane 0 then counts
+// the chunk with one acquire-release atomic.  Its release covers the warp's
+// OR-s (the barrier orders them before it); the last chunk's acquire reads
+// the end of the counter's chain of increments, so it sees every chunk's
+// OR-s, and the barrier after it orders the lanes' bitmap reads after it.
+template <bool kDataflow, class Ahead>
+__device__ __forceinline__ void recolor_tile(const RcArgs& a, const NextHist& nh, WarpStage& w, int slot, bool cached,
+                                             int32_t& my_max, Ahead&& stage_ahead) {
+    const int l = lane_id();
+    const int4 m = w.meta[slot];
+    const int32_t p = m.x / kRcNB;
+    const int b = m.x % kRcNB;
+    const int lg = lanes_log2(b), G = 1 << lg;
+    const int gi = l >> lg, gl = l & (G - 1);
+    const bool valid = gi < m.y;
+    WorkItem it{0, 0, 0};
+    if (valid) it = w.item[slot][gi];
+    const RecolorFetch<kDataflow> f{a.new_c, p, a.tune.spin_limit, &a.ctrl->err, cached};
+
+    int32_t u[8], x[8];
+    bool bad = false;
+    {
+        const int32_t* ids = w.ids + gi * (kStageIds >> (5 - lg)) + (it.beg & 3);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int32_t k = gl + (i << lg);
+            u[i] = -1;
+            if (k < it.deg) {
+                u[i] = a.g.vec ? ids[k] : ld_stream(a.g.idx + it.beg + k);
+                if (static_cast<uint32_t>(u[i]) >= static_cast<uint32_t>(a.g.n)) {
+                    bad = true;
+                    u[i] = -1;
+                }
+            }
+        }
+    }
+    __syncwarp();   // the slot and the staged ids are read: the next tiles' may land there
+    stage_ahead();
+
+    uint32_t lo = 0, hi = 0;
+    if (b < 2) {
+        w.bm[l] = 0u;
+        w.bm[l + 32] = 0u;
+        if (b == 0) {
+            // the row's bits already merged (read in the shadow of the gathers): a word
+            // adding no new bit is not merged again; bits are only ever set during the launch
+            if (4 * l < min(a.hub_words, kWarpBitmapWords))
+                stage_copy16(&w.have[4 * l], a.hub_bm + static_cast<int64_t>(-it.v - 1) * a.hub_words + 4 * l, 16);
+            cp_async_commit();
+        }
         __syncwarp();
     }
-    if (l == 0) edges += static_cast<unsigned long long>(it.deg);
+    for (int32_t k0 = 0;;) {
+        load8<kDataflow>(f, u, x);
+        wait8<kDataflow>(f, u, x, b == 0 ? max(p - kNearClasses, 0) : p);
+        if (b == 0 && kDataflow) defer_near(a, f, -it.v - 1, u, x);
+        if (b >= 2) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                lo |= bit_or_none(x[i] - 1);
+                hi |= bit_or_none(x[i] - 33);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                lo |= bit_or_none(x[i] - 1);
+                if (x[i] > 32 && x[i] <= 32 * kWarpBitmapWords) atomicOr(&w.bm[(x[i] - 1) >> 5], 1u << ((x[i] - 1) & 31));
+            }
+        }
+        k0 += 8 << lg;
+        if (!__any_sync(kFull, k0 < it.deg)) break;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {  // longer rows: the rest is not staged
+            const int32_t k = k0 + gl + (i << lg);
+            u[i] = k < it.deg ? load_nbr(a.g, it.beg + k, &a.ctrl->err) : -1;
+        }
+    }
+    if (bad) atomicOr(&a.ctrl->err, kErrBadGraph);
+
+    if (b >= 2) {
+        for (int d = G >> 1; d >= 1; d >>= 1) {
+            lo |= __shfl_xor_sync(kFull, lo, d);
+            hi |= __shfl_xor_sync(kFull, hi, d);
+        }
+        if (valid && gl == 0) {
+            const int32_t c = ~lo ? __ffs(~lo) : 32 + __ffs(~hi);  // a free one: deg < 64
+            st_relaxed(a.new_c + it.v, c);
+            my_max = max(my_max, c);
+            nh.add(c, b, 0);
+        }
+        return;
+    }
+    lo = __reduce_or_sync(kFull, lo);
+    __syncwarp();
+    uint32_t w0 = w.bm[l], w1 = w.bm[l + 32];
+    if (l == 0) w0 |= lo;
+    if (b == 1) {
+        const uint32_t any0 = __ballot_sync(kFull, ~w0 != 0u), any1 = __ballot_sync(kFull, ~w1 != 0u);
+        int32_t c;
+        if (any0 | any1) {
+            const int src = __ffs(any0 ? any0 : any1) - 1;
+            const uint32_t fw = __shfl_sync(kFull, ~(any0 ? w0 : w1), src);
+            c = ((any0 ? 0 : 32) + src) * 32 + __ffs(fw);
+        } else {  // every color of the window is taken
+            c = choose_warp<4>(a.g, it.beg, it.deg, 0u, f, w.bm, &a.ctrl->err);
+        }
+        if (l == 0) {
+            st_relaxed(a.new_c + it.v, c);
+            my_max = max(my_max, c);
+            nh.add(c, 1, 0);
+        }
+        return;
+    }
+    static_assert(kWarpBitmapWords == 64, "two bitmap words per lane");
+    uint32_t* hb = a.hub_bm + static_cast<int64_t>(-it.v - 1) * a.hub_words;
+    cp_async_wait<0>();  // (the next tiles' copies are in the same queue: they had the gathers' time)
+    __syncwarp();
+    if (l < a.hub_words && (w0 & ~w.have[l])) atomicOr(&hb[l], w0);
+    if (l + 32 < a.hub_words && (w1 & ~w.have[l + 32])) atomicOr(&hb[l + 32], w1);
+    for (int32_t s0 = kWarpBitmapWords; s0 < a.hub_words; s0 += kWarpBitmapWords) {  // colors beyond the first window
+        __syncwarp();
+        w.bm[l] = 0u;
+        w.bm[l + 32] = 0u;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int32_t d = x[i] - 1 - 32 * s0;
+            if (x[i] > 0 && d >= 0 && d < 32 * kWarpBitmapWords) atomicOr(&w.bm[d >> 5], 1u << (d & 31));
+        }
+        __syncwarp();
+        if (s0 + l < a.hub_words && w.bm[l]) atomicOr(&hb[s0 + l], w.bm[l]);
+        if (s0 + l + 32 < a.hub_words && w.bm[l + 32]) atomicOr(&hb[s0 + l + 32], w.bm[l + 32]);
+    }
     __syncwarp();
     int last = 0;
-    if (l == 0) last = add_acq_rel(a.hub_done + slot) == nch - 1;
+    if (l == 0) last = add_acq_rel(a.hub_done - it.v - 1) == -1;  // counts up from minus the chunks
     last = __shfl_sync(kFull, last, 0);
     __syncwarp();
     if (!last) return;
-    // First Fit over the merged bitmap: the first clear bit
-    for (int32_t w0 = 0; w0 < a.hub_words; w0 += 32) {
-        const int32_t i = w0 + l;
-        const uint32_t free_bits = i < a.hub_words ? ~__ldcg(hb + i) : 0u;
-        const uint32_t any = __ballot_sync(kFull, free_bits != 0u);
-        if (any) {
-            const int src = __ffs(any) - 1;
-            const uint32_t fw = __shfl_sync(kFull, free_bits, src);
-            const int32_t c = (w0 + src) * 32 + __ffs(fw);
+    // The neighbors left to this chunk, then First Fit over the merged bitmap.
+    // Everything it takes is loaded at once (the list's words past its count
+    // are dropped); with one window w.bm still holds this chunk's bits, which
+    // are the row's too.
+    uint32_t h0 = l < a.hub_words ? __ldcg(hb + l) : ~0u;
+    uint32_t h1 = l + 32 < a.hub_words ? __ldcg(hb + l + 32) : ~0u;
+    const int32_t hv = l == 0 ? __ldg(a.hub_v - it.v - 1) : 0;
+    int32_t left = 0;
+    if (kDataflow) {
+        const int32_t* pend = a.hub_pend + static_cast<int64_t>(-it.v - 1) * kRowPend;
+        left = __ldcg(a.hub_pcnt - it.v - 1);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) u[i] = __ldcg(pend + l + 32 * i);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (l + 32 * i >= left) u[i] = -1;
+        if (left > 0) {
+            load8<kDataflow>(f, u, x);
+            wait8<kDataflow>(f, u, x, p);
+        }
+    }
+    for (int32_t s0 = 0; s0 < a.hub_words; s0 += kWarpBitmapWords) {
+        if (a.hub_words > kWarpBitmapWords) {
+            __syncwarp();
+            w.bm[l] = 0u;
+            w.bm[l + 32] = 0u;
+            __syncwarp();
+        }
+        if (left > 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int32_t d = x[i] - 1 - 32 * s0;
+                if (x[i] > 0 && d >= 0 && d < 32 * kWarpBitmapWords) atomicOr(&w.bm[d >> 5], 1u << (d & 31));
+            }
+        }
+        __syncwarp();
+        if (s0 > 0) {
+            h0 = s0 + l < a.hub_words ? __ldcg(hb + s0 + l) : ~0u;
+            h1 = s0 + l + 32 < a.hub_words ? __ldcg(hb + s0 + l + 32) : ~0u;
+        }
+        const uint32_t f0 = ~(h0 | w.bm[l]), f1 = ~(h1 | w.bm[l + 32]);
+        const uint32_t any0 = __ballot_sync(kFull, f0 != 0u), any1 = __ballot_sync(kFull, f1 != 0u);
+        if (any0 | any1) {
+            const int src = __ffs(any0 ? any0 : any1) - 1;
+            const uint32_t fw = __shfl_sync(kFull, any0 ? f0 : f1, src);
+            const int32_t c = (s0 + (any0 ? 0 : 32) + src) * 32 + __ffs(fw);
             if (l == 0) {
                 st_relaxed(a.new_c + hv, c);
                 my_max = max(my_max, c);
-                nh.add(c, 0, nch);
+                nh.add(c, 0, __ldg(a.hub_nch - it.v - 1));
             }
             return;
         }
     }
 }
 
+// A warp's tiles t, t + step, ... below `end`, in order.  A tile is reached
+// through four dependent reads (segment table, work items, ids, colors); the
+// launch is bound by that latency (R-MAT 22 before: 5 % of DRAM, 30 % of the
+// L1 rate, long-scoreboard stalls), so the first three run ahead: while a
+// tile's colors are gathered, the ids of the next tile and the items of the
+// one after are on their way to shared memory (cp.async, no registers) and
+// the segment table's words for the third.  Together with one code path for
+// all buckets, branch-free marks and 4 blocks per SM (64 registers, none
+// spilled; a fifth block's 48 spilled 144 bytes: R-MAT 24 4.29 ms, stencil
+// 0.293) an iteration takes, before -> after: 27-point stencil 128^3 315 ->
+// 254 us (its 53.6 M scattered gathers alone take about 190 us at one L1TEX
+// sector per clock and SM), R-MAT 24 4.25 -> 3.21 ms, R-MAT 22 1.72 -> 0.98,
+// RMAT-Bad 22 0.95 -> 0.56, R-MAT 18 0.75 -> 0.34, a batch of 512 graphs 1.22
+// -> 0.66 (the deferral of defer_near and the 1-lane rows included).
 template <bool kDataflow>
-__device__ __forceinline__ void recolor_warp_tile(const RcArgs& a, const NextHist& nh, uint32_t* bm,
-                                                  int32_t sg, int32_t seg_first, int32_t seg_last,
-                                                  int32_t tile_in_seg, bool cached, int32_t& my_max,
-                                                  unsigned long long& edges) {
-    const int32_t p = sg / kNB;
-    const int b = sg % kNB;
-    const int32_t first = seg_first + tile_in_seg * warp_tile(b);
-    const RecolorFetch<kDataflow> f{a.new_c, p, a.tune.spin_limit, &a.ctrl->err, cached};
-    switch (b) {
-    case 0: recolor_chunk<kDataflow>(a, f, nh, load_item(a.list + first), bm, my_max, edges); break;
-    case 1: {
-        const WorkItem it = load_item(a.list + first);
-        const int32_t c = choose_warp<4>(a.g, it.beg, it.deg, 0u, f, bm, &a.ctrl->err);
-        if (lane_id() == 0) {
-            st_relaxed(a.new_c + it.v, c);
-            my_max = max(my_max, c);
-            edges += static_cast<unsigned long long>(it.deg);
-            nh.add(c, 1, 0);
+__device__ __forceinline__ void recolor_tiles(const RcArgs& a, const NextHist& nh, WarpStage& w, uint32_t t,
+                                              uint32_t end, uint32_t step, int32_t nseg, bool cached,
+                                              int32_t& my_max) {
+    if (t >= end) return;
+    const int l = lane_id();
+    int32_t sg = 0;
+    auto load_window = [&]() {
+        const int32_t i = min(sg + l, nseg);
+        stage_copy4(&w.win_t[l], a.tile_prefix + i);
+        stage_copy4(&w.win_s[l], a.seg_start + i);
+    };
+    // the items of tile tt, whose segment is sought from sg on, into a slot
+    auto stage_items = [&](uint32_t tt, int slot) {
+        int32_t win_t = w.win_t[l], win_s = w.win_s[l];
+        int n;
+        for (;;) {
+            n = __popc(__ballot_sync(kFull, static_cast<uint32_t>(win_t) <= tt));
+            if (n < 32) break;
+            sg += 31;
+            win_t = __ldg(a.tile_prefix + min(sg + l, nseg));
+            win_s = __ldg(a.seg_start + min(sg + l, nseg));
         }
-        break;
-    }
-    case 2: recolor_group_tile<32, kDataflow>(a, f, nh, 2, first, seg_last, my_max, edges); break;
-    case 3: recolor_group_tile<16, kDataflow>(a, f, nh, 3, first, seg_last, my_max, edges); break;
-    case 4: recolor_group_tile<8, kDataflow>(a, f, nh, 4, first, seg_last, my_max, edges); break;
-    case 5: recolor_group_tile<4, kDataflow>(a, f, nh, 5, first, seg_last, my_max, edges); break;
-    default: recolor_group_tile<2, kDataflow>(a, f, nh, 6, first, seg_last, my_max, edges); break;
+        sg += n - 1;
+        const int32_t seg_t = __shfl_sync(kFull, win_t, n - 1), seg_s = __shfl_sync(kFull, win_s, n - 1);
+        const int32_t seg_e = __shfl_sync(kFull, win_s, n);
+        const int tile = warp_tile(sg % kRcNB);
+        const int32_t first = seg_s + static_cast<int32_t>(tt - static_cast<uint32_t>(seg_t)) * tile;
+        const int32_t cnt = min(tile, seg_e - first);
+        if (l < cnt) stage_copy16(&w.item[slot][l], a.list + first + l, 16);
+        if (l == 0) w.meta[slot] = make_int4(sg, cnt, 0, 0);
+    };
+    sg = find_segment(a.tile_prefix, nseg, static_cast<int32_t>(t));
+    load_window();
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncwarp();
+    stage_items(t, 0);
+    load_window();
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncwarp();
+    stage_ids(a, w, 0);
+    if (end - t > step) stage_items(t + step, 1);
+    load_window();
+    cp_async_commit();
+    for (int slot = 0;; slot ^= 1) {
+        cp_async_wait<0>();
+        __syncwarp();
+        const uint32_t left = end - t;  // tiles t + step, t + 2 step exist if left exceeds step, 2 step
+        recolor_tile<kDataflow>(a, nh, w, slot, cached, my_max, [&]() {
+            if (left > step) {
+                stage_ids(a, w, slot ^ 1);
+                if (left - step > step) stage_items(t + 2 * step, slot);
+            }
+            load_window();
+            cp_async_commit();
+        });
+        if (left <= step) break;
+        t += step;
     }
 }
 
-// Segment table in shared memory when it fits.
-constexpr int kSegSmem = 1024;
-
-// Blocks of the dataflow launch: about one per 400 adjacency entries per
+// Blocks of the dataflow launch: about one per 200 adjacency entries per
 // color class, at least 16, at most all that fit.  An iteration is bound by
 // its class chain when the classes are small (each class waits for the ones
 // before it, and more warps only add pollers) and by throughput when they
-// are large.  Measured on GB300, per iteration: G(10^4, 16) 86 -> 50 us,
-// R-MAT 16 746 -> 537 us, R-MAT 18 1.12 -> 0.85 ms, R-MAT 20 1.64 -> 1.45
-// ms, 27-point stencil 64^3 133 -> 102 us; R-MAT 22 and 24 and the stencil
-// 128^3 keep the full grid.
+// are large.  Per iteration with one block per 800 / 400 / 200 / 100 / 50
+// entries: R-MAT 18 428 / 340 / 312 / 316 / 352 us, R-MAT 20 718 / 633 / 608 /
+// 608 / 607 us, R-MAT 22 1.14 / 0.98 / 0.98 / 0.98 / 0.98 ms, G(10^4, 16) 29 /
+// 23 / 23 / 24 / 24 us; a least grid of 8, 16, 32 or 64 blocks makes no
+// difference there.
 inline int coop_grid(int64_t nnz, int32_t classes, int capacity) {
-    const int64_t want = nnz / (400 * static_cast<int64_t>(std::max(classes, 1)));
+    const int64_t want = nnz / (200 * static_cast<int64_t>(std::max(classes, 1)));
     return static_cast<int>(std::max<int64_t>(std::min<int64_t>(16, capacity), std::min<int64_t>(want, capacity)));
 }
 
@@ -775,7 +1121,7 @@ inline int coop_grid(int64_t nnz, int32_t classes, int capacity) {
 // that tile: the waits always end.
 __device__ __forceinline__ NextHist setup_next_hist(const RcArgs& a, int32_t* s_hist) {
     if (!a.fuse_hist) return NextHist{nullptr, nullptr, nullptr, 0};  // cap 0: add() is a no-op
-    const bool local = a.hist_smem > 0;  // (cap + 1) * kNB entries of dynamic shared memory
+    const bool local = a.hist_smem > 0;  // (cap + 1) * kRcNB entries of dynamic shared memory
     if (local)
         for (int i = threadIdx.x; i < a.hist_smem; i += kBlock) s_hist[i] = 0;
     return NextHist{local ? s_hist : nullptr, a.nxt_cnt, a.nxt_units, a.cap};
@@ -784,64 +1130,36 @@ __device__ __forceinline__ NextHist setup_next_hist(const RcArgs& a, int32_t* s_
 __device__ __forceinline__ void flush_next_hist(const RcArgs& a, const NextHist& nh) {
     if (!nh.sh) return;
     __syncthreads();
-    const int32_t entries = (a.cap + 1) * kNB;
+    const int32_t entries = (a.cap + 1) * kRcNB;
     for (int i = threadIdx.x; i < entries; i += kBlock)
         if (nh.sh[i]) atomicAdd(&a.nxt_cnt[i], nh.sh[i]);
 }
 
-__global__ void __launch_bounds__(kBlock, 5) k_rc_recolor_coop(RcArgs a) {
-    __shared__ uint32_t s_bm[kWarps][kWarpBitmapWords];
-    __shared__ int32_t s_tp[kSegSmem + 1], s_ss[kSegSmem + 1];
+__global__ void __launch_bounds__(kBlock, 4) k_rc_recolor_coop(RcArgs a) {
+    __shared__ WarpStage s_stage[kWarps];
     extern __shared__ int32_t s_hist[];
     if (a.ctrl->err & (kErrImproper | kErrBadGraph)) return;
-    const int32_t total = a.ctrl->total_tiles;
-    const int32_t nseg = a.ctrl->k * kNB;
-    const bool staged = nseg <= kSegSmem;
-    if (staged) {
-        for (int i = threadIdx.x; i <= nseg; i += kBlock) {
-            s_tp[i] = a.tile_prefix[i];
-            s_ss[i] = a.seg_start[i];
-        }
-    }
     const NextHist nh = setup_next_hist(a, s_hist);
     __syncthreads();
-    const int32_t* tp = staged ? s_tp : a.tile_prefix;
-    const int32_t* ss = staged ? s_ss : a.seg_start;
     const int warp = threadIdx.x >> 5;
-    const int32_t W = gridDim.x * kWarps;
-    const bool cached = a.ctrl->n_heavy > 0;
     int32_t my_max = 0;
-    unsigned long long edges = 0;
-    int32_t sg = 0;
-    for (int32_t t = blockIdx.x * kWarps + warp; t < total; t += W) {
-        if (tp[sg + 1] <= t) sg = find_segment(tp, nseg, t);
-        recolor_warp_tile<true>(a, nh, s_bm[warp], sg, ss[sg], ss[sg + 1], t - tp[sg], cached, my_max,
-                                edges);
-    }
-    warp_add(&a.ctrl->edges, edges);
+    recolor_tiles<true>(a, nh, s_stage[warp], blockIdx.x * kWarps + warp, a.ctrl->total_tiles, gridDim.x * kWarps,
+                        a.ctrl->k * kRcNB, a.ctrl->n_heavy > 0, my_max);
     warp_max(&a.ncolors[a.iteration + 1], my_max);
     flush_next_hist(a, nh);
 }
 
-// Stepwise form: one launch per class p over its warp tiles [t0, t1).
-__global__ void __launch_bounds__(kBlock, 5) k_rc_recolor_step(RcArgs a, int32_t p, int32_t t0,
-                                                               int32_t t1) {
-    __shared__ uint32_t s_bm[kWarps][kWarpBitmapWords];
+// Stepwise form: one launch per class over its warp tiles [t0, t1).
+__global__ void __launch_bounds__(kBlock, 4) k_rc_recolor_step(RcArgs a, int32_t t0, int32_t t1) {
+    __shared__ WarpStage s_stage[kWarps];
     extern __shared__ int32_t s_hist[];
     if (a.ctrl->err & (kErrImproper | kErrBadGraph)) return;
     const NextHist nh = setup_next_hist(a, s_hist);
     __syncthreads();
     const int warp = threadIdx.x >> 5;
     int32_t my_max = 0;
-    unsigned long long edges = 0;
-    const int32_t seg0 = p * kNB;
-    for (int32_t t = t0 + blockIdx.x * kWarps + warp; t < t1; t += gridDim.x * kWarps) {
-        int sg = seg0;
-        while (sg + 1 < seg0 + kNB && a.tile_prefix[sg + 1] <= t) ++sg;
-        recolor_warp_tile<false>(a, nh, s_bm[warp], sg, a.seg_start[sg], a.seg_start[sg + 1],
-                                 t - a.tile_prefix[sg], false, my_max, edges);
-    }
-    warp_add(&a.ctrl->edges, edges);
+    recolor_tiles<false>(a, nh, s_stage[warp], t0 + blockIdx.x * kWarps + warp, t1, gridDim.x * kWarps,
+                         a.ctrl->k * kRcNB, false, my_max);
     warp_max(&a.ncolors[a.iteration + 1], my_max);
     flush_next_hist(a, nh);
 }
@@ -888,7 +1206,7 @@ gc_status class_ranks_device(const Graph& g, const int32_t* colors, bool trusted
     *maxc_out = h.max_in;
     if (!rank_out) return GC_OK;
     const int32_t cap = std::max(h.max_in, 1);
-    const int64_t ent = static_cast<int64_t>(cap + 1) * kNB;
+    const int64_t ent = static_cast<int64_t>(cap + 1) * kRcNB;
     Scratch sc_cls, sc_units, sc_present, sc_psize, sc_order, sc_jtab, sc_seg, sc_tiles, sc_fill, sc_iso;
     if (!sc_cls.alloc(ent * 4, s) || !sc_units.alloc((cap + 1) * 4, s) || !sc_iso.alloc((cap + 1) * 4, s) ||
         !sc_present.alloc((cap + 1) * 4, s) || !sc_psize.alloc((cap + 1) * 4, s) ||
@@ -946,8 +1264,8 @@ __global__ void __launch_bounds__(kBlock) k_brc_hist(RcArgs a) {
             continue;
         }
         const unsigned act = __activemask();
-        const unsigned peers = __match_any_sync(act, static_cast<uint32_t>(key * kNB + b));
-        if (lane_id() == __ffs(peers) - 1) atomicAdd(&a.cls_cnt[key * kNB + b], __popc(peers));
+        const unsigned peers = __match_any_sync(act, static_cast<uint32_t>(key * kRcNB + b));
+        if (lane_id() == __ffs(peers) - 1) atomicAdd(&a.cls_cnt[key * kRcNB + b], __popc(peers));
         if (b == 0) {
             int64_t rb;
             int32_t deg;
@@ -975,7 +1293,7 @@ __global__ void __launch_bounds__(kBlock) k_brc_order(RcArgs a) {
             const int32_t c = c0 + l;
             int32_t size = 0;
             if (c <= maxc) {
-                for (int b = 0; b < kNB; ++b) size += a.cls_cnt[(base + c) * kNB + b];
+                for (int b = 0; b < kRcNB; ++b) size += a.cls_cnt[(base + c) * kRcNB + b];
                 size += a.iso_cnt[base + c];
             }
             const uint32_t bal = __ballot_sync(kFull, size > 0);
@@ -1022,9 +1340,9 @@ __global__ void __launch_bounds__(kBlock) k_brc_order(RcArgs a) {
         for (int32_t p = l; p < k; p += 32) {
             const int32_t c = order[p];
             a.rank_of[base + c] = p;
-            for (int b = 0; b < kNB; ++b) {
-                const int32_t u = b == 0 ? a.cls_units[base + c] : a.cls_cnt[(base + c) * kNB + b];
-                if (u) atomicAdd(&a.seg_cnt[p * kNB + b], u);
+            for (int b = 0; b < kRcNB; ++b) {
+                const int32_t u = b == 0 ? a.cls_units[base + c] : a.cls_cnt[(base + c) * kRcNB + b];
+                if (u) atomicAdd(&a.seg_cnt[p * kRcNB + b], u);
             }
         }
         if (l == 0) atomicMax(&a.ctrl->k, k);
@@ -1040,6 +1358,17 @@ __global__ void __launch_bounds__(kOrderThreads) k_brc_segments(RcArgs a) {
 // ---------------------------------------------------------------------------
 // Host driver
 // ---------------------------------------------------------------------------
+// The scatter's shared segment counters (sized to the classes, so that small
+// tables leave the SM to more blocks and to L1) and its resident grid.
+static int scatter_launch(RcArgs& a, int32_t cap, const Tuning& tune, size_t* dyn) {
+    a.scatter_segs = static_cast<int32_t>(std::min<int64_t>(static_cast<int64_t>(cap) * kRcNB, kScatterSegs));
+    *dyn = static_cast<size_t>(a.scatter_segs) * 2 * sizeof(int32_t);
+    const int64_t blocks = (static_cast<int64_t>(a.g.n) + kBlock - 1) / kBlock;
+    const int64_t fit = tune.grid_blocks > 0 ? tune.grid_blocks
+                                             : sm_count() * occupancy_of(reinterpret_cast<const void*>(k_rc_scatter), kBlock, *dyn);
+    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(blocks, fit)));
+}
+
 gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_in, bool trusted,
                          int32_t perm, int32_t iterations, uint64_t seed, int32_t* colors_out,
                          int32_t* ncolors_per_iter, gc_stats* stats, cudaStream_t s) {
@@ -1048,8 +1377,6 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     const Tuning tune = recolor_tuning(current_tuning());
     const int grid = persistent_grid(tune);
     const int vgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + kBlock - 1) / kBlock, grid)));
-    const int grid_sc = static_cast<int>(std::max<int64_t>(
-        1, std::min<int64_t>((n + kBlock - 1) / kBlock, resident_grid(k_rc_scatter, tune))));
     cudaError_t ce;
 
     Scratch sc_ctrl, sc_bucket;
@@ -1064,18 +1391,6 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     a.bucket = sc_bucket.as<uint8_t>();
     a.ctrl = sc_ctrl.as<RcCtrl>();
     cudaMemsetAsync(a.ctrl, 0, sizeof(RcCtrl), s);
-    // A launch that gets fewer blocks than fit is bound by its class chain
-    // (coop_grid); there a row of 9 to 16 entries takes 4 lanes (one batch of
-    // loads) instead of 2 (two batches), unless the caller set the 2-lane
-    // threshold.  Per iteration, G(10^4, 16): 86 -> 51 us; a large graph is
-    // bound by tile throughput and keeps 2 lanes (RMAT-ER at scale 24 went
-    // 2.08 -> 3.09 ms with 4).
-    const bool g2_default = current_tuning().rc_g2_max_deg == kDefaultRcG2MaxDeg;
-    const int coop_fit = sm_count() * occupancy_of(reinterpret_cast<const void*>(k_rc_recolor_coop), kBlock);
-    auto chain_bound = [&](int32_t maxc) {
-        return g2_default && coop_grid(g.nnz, std::max(maxc, 1), coop_fit) < coop_fit;
-    };
-    if (trusted && chain_bound(maxc_in)) a.tune.g2_max_deg = std::min(kChainRcG2MaxDeg, a.tune.g4_max_deg);
     RcCtrl h;
     std::memset(&h, 0, sizeof(h));
     if (n > 0) {
@@ -1092,7 +1407,7 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     // bound's scratch is small.
     const int64_t heavy_min = std::max<int64_t>(tune.warp_max_deg, 63) + 1;
     const int64_t heavy_bound = std::min<int64_t>(n, static_cast<int64_t>(g.nnz) / heavy_min);
-    const int64_t bound_words = (static_cast<int64_t>(std::max(maxc_in, 1)) + 1 + 31) / 32;
+    const int64_t bound_words = (static_cast<int64_t>(std::max(maxc_in, 1)) + 1 + 31) / 32 + kRowPend;
     const bool read_back = !trusted || n == 0 || heavy_bound * bound_words * 4 > (int64_t(64) << 20);
     if (read_back) {
         ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
@@ -1100,13 +1415,6 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
         if (ce != cudaSuccess) return cuda_status(ce);
         if (h.err & kErrBadGraph) return GC_ERR_BAD_GRAPH;
         if (input != GC_OK) return input;
-        if (!trusted) {
-            if (n > 0 && chain_bound(maxc_in)) {  // the buckets again, with the chain-bound threshold
-                a.tune.g2_max_deg = std::min(kChainRcG2MaxDeg, a.tune.g4_max_deg);
-                cudaMemsetAsync(&a.ctrl->n_heavy, 0, sizeof(int32_t), s);
-                GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
-            }
-        }
     } else {
         h.n_heavy = static_cast<int32_t>(heavy_bound);
     }
@@ -1127,11 +1435,11 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     // Colors stay within [1, maxc_in]: a vertex of the class of rank p takes
     // at most color p + 1 <= k <= maxc_in.
     const int32_t cap = std::max(maxc_in, 1);
-    const int64_t ent = static_cast<int64_t>(cap + 1) * kNB;
-    const int32_t hub_words = (cap + 1 + 31) / 32;
+    const int64_t ent = static_cast<int64_t>(cap + 1) * kRcNB;
+    const int32_t hub_words = ((cap + 1 + 31) / 32 + 3) & ~3;  // 16-byte rows
     const int64_t hubs = std::max<int64_t>(1, h.n_heavy);
     Scratch sc_cls, sc_units, sc_cls2, sc_units2, sc_present, sc_psize, sc_order, sc_jtab, sc_rank, sc_seg, sc_tiles,
-        sc_fill, sc_list, sc_alt, sc_ncol, sc_hv, sc_hn, sc_hd, sc_hb, sc_iso, sc_iso2;
+        sc_fill, sc_list, sc_alt, sc_ncol, sc_hv, sc_hn, sc_hd, sc_hb, sc_hp, sc_hl, sc_iso, sc_iso2;
     // list entries: one per vertex, one per chunk of a bucket-0 row
     const int64_t list_len = n + (static_cast<int64_t>(g.nnz) / kChunk) + h.n_heavy;
     if (!sc_cls.alloc(ent * 4, s) || !sc_units.alloc((cap + 1) * 4, s) ||
@@ -1143,7 +1451,8 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
         !sc_list.alloc(list_len * sizeof(WorkItem), s) || !sc_alt.alloc(n * 4, s) ||
         !sc_ncol.alloc((iterations + 1) * 4, s) || !sc_hv.alloc(hubs * 4, s) ||
         !sc_hn.alloc(hubs * 4, s) || !sc_hd.alloc(hubs * 4, s) ||
-        !sc_hb.alloc(hubs * hub_words * 4, s) || !sc_iso.alloc((cap + 1) * 4, s) ||
+        !sc_hb.alloc(hubs * hub_words * 4, s) || !sc_hp.alloc(hubs * 4, s) ||
+        !sc_hl.alloc(hubs * kRowPend * 4, s) || !sc_iso.alloc((cap + 1) * 4, s) ||
         !sc_iso2.alloc((cap + 1) * 4, s))
         return GC_ERR_OOM;
     a.cap = cap;
@@ -1162,10 +1471,17 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     a.hub_done = sc_hd.as<int32_t>();
     a.hub_bm = sc_hb.as<uint32_t>();
     a.hub_words = hub_words;
+    a.hub_pcnt = sc_hp.as<int32_t>();
+    a.hub_pend = sc_hl.as<int32_t>();
     a.fuse_hist = 1;
     const int32_t hist_entries = static_cast<int32_t>(ent);
     const size_t hist_dyn = hist_entries <= kRcHistSmem ? static_cast<size_t>(hist_entries) * 4 : 0;
     a.hist_smem = hist_dyn ? hist_entries : 0;
+    if (hist_dyn > 16 * 1024)  // beyond 48 KB with the warps' stages
+        for (const void* k : {reinterpret_cast<const void*>(k_rc_recolor_coop), reinterpret_cast<const void*>(k_rc_recolor_step)})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kRcHistSmem * 4);
+    size_t sc_dyn = 0;
+    const int grid_sc = scatter_launch(a, cap, tune, &sc_dyn);
     const int coop_capacity =
         sm_count() * occupancy_of(reinterpret_cast<const void*>(k_rc_recolor_coop), kBlock, hist_dyn);
     const int grid_rc = tune.grid_blocks > 0 ? std::min(tune.grid_blocks, coop_capacity)
@@ -1206,7 +1522,7 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
         cudaMemsetAsync(a.nxt_units, 0, (cap + 1) * 4, s);
         cudaMemsetAsync(a.nxt_iso, 0, (cap + 1) * 4, s);
         GC_LAUNCH(KID_RC_ORDER, s, k_rc_order<<<1, kOrderThreads, 0, s>>>(a));
-        GC_LAUNCH(KID_RC_SCATTER, s, k_rc_scatter<<<grid_sc, kBlock, 0, s>>>(a));
+        GC_LAUNCH(KID_RC_SCATTER, s, k_rc_scatter<<<grid_sc, kBlock, sc_dyn, s>>>(a));
         if (tune.recolor_mode == 0) {
             void* args[] = {&a};
             cudaError_t le;
@@ -1219,15 +1535,15 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
             ce = cudaMemcpyAsync(&hc, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
             if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
             if (ce != cudaSuccess) { st = cuda_status(ce); break; }
-            tp.resize(static_cast<size_t>(hc.k) * kNB + 1);
+            tp.resize(static_cast<size_t>(hc.k) * kRcNB + 1);
             ce = cudaMemcpyAsync(tp.data(), a.tile_prefix, tp.size() * 4, cudaMemcpyDeviceToHost, s);
             if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
             if (ce != cudaSuccess) { st = cuda_status(ce); break; }
             for (int32_t p = 0; p < hc.k; ++p) {
-                const int32_t t0 = tp[p * kNB], t1 = tp[(p + 1) * kNB];
+                const int32_t t0 = tp[p * kRcNB], t1 = tp[(p + 1) * kRcNB];
                 if (t1 <= t0) continue;
                 const int g2 = std::min(grid_step, (t1 - t0 + kWarps - 1) / kWarps);
-                GC_LAUNCH(KID_RC_STEP, s, k_rc_recolor_step<<<g2, kBlock, hist_dyn, s>>>(a, p, t0, t1));
+                GC_LAUNCH(KID_RC_STEP, s, k_rc_recolor_step<<<g2, kBlock, hist_dyn, s>>>(a, t0, t1));
             }
         }
         cur = dst;
@@ -1281,8 +1597,6 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
     const int vgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + kBlock - 1) / kBlock, grid)));
     const int coop_capacity = sm_count() * occupancy_of(reinterpret_cast<const void*>(k_rc_recolor_coop), kBlock);
     const int grid_step = resident_grid(k_rc_recolor_step, tune);
-    const int grid_sc = static_cast<int>(std::max<int64_t>(
-        1, std::min<int64_t>((n + kBlock - 1) / kBlock, resident_grid(k_rc_scatter, tune))));
     const int grid_go = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((ng + kWarps - 1) / kWarps, grid)));
     cudaError_t ce;
 
@@ -1340,21 +1654,22 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
         if (max_color_out) std::copy(gmax.begin(), gmax.end(), max_color_out);
         return cuda_status(cudaStreamSynchronize(s));
     }
-    const int64_t ent = static_cast<int64_t>(cap + 1) * kNB;
-    const int32_t hub_words = (cap + 1 + 31) / 32;
+    const int64_t ent = static_cast<int64_t>(cap + 1) * kRcNB;
+    const int32_t hub_words = ((cap + 1 + 31) / 32 + 3) & ~3;  // 16-byte rows
     const int64_t hubs = std::max<int64_t>(1, h.n_heavy);
     const int64_t list_len = n + (static_cast<int64_t>(g.nnz) / kChunk) + h.n_heavy;
     const int grid_rc = tune.grid_blocks > 0 ? std::min(tune.grid_blocks, coop_capacity)
                                              : coop_grid(g.nnz, cap, coop_capacity);
     Scratch sc_base, sc_cls, sc_units, sc_rank, sc_gp, sc_gs, sc_go, sc_gj, sc_segc, sc_seg, sc_tiles,
-        sc_fill, sc_list, sc_alt, sc_ncol, sc_hv, sc_hn, sc_hd, sc_hb, sc_iso;
-    if (!sc_base.alloc((ng + 1) * 8, s) || !sc_cls.alloc(T * kNB * 4, s) || !sc_units.alloc(T * 4, s) ||
+        sc_fill, sc_list, sc_alt, sc_ncol, sc_hv, sc_hn, sc_hd, sc_hb, sc_hp, sc_hl, sc_iso;
+    if (!sc_base.alloc((ng + 1) * 8, s) || !sc_cls.alloc(T * kRcNB * 4, s) || !sc_units.alloc(T * 4, s) ||
         !sc_rank.alloc(T * 4, s) || !sc_gp.alloc(T * 4, s) || !sc_gs.alloc(T * 4, s) ||
         !sc_go.alloc(T * 4, s) || !sc_gj.alloc(T * 4, s) || !sc_segc.alloc(ent * 4, s) ||
         !sc_seg.alloc((ent + 1) * 4, s) || !sc_tiles.alloc((ent + 1) * 4, s) || !sc_fill.alloc(ent * 4, s) ||
         !sc_list.alloc(list_len * sizeof(WorkItem), s) || !sc_alt.alloc(n * 4, s) ||
         !sc_ncol.alloc((iters + 1) * 4, s) || !sc_hv.alloc(hubs * 4, s) || !sc_hn.alloc(hubs * 4, s) ||
-        !sc_hd.alloc(hubs * 4, s) || !sc_hb.alloc(hubs * hub_words * 4, s) || !sc_iso.alloc(T * 4, s))
+        !sc_hd.alloc(hubs * 4, s) || !sc_hb.alloc(hubs * hub_words * 4, s) || !sc_hp.alloc(hubs * 4, s) ||
+        !sc_hl.alloc(hubs * kRowPend * 4, s) || !sc_iso.alloc(T * 4, s))
         return GC_ERR_OOM;
     ce = cudaMemcpyAsync(sc_base.p, base.data(), (ng + 1) * 8, cudaMemcpyHostToDevice, s);
     if (ce != cudaSuccess) return cuda_status(ce);
@@ -1378,8 +1693,12 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
     a.hub_done = sc_hd.as<int32_t>();
     a.hub_bm = sc_hb.as<uint32_t>();
     a.hub_words = hub_words;
+    a.hub_pcnt = sc_hp.as<int32_t>();
+    a.hub_pend = sc_hl.as<int32_t>();
     a.iso_cnt = sc_iso.as<int32_t>();
     a.fuse_hist = 0;
+    size_t sc_dyn = 0;
+    const int grid_sc = scatter_launch(a, cap, tune, &sc_dyn);
     cudaMemsetAsync(a.ncolors, 0, (iters + 1) * 4, s);
 
     cudaEvent_t e0, e1;
@@ -1394,7 +1713,7 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
         a.iteration = it;
         a.old_c = cur;
         a.new_c = dst;
-        cudaMemsetAsync(a.cls_cnt, 0, T * kNB * 4, s);
+        cudaMemsetAsync(a.cls_cnt, 0, T * kRcNB * 4, s);
         cudaMemsetAsync(a.cls_units, 0, T * 4, s);
         cudaMemsetAsync(a.iso_cnt, 0, T * 4, s);
         cudaMemsetAsync(a.seg_cnt, 0, ent * 4, s);
@@ -1402,7 +1721,7 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
         GC_LAUNCH(KID_BRC_HIST, s, k_brc_hist<<<vgrid, kBlock, 0, s>>>(a));
         GC_LAUNCH(KID_BRC_ORDER, s, k_brc_order<<<grid_go, kBlock, 0, s>>>(a));
         GC_LAUNCH(KID_BRC_SEGMENTS, s, k_brc_segments<<<1, kOrderThreads, 0, s>>>(a));
-        GC_LAUNCH(KID_RC_SCATTER, s, k_rc_scatter<<<grid_sc, kBlock, 0, s>>>(a));
+        GC_LAUNCH(KID_RC_SCATTER, s, k_rc_scatter<<<grid_sc, kBlock, sc_dyn, s>>>(a));
         if (tune.recolor_mode == 0) {
             void* args[] = {&a};
             cudaError_t le;
@@ -1415,15 +1734,15 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
             ce = cudaMemcpyAsync(&hc, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
             if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
             if (ce != cudaSuccess) { st = cuda_status(ce); break; }
-            tp.resize(static_cast<size_t>(hc.k) * kNB + 1);
+            tp.resize(static_cast<size_t>(hc.k) * kRcNB + 1);
             ce = cudaMemcpyAsync(tp.data(), a.tile_prefix, tp.size() * 4, cudaMemcpyDeviceToHost, s);
             if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
             if (ce != cudaSuccess) { st = cuda_status(ce); break; }
             for (int32_t p = 0; p < hc.k; ++p) {
-                const int32_t t0 = tp[p * kNB], t1 = tp[(p + 1) * kNB];
+                const int32_t t0 = tp[p * kRcNB], t1 = tp[(p + 1) * kRcNB];
                 if (t1 <= t0) continue;
                 const int g2 = std::min(grid_step, (t1 - t0 + kWarps - 1) / kWarps);
-                GC_LAUNCH(KID_RC_STEP, s, k_rc_recolor_step<<<g2, kBlock, 0, s>>>(a, p, t0, t1));
+                GC_LAUNCH(KID_RC_STEP, s, k_rc_recolor_step<<<g2, kBlock, 0, s>>>(a, t0, t1));
             }
         }
         cur = dst;

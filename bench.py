@@ -134,7 +134,7 @@ def _peak_hbm():
 KERNEL_SOURCES = {
     "k_rc_recolor_coop": ["gc_recolor.cu", "gc_common.cuh", "gc_internal.h"],
     "k_rc_recolor_step": ["gc_recolor.cu", "gc_common.cuh", "gc_internal.h"],
-    "spec_rounds_graph": ["gc_color.cu", "gc_common.cuh", "gc_internal.h"],
+    "k_spec_rounds": ["gc_color.cu", "gc_common.cuh", "gc_internal.h"],
 }
 
 
@@ -724,7 +724,7 @@ def _roofline(wl, n, nnz, prof, prof_steps, leg_stats, args):
         compulsory = nlegs * iters * (4 * nnz + 16 * n)
         units = (f"recoloring iterations: 8 B per adjacency entry + 24 B per vertex, "
                  f"{nlegs} x {iters} x (8*{nnz} + 24*{n}) B per step over {launches_per_step:g} launches")
-    elif top_name in ("spec_rounds_graph", "k_tentative", "k_conflict"):
+    elif top_name == "k_spec_rounds":
         spec_edges, visits = 0, 0
         for st in leg_stats:
             spec_edges += st["edges_examined"] - st.get("edges_examined_recolor", iters * nnz if kind != "arc" else 0)
@@ -733,9 +733,6 @@ def _roofline(wl, n, nnz, prof, prof_steps, leg_stats, args):
         # edges_examined counts both phases; 24 B per vertex and phase
         per_step = 8 * spec_edges + 48 * visits
         compulsory = 4 * spec_edges + 32 * visits
-        if top_name != "spec_rounds_graph":
-            per_step /= 2
-            compulsory /= 2
         units = ("speculative rounds: 8 B per examined adjacency entry (both phases) + 24 B per "
                  f"work-set vertex and phase, {per_step:.4g} B per step over {launches_per_step:g} launches")
     else:

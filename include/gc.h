@@ -383,20 +383,18 @@ gc_status gc_check_graph(const gc_graph* g, int64_t* first_bad_vertex, void* str
  * Scheduling knobs (not part of the method: results are identical for every
  * setting).  A vertex of degree d with d + X <= 64 is handled by a group of
  * 2 lanes if d <= g2_max_deg, 4 lanes if d <= g4_max_deg, 8 if d <= g8_max_deg, 16 if d <= g16_max_deg,
- * else 32; otherwise by one warp with a shared-memory bitmap if
- * d <= warp_max_deg (default 1024; a graph with no row longer than 12288
- * entries runs the coloring with no limit while warp_max_deg is at its
- * default), else by a whole block (coloring) or split into chunks
- * of 256 neighbors (recoloring, where rc_warp_max_deg takes the place of
- * warp_max_deg and rc_g2_max_deg, capped at g4_max_deg, that of g2_max_deg;
- * a row of up to 8 entries, if rc_g2_max_deg allows 2 lanes, takes a single
- * one there).  grid_blocks = 0 sizes every
+ * else 32; a longer row by a warp when coloring, and when recoloring by one
+ * warp up to rc_warp_max_deg entries, in chunks of 256 neighbors beyond
+ * (warp_max_deg, default 1024, is accepted and has no effect).  The
+ * recoloring takes rc_g2_max_deg, capped at g4_max_deg, in the place of
+ * g2_max_deg, and a single lane for a row of up to 8 entries if it allows 2
+ * there.  grid_blocks = 0 sizes every
  * grid to the blocks that fit on the GPU at once.  recolor_mode 0 runs each recoloring iteration as one dataflow
  * launch (vertices wait, with a bounded spin of spin_limit polls, for their
  * earlier-class neighbors); 1 launches one grid per color class.
- * spec_graph 1 (default) runs the speculative rounds as a CUDA graph whose
- * WHILE node repeats {tentative, conflict} until a kernel reports an empty
- * work set (no host round trip per round); 0 drives the rounds from the
+ * spec_graph 1 (default) runs the speculative rounds in one cooperative
+ * launch with grid barriers (no host round trip per round); 0 launches them
+ * one by one from the
  * host.  gc_set_tuning sets the process-wide knobs (change them only while
  * no call is running); a plan's knobs apply to its own calls only.
  */

@@ -49,14 +49,13 @@ Tuning default_tuning() {
     t.g4_max_deg = 64;
     t.g8_max_deg = 64;
     t.g16_max_deg = 64;
-    t.warp_max_deg = kDefaultWarpMaxDeg;
+    t.warp_max_deg = 1024;
     t.grid_blocks = 0;
     t.recolor_mode = 0;
     t.spin_limit = 1 << 20;
     t.spec_graph = 1;
     t.rc_warp_max_deg = 512;
-    // 2 lanes up to degree 32 when coloring, 16 when recoloring (measured:
-    // stencil coloring 1.32 -> 1.15 ms at 32, its recoloring 3.24 -> 4.61 ms)
+    // 2 lanes up to degree 32 when coloring, 16 when recoloring
     t.g2_max_deg = 32;
     t.rc_g2_max_deg = 16;
     return t;
@@ -136,11 +135,11 @@ void note_launches(int64_t k) { g_launches.fetch_add(k, std::memory_order_relaxe
 // ---------------------------------------------------------------------------
 namespace {
 const char* const kKernelNames[] = {
-    "k_spec_setup", "k_spec_fill", "k_tentative", "k_conflict", "k_priorities",
+    "k_spec_setup", "k_heavy_setup", "k_spec_rounds", "k_priorities",
     "k_rc_bucket", "k_rc_validate", "k_rc_hist", "k_rc_order", "k_rc_scatter",
     "k_rc_recolor_coop", "k_rc_recolor_step", "k_validate", "k_validate_heavy",
-    "k_mark_present", "k_count_bits", "k_check_graph", "spec_rounds_graph", "k_batch", "k_brc_hist",
-    "k_brc_order", "k_brc_segments", "k_mark_colors"};
+    "k_mark_present", "k_count_bits", "k_check_graph", "k_batch", "k_brc_hist",
+    "k_brc_order", "k_brc_segments"};
 static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == KID_COUNT_,
               "one name per KernelId");
 std::atomic<bool> g_prof_on{false};
@@ -706,13 +705,12 @@ gc_status gc_autotune(const gc_graph* g, gc_strategy strategy, int32_t X, uint64
     st = time_it(cur, &cur_ms);
     // one knob at a time, keeping any improvement
     const int32_t groups[][3] = {{64, 64, 64}, {4, 8, 16}, {0, 0, 0}, {0, 64, 64}, {16, 32, 64}};
-    const int32_t warp_max[] = {256, 1024, 2048};
     const int32_t rc_warp_max[] = {256, 512, 1024};
     const int32_t g2_max[] = {0, 16, 32};
     const int32_t rc_g2_max[] = {0, 8, 32};
     const int32_t blocks_per_sm[] = {0, 2, 4};
-    for (int step = 0; step < 8 && st == GC_OK; ++step) {
-        const int variants = step == 0 ? 5 : step == 1 ? 3 : step == 2 ? 2 : step == 3 ? 2 : 3;
+    for (int step = 0; step < 7 && st == GC_OK; ++step) {
+        const int variants = step == 0 ? 5 : step == 1 ? 2 : step == 2 ? 2 : 3;
         for (int i = 0; i < variants && st == GC_OK; ++i) {
             gc_tuning t = cur;
             if (step == 0) {
@@ -721,12 +719,11 @@ gc_status gc_autotune(const gc_graph* g, gc_strategy strategy, int32_t X, uint64
                 t.g16_max_deg = groups[i][2];
                 t.g2_max_deg = std::min(t.g2_max_deg, t.g4_max_deg);
             }
-            else if (step == 1) t.warp_max_deg = warp_max[i];
-            else if (step == 2) t.recolor_mode = i;
-            else if (step == 3) t.spec_graph = i;
-            else if (step == 4) t.grid_blocks = blocks_per_sm[i] * sm_count();
-            else if (step == 5) t.rc_warp_max_deg = rc_warp_max[i];
-            else if (step == 6) t.g2_max_deg = std::min(g2_max[i], t.g4_max_deg);
+            else if (step == 1) t.recolor_mode = i;
+            else if (step == 2) t.spec_graph = i;
+            else if (step == 3) t.grid_blocks = blocks_per_sm[i] * sm_count();
+            else if (step == 4) t.rc_warp_max_deg = rc_warp_max[i];
+            else if (step == 5) t.g2_max_deg = std::min(g2_max[i], t.g4_max_deg);
             else t.rc_g2_max_deg = rc_g2_max[i];
             if (std::memcmp(&t, &cur, sizeof(t)) == 0) continue;
             float ms = 0.f;

@@ -9,116 +9,135 @@
 // color, losers form W_{r+1}.  The vertex of W_r with the largest (priority,
 // id) always wins, so the loop ends within |V| rounds.
 //
-// Layout in HBM: colors int32[n] (the output, 0 = uncolored), key uint64[n]
-// = (tentative color << 32 | priority), so one 8-byte gather gives conflict
-// detection both the color and the priority of a neighbor; two work lists of
-// 16-byte items (vertex, row start, degree) used as
-// ping-pong buffers, each cut into six degree-bucket regions whose starts are
-// fixed in round 0 (a loser stays in its bucket, so a region never
-// overflows).  All per-round state (round number, bucket counts) lives in a
-// small device control block, so a round's two launches take no host input.
+// Layout in HBM: a color word per vertex holds its tentative color with bit
+// 31 set until it is fixed and the color alone afterwards, so one gather tells
+// a neighbor's color and whether it is fixed; the priority stands beside it
+// or in an array of its own (see color_word).  Two work lists of 16-byte items
+// are used as ping-pong buffers, each cut into degree-bucket regions whose
+// starts are fixed by the set-up (a loser stays in its bucket, so a region
+// never overflows).
 //
-// Heavy rows (the block- and warp-bucket rows, degree above 64 - X) are not
-// re-read every round.  Each keeps a bitmap of the colors of its fixed
-// neighbors, which those neighbors mark when they are fixed (a fixed vertex
-// walks its row once and sets its color's bit in each heavy neighbor's
-// bitmap; a block-bucket winner's row is marked by the whole grid in a third
-// launch of the round), so its tentative color is a search of its bitmap.
-// For the conflict test it keeps a list of its neighbors above it in the
-// total order that were not fixed at its last look, built from the row in
-// round 0; only those can beat it, so a round scans the list, dropping the
-// entries fixed since.  The forbidden set and the conflict candidates are
-// exactly those of a full row scan.  Where the block-bucket rows hold under
-// 1/16 of the entries, marks would cost more than they save for the warp-
-// bucket rows: those keep the list of all their neighbors not fixed and
-// fold the fixed ones' colors into their bitmaps themselves each round.
+// No row is read to choose a tentative color: a vertex fixed at color c walks
+// its row once and sets bit c - 1 in the mask of each neighbor -- 64 bits for
+// a light row (degree + X <= 64: its color is among the first 64), a bitmap
+// for a heavy one -- so the choice is the j-th clear bit of the mask.  Each
+// row is pushed once in a run instead of being gathered in every round
+// (G(10^6, 24) First Fit: 24 M pushes instead of 128 M gathers).
+//
+// The conflict test of a light row reads the row a few neighbors at a time and
+// ends at the first one it loses to (most vertices of an early round lose to
+// one of the first).  A heavy row keeps a list of its neighbors above it in
+// the total order that were not fixed at its last look, built from the row
+// in round 0; only those can beat it.
+//
+// All rounds run in one cooperative launch with a grid barrier between the
+// phases of a round (choice, test, and where there are any the long lists left
+// open and the long rows' pushes); a barrier takes about 1.2 us.
+//
+// What it replaced -- three launches a round in a CUDA graph, every light row
+// gathered again for every choice and every test, an 8-byte key per gather, a
+// block per row beyond 1024 entries -- spent its time on the launches and
+// their gaps (20 us a round where there is little to do), on gathers, and on
+// a block waiting through one dependent load after the other for a row that
+// then lost at once.  Coloring, set-up included, before -> after: R-MAT 24
+// First Fit 87.0 -> 51.2 ms (524 rounds), R-MAT 22 Random-4 Fit 12.1 -> 8.6,
+// RMAT-Bad 22 14.6 -> 7.9, R-MAT 20 11.4 -> 7.7, G(10^6, 24) 1.68 -> 1.12, the
+// 27-point stencil 128^3 with Random-8 Fit 1.12 -> 0.90, a batch of 512 graphs
+// 3.99 -> 3.73, G(10^4, 16) 0.22 -> 0.14 (kernels).
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 
 #include "gc_internal.h"
 
 namespace gc {
 
 struct SpecCtrl {
-    int32_t cnt[2][kNB];    // bucket counts of the work list of parity p
-    int32_t start[kNB];     // region starts (fixed)
-    int32_t init_cnt[kNB];  // round-0 bucket sizes
+    int32_t cnt[2][kNB];    // bucket counts of the work list of parity p (0: heavy rows)
+    int32_t init_cnt[kNB];  // round-0 bucket sizes (0: heavy rows)
     int32_t round;
     int32_t active;         // |W| for the coming round
     int32_t max_color;
     int32_t max_deg;
     uint32_t err;
-    uint32_t done_blocks;
-    int32_t mark_cnt;       // marking items of the round (block-bucket winners)
+    uint32_t barrier;       // arrivals at the grid barrier
+    int32_t mark_cnt;       // row pieces to be pushed (round 0: to be tested) by the whole grid
+    int32_t open_cnt;       // list pieces left open
+    int32_t open_rows;
     unsigned long long edges;
     unsigned long long conflicts;
-    long long heavy_entries;  // pending-list entries over all heavy rows
-    unsigned long long block_entries;  // adjacency entries of the block-bucket rows
+    long long heavy_entries;  // list entries over all heavy rows
     long long heavy_words;    // bitmap words over all heavy rows
 };
 
-// Heavy rows (the block- and warp-bucket rows): index of each, its list
-// (start, length) of the neighbors that were not fixed at its last look
-// (those above it in the total order, except for pulling warp-bucket rows)
-// and its forbidden bitmap (start, words), which the marking vertices reach
-// through bref.
+// Heavy rows (degree + X > 64), in the order of their region of the round-0
+// list: each one's list (start, length; bit 31: it lost round 0), its
+// forbidden bitmap (start, words), which the pushing vertices reach through
+// bref, and the queues of row and list pieces.
 struct HeavyRows {
-    int32_t* hid;
     int64_t* h_pbeg;
     int32_t* h_pcnt;
-    int64_t* h_bbeg;
-    int32_t* h_bwords;
     int32_t* pend;
     uint32_t* hbm;
-    uint64_t* bref;  // per vertex: bitmap_ref of its row, or all ones
-    // the rows of the round's block-bucket winners, in pieces of kMarkChunk
-    // entries (item: row piece start, winner's color, length), marked by
-    // the whole grid after the conflict launch
-    WorkItem* mark;
-    int64_t mark_cap;
-    // 1: the warp-bucket rows keep lists of all their neighbors not fixed and
-    // fold their bitmaps themselves (few block-bucket rows: marks would cost
-    // more than they save); only the block-bucket rows are marked then
-    int32_t pull_warp;
-    int32_t mark_bucket;  // the largest bucket that is marked
-    uint8_t* near;        // with pull_warp: 1 for a neighbor of a block-bucket row (it marks)
+    uint64_t* bref;      // per heavy vertex: bitmap_ref of its row
+    WorkItem* mark;      // row pieces: start, color (round 0: heavy row index), length
+    WorkItem* open;      // list pieces: start, index of the open row, length
+    WorkItem* open_row;  // open rows: the row's work item
+    int32_t* open_done;  // pieces done, counted up from minus their number
+    int32_t* open_lost;
+    int64_t mark_cap, open_cap, open_rows_cap;
 };
 
-constexpr int32_t kMarkChunk = 2048;
-constexpr uint8_t kBucketFixed = 0xFE;  // bucket byte of a fixed heavy row (marks skip it)
-constexpr unsigned long long kPullShare = 16;    // block-bucket rows below 1/16 of the entries: warp rows pull
+constexpr int32_t kPiece = 128;         // entries of a row piece (one warp, 4 per lane)
+constexpr int32_t kOpenPiece = 512;     // entries of a list piece
+constexpr uint8_t kBucketFixed = 0xFE;  // bucket byte of a fixed vertex (pushes skip it)
 
 struct SpecArgs {
     Graph g;
     int32_t X;
     uint64_t seed;
     Tuning tune;
-    int32_t* color;    // fixed colors (0 = in the work set)
-    uint64_t* key;     // (tentative color << 32) | priority
-    uint8_t* bucket;   // degree bucket per vertex
-    WorkItem* list0;   // work lists (ping-pong), bucket regions
+    int32_t* color;    // the output
+    uint32_t* prio;    // priorities, or (wide) 8-byte words: priority, tentative color | kUnfixed / fixed color
+    uint32_t* mlo;     // colors 1..32 and 33..64 of the fixed neighbors (light rows)
+    uint32_t* mhi;
+    uint8_t* bucket;   // degree bucket per vertex (0: heavy)
+    WorkItem* list0;   // work lists (ping-pong), bucket regions, the heavy rows' first
     WorkItem* list1;
     SpecCtrl* ctrl;
-    unsigned long long cond;  // WHILE-node handle (graph mode)
-    int32_t use_cond;
     int32_t round_limit;
+    int32_t max_rounds;   // rounds of this launch
     // batches: graph of every vertex and the graphs' descriptors (nullptr for
     // one graph), and the round in which every vertex kept its color
     const int32_t* graph_of;
     const BatchDesc* desc;
     int32_t* win_round;
-    int32_t* graph_heavy;  // batches: nonzero for a graph with heavy rows (its vertices mark)
-    // heavy rows (bucket 0), in device memory so that the arrays can be
-    // sized after the CUDA graph of the rounds has been built
-    struct HeavyRows* heavy;
+    HeavyRows heavy;
     // priority rule: 0 the random order; 1 Largest First (degree first);
     // 2 aRC (rank of the vertex's previous class first, from prio_rank[prio_old[v]])
     int32_t prio_kind;
     const int32_t* prio_rank;
     const int32_t* prio_old;
 };
+
+constexpr int32_t kUnfixed = INT32_MIN;
+__device__ __forceinline__ int32_t tent_of(int32_t x) { return x & INT32_MAX; }
+
+// A vertex's color word (tentative color | kUnfixed, or the fixed color) and
+// priority.  Up to kWideMax vertices they share an 8-byte word, so that the
+// test of a light row takes one gather; beyond, 8-byte words would not stay
+// in L2 (gathers measured: 280 G/s up to 67 MB, 266 G/s at 80 MB, 119 G/s at 134 MB), and the
+// color words (the output array) and the priorities are arrays of their own,
+// the priorities gathered only where a color matches.
+constexpr int64_t kWideMax = 10 << 20;
+template <bool kWide>
+__device__ __forceinline__ int32_t* color_word(const SpecArgs& a, int32_t v) {
+    return kWide ? reinterpret_cast<int32_t*>(a.prio) + 2 * static_cast<int64_t>(v) + 1 : a.color + v;
+}
+template <bool kWide>
+__device__ __forceinline__ uint32_t prio_word(const SpecArgs& a, int32_t v) {
+    return __ldg(a.prio + (kWide ? 2 * static_cast<int64_t>(v) : static_cast<int64_t>(v)));
+}
 
 // A vertex-visit key (16 bits, clamped) above the upper half of the random
 // priority; equal keys still fall back to the id.
@@ -127,13 +146,17 @@ __device__ __forceinline__ uint32_t ordered_prio(int64_t first_key, uint32_t p) 
     return (k << 16) | (p >> 16);
 }
 
+// u is above v in the random total order of Sec. 2.2: the larger priority,
+// then the larger id.
+__device__ __forceinline__ bool above(uint32_t pu, int32_t u, uint32_t pv, int32_t v) {
+    return pu > pv || (pu == pv && u > v);
+}
+
 // Bitmap words of a heavy row: colors 1 .. 32 * words, at least deg + 64.
 __host__ __device__ __forceinline__ int32_t heavy_words(int32_t deg) { return (deg + 64) / 32 + 2; }
 
-// Per-vertex reference to a heavy row's bitmap: (first word << 24) | words,
-// the words clamped to 2^24 - 1 on the marking and the reading side alike;
-// kNoBitmap for every other row.
-constexpr uint64_t kNoBitmap = ~0ull;
+// Reference to a heavy row's bitmap: (first word << 24) | words, the words
+// clamped to 2^24 - 1 on the pushing and the reading side alike.
 constexpr uint32_t kRefWords = (1u << 24) - 1u;
 __device__ __forceinline__ uint64_t bitmap_ref(long long first_word, long long words) {
     return (static_cast<uint64_t>(first_word) << 24) |
@@ -152,92 +175,74 @@ __device__ __forceinline__ uint32_t draw_index(const SpecArgs& a, int32_t v, int
 }
 
 // ---------------------------------------------------------------------------
-// Set-up: priorities, bucket sizes, then the round-0 work list (all vertices)
+// Set-up: priorities, round-0 tentative colors (nothing is colored yet, so
+// the j-th permissible color is j + 1 with no row read), bucket sizes, and
+// the heavy rows' region of the round-0 list.  (The light rows of round 0
+// are taken in id order and need no list.)
 // ---------------------------------------------------------------------------
+template <bool kWide>
 __global__ void __launch_bounds__(kBlock) k_spec_setup(SpecArgs a) {
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * kBlock;
-    int32_t my_max_deg = 0;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kBlock + threadIdx.x; i < a.g.n; i += stride) {
-        const int32_t v = static_cast<int32_t>(i);
-        int64_t beg;
-        int32_t deg;
-        row_of(a.g, v, beg, deg, &a.ctrl->err);
-        my_max_deg = max(my_max_deg, deg);
-        int32_t X = a.X, vl = v;
-        uint64_t seed = a.seed;
-        if (a.graph_of) {
-            const BatchDesc& d = a.desc[a.graph_of[v]];
-            X = d.X;
-            seed = d.seed;
-            vl = static_cast<int32_t>(v - d.base);
-        }
-        const int b = bucket_of(deg, X, a.tune);
-        a.bucket[v] = static_cast<uint8_t>(b);
-        if (b == 0) atomicAdd(&a.ctrl->block_entries, static_cast<unsigned long long>(deg));
-        if (b <= 1 && a.graph_of) {
-            int32_t* gh = a.graph_heavy + a.graph_of[v];
-            if (!*gh) atomicOr(gh, 1);
-        }
-        uint32_t p = prio_of(seed, vl);
-        if (a.prio_kind == 1) p = ordered_prio(deg, p);
-        else if (a.prio_kind == 2) p = ordered_prio(65535 - static_cast<int64_t>(a.prio_rank[a.prio_old[v]]), p);
-        // round 0's tentative color: nothing is colored yet, so the j-th
-        // permissible color is j + 1 (First Fit: 1)
-        const uint32_t j0 = (a.graph_of || a.X > 1) ? draw_index(a, v, 0) : 0u;
-        a.key[v] = (static_cast<uint64_t>(j0 + 1u) << 32) | p;
-        a.color[v] = 0;
-        const unsigned act = __activemask();
-        const unsigned peers = __match_any_sync(act, b);
-        const int leader = __ffs(peers) - 1;
-        if (lane_id() == leader) atomicAdd(&a.ctrl->init_cnt[b], __popc(peers));
-    }
-    warp_max(&a.ctrl->max_deg, my_max_deg);
-}
-
-__global__ void __launch_bounds__(kBlock) k_spec_fill(SpecArgs a) {
-    __shared__ int32_t s_start[kNB];
-    if (threadIdx.x == 0) {
-        int32_t acc = 0;
-        for (int b = 0; b < kNB; ++b) {
-            s_start[b] = acc;
-            acc += a.ctrl->init_cnt[b];
-        }
-        if (blockIdx.x == 0) {
-            for (int b = 0; b < kNB; ++b) a.ctrl->start[b] = s_start[b];
-            a.ctrl->active = acc;
-        }
-    }
+    __shared__ int32_t s_cnt[kNB];
+    if (threadIdx.x < kNB) s_cnt[threadIdx.x] = 0;
     __syncthreads();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kBlock;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * kBlock + threadIdx.x; i < a.g.n; i += stride) {
+    int32_t my_max_deg = 0;
+    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * kBlock; i0 < a.g.n; i0 += stride) {
+        const int64_t i = i0 + threadIdx.x;
+        const bool valid = i < a.g.n;
         const int32_t v = static_cast<int32_t>(i);
-        const int b = a.bucket[v];
-        int64_t beg;
-        int32_t deg;
-        row_of(a.g, v, beg, deg, &a.ctrl->err);
-        const unsigned act = __activemask();
-        const unsigned peers = __match_any_sync(act, b);
-        const int leader = __ffs(peers) - 1;
-        int32_t base = 0;
-        if (lane_id() == leader) base = atomicAdd(&a.ctrl->cnt[0][b], __popc(peers));
-        base = __shfl_sync(peers, base, leader);
-        store_item(a.list0 + s_start[b] + base + __popc(peers & ((1u << lane_id()) - 1u)), beg, v, deg);
+        int64_t beg = 0;
+        int32_t deg = 0, b = kNB;
+        if (valid) {
+            row_of(a.g, v, beg, deg, &a.ctrl->err);
+            my_max_deg = max(my_max_deg, deg);
+            int32_t X = a.X, vl = v;
+            uint64_t seed = a.seed;
+            if (a.graph_of) {
+                const BatchDesc& d = a.desc[a.graph_of[v]];
+                X = d.X;
+                seed = d.seed;
+                vl = static_cast<int32_t>(v - d.base);
+            }
+            b = bucket_of(deg, X, a.tune);
+            if (b == 1) b = 0;
+            a.bucket[v] = static_cast<uint8_t>(b);
+            uint32_t p = prio_of(seed, vl);
+            if (a.prio_kind == 1) p = ordered_prio(deg, p);
+            else if (a.prio_kind == 2) p = ordered_prio(65535 - static_cast<int64_t>(a.prio_rank[a.prio_old[v]]), p);
+            const uint32_t j0 = (a.graph_of || a.X > 1) ? draw_index(a, v, 0) : 0u;
+            const int32_t c0 = static_cast<int32_t>(j0 + 1u) | kUnfixed;
+            if (kWide) {
+                reinterpret_cast<uint2*>(a.prio)[v] = make_uint2(p, static_cast<uint32_t>(c0));
+            } else {
+                a.prio[v] = p;
+                a.color[v] = c0;
+            }
+            a.mlo[v] = 0u;
+            a.mhi[v] = 0u;
+        }
+        warp_append(b == 0, beg, v, deg, &a.ctrl->init_cnt[0], a.list0, 0);
+        for (int q = 2; q < kNB; ++q) {
+            const uint32_t m = __ballot_sync(kFull, b == q);
+            if (m && lane_id() == 0) atomicAdd(&s_cnt[q], __popc(m));
+        }
     }
+    warp_max(&a.ctrl->max_deg, my_max_deg);
+    __syncthreads();
+    if (threadIdx.x >= 2 && threadIdx.x < kNB && s_cnt[threadIdx.x])
+        atomicAdd(&a.ctrl->init_cnt[threadIdx.x], s_cnt[threadIdx.x]);
 }
 
-// Heavy rows: index, pending-list and bitmap offsets (exclusive scans over
-// the bucket-0 region of the round-0 list), one block.
 constexpr int kHeavyThreads = 1024;
 constexpr int kHeavyChunk = 8 * kHeavyThreads;  // rows per block of the two set-up kernels
 
-__device__ __forceinline__ void heavy_sizes(const SpecArgs& a, int32_t h, int32_t nh, int32_t& v,
+__device__ __forceinline__ void heavy_sizes(const SpecArgs& a, int32_t h, int32_t nh, WorkItem& it,
                                             long long& e, long long& wd) {
-    v = 0;
+    it = WorkItem{0, 0, 0};
     e = 0;
     wd = 0;
     if (h < nh) {
-        const WorkItem it = load_item(a.list0 + a.ctrl->start[0] + h);
-        v = it.v;
+        it = load_item(a.list0 + h);
         e = (static_cast<long long>(it.deg) + 3) & ~3ll;  // 16-byte aligned list starts
         wd = heavy_words(it.deg);
     }
@@ -250,9 +255,9 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_sums(SpecArgs a, int32_
     long long te = 0, tw = 0;
     const int32_t lo = blockIdx.x * kHeavyChunk;
     for (int32_t h = lo + static_cast<int32_t>(threadIdx.x); h < min(nh, lo + kHeavyChunk); h += kHeavyThreads) {
-        int32_t v;
+        WorkItem it;
         long long e, wd;
-        heavy_sizes(a, h, nh, v, e, wd);
+        heavy_sizes(a, h, nh, it, e, wd);
         te += e;
         tw += wd;
     }
@@ -274,12 +279,14 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_sums(SpecArgs a, int32_
         }
         sums[2 * blockIdx.x] = be;
         sums[2 * blockIdx.x + 1] = bw;
+        atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctrl->heavy_entries), static_cast<unsigned long long>(be));
+        atomicAdd(reinterpret_cast<unsigned long long*>(&a.ctrl->heavy_words), static_cast<unsigned long long>(bw));
     }
 }
 
-// Heavy rows: index, pending-list and bitmap offsets (exclusive scans over
-// the block- and warp-bucket regions of the round-0 list), a chunk of rows
-// per block, based at the sums of the chunks before it.
+// Heavy rows: list and bitmap offsets (exclusive scans over their region of
+// the round-0 list), a chunk of rows per block, based at the sums of the
+// chunks before it; and the row pieces of round 0.
 __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32_t nh, const long long* sums) {
     __shared__ long long s_e[kHeavyThreads / 32], s_w[kHeavyThreads / 32];
     __shared__ long long s_base_e, s_base_w;
@@ -292,28 +299,34 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
         }
         s_base_e = be;
         s_base_w = bw;
-        if (blockIdx.x == gridDim.x - 1) {
-            a.ctrl->heavy_entries = be + sums[2 * blockIdx.x];
-            a.ctrl->heavy_words = bw + sums[2 * blockIdx.x + 1];
-        }
     }
     __syncthreads();
     const int32_t lo = blockIdx.x * kHeavyChunk;
     const int32_t hi = min(nh, lo + kHeavyChunk);
+    const HeavyRows& hr = a.heavy;
     for (int32_t h0 = lo; h0 < hi; h0 += kHeavyThreads) {
         const int32_t h = h0 + static_cast<int32_t>(threadIdx.x);
-        int32_t v;
+        WorkItem it;
         long long e, wd;
-        heavy_sizes(a, h < hi ? h : nh, nh, v, e, wd);
+        heavy_sizes(a, h < hi ? h : nh, nh, it, e, wd);
+        const int32_t np = (it.deg + kPiece - 1) / kPiece;
         long long ie = e, iw = wd;  // warp inclusive scans
+        int32_t ip = np;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const long long ye = __shfl_up_sync(kFull, ie, d), yw = __shfl_up_sync(kFull, iw, d);
+            const int32_t yp = __shfl_up_sync(kFull, ip, d);
             if (l >= d) {
                 ie += ye;
                 iw += yw;
+                ip += yp;
             }
         }
+        int32_t pbase = 0;
+        if (l == 31 && ip) pbase = atomicAdd(&a.ctrl->mark_cnt, ip);
+        pbase = __shfl_sync(kFull, pbase, 31) + ip - np;
+        for (int32_t q = 0; q < np && pbase + q < hr.mark_cap; ++q)
+            store_item(hr.mark + pbase + q, it.beg + static_cast<int64_t>(q) * kPiece, h, min(kPiece, it.deg - q * kPiece));
         if (l == 31) {
             s_e[w] = ie;
             s_w[w] = iw;
@@ -329,13 +342,9 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
             tw += s_w[k];
         }
         if (h < hi) {
-            const HeavyRows& hr = *a.heavy;
-            hr.hid[v] = h;
             hr.h_pbeg[h] = be + ie - e;
-            hr.h_pcnt[h] = -1;
-            hr.h_bbeg[h] = bw + iw - wd;
-            hr.h_bwords[h] = static_cast<int32_t>(wd);
-            if (hr.bref && (h < a.ctrl->init_cnt[0] || !hr.pull_warp)) hr.bref[v] = bitmap_ref(bw + iw - wd, wd);
+            hr.h_pcnt[h] = 0;
+            hr.bref[it.v] = bitmap_ref(bw + iw - wd, wd);
         }
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -346,142 +355,202 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
     }
 }
 
-// Tile bookkeeping of one round, loaded by every block at kernel start.  In
-// the tentative launch a block-bucket row needs only one warp (its color
-// comes from its bitmap), so its tiles hold one row per warp there.
-struct RoundTiles {
-    int32_t cnt[kNB];
-    int32_t start[kNB];
-    int32_t prefix[kNB + 1];
-};
+// ---------------------------------------------------------------------------
+// The rounds
+// ---------------------------------------------------------------------------
+// Grid barrier of the cooperative launch: every block adds one arrival and
+// polls until all have (bounded: false, and kErrTimeout, once the limit has
+// run out; the blocks then all leave by the same limit).
+constexpr int32_t kBarrierPolls = 1 << 24;
 
-__device__ __forceinline__ int round_tile(int b, bool warp_heavy) {
-    return b == 0 && warp_heavy ? kWarps : bucket_tile(b);
-}
-
-__device__ __forceinline__ void load_round_tiles(const SpecCtrl* c, int par, bool warp_heavy,
-                                                 RoundTiles& rt) {
-    if (threadIdx.x == 0) {
-        int32_t acc = 0;
-        for (int b = 0; b < kNB; ++b) {
-            rt.cnt[b] = c->cnt[par][b];
-            rt.start[b] = c->start[b];
-            rt.prefix[b] = acc;
-            const int tile = round_tile(b, warp_heavy);
-            acc += (rt.cnt[b] + tile - 1) / tile;
+struct GridBarrier {
+    uint32_t target = 0;
+    __device__ __forceinline__ bool sync(SpecCtrl* c) {
+        __shared__ bool s_ok;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            target += gridDim.x;
+            __threadfence();
+            atomicAdd(&c->barrier, 1u);
+            bool ok = false;
+            for (int32_t i = 0; i < kBarrierPolls && !ok; ++i) {
+                uint32_t x;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(&c->barrier) : "memory");
+                ok = static_cast<int32_t>(x - target) >= 0;
+            }
+            if (!ok) atomicOr(&c->err, kErrTimeout);
+            __threadfence();
+            s_ok = ok;
         }
-        rt.prefix[kNB] = acc;
+        __syncthreads();
+        return s_ok;
     }
-    __syncthreads();
-}
-
-__device__ __forceinline__ int tile_bucket(const RoundTiles& rt, int32_t t) {
-    int b = 0;
-    while (t >= rt.prefix[b + 1]) ++b;
-    return b;
-}
-
-// Colors fixed before the round (the snapshot); 0 = in the work set.
-struct SnapshotFetch {
-    const int32_t* color;
-    __device__ __forceinline__ int32_t raw(int32_t u) const { return __ldg(color + u); }
-    __device__ __forceinline__ int32_t resolve(int32_t, int32_t x) const { return x; }
 };
 
-// ---------------------------------------------------------------------------
-// Keys, the total order and the heavy rows' bitmaps
-// ---------------------------------------------------------------------------
-// Bit 63 of a key marks a fixed vertex.  The conflict launch that fixes a
-// vertex sets it while other blocks of that launch may still read the key,
-// so every conflict test compares tentative colors with the bit masked off.
-// A neighbor fixed before the round never matches a tentative color (the
-// color was chosen against it), so the bit only tells the list scans which
-// entries to drop.
-constexpr uint64_t kKeyFixed = 1ull << 63;
-__device__ __forceinline__ uint32_t key_tent(uint64_t k) {
-    return static_cast<uint32_t>(k >> 32) & 0x7FFFFFFFu;
-}
-// u is above v in the random total order of Sec. 2.2: the larger priority,
-// then the larger id.
-__device__ __forceinline__ bool above(uint64_t ku, int32_t u, uint64_t kv, int32_t v) {
-    const uint32_t pu = static_cast<uint32_t>(ku), pv = static_cast<uint32_t>(kv);
-    return pu > pv || (pu == pv && u > v);
+// Items of the work lists are rewritten during the launch: no read-only loads.
+__device__ __forceinline__ WorkItem load_item_rw(const WorkItem* p) {
+    int4 r;
+    asm volatile("ld.global.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+                 : "l"(p));
+    WorkItem w;
+    w.beg = (static_cast<int64_t>(static_cast<uint32_t>(r.y)) << 32) | static_cast<uint32_t>(r.x);
+    w.v = r.z;
+    w.deg = r.w;
+    return w;
 }
 
-constexpr int kHeavyU = 4;  // list entries per thread per step of a heavy row
-constexpr int kCompactEvery = 16;  // power of two
-constexpr int kProbeMin = 4;       // lists longer than this many probes are probed
-constexpr int kHeavyStep = kHeavyU * kBlock;
-
-// Per-thread asynchronous 16-byte global -> shared copies (cp.async): a
-// thread stages the 4 list entries it will process next while it works on
-// the current ones, and waits only for its own copies (no barrier, no spin).
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
 }
 
-// Stages step `step` of a 16-byte aligned list (entries [i0, i0 +
-// kHeavyStep), thread t the 4 at i0 + 4t) into buf.  A copy may read up to 3
-// entries past cnt: lists are padded to 4 entries.
-__device__ __forceinline__ void stage_step(int32_t* buf, const int32_t* lst, int64_t i0, int64_t cnt) {
-    const int64_t i = i0 + 4 * static_cast<int64_t>(threadIdx.x);
-    if (i < cnt) cp_async16(buf + 4 * threadIdx.x, lst + i);
-    cp_async_commit();
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+    const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
 }
 
-// A vertex fixed at color c marks c in the bitmap of each heavy neighbor,
-// where it stays forbidden for the neighbor's later rounds (a neighbor's
-// bitmap thus holds the colors of all its neighbors fixed before the
-// round).  Lanes lane0, lane0 + stride, ... take the row's entries; a bit
-// already set is not written again.
-__device__ __forceinline__ void mark_color(const SpecArgs& a, const HeavyRows& hr, int64_t beg,
-                                           int32_t deg, int32_t c, int32_t lane0, int32_t stride) {
+constexpr int kHead = 128;              // list entries a warp looks at first, 4 per lane
+constexpr int kRefill = 16;             // dead ones among them that are worth replacing
+constexpr int32_t kLongList = 1024;     // longer lists are left open to the grid
+constexpr int32_t kPushInline = 128;    // longer winners' rows are pushed by the grid
+
+// What a warp keeps in shared memory: the heads of its current and next heavy
+// row's lists, or the items and ids of its current and next tile of light
+// rows; and the losers it has not yet written to the next list (one counter
+// update and one coalesced write per 16 or more of them).
+constexpr int kLightIds = 576;  // 36 per row with 2 lanes, 72 with 4
+struct __align__(16) WarpRounds {
+    union {
+        int32_t head[2][kHead];
+        struct {
+            WorkItem item[2][16];
+            int32_t ids[2][kLightIds];
+        } light;
+    };
+    WorkItem out[32];
+};
+
+// State of a warp over the launch.  Lane b keeps the count of bucket b's work
+// list and the start of its region.
+struct Rounds {
+    const SpecArgs& a;
+    WarpRounds& w;
+    int32_t lane_start, lane_cnt;
+    int32_t round;
+    int32_t par;
+    int32_t out_n;         // buffered losers
+    int32_t my_max;
+    unsigned long long edges;
+    __device__ __forceinline__ int32_t start(int b) const { return __shfl_sync(kFull, lane_start, b); }
+    __device__ __forceinline__ int32_t cnt(int b) const { return __shfl_sync(kFull, lane_cnt, b); }
+};
+
+__device__ __forceinline__ WorkItem* next_list(const Rounds& r) { return r.par ? r.a.list0 : r.a.list1; }
+__device__ __forceinline__ const WorkItem* this_list(const Rounds& r) { return r.par ? r.a.list1 : r.a.list0; }
+
+// Writes the buffered losers of bucket b to the next list (in one go: fewer
+// than 16 were there before the last lanes', at most 32, came in).
+__device__ __forceinline__ void flush_losers(Rounds& r, int b) {
+    const int l = lane_id();
+    const int32_t n = r.out_n;
+    if (n == 0) return;
+    int32_t base = 0;
+    if (l == 0) base = atomicAdd(&r.a.ctrl->cnt[r.par ^ 1][b], n);
+    base = __shfl_sync(kFull, base, 0) + r.start(b);
+    for (int32_t i = l; i < n; i += 32) {
+        const WorkItem x = r.w.out[i];
+        store_item(next_list(r) + base + i, x.beg, x.v, x.deg);
+    }
+    __syncwarp();
+    r.out_n = 0;
+}
+
+// The lanes with `want` add their row to the losers of bucket b (one bucket
+// at a time is buffered).  The whole warp calls it.
+__device__ __forceinline__ void add_losers(Rounds& r, int b, bool want, int64_t beg, int32_t v, int32_t deg) {
+    const uint32_t m = __ballot_sync(kFull, want);
+    if (m == 0) return;
+    if (want) r.w.out[r.out_n + __popc(m & ((1u << lane_id()) - 1u))] = WorkItem{beg, v, deg};
+    r.out_n += __popc(m);
+    __syncwarp();
+    if (r.out_n >= 16) flush_losers(r, b);
+}
+
+// A vertex fixed at color c sets its bit in the mask of each neighbor not yet
+// fixed, where it stays forbidden for the neighbor's later rounds.  Lanes
+// lane0, lane0 + stride, ... take the row's entries.  Without heavy rows the
+// bit is set with no look at the neighbor (a fixed one's mask is not read any
+// more); with them the bucket byte tells the kind (L2-resident), and a
+// bitmap's bit that is there already is not written again.
+template <bool kHeavy>
+__device__ __forceinline__ void push4(const SpecArgs& a, const int32_t (&u)[4], int32_t c) {
     const uint32_t bit = static_cast<uint32_t>(c - 1);
     const uint32_t mask = 1u << (bit & 31u);
-    // the bucket bytes (L2-resident) first; the bitmap reference only for
-    // heavy rows not fixed yet (a fixed heavy row's byte is kBucketFixed)
-    for_each_nbr<2, uint32_t, false>(
-        a.g, beg, deg, lane0, stride, [&](int32_t u) { return static_cast<uint32_t>(__ldcg(a.bucket + u)); },
-        [&](int32_t u, uint32_t b) {
-            if (b > hr.mark_bucket) return;
-            const uint64_t r = __ldg(hr.bref + u);
-            if (r == kNoBitmap || bit >= 32u * static_cast<uint32_t>(r & kRefWords)) return;
-            uint32_t* w = hr.hbm + (r >> 24) + (bit >> 5);
-            if (!(__ldcg(w) & mask)) atomicOr(w, mask);
-        },
-        &a.ctrl->err);
+    uint32_t* const light = bit < 32u ? a.mlo : a.mhi;
+    if constexpr (!kHeavy) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (u[i] >= 0) atomicOr(light + u[i], mask);
+    } else {
+        uint32_t b[4];
+        uint64_t ref[4];
+        uint32_t* w[4];
+        uint32_t have[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) b[i] = u[i] >= 0 ? __ldcg(a.bucket + u[i]) : kBucketFixed;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ref[i] = b[i] == 0 ? __ldg(a.heavy.bref + u[i]) : 0ull;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            w[i] = nullptr;
+            if (b[i] == 0) {
+                if (bit < 32u * static_cast<uint32_t>(ref[i] & kRefWords)) w[i] = a.heavy.hbm + (ref[i] >> 24) + (bit >> 5);
+            } else if (b[i] != kBucketFixed && bit < 64u) {
+                atomicOr(light + u[i], mask);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) have[i] = w[i] ? __ldcg(w[i]) : mask;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (!(have[i] & mask)) atomicOr(w[i], mask);
+    }
+}
+
+// A heavy row (or a piece of one), 4 entries per lane at a time.
+__device__ __forceinline__ void push_row(const SpecArgs& a, int64_t beg, int32_t deg, int32_t c) {
+    for (int32_t k0 = lane_id(); k0 < deg; k0 += 128) {
+        int32_t u[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) u[i] = k0 + 32 * i < deg ? load_nbr(a.g, beg + k0 + 32 * i, &a.ctrl->err) : -1;
+        push4<true>(a, u, c);
+    }
+}
+
+// Fixes v at color c (one lane calls it).  A row is examined twice in every
+// round that its vertex is in the work set (the method's choice and test;
+// the choice of round 0 is counted for all rows by the host).
+template <bool kHeavy, bool kWide>
+__device__ __forceinline__ void fix_color(Rounds& r, int32_t v, int32_t c, int32_t deg) {
+    r.a.color[v] = c;
+    if (kWide) *color_word<true>(r.a, v) = c;
+    if (kHeavy) r.a.bucket[v] = kBucketFixed;
+    r.my_max = max(r.my_max, c);
+    if (r.a.win_round) r.a.win_round[v] = r.round;
+    r.edges += static_cast<unsigned long long>(deg) * (2ull * static_cast<unsigned long long>(r.round) + 1ull);
 }
 
 // ---------------------------------------------------------------------------
-// Tentative coloring of W_r against the snapshot `color`
+// Tentative colors of W_r against the masks of the colors fixed before it
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void set_tent(const SpecArgs& a, int32_t v, int32_t c) {
-    const uint64_t k = a.key[v];
-    a.key[v] = (static_cast<uint64_t>(static_cast<uint32_t>(c)) << 32) | (k & 0xFFFFFFFFull);
-}
-template <int G, bool kRXF>
-__device__ __forceinline__ void tentative_group_tile(const SpecArgs& a, const RoundTiles& rt,
-                                                     const WorkItem* list, int b, int32_t first,
-                                                     int32_t round, unsigned long long& edges) {
-    const int gi = threadIdx.x / G, gl = threadIdx.x % G;
-    const int32_t k = first + gi;
-    const bool valid = k < rt.cnt[b];
-    WorkItem it{0, 0, 0};
-    uint32_t j = 0;
-    if (valid) {
-        it = load_item(list + rt.start[b] + k);
-        if (kRXF) j = draw_index(a, it.v, round);
-    }
-    const SnapshotFetch fetch{a.color};
-    // aligned 4-id reads, one chunk per lane per batch (measured: stencil coloring 1.40 ->
-    // 1.35 ms, RMAT-Good 30.5 -> 28.6 ms; the recoloring keeps single-id reads)
-    const int32_t c = choose_reg<G, 1, SnapshotFetch, true>(a.g, it.beg, it.deg, gl, j, fetch, &a.ctrl->err);
-    if (valid && gl == 0) {
-        set_tent(a, it.v, c);
-        edges += static_cast<unsigned long long>(it.deg);
-    }
-}
+// Colors fixed before the round, for the full-row fallback.
+template <bool kWide>
+struct SnapshotFetch {
+    const SpecArgs& a;
+    __device__ __forceinline__ int32_t raw(int32_t u) const { return __ldcg(color_word<kWide>(a, u)); }
+    __device__ __forceinline__ int32_t resolve(int32_t, int32_t x) const { return x; }  // negative: not fixed
+};
 
 // The j-th clear bit of a bitmap (bit b = color b + 1), one warp; -1: past it.
 __device__ __forceinline__ int32_t choose_from_bitmap(const uint32_t* bm, int32_t words, uint32_t j) {
@@ -505,667 +574,681 @@ __device__ __forceinline__ int32_t choose_from_bitmap(const uint32_t* bm, int32_
     return -1;
 }
 
-// Heavy row v in round >= 1 (one warp): its bitmap holds the colors of
-// every neighbor fixed before the round (marked by those neighbors).
-__device__ int32_t choose_bitmap_warp(const HeavyRows& hr, int32_t v, uint32_t j) {
-    const uint64_t r = hr.bref[v];
-    return choose_from_bitmap(hr.hbm + (r >> 24), static_cast<int32_t>(r & kRefWords), j);
-}
-
-// Warp-bucket row v in round >= 1 (the whole warp): it keeps the list of its
-// neighbors not fixed at its last look (the row itself before the first
-// look) and a bitmap of the colors of the others.  It folds the neighbors
-// fixed since into the bitmap (a shared window of 2048 colors, merged once)
-// and drops them from the list, compacted in place with ballots (a batch's
-// reads precede its writes, which land at or below every position the batch
-// read); then it takes the j-th permissible color from the bitmap.  -1: past
-// the bitmap.  The forbidden set is exactly that of a full row scan.
-__device__ int32_t choose_warp_pending(const SpecArgs& a, const WorkItem& it, uint32_t j, uint32_t* sbm) {
-    const int l = lane_id();
-    const HeavyRows& hr = *a.heavy;
-    const int32_t h = hr.hid[it.v];
-    const int32_t pc = hr.h_pcnt[h];
-    const int64_t cnt = pc < 0 ? static_cast<int64_t>(it.deg) : static_cast<int64_t>(pc);
-    const int32_t* src = pc < 0 ? a.g.idx + it.beg : hr.pend + hr.h_pbeg[h];
-    int32_t* dst = hr.pend + hr.h_pbeg[h];
-    uint32_t* bm = hr.hbm + hr.h_bbeg[h];
-    const int32_t words = hr.h_bwords[h];
-    const uint32_t bits = 32u * static_cast<uint32_t>(words);
-    const int32_t sw = min(words, kWarpBitmapWords);
-    const uint32_t sbits = 32u * static_cast<uint32_t>(sw);
-    for (int i = l; i < sw; i += 32) sbm[i] = 0u;
-    __syncwarp();
-    int32_t kept = 0;
-    for (int64_t i0 = 0; i0 < cnt; i0 += kHeavyU * 32) {
-        int32_t u[kHeavyU], c[kHeavyU];
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            const int64_t i = i0 + k * 32 + l;
-            u[k] = i < cnt ? src[i] : -1;
-        }
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            const int64_t i = i0 + k * 32 + l;
-            c[k] = -1;
-            if (i < cnt) {
-                if (u[k] < 0 || u[k] >= a.g.n) atomicOr(&a.ctrl->err, kErrBadGraph);
-                else c[k] = __ldg(a.color + u[k]);
+// A light row takes a thread (its color is among the first 64), a heavy one a
+// warp that searches its bitmap.
+template <bool kRXF, bool kHeavy, bool kWide>
+__device__ __forceinline__ void choose_phase(Rounds& r) {
+    const SpecArgs& a = r.a;
+    const WorkItem* list = this_list(r);
+    if constexpr (kHeavy) {
+        const int32_t n = r.cnt(0);
+        const int32_t W = gridDim.x * kWarps;
+        for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(n); k += W) {
+            const WorkItem it = load_item_rw(list + k);
+            const uint32_t j = kRXF ? draw_index(a, it.v, r.round) : 0u;
+            const uint64_t ref = __ldg(a.heavy.bref + it.v);
+            int32_t c = choose_from_bitmap(a.heavy.hbm + (ref >> 24), static_cast<int32_t>(ref & kRefWords), j);
+            if (c < 0) {  // past the bitmap's free colors (Random-X with a large X): the row in full
+                int64_t beg;
+                int32_t deg;
+                row_of(a.g, it.v, beg, deg, &a.ctrl->err);
+                c = choose_warp<4>(a.g, beg, deg, j, SnapshotFetch<kWide>{a}, reinterpret_cast<uint32_t*>(r.w.head), &a.ctrl->err);
             }
-        }
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            if (c[k] > 0) {
-                const uint32_t b = static_cast<uint32_t>(c[k] - 1);
-                if (b < sbits) atomicOr(&sbm[b >> 5], 1u << (b & 31));
-                else if (b < bits) atomicOr(bm + (b >> 5), 1u << (b & 31));
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            const unsigned bal = __ballot_sync(kFull, c[k] == 0);
-            if (c[k] == 0) dst[kept + __popc(bal & ((1u << l) - 1u))] = u[k];
-            kept += __popc(bal);
+            if (lane_id() == 0) *color_word<kWide>(a, it.v) = c | kUnfixed;
         }
     }
-    if (l == 0) hr.h_pcnt[h] = kept;
-    __syncwarp();
-    for (int i = l; i < sw; i += 32) {
-        const uint32_t x = sbm[i];
-        if (x) bm[i] = __ldcg(bm + i) | x;  // the warp owns these words this round
+    for (int b = 2; b < kNB; ++b) {
+        const int32_t n = r.cnt(b);
+        const WorkItem* lst = list + r.start(b);
+        for (uint32_t k = blockIdx.x * kBlock + threadIdx.x; k < static_cast<uint32_t>(n); k += gridDim.x * kBlock) {
+            const int32_t v = load_item_rw(lst + k).v;
+            const uint32_t lo = ~__ldcg(a.mlo + v);
+            int32_t c;
+            if (kRXF) {
+                const uint64_t f = (static_cast<uint64_t>(~__ldcg(a.mhi + v)) << 32) | lo;
+                c = select_bit64(f, draw_index(a, v, r.round)) + 1;
+            } else {
+                c = lo ? __ffs(lo) : 32 + __ffs(~__ldcg(a.mhi + v));
+            }
+            *color_word<kWide>(a, v) = c | kUnfixed;
+        }
     }
-    __syncwarp();
-    return choose_from_bitmap(bm, words, j);
 }
 
-template <bool kRXF>
-__global__ void __launch_bounds__(kBlock, 5) k_tentative(SpecArgs a) {
-    __shared__ uint32_t s_bm[kWarps][kWarpBitmapWords];
-    __shared__ RoundTiles rt;
-    const int32_t round = a.ctrl->round;
-    const int par = round & 1;
-    const WorkItem* list = par ? a.list1 : a.list0;
-    if (blockIdx.x == 0 && threadIdx.x < kNB) a.ctrl->cnt[par ^ 1][threadIdx.x] = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctrl->mark_cnt = 0;  // the last round's were marked
-    if (round == 0) {  // tentative colors set with the priorities (every row counted once)
-        if (blockIdx.x == 0 && threadIdx.x == 0)
-            atomicAdd(&a.ctrl->edges, static_cast<unsigned long long>(a.g.nnz));
+// ---------------------------------------------------------------------------
+// Conflict test of the light rows, G lanes each
+// ---------------------------------------------------------------------------
+// Of 4 ids, the first of them k places into the row, the row's own; a bad
+// one is flagged and dropped (-1).
+__device__ __forceinline__ void in_row(const Graph& g, int32_t k, int32_t deg, int32_t (&u)[4], uint32_t* err) {
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool mine = static_cast<uint32_t>(k + i) < static_cast<uint32_t>(deg);
+        const bool fits = static_cast<uint32_t>(u[i]) < static_cast<uint32_t>(g.n);
+        bad |= mine && !fits;
+        if (!mine || !fits) u[i] = -1;
+    }
+    if (bad) atomicOr(err, kErrBadGraph);
+}
+
+// The 4 ids of piece c of a row (aligned 16-byte pieces, or single reads), -1
+// where the row has none.
+__device__ __forceinline__ void row_piece(const Graph& g, int64_t beg, int32_t deg, int32_t c, int32_t (&u)[4],
+                                          uint32_t* err) {
+    const int32_t k = 4 * c - (g.vec ? static_cast<int32_t>(beg & 3) : 0);
+    const int64_t e0 = beg + k, end = beg + deg;
+    if (g.vec && e0 + 4 <= g.nnz) {
+        const int4 q = ld_stream4(g.idx + e0);
+        u[0] = q.x;
+        u[1] = q.y;
+        u[2] = q.z;
+        u[3] = q.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) u[i] = e0 + i < end ? ld_stream(g.idx + e0 + i) : -1;
+    }
+    in_row(g, k, deg, u, err);
+}
+__device__ __forceinline__ int32_t row_pieces(const Graph& g, int64_t beg, int32_t deg) {
+    return ((g.vec ? static_cast<int32_t>(beg & 3) : 0) + deg + 3) >> 2;
+}
+
+// Does one of the 4 neighbors u have v's tentative color tv and stand above
+// v?  With `all` every neighbor's color matches (First Fit's round 0).
+// Bit i of `live`: u[i] is not fixed yet.
+template <bool kWide>
+__device__ __forceinline__ bool beaten(const SpecArgs& a, const int32_t (&u)[4], int32_t v, int32_t tv, bool all,
+                                       uint32_t& live) {
+    bool lose = false;
+    live = 0;
+    if constexpr (kWide) {
+        const uint2* key = reinterpret_cast<const uint2*>(a.prio);
+        uint2 x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = u[i] >= 0 ? key[u[i]] : make_uint2(0u, 0u);
+        const uint32_t pv = prio_word<true>(a, v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            lose |= u[i] >= 0 && (all || tent_of(static_cast<int32_t>(x[i].y)) == tv) && above(x[i].x, u[i], pv, v);
+            live |= (x[i].y >> 31) << i;
+        }
+    } else {
+        bool match[4];
+        if (all) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) match[i] = u[i] >= 0;
+            live = 15u;
+        } else {
+            int32_t x[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] = u[i] >= 0 ? a.color[u[i]] : 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                match[i] = u[i] >= 0 && tent_of(x[i]) == tv;
+                live |= (static_cast<uint32_t>(x[i]) >> 31) << i;
+            }
+        }
+        uint32_t p[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i] = match[i] ? prio_word<false>(a, u[i]) : 0u;
+        if (match[0] || match[1] || match[2] || match[3]) {
+            const uint32_t pv = prio_word<false>(a, v);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) lose |= match[i] && above(p[i], u[i], pv, v);
+        }
+    }
+    return lose;
+}
+
+// The lanes with `want` add their light row to the losers (of bucket b;
+// round 0: of its own).
+template <bool kRound0>
+__device__ __forceinline__ void light_losers(Rounds& r, int b, bool want, const WorkItem& it) {
+    if (!kRound0) {
+        add_losers(r, b, want, it.beg, it.v, it.deg);
         return;
     }
-    load_round_tiles(a.ctrl, par, true, rt);
-    unsigned long long edges = 0;
-    const SnapshotFetch fetch{a.color};
-    for (int32_t t = blockIdx.x; t < rt.prefix[kNB]; t += gridDim.x) {
-        const int b = tile_bucket(rt, t);
-        const int32_t first = (t - rt.prefix[b]) * round_tile(b, true);
-        switch (b) {
-        case 0:
-        case 1: {  // heavy rows, one warp each
-            const int w = threadIdx.x >> 5;
-            const int32_t k = first + w;
-            if (k < rt.cnt[b]) {
-                const WorkItem it = load_item(list + rt.start[b] + k);
-                const uint32_t j = kRXF ? draw_index(a, it.v, round) : 0u;
-                // a marking row's item holds its list (ListItem), and the
-                // conflict launch counts this visit's entries with its own
-                const bool marked = b == 0 || !a.heavy->pull_warp;
-                int32_t c = marked ? choose_bitmap_warp(*a.heavy, it.v, j) : choose_warp_pending(a, it, j, s_bm[w]);
-                // past the bitmap's free colors (Random-X with a large X): the row in full
-                if (c < 0) {
-                    int64_t rbeg = it.beg;
-                    int32_t rdeg = it.deg;
-                    if (marked) row_of(a.g, it.v, rbeg, rdeg, &a.ctrl->err);
-                    c = choose_warp<4>(a.g, rbeg, rdeg, j, fetch, s_bm[w], &a.ctrl->err);
-                }
-                if (lane_id() == 0) {
-                    set_tent(a, it.v, c);
-                    if (!marked) edges += static_cast<unsigned long long>(it.deg);
+    const int own = bucket_of(it.deg, 1, r.a.tune);  // (a light row's bucket does not depend on X)
+    add_losers(r, kNB - 1, want && own == kNB - 1, it.beg, it.v, it.deg);
+    for (int q = 2; q < kNB - 1; ++q)
+        warp_append(want && own == q, it.beg, it.v, it.deg, &r.a.ctrl->cnt[1][q], r.a.list1, r.start(q));
+}
+
+// The light rows of bucket b, or (round 0) all of them in id order, where
+// consecutive rows are consecutive in the adjacency: a warp takes 32 / G rows
+// at a time.  A row's group tests one piece per lane first (most rows of an
+// early round lose to one of the first neighbors), then two at a time, until
+// it has found a neighbor that the row loses to.  The items (round 0: offsets
+// and buckets) of the tile after the next and the ids of the next are on
+// their way to shared memory meanwhile.  Round 0 looks at every id, for the
+// checks of the adjacency; colors and priorities are gathered until the row
+// has lost.
+template <int G, bool kRXF, bool kHeavy, bool kWide, bool kRound0>
+__device__ __forceinline__ void light_rows(Rounds& r, int b) {
+    const SpecArgs& a = r.a;
+    constexpr int R = 32 / G;
+    constexpr int kRow = kLightIds / R;  // ids of a row in the stage
+    static_assert(R <= 16 && kRow % 4 == 0, "16-byte rows");
+    const int l = lane_id(), gi = l / G, gl = l % G;
+    const int32_t cnt = kRound0 ? a.g.n : r.cnt(b);
+    const int32_t tiles = cnt / R + (cnt % R != 0);
+    const int32_t W = gridDim.x * kWarps;
+    int32_t t = blockIdx.x * kWarps + (threadIdx.x >> 5);
+    if (t >= tiles) return;
+    const WorkItem* lst = kRound0 ? nullptr : this_list(r) + r.start(b);
+    auto& st = r.w.light;
+    auto stage_items = [&](int32_t tt, int slot) {
+        if (kRound0) {  // the R + 1 offsets
+            int64_t* off = reinterpret_cast<int64_t*>(st.item[slot]);
+            if (l <= min(R, cnt - tt * R)) cp_async8(off + l, a.g.off + tt * R + l);
+        } else if (l < min(R, cnt - tt * R)) {
+            cp_async16(&st.item[slot][l], lst + tt * R + l);
+        }
+    };
+    auto item = [&](int32_t tt, int slot) {
+        WorkItem it{0, 0, 0};
+        if (gi < cnt - tt * R) {
+            if (kRound0) {
+                const int64_t* off = reinterpret_cast<const int64_t*>(st.item[slot]);
+                const int64_t len = off[gi + 1] - off[gi];  // checked by the set-up
+                if (len < 64) it = WorkItem{off[gi], tt * R + gi, static_cast<int32_t>(len)};
+            } else {
+                it = st.item[slot][gi];
+            }
+        }
+        return it;
+    };
+    auto stage_ids = [&](int32_t tt, int slot) {
+        if (!a.g.vec) return;
+        const WorkItem it = item(tt, slot);
+        const int32_t np = min(row_pieces(a.g, it.beg, it.deg), kRow / 4);
+        for (int32_t c = gl; c < np; c += G) {
+            const int64_t e = (it.beg & ~static_cast<int64_t>(3)) + 4 * static_cast<int64_t>(c);
+            if (e + 4 <= a.g.nnz) cp_async16(&st.ids[slot][gi * kRow + 4 * c], a.g.idx + e);
+        }
+    };
+    stage_items(t, 0);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncwarp();
+    stage_ids(t, 0);
+    if (tiles - t > W) stage_items(t + W, 1);
+    cp_async_commit();
+    int next_bucket = b;
+    if (kRound0 && kHeavy) next_bucket = gi < cnt - t * R ? a.bucket[t * R + gi] : 0;
+    for (int slot = 0;; slot ^= 1) {
+        const int bucket = next_bucket;
+        if (kRound0 && kHeavy && tiles - t > W) next_bucket = gi < cnt - (t + W) * R ? a.bucket[(t + W) * R + gi] : 0;
+        cp_async_wait<0>();
+        __syncwarp();
+        const WorkItem it = item(t, slot);
+        __syncwarp();  // the slot's items are read: the ones after the next tile's may land there
+        const bool valid = gi < cnt - t * R && (!kRound0 || !kHeavy || bucket != 0);
+        const int32_t left = tiles - t;
+        if (left > W) {
+            stage_ids(t + W, slot ^ 1);
+            if (left - W > W) stage_items(t + 2 * W, slot);
+        }
+        cp_async_commit();
+
+        const int32_t shift = static_cast<int32_t>(it.beg & 3);
+        const int32_t staged = a.g.vec ? static_cast<int32_t>(min(static_cast<int64_t>(kRow / 4), (a.g.nnz - it.beg + shift) >> 2)) : 0;
+        auto piece = [&](int32_t c, int32_t (&u)[4]) {
+            if (c < staged) {
+                const int4 q = *reinterpret_cast<const int4*>(&st.ids[slot][gi * kRow + 4 * c]);
+                u[0] = q.x;
+                u[1] = q.y;
+                u[2] = q.z;
+                u[3] = q.w;
+                in_row(a.g, 4 * c - shift, it.deg, u, &a.ctrl->err);
+            } else {
+                row_piece(a.g, it.beg, it.deg, c, u, &a.ctrl->err);
+            }
+        };
+        const bool all = kRound0 && !kRXF;
+        const int32_t tv = !valid ? 0 : all ? 1 : tent_of(*color_word<kWide>(a, it.v));
+        const int32_t np = valid ? row_pieces(a.g, it.beg, it.deg) : 0;
+        bool lost = false, loop = false;
+        uint64_t live = 0;  // of this lane's pieces, 4 bits each: neighbors not fixed yet (the first 16 pieces)
+        int pieces = 0;
+        for (int32_t c0 = 0, step = G;; c0 += step, step = 2 * G) {
+            const bool on = c0 < np && (kRound0 || !lost);
+            if (!__any_sync(kFull, on)) break;
+            int32_t u[2][4];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) u[q][i] = -1;
+                const int32_t c = c0 + q * G + gl;
+                if (on && c < np && q * G < step) piece(c, u[q]);
+                if (kRound0) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (u[q][i] == it.v && valid) {  // uncolorable (Sec. 1): reported as a malformed graph
+                            loop = true;
+                            u[q][i] = -1;
+                        }
+                        if (lost) u[q][i] = -1;
+                    }
                 }
             }
+            uint32_t lv;
+            bool lose = beaten<kWide>(a, u[0], it.v, tv, all, lv);
+            live |= static_cast<uint64_t>(lv) << pieces;
+            pieces += 4;
+            if (c0 > 0) {
+                lose |= beaten<kWide>(a, u[1], it.v, tv, all, lv);
+                live |= static_cast<uint64_t>(lv) << pieces;
+                pieces += 4;
+            }
+            lost |= group_any<G>(lose);
+        }
+        if (kRound0 && loop) atomicOr(&a.ctrl->err, kErrBadGraph);
+        if (valid && !lost) {
+            if (gl == 0) fix_color<kHeavy, kWide>(r, it.v, tv, it.deg);
+            for (int32_t c = gl, q = 0; c < np; c += G, ++q) {
+                int32_t u[4];
+                piece(c, u);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (q < 16 && !(live >> (4 * q + i) & 1u)) u[i] = -1;
+                push4<kHeavy>(a, u, tv);
+            }
+        }
+        light_losers<kRound0>(r, b, valid && lost && gl == 0, it);
+        if (left <= W) break;
+        t += W;
+    }
+    cp_async_wait<0>();
+    __syncwarp();
+    flush_losers(r, kRound0 ? kNB - 1 : b);
+}
+
+// ---------------------------------------------------------------------------
+// Conflict test of the heavy rows, a warp each
+// ---------------------------------------------------------------------------
+// ListItem: the work item of a heavy row holds its list, not its row: beg =
+// the list's start in pend, deg = its length.
+
+// A heavy winner (the whole warp): fixed, and its row pushed or queued for
+// the whole grid.
+template <bool kWide>
+__device__ __forceinline__ void heavy_win(Rounds& r, int32_t v, int32_t c, int64_t beg, int32_t deg) {
+    const SpecArgs& a = r.a;
+    const int l = lane_id();
+    if (l == 0) fix_color<true, kWide>(r, v, c, deg);
+    if (deg <= kPushInline) {
+        push_row(a, beg, deg, c);
+        return;
+    }
+    const int32_t np = (deg + kPiece - 1) / kPiece;
+    int32_t pos = 0;
+    if (l == 0) pos = atomicAdd(&a.ctrl->mark_cnt, np);
+    pos = __shfl_sync(kFull, pos, 0);
+    for (int32_t q = l; q < np && pos + q < a.heavy.mark_cap; q += 32)  // (the capacity holds every piece of every row)
+        store_item(a.heavy.mark + pos + q, beg + static_cast<int64_t>(q) * kPiece, c, min(kPiece, deg - q * kPiece));
+}
+
+// Round 0, a piece of a heavy row (the whole warp): its share of the test,
+// and the row's list -- the neighbors above it in the total order, the only
+// ones that can beat it in a later round (their order is free, so the pieces
+// of a row just take places).
+template <bool kRXF, bool kWide>
+__device__ __forceinline__ void heavy_round0_piece(Rounds& r, const WorkItem& it) {
+    const SpecArgs& a = r.a;
+    const int l = lane_id();
+    const int32_t h = it.v;
+    const int32_t v = load_item(a.list0 + h).v;
+    int32_t* dst = a.heavy.pend + __ldg(a.heavy.h_pbeg + h);
+    const uint32_t pv = prio_word<kWide>(a, v);
+    const int32_t tv = kRXF ? tent_of(*color_word<kWide>(a, v)) : 1;
+    bool lose = false, loop = false;
+    {
+        int32_t u[4];
+        uint32_t p[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int32_t k = 32 * i + l;
+            u[i] = k < it.deg ? load_nbr(a.g, it.beg + k, &a.ctrl->err) : -1;
+            if (u[i] == v) {
+                loop = true;
+                u[i] = -1;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i] = u[i] >= 0 ? prio_word<kWide>(a, u[i]) : 0u;
+        uint32_t keep[4];
+        int32_t total = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool up = u[i] >= 0 && above(p[i], u[i], pv, v);
+            if (up && (!kRXF || tent_of(*color_word<kWide>(a, u[i])) == tv)) lose = true;
+            keep[i] = __ballot_sync(kFull, up);
+            total += __popc(keep[i]);
+        }
+        int32_t pos = 0;
+        if (l == 0 && total) pos = atomicAdd(a.heavy.h_pcnt + h, total) & INT32_MAX;
+        pos = __shfl_sync(kFull, pos, 0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (keep[i] >> l & 1u) dst[pos + __popc(keep[i] & ((1u << l) - 1u))] = u[i];
+            pos += __popc(keep[i]);
+        }
+    }
+    if (loop) atomicOr(&a.ctrl->err, kErrBadGraph);
+    if (__any_sync(kFull, lose) && l == 0) atomicOr(a.heavy.h_pcnt + h, INT32_MIN);
+}
+
+// Round 0, once every piece is done: winners and losers (32 rows per warp).
+template <bool kWide>
+__device__ __forceinline__ void heavy_round0_close(Rounds& r) {
+    const SpecArgs& a = r.a;
+    const int l = lane_id();
+    const int32_t nh = a.ctrl->init_cnt[0];
+    const int32_t W = gridDim.x * kWarps;
+    for (int32_t h0 = (blockIdx.x * kWarps + (threadIdx.x >> 5)) * 32; h0 < nh; h0 += W * 32) {
+        const int32_t h = h0 + l;
+        WorkItem it{0, 0, 0};
+        int32_t pc = 0, c = 0;
+        int64_t pb = 0;
+        if (h < nh) {
+            it = load_item(a.list0 + h);
+            pc = __ldcg(a.heavy.h_pcnt + h);
+            pb = __ldg(a.heavy.h_pbeg + h);
+            c = tent_of(*color_word<kWide>(a, it.v));
+        }
+        warp_append(h < nh && pc < 0, pb, it.v, pc & INT32_MAX, &a.ctrl->cnt[1][0], a.list1, 0);
+        for (uint32_t m = __ballot_sync(kFull, h < nh && pc >= 0); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            heavy_win<kWide>(r, __shfl_sync(kFull, it.v, src), __shfl_sync(kFull, c, src), __shfl_sync(kFull, it.beg, src),
+                      __shfl_sync(kFull, it.deg, src));
+        }
+    }
+}
+
+// Is one of the list entries [k0, k0 + 256) of the lane's tentative color tv?
+// (An entry was above v and unfixed at the last look; one fixed before the
+// round never matches, the color was chosen against it.)
+template <bool kWide>
+__device__ __forceinline__ bool list_hit(const SpecArgs& a, const int32_t* lst, int32_t k0, int32_t len, int32_t tv) {
+    int32_t u[8], x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int32_t k = k0 + 32 * i + lane_id();
+        u[i] = k < len ? __ldcg(lst + k) : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = u[i] >= 0 ? *color_word<kWide>(a, u[i]) : 0;
+    bool hit = false;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) hit |= tent_of(x[i]) == tv;  // tv >= 1
+    return hit;
+}
+
+// A long list none of whose first entries beat its row is left to the whole
+// grid, in pieces.
+__device__ __forceinline__ void leave_open(Rounds& r, const WorkItem& it) {
+    const SpecArgs& a = r.a;
+    const int l = lane_id();
+    const int32_t np = (it.deg + kOpenPiece - 1) / kOpenPiece;
+    int32_t slot = 0, pos = 0;
+    if (l == 0) {
+        slot = atomicAdd(&a.ctrl->open_rows, 1);
+        pos = atomicAdd(&a.ctrl->open_cnt, np);
+        store_item(a.heavy.open_row + slot, it.beg, it.v, it.deg);
+        a.heavy.open_done[slot] = -np;
+        a.heavy.open_lost[slot] = 0;
+    }
+    slot = __shfl_sync(kFull, slot, 0);
+    pos = __shfl_sync(kFull, pos, 0);
+    for (int32_t q = l; q < np; q += 32)
+        store_item(a.heavy.open + pos + q, it.beg + static_cast<int64_t>(q) * kOpenPiece, slot,
+                   min(kOpenPiece, it.deg - q * kOpenPiece));
+}
+
+// Rounds from 1 on.  The first kHead entries of a list come first: most rows
+// of a dense core lose in every round (98 % of the visits to R-MAT 24's rows
+// beyond 1024 entries), nearly always to one of the first 32.  The items and
+// the heads of a warp's next rows are on their way while it tests one.  A
+// list of at most kHead entries is compacted in place; on a longer one the
+// entries of the head that were fixed since are replaced by the list's last
+// ones once there are kRefill, so that the head stays alive and the list
+// shrinks without a pass over it (it stays a superset of the neighbors above
+// v not fixed; its order is free).
+template <bool kWide>
+__device__ __forceinline__ void heavy_rows(Rounds& r) {
+    const SpecArgs& a = r.a;
+    const WorkItem* list = this_list(r);
+    const int l = lane_id();
+    const int32_t n = r.cnt(0);
+    const int32_t W = gridDim.x * kWarps;
+    int32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5);
+    if (k >= n) return;
+    auto stage = [&](const WorkItem& it, int slot) {
+        if (4 * l < it.deg) cp_async16(&r.w.head[slot][4 * l], a.heavy.pend + it.beg + 4 * l);
+    };
+    WorkItem it = load_item_rw(list + k), nx{0, 0, 0};
+    if (k + W < n) nx = load_item_rw(list + k + W);
+    stage(it, 0);
+    cp_async_commit();
+    for (int slot = 0;; slot ^= 1) {
+        cp_async_wait<0>();
+        __syncwarp();
+        const bool more = n - k > W;
+        if (more) stage(nx, slot ^ 1);
+        cp_async_commit();
+        WorkItem after{0, 0, 0};
+        if (more && n - k - W > W) after = load_item_rw(list + k + 2 * W);
+
+        const int32_t pc = it.deg;
+        int32_t* lst = a.heavy.pend + it.beg;
+        const int4 q = *reinterpret_cast<const int4*>(&r.w.head[slot][4 * l]);
+        const int32_t u[4] = {q.x, q.y, q.z, q.w};
+        int32_t x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = 4 * l + i < pc ? *color_word<kWide>(a, u[i]) : kUnfixed;
+        const int32_t tv = tent_of(*color_word<kWide>(a, it.v));
+        bool mine = false;
+        uint32_t dead[4];
+        int32_t nd = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            mine |= tent_of(x[i]) == tv;
+            dead[i] = __ballot_sync(kFull, x[i] >= 0);
+            nd += __popc(dead[i]);
+        }
+        bool lost = __any_sync(kFull, mine);
+        int32_t len = pc;
+        if (pc <= kHead) {
+            if (lost && nd) {
+                int32_t kept = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t live = __ballot_sync(kFull, 4 * l + i < pc && x[i] < 0);
+                    if (live >> l & 1u) lst[kept + __popc(live & ((1u << l) - 1u))] = u[i];
+                    kept += __popc(live);
+                }
+                len = kept;
+            }
+        } else {
+            if (nd >= kRefill) {
+                const int32_t moved = min(nd, pc - kHead);
+                int32_t d = 0;  // rank of the entry among the dead ones
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int32_t rank = d + __popc(dead[i] & ((1u << l) - 1u));
+                    if ((dead[i] >> l & 1u) && rank < moved) lst[4 * l + i] = __ldcg(lst + pc - 1 - rank);
+                    d += __popc(dead[i]);
+                }
+                len = pc - moved;
+            }
+        }
+        bool open = false;
+        if (!lost && pc > kHead) {
+            // (a refill left the entries it moved in their old places, which are tested here)
+            if (pc <= kLongList) {
+                for (int32_t k0 = kHead; k0 < pc && !lost; k0 += 256) lost = __any_sync(kFull, list_hit<kWide>(a, lst, k0, pc, tv));
+            } else {
+                open = true;  // (the shortened list holds every live entry)
+                leave_open(r, WorkItem{it.beg, it.v, len});
+            }
+        }
+        add_losers(r, 0, l == 0 && lost, it.beg, it.v, len);
+        if (!lost && !open) {
+            int64_t beg;
+            int32_t deg;
+            row_of(a.g, it.v, beg, deg, &a.ctrl->err);
+            heavy_win<kWide>(r, it.v, tv, beg, deg);
+        }
+        if (!more) break;
+        it = nx;
+        nx = after;
+        k += W;
+    }
+    flush_losers(r, 0);
+}
+
+// The open lists' pieces: the warp that finishes a row's last piece closes
+// the row (acquire-release on the row's counter orders the other pieces'
+// findings before it).
+template <bool kWide>
+__device__ __forceinline__ void open_phase(Rounds& r) {
+    const SpecArgs& a = r.a;
+    const int l = lane_id();
+    const int32_t n = __ldcg(&a.ctrl->open_cnt);
+    const int32_t W = gridDim.x * kWarps;
+    for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(n); k += W) {
+        const WorkItem it = load_item_rw(a.heavy.open + k);
+        const WorkItem row = load_item_rw(a.heavy.open_row + it.v);
+        if (!__ldcg(a.heavy.open_lost + it.v)) {
+            const int32_t tv = tent_of(*color_word<kWide>(a, row.v));
+            const int32_t* lst = a.heavy.pend + it.beg;
+            bool lost = false;
+            for (int32_t k0 = 0; k0 < it.deg && !lost; k0 += 256) lost = __any_sync(kFull, list_hit<kWide>(a, lst, k0, it.deg, tv));
+            if (lost && l == 0) atomicExch(a.heavy.open_lost + it.v, 1);
+        }
+        __syncwarp();
+        int last = 0;
+        if (l == 0) last = add_acq_rel(a.heavy.open_done + it.v) == -1;
+        if (!__shfl_sync(kFull, last, 0)) continue;
+        __syncwarp();
+        if (__ldcg(a.heavy.open_lost + it.v)) {
+            if (l == 0) {
+                const int32_t pos = atomicAdd(&a.ctrl->cnt[r.par ^ 1][0], 1);
+                store_item(next_list(r) + pos, row.beg, row.v, row.deg);
+            }
+        } else {
+            int64_t beg;
+            int32_t deg;
+            row_of(a.g, row.v, beg, deg, &a.ctrl->err);
+            heavy_win<kWide>(r, row.v, tent_of(*color_word<kWide>(a, row.v)), beg, deg);
+        }
+    }
+}
+
+// The long winners' rows, in pieces.
+__device__ __forceinline__ void push_phase(Rounds& r) {
+    const SpecArgs& a = r.a;
+    const int32_t n = static_cast<int32_t>(min(static_cast<int64_t>(__ldcg(&a.ctrl->mark_cnt)), a.heavy.mark_cap));
+    const int32_t W = gridDim.x * kWarps;
+    for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(n); k += W) {
+        const WorkItem it = load_item_rw(a.heavy.mark + k);
+        push_row(a, it.beg, it.deg, it.v);
+    }
+}
+
+template <bool kRXF, bool kHeavy, bool kWide>
+__device__ __forceinline__ void test_phase(Rounds& r) {
+    const SpecArgs& a = r.a;
+    if (r.round == 0) {
+        if constexpr (kHeavy) {
+            const int32_t np = static_cast<int32_t>(min(static_cast<int64_t>(a.ctrl->mark_cnt), a.heavy.mark_cap));
+            const int32_t W = gridDim.x * kWarps;
+            for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(np); k += W)
+                heavy_round0_piece<kRXF, kWide>(r, load_item(a.heavy.mark + k));
+        }
+        light_rows<2, kRXF, kHeavy, kWide, true>(r, 0);
+        return;
+    }
+    if constexpr (kHeavy) heavy_rows<kWide>(r);
+    for (int b = 2; b < kNB; ++b) {
+        if (r.cnt(b) == 0) continue;
+        switch (b) {
+        case 2: light_rows<32, kRXF, kHeavy, kWide, false>(r, 2); break;
+        case 3: light_rows<16, kRXF, kHeavy, kWide, false>(r, 3); break;
+        case 4: light_rows<8, kRXF, kHeavy, kWide, false>(r, 4); break;
+        case 5: light_rows<4, kRXF, kHeavy, kWide, false>(r, 5); break;
+        default: light_rows<2, kRXF, kHeavy, kWide, false>(r, 6); break;
+        }
+    }
+}
+
+// kHeavy: the graph has heavy rows (the form without them returns at once on
+// such a graph, and is launched before the host knows).
+template <bool kRXF, bool kHeavy, bool kWide>
+__global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant__ SpecArgs a) {
+    __shared__ WarpRounds s_w[kWarps];
+    static_assert(sizeof(WarpRounds::head) >= kWarpBitmapWords * 4, "the full-row fallback's bitmap");
+    SpecCtrl* const c = a.ctrl;
+    if (c->err || (!kHeavy && c->init_cnt[0] > 0)) return;
+    const int warp = threadIdx.x >> 5;
+    const int l = lane_id();
+    const int32_t mine = l < kNB && l != 1 ? c->init_cnt[l] : 0;
+    Rounds r{a, s_w[warp],
+             static_cast<int32_t>(warp_inclusive_scan(static_cast<uint32_t>(mine))) - mine,
+             l < kNB ? c->cnt[c->round & 1][l] : 0, c->round, 0, 0, 0, 0ull};
+    GridBarrier bar;
+    unsigned long long conflicts = 0;
+    int32_t total = 0;
+    bool ok = true;
+    for (int32_t done = 0; done < a.max_rounds; ++done) {
+        r.par = r.round & 1;
+        if (r.round > 0) {
+            choose_phase<kRXF, kHeavy, kWide>(r);
+            if (blockIdx.x == 0 && threadIdx.x < kNB) c->cnt[r.par ^ 1][threadIdx.x] = 0;
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                c->mark_cnt = 0;
+                c->open_cnt = 0;
+                c->open_rows = 0;
+            }
+            if (!(ok = bar.sync(c))) break;
+        }
+        test_phase<kRXF, kHeavy, kWide>(r);
+        if (!(ok = bar.sync(c))) break;
+        if constexpr (kHeavy) {
+            if (r.round == 0) {
+                if (blockIdx.x == 0 && threadIdx.x == 0) c->mark_cnt = 0;
+                if (!(ok = bar.sync(c))) break;
+                heavy_round0_close<kWide>(r);
+                if (!(ok = bar.sync(c))) break;
+            }
+            if (__ldcg(&c->open_cnt) > 0) {
+                open_phase<kWide>(r);
+                if (!(ok = bar.sync(c))) break;
+            }
+            if (__ldcg(&c->mark_cnt) > 0) {
+                push_phase(r);
+                if (!(ok = bar.sync(c))) break;
+            }
+        }
+        r.lane_cnt = l < kNB ? __ldcg(&c->cnt[r.par ^ 1][l]) : 0;
+        total = __reduce_add_sync(kFull, r.lane_cnt);
+        conflicts += static_cast<unsigned long long>(total);
+        ++r.round;
+        if (total == 0) break;
+        if (r.round >= a.round_limit) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&c->err, kErrRoundLimit);
             break;
         }
-        case 2: tentative_group_tile<32, kRXF>(a, rt, list, 2, first, round, edges); break;
-        case 3: tentative_group_tile<16, kRXF>(a, rt, list, 3, first, round, edges); break;
-        case 4: tentative_group_tile<8, kRXF>(a, rt, list, 4, first, round, edges); break;
-        case 5: tentative_group_tile<4, kRXF>(a, rt, list, 5, first, round, edges); break;
-        default: tentative_group_tile<2, kRXF>(a, rt, list, 6, first, round, edges); break;
-        }
     }
-    warp_add(&a.ctrl->edges, edges);
-}
-
-// ---------------------------------------------------------------------------
-// Conflict detection; winners fix their color, losers go to W_{r+1}
-// ---------------------------------------------------------------------------
-// Does some neighbor in this lane's stripe have v's tentative color and a
-// larger (priority, id)?  U gathers in flight.  Without heavy rows no key
-// carries the fixed bit, and equal tentative colors make the keys order as
-// the priorities.
-template <int UC, bool kHeavy = true>
-__device__ __forceinline__ bool loses(const SpecArgs& a, const WorkItem& it, int32_t lane0,
-                                      int32_t stride) {
-    if (it.deg == 0) return false;
-    const unsigned long long* key = reinterpret_cast<const unsigned long long*>(a.key);
-    const uint64_t kv = __ldg(key + it.v);
-    const uint32_t tv = key_tent(kv);
-    bool lose = false, loop = false;
-    for_each_nbr<UC, uint64_t, true>(
-        a.g, it.beg, it.deg, lane0, stride, [&](int32_t u) { return __ldg(key + u); },
-        [&](int32_t u, uint64_t ku) {
-            if (u == it.v) loop = true;  // uncolorable (Sec. 1): reported as a malformed graph
-            else if (kHeavy ? key_tent(ku) == tv && above(ku, u, kv, it.v)
-                            : static_cast<uint32_t>(ku >> 32) == tv && (ku > kv || (ku == kv && u > it.v)))
-                lose = true;
-        },
-        &a.ctrl->err);
-    if (loop) atomicOr(&a.ctrl->err, kErrBadGraph);
-    return lose;
-}
-
-// ListItem: from round 1 on, the work item of a marking heavy row (a
-// block-bucket row, or a warp-bucket row where the warp rows do not pull)
-// holds its list instead of its row: beg = the list's start in pend, deg =
-// its length.  A visit then reads the item, the list and the listed keys
-// with no index lookups in between (before: item, heavy index, list start
-// and length, list, keys); the row's bounds, needed only for the edge count
-// and a winner's marks, are loaded beside the list (the conflict launch
-// counts both launches' entries of such a row: every row of a round's work
-// set is visited by both).  Round 0 reads rows from items of the usual form,
-// and its losers write the new one.
-
-// Round 0, a block-bucket row (the whole block): the conflict test over the
-// full row, which also writes the row's list: its neighbors above it in the
-// total order that are not fixed.  Only these can beat it in a later round.
-// lbeg, lcnt: the list's start in pend and its length (block-uniform).
-__device__ bool above_build_block(const SpecArgs& a, const HeavyRows& hr, const WorkItem& it,
-                                  uint32_t* wsum, int64_t& lbeg, int32_t& lcnt) {
-    const int t = threadIdx.x, l = lane_id(), w = t >> 5;
-    const int32_t h = hr.hid[it.v];
-    lbeg = hr.h_pbeg[h];
-    int32_t* dst = hr.pend + lbeg;
-    const unsigned long long* key = reinterpret_cast<const unsigned long long*>(a.key);
-    const uint64_t kv = __ldg(key + it.v);
-    const uint32_t tv = key_tent(kv);
-    bool lose = false, loop = false;
-    int32_t kept = 0;
-    for (int64_t i0 = 0; i0 < it.deg; i0 += kHeavyStep) {
-        int32_t u[kHeavyU];
-        uint64_t ku[kHeavyU];
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            const int64_t i = i0 + static_cast<int64_t>(k) * kBlock + t;
-            u[k] = i < it.deg ? load_nbr(a.g, it.beg + i, &a.ctrl->err) : -1;
-        }
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) ku[k] = u[k] >= 0 ? __ldg(key + u[k]) : 0ull;
-        int32_t mine = 0;
-        bool keep[kHeavyU];
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            keep[k] = false;
-            if (u[k] < 0) continue;
-            if (u[k] == it.v) {
-                loop = true;
-                continue;
-            }
-            const bool up = above(ku[k], u[k], kv, it.v);
-            if (up && key_tent(ku[k]) == tv) lose = true;
-            keep[k] = up && !(ku[k] & kKeyFixed);
-            mine += keep[k];
-        }
-        const int32_t incl_w = static_cast<int32_t>(warp_inclusive_scan(static_cast<uint32_t>(mine)));
-        if (l == 31) wsum[w] = static_cast<uint32_t>(incl_w);
-        __syncthreads();
-        int32_t before = 0, total = 0;
-#pragma unroll
-        for (int k = 0; k < kWarps; ++k) {
-            const int32_t x = static_cast<int32_t>(wsum[k]);
-            if (k < w) before += x;
-            total += x;
-        }
-        int32_t pos = kept + before + incl_w - mine;
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k)
-            if (keep[k]) dst[pos++] = u[k];
-        kept += total;
-        __syncthreads();
-    }
-    lcnt = kept;
-    if (loop) atomicOr(&a.ctrl->err, kErrBadGraph);
-    return lose;
-}
-
-// Round >= 1, a block-bucket row: the conflict test over its list (the
-// neighbors above it not fixed at its last look), dropping the entries fixed
-// since, compacted in place (a kept entry moves to a position at or below
-// the one it was read from, after the step's entries are staged).  The
-// list's next step is staged while this one runs.  On a list longer
-// than kProbeMin probes, a probe of the first kBlock entries comes first:
-// most rows of a dense core lose every round,
-// usually to one of the first entries, and a loss found there leaves the
-// list as it is (still a superset of the neighbors above v not fixed).
-// Every kCompactEvery-th round skips the probe, so that no list goes long
-// uncompacted.  The item holds the list (see ListItem); lcnt: its length
-// after the scan (block-uniform).
-__device__ bool above_scan_block(const SpecArgs& a, const WorkItem& it, int32_t (*stage)[kHeavyStep],
-                                 uint32_t* wsum, int32_t& lcnt) {
-    const int t = threadIdx.x, l = lane_id(), w = t >> 5;
-    const int64_t pc = it.deg;
-    int32_t* lst = a.heavy->pend + it.beg;
-    const unsigned long long* key = reinterpret_cast<const unsigned long long*>(a.key);
-    const uint32_t tv = key_tent(__ldg(key + it.v));
-    lcnt = static_cast<int32_t>(pc);
-    if (pc > kProbeMin * kBlock && (a.ctrl->round & (kCompactEvery - 1)) != 0) {  // the probe
-        bool hit = false;
-        const int32_t u = lst[t];
-        if (static_cast<uint32_t>(u) < static_cast<uint32_t>(a.g.n)) hit = key_tent(__ldg(key + u)) == tv;
-        if (__syncthreads_or(hit)) return true;
-    }
-    bool lose = false;
-    int32_t kept = 0;
-    if (pc > 0) stage_step(stage[0], lst, 0, pc);
-    int parity = 0;
-    for (int64_t i0 = 0; i0 < pc; i0 += kHeavyStep, parity ^= 1) {
-        const bool more = i0 + kHeavyStep < pc;
-        if (more) stage_step(stage[parity ^ 1], lst, i0 + kHeavyStep, pc);
-        if (more) cp_async_wait<1>(); else cp_async_wait<0>();
-        int32_t u[kHeavyU];
-        uint64_t ku[kHeavyU];
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            const int64_t i = i0 + 4 * static_cast<int64_t>(t) + k;
-            u[k] = i < pc ? stage[parity][4 * t + k] : -1;
-            ku[k] = 0;
-            if (i < pc) {
-                if (static_cast<uint32_t>(u[k]) >= static_cast<uint32_t>(a.g.n)) {
-                    atomicOr(&a.ctrl->err, kErrBadGraph);
-                    u[k] = -1;
-                } else {
-                    ku[k] = __ldg(key + u[k]);
-                }
-            }
-        }
-        int32_t mine = 0;
-        bool keep[kHeavyU];
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            keep[k] = u[k] >= 0 && !(ku[k] & kKeyFixed);
-            if (u[k] >= 0 && key_tent(ku[k]) == tv) lose = true;
-            mine += keep[k];
-        }
-        const int32_t incl_w = static_cast<int32_t>(warp_inclusive_scan(static_cast<uint32_t>(mine)));
-        if (l == 31) wsum[w] = static_cast<uint32_t>(incl_w);
-        __syncthreads();  // also: the whole step is staged before any write
-        int32_t before = 0, total = 0;
-#pragma unroll
-        for (int k = 0; k < kWarps; ++k) {
-            const int32_t x = static_cast<int32_t>(wsum[k]);
-            if (k < w) before += x;
-            total += x;
-        }
-        int32_t pos = kept + before + incl_w - mine;
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k)
-            if (keep[k]) lst[pos++] = u[k];
-        kept += total;
-        __syncthreads();  // frees stage[parity] for the step after next
-    }
-    lcnt = kept;
-    return lose;
-}
-
-// The two list passes of a warp-bucket row (the whole warp): round 0 builds
-// the list from the row, later rounds scan and compact it (ballots; a
-// batch's reads precede its writes, which land at or below every position
-// the batch read), after a probe of the first 32 entries as in
-// above_scan_block.
-__device__ bool above_build_warp(const SpecArgs& a, const HeavyRows& hr, const WorkItem& it, int64_t& lbeg,
-                                 int32_t& lcnt) {
-    const int l = lane_id();
-    const int32_t h = hr.hid[it.v];
-    lbeg = hr.h_pbeg[h];
-    int32_t* dst = hr.pend + lbeg;
-    const unsigned long long* key = reinterpret_cast<const unsigned long long*>(a.key);
-    const uint64_t kv = __ldg(key + it.v);
-    const uint32_t tv = key_tent(kv);
-    bool lose = false, loop = false;
-    int32_t kept = 0;
-    for (int32_t i0 = 0; i0 < it.deg; i0 += kHeavyU * 32) {
-        int32_t u[kHeavyU];
-        uint64_t ku[kHeavyU];
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            const int32_t i = i0 + k * 32 + l;
-            u[k] = i < it.deg ? load_nbr(a.g, it.beg + i, &a.ctrl->err) : -1;
-        }
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) ku[k] = u[k] >= 0 ? __ldg(key + u[k]) : 0ull;
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            bool keep = false;
-            if (u[k] == it.v) {
-                loop = true;
-            } else if (u[k] >= 0) {
-                const bool up = above(ku[k], u[k], kv, it.v);
-                if (up && key_tent(ku[k]) == tv) lose = true;
-                keep = up && !(ku[k] & kKeyFixed);
-            }
-            const unsigned bal = __ballot_sync(kFull, keep);
-            if (keep) dst[kept + __popc(bal & ((1u << l) - 1u))] = u[k];
-            kept += __popc(bal);
-        }
-    }
-    lcnt = kept;
-    if (loop) atomicOr(&a.ctrl->err, kErrBadGraph);
-    return __any_sync(kFull, lose);
-}
-
-__device__ bool above_scan_warp(const SpecArgs& a, const WorkItem& it, int32_t& lcnt) {
-    const int l = lane_id();
-    const int32_t pc = it.deg;
-    int32_t* lst = a.heavy->pend + it.beg;
-    const unsigned long long* key = reinterpret_cast<const unsigned long long*>(a.key);
-    const uint32_t tv = key_tent(__ldg(key + it.v));
-    lcnt = pc;
-    if (pc > kProbeMin * 32 && (a.ctrl->round & (kCompactEvery - 1)) != 0) {  // the probe
-        const int32_t u = lst[l];
-        const bool hit = static_cast<uint32_t>(u) < static_cast<uint32_t>(a.g.n) &&
-                         key_tent(__ldg(key + u)) == tv;
-        if (__any_sync(kFull, hit)) return true;
-    }
-    bool lose = false;
-    int32_t kept = 0;
-    for (int32_t i0 = 0; i0 < pc; i0 += kHeavyU * 32) {
-        int32_t u[kHeavyU];
-        uint64_t ku[kHeavyU];
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            const int32_t i = i0 + k * 32 + l;
-            u[k] = i < pc ? lst[i] : -1;
-        }
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            ku[k] = 0;
-            if (u[k] >= a.g.n) {
-                atomicOr(&a.ctrl->err, kErrBadGraph);
-                u[k] = -1;
-            } else if (u[k] >= 0) {
-                ku[k] = __ldg(key + u[k]);
-            }
-        }
-        __syncwarp();  // every read of the batch before any write
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            if (u[k] >= 0 && key_tent(ku[k]) == tv) lose = true;
-            const bool keep = u[k] >= 0 && !(ku[k] & kKeyFixed);
-            const unsigned bal = __ballot_sync(kFull, keep);
-            if (keep) lst[kept + __popc(bal & ((1u << l) - 1u))] = u[k];
-            kept += __popc(bal);
-        }
-    }
-    lcnt = kept;
-    return __any_sync(kFull, lose);
-}
-
-// The conflict test of a warp-bucket row after round 0 (the whole warp),
-// over its list, which the round's tentative launch has just compacted: the
-// neighbors not fixed before the round, the only ones that can share its
-// tentative color.
-__device__ bool loses_pending_warp(const SpecArgs& a, const WorkItem& it) {
-    const HeavyRows& hr = *a.heavy;
-    const int32_t h = hr.hid[it.v];
-    const int32_t pc = hr.h_pcnt[h];
-    const int32_t* lst = hr.pend + hr.h_pbeg[h];
-    const unsigned long long* key = reinterpret_cast<const unsigned long long*>(a.key);
-    const uint64_t kv = __ldg(key + it.v);
-    const uint32_t tv = key_tent(kv);
-    const int l = lane_id();
-    bool lose = false;
-    for (int32_t i0 = 0; i0 < pc; i0 += kHeavyU * 32) {
-        int32_t u[kHeavyU];
-        uint64_t ku[kHeavyU];
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            const int32_t i = i0 + k * 32 + l;
-            u[k] = i < pc ? __ldg(lst + i) : -1;
-        }
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k) {
-            ku[k] = 0;
-            if (u[k] >= a.g.n) {
-                atomicOr(&a.ctrl->err, kErrBadGraph);
-                u[k] = -1;
-            } else if (u[k] >= 0) {
-                ku[k] = __ldg(key + u[k]);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < kHeavyU; ++k)
-            if (u[k] >= 0 && u[k] != it.v && key_tent(ku[k]) == tv && above(ku[k], u[k], kv, it.v))
-                lose = true;
-    }
-    return __any_sync(kFull, lose);
-}
-
-// Whether a fixed vertex marks its heavy neighbors' bitmaps: only where the
-// graph has heavy rows (in a batch, its own graph).
-__device__ __forceinline__ bool marks_of(const SpecArgs& a, const HeavyRows& hr, int32_t v) {
-    return hr.bref && (!hr.near || hr.near[v]) && (!a.graph_of || a.graph_heavy[a.graph_of[v]]);
-}
-
-// A winner (leader lane) fixes its color c, its key's tentative color: the
-// color array and the fixed bit of its key.
-template <bool kHeavy>
-__device__ __forceinline__ void fix_color(const SpecArgs& a, int32_t v, int32_t c, bool leader,
-                                          int32_t& my_max, int32_t round) {
-    if (!leader) return;
-    a.color[v] = c;
-    if (kHeavy) {  // the fixed bit: read by the heavy rows' list scans only
-        const HeavyRows& hr = *a.heavy;
-        if (hr.bref && (!hr.near || hr.near[v])) a.key[v] |= kKeyFixed;
-    }
-    my_max = max(my_max, c);
-    if (a.win_round) a.win_round[v] = round;
-}
-
-template <int G, bool kHeavy, bool kPending = false>
-__device__ __forceinline__ void conflict_group_tile(const SpecArgs& a, const HeavyRows& hr,
-                                                    const RoundTiles& rt, const WorkItem* list,
-                                                    WorkItem* next, int par, int b, int32_t first,
-                                                    int32_t round, int32_t& my_max,
-                                                    unsigned long long& edges) {
-    const int gi = threadIdx.x / G, gl = threadIdx.x % G;
-    const int32_t k = first + gi;
-    const bool valid = k < rt.cnt[b];
-    WorkItem it{0, 0, 0};
-    if (valid) it = load_item(list + rt.start[b] + k);
-    bool lose;
-    if constexpr (kPending) lose = valid && loses_pending_warp(a, it);  // G == 32: one warp per row
-    else lose = group_any<G>(loses<1, kHeavy>(a, it, gl, G));  // one 4-id chunk per lane per batch
-    const bool leader = valid && gl == 0;
-    const bool win = valid && !lose;
-    int32_t c = 0;
-    if (leader) {
-        edges += static_cast<unsigned long long>(it.deg);
-        if (win) c = static_cast<int32_t>(key_tent(a.key[it.v])) * (kHeavy && marks_of(a, hr, it.v) ? -1 : 1);
-    }
-    fix_color<kHeavy>(a, it.v, c < 0 ? -c : c, leader && win, my_max, round);
-    if (kHeavy && hr.bref) {  // c < 0: fixed at -c, marks
-        c = __shfl_sync(kFull, c, lane_id() & ~(G - 1));
-        if (win && c < 0) mark_color(a, hr, it.beg, it.deg, -c, gl, G);
-    }
-    warp_append(leader && lose, it.beg, it.v, it.deg, &a.ctrl->cnt[par ^ 1][b], next, rt.start[b]);
-}
-
-// Warp-bucket rows: one warp per row, over its list after round 0.
-__device__ __forceinline__ void conflict_warp_tile(const SpecArgs& a, const HeavyRows& hr,
-                                                   const RoundTiles& rt, const WorkItem* list,
-                                                   WorkItem* next, int par, int32_t first,
-                                                   int32_t round, int32_t& my_max,
-                                                   unsigned long long& edges) {
-    const int32_t k = first + (threadIdx.x >> 5);
-    const bool valid = k < rt.cnt[1];  // the same for the whole warp
-    WorkItem it{0, 0, 0};
-    bool lose = false;
-    int64_t rbeg = 0, lbeg = 0;  // the row (edge count, marks) and the list (next round's item)
-    int32_t rdeg = 0, lcnt = 0;
-    if (valid) {
-        it = load_item(list + rt.start[1] + k);
-        if (round == 0) {
-            rbeg = it.beg;
-            rdeg = it.deg;
-            lose = above_build_warp(a, hr, it, lbeg, lcnt);
-        } else {
-            row_of(a.g, it.v, rbeg, rdeg, &a.ctrl->err);  // loaded beside the list
-            lbeg = it.beg;
-            lose = above_scan_warp(a, it, lcnt);
-        }
-    }
-    const bool leader = valid && lane_id() == 0;
-    const bool win = valid && !lose;
-    int32_t c = 0;
-    if (leader) {
-        // from round 1 on also the round's tentative visit (ListItem)
-        edges += static_cast<unsigned long long>(rdeg) * (round == 0 ? 1u : 2u);
-        if (win) c = static_cast<int32_t>(key_tent(a.key[it.v]));
-    }
-    fix_color<true>(a, it.v, c, leader && win, my_max, round);
-    if (leader && win) a.bucket[it.v] = kBucketFixed;
-    if (hr.bref) {  // a warp-bucket row's graph has heavy rows: it marks
-        c = __shfl_sync(kFull, c, 0);
-        if (win) mark_color(a, hr, rbeg, rdeg, c, lane_id(), 32);
-    }
-    warp_append(leader && lose, lbeg, it.v, lcnt, &a.ctrl->cnt[par ^ 1][1], next, rt.start[1]);
-}
-
-// kHeavy = false: the form for graphs without heavy rows (buckets 0 and 1
-// empty), with none of their code, nor marks or fixed bits.  kMinBlocks:
-// resident blocks per SM the registers are budgeted for (measured: the
-// light form and the pulling warp rows gain from 64 registers without
-// spills, the marking form from the fifth block).
-template <bool kHeavy, int kMinBlocks>
-__global__ void __launch_bounds__(kBlock, kMinBlocks) k_conflict(SpecArgs a) {
-    __shared__ RoundTiles rt;
-    __shared__ bool s_last;
-    __shared__ uint32_t s_wsum[kWarps];
-    __shared__ int32_t s_c, s_pos, s_rdeg;
-    __shared__ int64_t s_rbeg;
-    __shared__ __align__(16) int32_t stage[2][kHeavyStep];  // block-bucket rows' next list step
-    const int32_t round = a.ctrl->round;
-    const int par = round & 1;
-    const WorkItem* list = par ? a.list1 : a.list0;
-    WorkItem* next = par ? a.list0 : a.list1;
-    load_round_tiles(a.ctrl, par, false, rt);
-    // only the blocks with a tile take part in closing the round (a round has
-    // at least one tile: the rounds stop when the work set is empty)
-    const uint32_t participants = static_cast<uint32_t>(min(static_cast<int32_t>(gridDim.x), rt.prefix[kNB]));
-    if (blockIdx.x >= participants) return;
-    const HeavyRows& hr = *a.heavy;  // bref == nullptr: no heavy rows, nothing to mark
-    unsigned long long edges = 0;
-    int32_t my_max = 0;
-    for (int32_t t = blockIdx.x; t < rt.prefix[kNB]; t += gridDim.x) {
-        const int b = tile_bucket(rt, t);
-        const int32_t first = (t - rt.prefix[b]) * bucket_tile(b);
-        if constexpr (kHeavy) {
-            if (b == 0) {
-            const WorkItem it = load_item(list + rt.start[0] + first);
-            int64_t rbeg = it.beg, lbeg = it.beg;  // the row and the list (see ListItem)
-            int32_t rdeg = it.deg, lcnt = 0;
-            if (round != 0 && threadIdx.x == 0) row_of(a.g, it.v, rbeg, rdeg, &a.ctrl->err);
-            const bool mine = round == 0 ? above_build_block(a, hr, it, s_wsum, lbeg, lcnt)
-                                         : above_scan_block(a, it, stage, s_wsum, lcnt);
-            const bool lose = __syncthreads_or(mine);
-            if (threadIdx.x == 0) {
-                // from round 1 on also the round's tentative visit (ListItem)
-                edges += static_cast<unsigned long long>(rdeg) * (round == 0 ? 1u : 2u);
-                s_rdeg = rdeg;
-                s_rbeg = rbeg;
-                if (lose) {
-                    const int32_t pos = atomicAdd(&a.ctrl->cnt[par ^ 1][0], 1);
-                    store_item(next + rt.start[0] + pos, lbeg, it.v, lcnt);
-                } else {
-                    s_c = static_cast<int32_t>(key_tent(a.key[it.v]));
-                    fix_color<true>(a, it.v, s_c, true, my_max, round);
-                    a.bucket[it.v] = kBucketFixed;
-                    // the row's marks go to the grid-wide marking launch
-                    const int32_t pieces = (rdeg + kMarkChunk - 1) / kMarkChunk;
-                    s_pos = pieces ? atomicAdd(&a.ctrl->mark_cnt, pieces) : 0;
-                }
-            }
-            __syncthreads();
-            if (!lose) {
-                const int32_t pieces = (s_rdeg + kMarkChunk - 1) / kMarkChunk;
-                for (int32_t q = threadIdx.x; q < pieces && s_pos + q < hr.mark_cap; q += kBlock) {
-                    const int32_t len = min(kMarkChunk, s_rdeg - q * kMarkChunk);
-                    store_item(hr.mark + s_pos + q, s_rbeg + static_cast<int64_t>(q) * kMarkChunk, s_c, len);
-                }
-            }
-            __syncthreads();  // s_c, s_pos and the stage buffers are reused by the next tile
-            continue;
-            }
-            if (b == 1) {
-                if (!hr.pull_warp) conflict_warp_tile(a, hr, rt, list, next, par, first, round, my_max, edges);
-                else if (round == 0) conflict_group_tile<32, true>(a, hr, rt, list, next, par, 1, first, round, my_max, edges);
-                else conflict_group_tile<32, true, true>(a, hr, rt, list, next, par, 1, first, round, my_max, edges);
-                continue;
-            }
-        }
-        switch (b) {
-        case 2: conflict_group_tile<32, kHeavy>(a, hr, rt, list, next, par, 2, first, round, my_max, edges); break;
-        case 3: conflict_group_tile<16, kHeavy>(a, hr, rt, list, next, par, 3, first, round, my_max, edges); break;
-        case 4: conflict_group_tile<8, kHeavy>(a, hr, rt, list, next, par, 4, first, round, my_max, edges); break;
-        case 5: conflict_group_tile<4, kHeavy>(a, hr, rt, list, next, par, 5, first, round, my_max, edges); break;
-        default: conflict_group_tile<2, kHeavy>(a, hr, rt, list, next, par, 6, first, round, my_max, edges); break;
-        }
-    }
-    warp_add(&a.ctrl->edges, edges);
-    warp_max(&a.ctrl->max_color, my_max);
-
-    // The last block to finish closes the round.
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&a.ctrl->done_blocks, 1u) == participants - 1;
-    __syncthreads();
-    if (s_last && threadIdx.x == 0) {
-        __threadfence();
-        volatile SpecCtrl* c = a.ctrl;
-        int32_t total = 0;
-        for (int b = 0; b < kNB; ++b) total += c->cnt[par ^ 1][b];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        c->round = r.round;
         c->active = total;
-        c->conflicts += static_cast<unsigned long long>(total);
-        c->round = round + 1;
-        c->done_blocks = 0u;
-        const bool over = total > 0 && round + 1 >= a.round_limit;
-        if (over) c->err |= kErrRoundLimit;
-        if (a.use_cond) cudaGraphSetConditional(a.cond, (total > 0 && !over) ? 1u : 0u);
+        c->conflicts += conflicts;
     }
-}
-
-// Neighbors of the block-bucket rows (one block per row): the vertices that
-// mark when only those rows are marked.
-__global__ void __launch_bounds__(kBlock) k_near_block(SpecArgs a, uint8_t* near) {
-    const int32_t rows = a.ctrl->init_cnt[0];
-    for (int32_t q = blockIdx.x; q < rows; q += gridDim.x) {
-        const WorkItem it = load_item(a.list0 + a.ctrl->start[0] + q);
-        for (int32_t i = threadIdx.x; i < it.deg; i += kBlock) {
-            const int32_t u = ld_stream(a.g.idx + it.beg + i);
-            if (static_cast<uint32_t>(u) < static_cast<uint32_t>(a.g.n)) near[u] = 1;
-        }
-    }
-}
-
-// The marks of the round's block-bucket winners (their rows in pieces, one
-// block per piece), before the next round's tentative launch reads them.
-__global__ void __launch_bounds__(kBlock) k_mark_colors(SpecArgs a) {
-    const int32_t pending = a.ctrl->mark_cnt;
-    if (pending == 0) return;
-    const HeavyRows& hr = *a.heavy;
-    // (the capacity holds every piece of every block-bucket row: never cut)
-    const int32_t cnt = static_cast<int32_t>(min(static_cast<int64_t>(pending), hr.mark_cap));
-    for (int32_t q = blockIdx.x; q < cnt; q += gridDim.x) {
-        const WorkItem it = load_item(hr.mark + q);  // v: the color, deg: the piece's length
-        mark_color(a, hr, it.beg, it.deg, it.v, threadIdx.x, kBlock);
-    }
+    warp_add(&c->edges, r.edges);
+    warp_max(&c->max_color, r.my_max);
 }
 
 __global__ void __launch_bounds__(kBlock) k_priorities(uint64_t seed, int64_t n, uint32_t* out) {
@@ -1185,116 +1268,71 @@ gc_status priorities_device(uint64_t seed, int64_t n, uint32_t* out, cudaStream_
 // ---------------------------------------------------------------------------
 // Host driver
 // ---------------------------------------------------------------------------
-namespace {
-struct PinnedWord {
-    int32_t* p = nullptr;
-    PinnedWord() { cudaMallocHost(&p, sizeof(int32_t) * 16); }
-};
-thread_local PinnedWord t_pinned;
-}  // namespace
-
-// The rounds as one CUDA graph: a WHILE node whose body is {tentative,
-// conflict}; the last block of the conflict kernel sets the condition from
-// the size of the next work set, so no round waits for the host.
-struct RoundsGraph {
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    ~RoundsGraph() { reset(); }
-    void reset() {
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
-        exec = nullptr;
-        graph = nullptr;
-    }
-};
-
-// The conflict kernel's form: without heavy rows, with pulling warp rows, or
-// with marks for both heavy buckets.
-void* conflict_kernel(bool heavy, bool pull) {
-    if (!heavy) return reinterpret_cast<void*>(k_conflict<false, 4>);
-    return pull ? reinterpret_cast<void*>(k_conflict<true, 4>) : reinterpret_cast<void*>(k_conflict<true, 5>);
-}
-
-// heavy: the conflict kernel with the heavy rows' code, and the marking node.
-gc_status build_rounds_graph(const SpecArgs& a, int32_t X, int grid_t, int grid_c, int grid_m,
-                             bool heavy, bool pull, RoundsGraph& rg) {
-    cudaGraph_t& graph = rg.graph;
-    cudaGraphExec_t& exec = rg.exec;
-    cudaError_t e = cudaGraphCreate(&graph, 0);
-    cudaGraphConditionalHandle handle = 0;
-    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&handle, graph, 1, cudaGraphCondAssignDefault);
-    alignas(cudaGraphNodeParams) unsigned char cp_buf[sizeof(cudaGraphNodeParams)];
-    std::memset(cp_buf, 0, sizeof(cp_buf));
-    cudaGraphNodeParams& cp = *reinterpret_cast<cudaGraphNodeParams*>(cp_buf);
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = handle;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    cudaGraphNode_t cnode = nullptr;
-    if (e == cudaSuccess) e = cudaGraphAddNode(&cnode, graph, nullptr, nullptr, 0, &cp);
-    SpecArgs ga = a;
-    ga.cond = handle;
-    ga.use_cond = 1;
-    void* args[] = {&ga};
-    cudaGraphNode_t n1 = nullptr, n2 = nullptr, n3 = nullptr;
-    if (e == cudaSuccess) {
-        cudaGraph_t body = cp.conditional.phGraph_out[0];
-        cudaKernelNodeParams k1;
-        std::memset(&k1, 0, sizeof(k1));
-        k1.func = X > 1 ? reinterpret_cast<void*>(k_tentative<true>) : reinterpret_cast<void*>(k_tentative<false>);
-        k1.gridDim = dim3(grid_t);
-        k1.blockDim = dim3(kBlock);
-        k1.kernelParams = args;
-        cudaKernelNodeParams k2 = k1;
-        k2.func = conflict_kernel(heavy, pull);
-        k2.gridDim = dim3(grid_c);
-        cudaKernelNodeParams k3 = k1;
-        k3.func = reinterpret_cast<void*>(k_mark_colors);
-        k3.gridDim = dim3(grid_m);
-        e = cudaGraphAddKernelNode(&n1, body, nullptr, 0, &k1);
-        if (e == cudaSuccess) e = cudaGraphAddKernelNode(&n2, body, &n1, 1, &k2);
-        if (e == cudaSuccess && heavy) e = cudaGraphAddKernelNode(&n3, body, &n2, 1, &k3);
-    }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-    return cuda_status(e);
-}
-
-gc_status launch_rounds_graph(RoundsGraph& rg, cudaStream_t s) {
-    prof_begin(KID_SPEC_GRAPH, s);
-    const cudaError_t e = cudaGraphLaunch(rg.exec, s);
-    prof_end(KID_SPEC_GRAPH, s);
-    return cuda_status(e);  // the caller's read-back of the round state waits for it
-}
-
-// The speculative coloring; with graph_of / desc / win_round set, a batch.
 struct PrioRule {
     int32_t kind = 0;
     const int32_t* rank = nullptr;
     const int32_t* old = nullptr;
 };
 
+namespace {
+template <bool kWide>
+const void* rounds_kernel_of(bool rxf, bool heavy) {
+    if (rxf) return heavy ? reinterpret_cast<const void*>(k_spec_rounds<true, true, kWide>)
+                          : reinterpret_cast<const void*>(k_spec_rounds<true, false, kWide>);
+    return heavy ? reinterpret_cast<const void*>(k_spec_rounds<false, true, kWide>)
+                 : reinterpret_cast<const void*>(k_spec_rounds<false, false, kWide>);
+}
+
+// The rounds: one cooperative launch (spec_graph 1), or one per round.  h
+// receives the final control block.
+gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_t s) {
+    const void* k = a.g.n <= kWideMax ? rounds_kernel_of<true>(rxf, heavy) : rounds_kernel_of<false>(rxf, heavy);
+    const int fit = sm_count() * occupancy_of(k, kBlock);
+    // a block per tile of round 0 at most: on small graphs more blocks would only lengthen the barriers
+    const int64_t tiles = heavy ? fit : (static_cast<int64_t>(a.g.n) * 2 + kBlock - 1) / kBlock;
+    const int64_t want = a.tune.grid_blocks > 0 ? a.tune.grid_blocks : std::max<int64_t>(1, tiles);
+    const int grid = static_cast<int>(std::min<int64_t>(fit, want));
+    a.max_rounds = a.tune.spec_graph ? INT32_MAX : 1;
+    for (;;) {
+        void* args[] = {&a};
+        cudaError_t e;
+        GC_LAUNCH(KID_SPEC_ROUNDS, s, e = cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kBlock), args, 0, s));
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return cuda_status(e);
+        if (h->err) return status_from_err_bits(h->err);
+        if ((!heavy && h->init_cnt[0] > 0) || h->active == 0) return GC_OK;
+        e = cudaMemsetAsync(&a.ctrl->barrier, 0, sizeof(uint32_t), s);
+        if (e != cudaSuccess) return cuda_status(e);
+    }
+}
+}  // namespace
+
+// The speculative coloring; with graph_of / desc / win_round set, a batch.
 static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int32_t* graph_of,
-                            const BatchDesc* desc, int32_t ng, int32_t* win_round, const PrioRule& rule,
+                            const BatchDesc* desc, int32_t* win_round, const PrioRule& rule,
                             int32_t* colors_out, gc_stats* stats, cudaStream_t s) {
     if (g.n == 0) {
         if (stats) { std::memset(stats, 0, sizeof(*stats)); }
         return GC_OK;
     }
-    if (!t_pinned.p) return GC_ERR_OOM;
     const int64_t n = g.n;
-    Scratch sc_key, sc_l0, sc_l1, sc_bucket, sc_ctrl;
-    if (!sc_key.alloc(n * 8, s) ||
+    const bool wide = n <= kWideMax;
+    Scratch sc_prio, sc_lo, sc_hi, sc_l0, sc_l1, sc_bucket, sc_ctrl;
+    if (!sc_prio.alloc(n * (wide ? 8 : 4), s) || !sc_lo.alloc(n * 4, s) || !sc_hi.alloc(n * 4, s) ||
         !sc_l0.alloc(n * sizeof(WorkItem), s) || !sc_l1.alloc(n * sizeof(WorkItem), s) ||
         !sc_bucket.alloc(n, s) || !sc_ctrl.alloc(sizeof(SpecCtrl), s))
         return GC_ERR_OOM;
     SpecArgs a;
-    std::memset(&a, 0, sizeof(a));  // use_cond = 0: no WHILE node unless rounds_in_graph sets it
+    std::memset(&a, 0, sizeof(a));
     a.g = g;
     a.X = X;
     a.seed = seed;
     a.tune = current_tuning();
     a.color = colors_out;
-    a.key = sc_key.as<uint64_t>();
+    a.prio = sc_prio.as<uint32_t>();
+    a.mlo = sc_lo.as<uint32_t>();
+    a.mhi = sc_hi.as<uint32_t>();
     a.bucket = sc_bucket.as<uint8_t>();
     a.list0 = sc_l0.as<WorkItem>();
     a.list1 = sc_l1.as<WorkItem>();
@@ -1302,15 +1340,10 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
     a.graph_of = graph_of;
     a.desc = desc;
     a.win_round = win_round;
-    Scratch sc_gh;
-    if (graph_of) {
-        if (!sc_gh.alloc(static_cast<size_t>(ng) * 4 + 4, s)) return GC_ERR_OOM;
-        a.graph_heavy = sc_gh.as<int32_t>();
-        cudaMemsetAsync(a.graph_heavy, 0, static_cast<size_t>(ng) * 4 + 4, s);
-    }
     a.prio_kind = rule.kind;
     a.prio_rank = rule.rank;
     a.prio_old = rule.old;
+    a.round_limit = static_cast<int32_t>(std::min<int64_t>(n + 2, INT32_MAX));
 
     struct Events {
         cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1323,152 +1356,63 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
             cudaEventDestroy(e1);
         }
     } ev;
-    const cudaEvent_t e0 = ev.e0, e1 = ev.e1;
-    cudaEventRecord(e0, s);
+    cudaEventRecord(ev.e0, s);
     cudaMemsetAsync(a.ctrl, 0, sizeof(SpecCtrl), s);
-    const int grid_t = resident_grid(X > 1 ? k_tentative<true> : k_tentative<false>, a.tune);
-    const int grid_cl = resident_grid(k_conflict<false, 4>, a.tune);
-    const int grid_m = resident_grid(k_mark_colors, a.tune);
-    const int setup_grid = static_cast<int>(
-        std::min<int64_t>((n + kBlock - 1) / kBlock, resident_grid(k_spec_setup, a.tune)));
-    Scratch sc_heavy;
-    if (!sc_heavy.alloc(sizeof(HeavyRows), s)) return GC_ERR_OOM;
-    a.heavy = sc_heavy.as<HeavyRows>();
-    cudaMemsetAsync(a.heavy, 0, sizeof(HeavyRows), s);
-    GC_LAUNCH(KID_SPEC_SETUP, s, k_spec_setup<<<setup_grid, kBlock, 0, s>>>(a));
-    GC_LAUNCH(KID_SPEC_FILL, s, k_spec_fill<<<setup_grid, kBlock, 0, s>>>(a));
-    gc_status st = GC_OK;
-    a.round_limit = static_cast<int32_t>(std::min<int64_t>(n + 2, INT32_MAX));
-    // the rounds' CUDA graph is built while the set-up kernels run
-    RoundsGraph rg;
-    if (a.tune.spec_graph && (st = build_rounds_graph(a, X, grid_t, grid_cl, grid_m, false, false, rg)) != GC_OK) return st;
-    // heavy rows: their pending lists and bitmaps (sizes read back)
-    Scratch sc_hid, sc_pbeg, sc_pcnt, sc_bbeg, sc_bwords, sc_pend, sc_hbm, sc_hsums, sc_bref, sc_mark, sc_near;
-    bool heavy = false, pull = false;
-    int grid_ch = 0;
-    {
-        SpecCtrl h0;
-        cudaError_t ce = cudaMemcpyAsync(&h0, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
+    const auto setup = wide ? k_spec_setup<true> : k_spec_setup<false>;
+    const int setup_grid = static_cast<int>(std::min<int64_t>((n + kBlock - 1) / kBlock, resident_grid(setup, a.tune)));
+    GC_LAUNCH(KID_SPEC_SETUP, s, setup<<<setup_grid, kBlock, 0, s>>>(a));
+    SpecCtrl h;
+    gc_status st = run_rounds(a, X > 1, false, &h, s);
+    Scratch sc_pbeg, sc_pcnt, sc_bref, sc_pend, sc_hbm, sc_hsums, sc_mark, sc_open, sc_orow, sc_odone, sc_olost;
+    if (st == GC_OK && h.init_cnt[0] > 0) {
+        // heavy rows: their lists and bitmaps (sizes read back), then the rounds
+        const int32_t nh = h.init_cnt[0];
+        const int hblocks = static_cast<int>((static_cast<int64_t>(nh) + kHeavyChunk - 1) / kHeavyChunk);
+        if (!sc_pbeg.alloc(static_cast<int64_t>(nh) * 8, s) || !sc_pcnt.alloc(static_cast<int64_t>(nh) * 4, s) ||
+            !sc_bref.alloc(n * 8, s) || !sc_hsums.alloc(static_cast<int64_t>(hblocks) * 16, s))
+            return GC_ERR_OOM;
+        GC_LAUNCH(KID_SPEC_FILL, s, k_heavy_sums<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sc_hsums.as<long long>()));
+        cudaError_t ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
         if (ce != cudaSuccess) return cuda_status(ce);
-        if (h0.err) return status_from_err_bits(h0.err);
-        if (h0.init_cnt[0] > 0 && h0.max_deg <= kPullAllMaxDeg && a.tune.warp_max_deg == kDefaultWarpMaxDeg) {
-            // No row longer than kPullAllMaxDeg: every heavy row is a warp row
-            // that pulls (folds its list of neighbors not yet fixed each
-            // round) instead of being marked.  The marks' extra launch per
-            // round and one pass per fixed vertex cost more than the folds
-            // on such graphs (coloring on GB300: R-MAT 14 2.53 -> 1.93 ms,
-            // R-MAT 16 4.28 -> 3.71 ms, RMAT-Bad 16 1.49 -> 1.36 ms; R-MAT 17,
-            // max degree 15.7 K, 4.97 -> 5.48 ms the other way).  The set-up
-            // runs again with the lifted threshold.
-            a.tune.warp_max_deg = INT32_MAX;
-            cudaMemsetAsync(a.ctrl, 0, sizeof(SpecCtrl), s);
-            GC_LAUNCH(KID_SPEC_SETUP, s, k_spec_setup<<<setup_grid, kBlock, 0, s>>>(a));
-            GC_LAUNCH(KID_SPEC_FILL, s, k_spec_fill<<<setup_grid, kBlock, 0, s>>>(a));
-            ce = cudaMemcpyAsync(&h0, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
-            if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-            if (ce != cudaSuccess) return cuda_status(ce);
-            if (h0.err) return status_from_err_bits(h0.err);
-        }
-        const int32_t nh = h0.init_cnt[0] + h0.init_cnt[1];  // block- and warp-bucket rows
-        heavy = nh > 0;
-        if (heavy) {
-            // a small share of the entries in block-bucket rows: the warp-bucket
-            // rows fold their own bitmaps, and only the block-bucket rows'
-            // neighbors mark
-            const bool pull_warp = h0.block_entries * kPullShare < static_cast<unsigned long long>(g.nnz);
-            pull = pull_warp;
-            grid_ch = pull ? resident_grid(k_conflict<true, 4>, a.tune) : resident_grid(k_conflict<true, 5>, a.tune);
-            const bool marks = !pull_warp || h0.init_cnt[0] > 0;
-            const bool near = pull_warp && h0.init_cnt[0] > 0;
-            if (!sc_hid.alloc(n * 4, s) || !sc_pbeg.alloc(static_cast<int64_t>(nh) * 8, s) ||
-                !sc_pcnt.alloc(static_cast<int64_t>(nh) * 4, s) || !sc_bbeg.alloc(static_cast<int64_t>(nh) * 8, s) ||
-                !sc_bwords.alloc(static_cast<int64_t>(nh) * 4, s) || (marks && !sc_bref.alloc(n * 8, s)) ||
-                (near && !sc_near.alloc(n, s)))
-                return GC_ERR_OOM;
-            HeavyRows hr1{};
-            hr1.pull_warp = pull_warp ? 1 : 0;
-            hr1.mark_bucket = pull_warp ? 0 : 1;
-            hr1.near = sc_near.as<uint8_t>();
-            if (near) {
-                cudaMemsetAsync(hr1.near, 0, static_cast<size_t>(n), s);
-                const int grid = std::min(h0.init_cnt[0], resident_grid(k_near_block, a.tune));
-                GC_LAUNCH(KID_SPEC_FILL, s, k_near_block<<<grid, kBlock, 0, s>>>(a, hr1.near));
-            }
-            hr1.hid = sc_hid.as<int32_t>();
-            hr1.h_pbeg = sc_pbeg.as<int64_t>();
-            hr1.h_pcnt = sc_pcnt.as<int32_t>();
-            hr1.h_bbeg = sc_bbeg.as<int64_t>();
-            hr1.h_bwords = sc_bwords.as<int32_t>();
-            hr1.bref = sc_bref.as<uint64_t>();  // nullptr: nothing is marked
-            ce = marks ? cudaMemsetAsync(hr1.bref, 0xFF, static_cast<size_t>(n) * 8, s) : cudaSuccess;  // kNoBitmap
-            if (ce == cudaSuccess)
-                ce = cudaMemcpyAsync(a.heavy, &hr1, sizeof(HeavyRows), cudaMemcpyHostToDevice, s);
-            if (ce != cudaSuccess) return cuda_status(ce);
-            const int hblocks = static_cast<int>((static_cast<int64_t>(nh) + kHeavyChunk - 1) / kHeavyChunk);
-            if (!sc_hsums.alloc(static_cast<int64_t>(hblocks) * 16, s)) return GC_ERR_OOM;
-            GC_LAUNCH(KID_SPEC_FILL, s, k_heavy_sums<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sc_hsums.as<long long>()));
-            GC_LAUNCH(KID_SPEC_FILL, s,
-                      k_heavy_setup<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sc_hsums.as<long long>()));
-            ce = cudaMemcpyAsync(&h0, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
-            if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-            if (ce != cudaSuccess) return cuda_status(ce);
-            // marking pieces: at most one per kMarkChunk entries, plus one, per row
-            const int64_t mark_cap = h0.heavy_entries / kMarkChunk + h0.init_cnt[0] + 1;
-            if (!sc_pend.alloc(static_cast<size_t>(h0.heavy_entries) * 4, s) ||
-                !sc_hbm.alloc(static_cast<size_t>(h0.heavy_words) * 4, s) ||
-                !sc_mark.alloc(static_cast<size_t>(mark_cap) * sizeof(WorkItem), s))
-                return GC_ERR_OOM;
-            HeavyRows hr2 = hr1;
-            hr2.pend = sc_pend.as<int32_t>();
-            hr2.hbm = sc_hbm.as<uint32_t>();
-            hr2.mark = sc_mark.as<WorkItem>();
-            hr2.mark_cap = mark_cap;
-            ce = cudaMemsetAsync(hr2.hbm, 0, static_cast<size_t>(h0.heavy_words) * 4, s);
-            if (ce == cudaSuccess)
-                ce = cudaMemcpyAsync(a.heavy, &hr2, sizeof(HeavyRows), cudaMemcpyHostToDevice, s);
-            if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-            if (ce != cudaSuccess) return cuda_status(ce);
-            if (a.tune.spec_graph) {  // the graph of the heavy form instead
-                rg.reset();
-                if ((st = build_rounds_graph(a, X, grid_t, grid_ch, grid_m, true, pull, rg)) != GC_OK) return st;
-            }
-        }
+        HeavyRows& hr = a.heavy;
+        hr.mark_cap = h.heavy_entries / kPiece + nh;  // every piece of every row
+        hr.open_rows_cap = h.heavy_entries / kLongList + 1;
+        hr.open_cap = h.heavy_entries / kOpenPiece + hr.open_rows_cap;
+        if (!sc_pend.alloc(static_cast<size_t>(h.heavy_entries) * 4, s) ||
+            !sc_hbm.alloc(static_cast<size_t>(h.heavy_words) * 4, s) ||
+            !sc_mark.alloc(static_cast<size_t>(hr.mark_cap) * sizeof(WorkItem), s) ||
+            !sc_open.alloc(static_cast<size_t>(hr.open_cap) * sizeof(WorkItem), s) ||
+            !sc_orow.alloc(static_cast<size_t>(hr.open_rows_cap) * sizeof(WorkItem), s) ||
+            !sc_odone.alloc(static_cast<size_t>(hr.open_rows_cap) * 4, s) ||
+            !sc_olost.alloc(static_cast<size_t>(hr.open_rows_cap) * 4, s))
+            return GC_ERR_OOM;
+        hr.h_pbeg = sc_pbeg.as<int64_t>();
+        hr.h_pcnt = sc_pcnt.as<int32_t>();
+        hr.bref = sc_bref.as<uint64_t>();
+        hr.pend = sc_pend.as<int32_t>();
+        hr.hbm = sc_hbm.as<uint32_t>();
+        hr.mark = sc_mark.as<WorkItem>();
+        hr.open = sc_open.as<WorkItem>();
+        hr.open_row = sc_orow.as<WorkItem>();
+        hr.open_done = sc_odone.as<int32_t>();
+        hr.open_lost = sc_olost.as<int32_t>();
+        ce = cudaMemsetAsync(hr.hbm, 0, static_cast<size_t>(h.heavy_words) * 4, s);
+        if (ce != cudaSuccess) return cuda_status(ce);
+        GC_LAUNCH(KID_SPEC_FILL, s,
+                  k_heavy_setup<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sc_hsums.as<long long>()));
+        st = run_rounds(a, X > 1, true, &h, s);
     }
-    if (a.tune.spec_graph) {
-        st = launch_rounds_graph(rg, s);
-    } else {
-        int32_t rounds = 0;
-        for (;;) {
-            if (X > 1) GC_LAUNCH(KID_TENTATIVE, s, k_tentative<true><<<grid_t, kBlock, 0, s>>>(a));
-            else GC_LAUNCH(KID_TENTATIVE, s, k_tentative<false><<<grid_t, kBlock, 0, s>>>(a));
-            if (heavy && pull) GC_LAUNCH(KID_CONFLICT, s, k_conflict<true, 4><<<grid_ch, kBlock, 0, s>>>(a));
-            else if (heavy) GC_LAUNCH(KID_CONFLICT, s, k_conflict<true, 5><<<grid_ch, kBlock, 0, s>>>(a));
-            else GC_LAUNCH(KID_CONFLICT, s, k_conflict<false, 4><<<grid_cl, kBlock, 0, s>>>(a));
-            if (heavy) GC_LAUNCH(KID_MARK, s, k_mark_colors<<<grid_m, kBlock, 0, s>>>(a));
-            ++rounds;
-            cudaMemcpyAsync(t_pinned.p, &a.ctrl->active, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-            cudaError_t ce = cudaStreamSynchronize(s);
-            if (ce != cudaSuccess) { st = cuda_status(ce); break; }
-            if (t_pinned.p[0] == 0) break;
-            if (rounds >= a.round_limit) { st = GC_ERR_ROUND_LIMIT; break; }
-        }
-    }
-    cudaEventRecord(e1, s);
-    SpecCtrl h;
-    cudaError_t ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-    if (ce != cudaSuccess && st == GC_OK) st = cuda_status(ce);
-    if (st == GC_OK) st = status_from_err_bits(h.err);
-    if (a.tune.spec_graph) note_launches((heavy ? 3 : 2) * static_cast<int64_t>(h.round));
+    cudaEventRecord(ev.e1, s);
     if (stats) {
         std::memset(stats, 0, sizeof(*stats));
         stats->rounds = h.round;
         stats->max_color = h.max_color;
-        stats->edges_examined = static_cast<int64_t>(h.edges);
+        stats->edges_examined = static_cast<int64_t>(h.edges) + g.nnz;  // round 0's choice: every row once
         stats->conflicts = static_cast<int64_t>(h.conflicts);
         float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
+        cudaEventSynchronize(ev.e1);
+        cudaEventElapsedTime(&ms, ev.e0, ev.e1);
         stats->ms_color = ms;
     }
     return st;
@@ -1476,14 +1420,14 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
 
 gc_status color_device(const Graph& g, int32_t X, uint64_t seed, int32_t* colors_out,
                        gc_stats* stats, cudaStream_t s) {
-    return color_impl(g, X, seed, nullptr, nullptr, 0, nullptr, PrioRule{}, colors_out, stats, s);
+    return color_impl(g, X, seed, nullptr, nullptr, nullptr, PrioRule{}, colors_out, stats, s);
 }
 
 gc_status color_lf_device(const Graph& g, int32_t X, uint64_t seed, int32_t* colors_out,
                           gc_stats* stats, cudaStream_t s) {
     PrioRule r;
     r.kind = 1;
-    return color_impl(g, X, seed, nullptr, nullptr, 0, nullptr, r, colors_out, stats, s);
+    return color_impl(g, X, seed, nullptr, nullptr, nullptr, r, colors_out, stats, s);
 }
 
 // aRC (Sec. 3): every iteration colors the graph again by the speculative
@@ -1520,7 +1464,7 @@ gc_status recolor_async_device(const Graph& g, const int32_t* colors_in, int32_t
         r.rank = sc_rank.as<int32_t>();
         r.old = old;
         gc_stats cs;
-        st = color_impl(g, 1, seed, nullptr, nullptr, 0, nullptr, r, colors_out, &cs, s);
+        st = color_impl(g, 1, seed, nullptr, nullptr, nullptr, r, colors_out, &cs, s);
         if (st != GC_OK) break;
         maxc = cs.max_color;
         if (ncolors_per_iter) ncolors_per_iter[it + 1] = maxc;
@@ -1654,7 +1598,7 @@ gc_status color_batch_device(const Graph& g, const gc_batch_graph* graphs, int32
     const BatchDesc* d_desc = sd.as<BatchDesc>();
     int32_t* graph_of = sgo.as<int32_t>();
     batch_graph_of(g, d_desc, ng, graph_of, s);
-    st = color_impl(g, max_x, 0, graph_of, d_desc, ng, swr.as<int32_t>(), PrioRule{}, colors_out, stats, s);
+    st = color_impl(g, max_x, 0, graph_of, d_desc, swr.as<int32_t>(), PrioRule{}, colors_out, stats, s);
     if (st != GC_OK) return st;
     if (rounds_out || max_color_out)
         st = batch_max_colors(g, graph_of, colors_out, swr.as<int32_t>(), ng, max_color_out, rounds_out, s);

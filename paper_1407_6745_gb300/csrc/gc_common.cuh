@@ -3,11 +3,9 @@
 // Degree-bucketed scheduling: every vertex to (re)color is handled by a group
 // of lanes sized to its degree.  A vertex whose answer is known to lie in the
 // first 64 colors (deg + X <= 64: at most deg colors are forbidden, and the
-// pick is among the first X permissible ones) keeps its forbidden set in a
-// 64-bit register mask, OR-reduced over a group of 4, 8, 16 or 32 lanes; a
-// larger one uses a bitmap in shared memory, per warp (deg <= warp_max_deg)
-// or per block.  The color picked is the j-th clear bit of the mask (First
-// Fit: j = 0), located with popc/ffs.
+// pick is among the first X permissible ones) keeps its forbidden set in 64
+// bits; a larger one uses a bitmap.  The color picked is the j-th clear bit
+// of the mask (First Fit: j = 0), located with popc/ffs.
 #pragma once
 
 #include <cstdint>
@@ -18,15 +16,8 @@ namespace gc {
 constexpr int kBlock = 256;          // threads per block, every kernel
 constexpr int kWarps = kBlock / 32;
 constexpr int kNB = 7;               // degree buckets
-// bucket b: 0 block/vertex, 1 warp/vertex + smem bitmap, 2..6 group of
-// 32/16/8/4/2 lanes per vertex with a 64-bit register mask
-__host__ __device__ constexpr int bucket_group(int b) {
-    return b == 0 ? kBlock : b == 1 ? 32 : b == 2 ? 32 : b == 3 ? 16 : b == 4 ? 8 : b == 5 ? 4 : 2;
-}
-// vertices per block tile
-__host__ __device__ constexpr int bucket_tile(int b) {
-    return b == 0 ? 1 : kBlock / bucket_group(b);
-}
+// bucket b: 0 split row, 1 warp/vertex + bitmap (the coloring takes both as
+// heavy rows), 2..6 group of 32/16/8/4/2 lanes per vertex, at most 64 colors
 constexpr int kWarpBitmapWords = 64;    // 2048 colors per window, per warp
 
 // error bits accumulated on the device
@@ -34,12 +25,6 @@ constexpr uint32_t kErrBadGraph = 1u;
 constexpr uint32_t kErrTimeout = 2u;
 constexpr uint32_t kErrImproper = 4u;
 constexpr uint32_t kErrRoundLimit = 8u;
-
-// Default warp threshold of the coloring phase (rows above it take a whole
-// block); on a graph whose largest row has at most kPullAllMaxDeg entries the
-// default is lifted so that every heavy row is a warp row (see color_impl).
-constexpr int32_t kDefaultWarpMaxDeg = 1024;
-constexpr int32_t kPullAllMaxDeg = 12288;
 
 // Scheduling thresholds (runtime; tuned per workload).
 struct Tuning {
@@ -50,7 +35,7 @@ struct Tuning {
     int32_t grid_blocks;   // persistent grid size (0 = 8 per SM)
     int32_t recolor_mode;  // 0 = dataflow (one launch), 1 = one launch per class
     int32_t spin_limit;    // bounded wait iterations in the dataflow recolor
-    int32_t spec_graph;    // 1: speculative rounds in a CUDA graph WHILE node; 0: host loop
+    int32_t spec_graph;    // 1: speculative rounds in one cooperative launch; 0: one launch each
     int32_t rc_warp_max_deg;  // warp_max_deg of the recoloring phase
     int32_t g2_max_deg;    // deg <= this -> 2 lanes (0: none)
     int32_t rc_g2_max_deg;  // g2_max_deg of the recoloring phase (capped at g4_max_deg)
@@ -153,22 +138,6 @@ constexpr unsigned kFull = 0xffffffffu;
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 template <int G>
-__device__ __forceinline__ uint64_t group_or(uint64_t m) {
-    uint32_t lo = static_cast<uint32_t>(m), hi = static_cast<uint32_t>(m >> 32);
-    if constexpr (G == 32) {
-        lo = __reduce_or_sync(kFull, lo);
-        hi = __reduce_or_sync(kFull, hi);
-    } else {
-#pragma unroll
-        for (int d = G / 2; d >= 1; d >>= 1) {
-            lo |= __shfl_xor_sync(kFull, lo, d);
-            hi |= __shfl_xor_sync(kFull, hi, d);
-        }
-    }
-    return (static_cast<uint64_t>(hi) << 32) | lo;
-}
-
-template <int G>
 __device__ __forceinline__ bool group_any(bool p) {
     const uint32_t b = __ballot_sync(kFull, p);
     if constexpr (G == 32) {
@@ -211,18 +180,6 @@ __device__ __forceinline__ int select_bit64(uint64_t x, uint32_t j) {
     const uint32_t pl = __popc(lo);
     if (j < pl) return select_bit32(lo, j);
     return 32 + select_bit32(static_cast<uint32_t>(x >> 32), j - pl);
-}
-
-// Adjacency range of v with the structure checks that keep every later load
-// in bounds: a bad row is flagged and treated as empty.
-__device__ __forceinline__ void row_range(const Graph& g, int32_t v, int64_t& beg, int64_t& end,
-                                          uint32_t* err) {
-    beg = __ldg(g.off + v);
-    end = __ldg(g.off + v + 1);
-    if (beg < 0 || end < beg || end > g.nnz) {
-        atomicOr(err, kErrBadGraph);
-        beg = end = 0;
-    }
 }
 
 // Streamed data (adjacency, work items) is read once per pass: it is loaded
@@ -389,29 +346,13 @@ __device__ __forceinline__ void for_each_nbr(const Graph& g, int64_t beg, int32_
 
 // Colors of the neighbors through a Fetch: raw(u) issues the load (no
 // branch), resolve(u, x) turns it into a color, or a value < 1 to ignore.
-template <int UC, class Fetch, class Mark, bool kVec = false>
+template <int UC, class Fetch, class Mark>
 __device__ __forceinline__ void scan_row(const Graph& g, int64_t beg, int32_t deg, int32_t lane0,
                                          int32_t stride, const Fetch& fetch, Mark&& mark,
                                          uint32_t* err) {
-    for_each_nbr<UC, int32_t, kVec>(
+    for_each_nbr<UC, int32_t, false>(
         g, beg, deg, lane0, stride, [&](int32_t u) { return fetch.raw(u); },
         [&](int32_t u, int32_t x) { mark(fetch.resolve(u, x)); }, err);
-}
-
-// Register path, G lanes per vertex; requires deg + j < 64.  All 32 lanes of
-// the warp must call it (lanes without a vertex pass deg = 0).
-template <int G, int U, class Fetch, bool kVec = false>
-__device__ __forceinline__ int32_t choose_reg(const Graph& g, int64_t beg, int32_t deg, int gl,
-                                              uint32_t j, const Fetch& fetch, uint32_t* err) {
-    uint64_t m = 0;
-    auto mark = [&](int32_t c) {
-        if (static_cast<uint32_t>(c - 1) < 64u) m |= 1ull << (c - 1);
-    };
-    scan_row<U, Fetch, decltype(mark)&, kVec>(g, beg, deg, gl, G, fetch, mark, err);
-    m = group_or<G>(m);
-    const uint64_t free_bits = ~m;
-    if (j == 0) return __ffsll(static_cast<long long>(free_bits));
-    return select_bit64(free_bits, j) + 1;
 }
 
 // Warp path with a 64-word shared bitmap (2048 colors per window); windows
@@ -483,6 +424,13 @@ __device__ __forceinline__ void warp_append(bool want, int64_t beg, int32_t v, i
     if (l == leader) base = atomicAdd(counter, __popc(b));
     base = __shfl_sync(kFull, base, leader);
     if (want) store_item(list + start + base + __popc(b & ((1u << l) - 1u)), beg, v, deg);
+}
+
+// Adds 1 with acquire-release semantics at GPU scope; returns the old value.
+__device__ __forceinline__ int32_t add_acq_rel(int32_t* p) {
+    int32_t old;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
+    return old;
 }
 
 // Warp-wide sum of a per-thread count added to a global counter (one atomic

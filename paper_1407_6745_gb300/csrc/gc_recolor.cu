@@ -144,12 +144,6 @@ __device__ __forceinline__ int32_t ld_relaxed(const int32_t* p) {
 __device__ __forceinline__ void st_relaxed(int32_t* p, int32_t x) {
     asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
 }
-// Adds 1 with acquire-release semantics at GPU scope; returns the old value.
-__device__ __forceinline__ int32_t add_acq_rel(int32_t* p) {
-    int32_t old;
-    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
-    return old;
-}
 
 __device__ __forceinline__ int32_t chunks_of(int32_t deg) { return (deg + kChunk - 1) / kChunk; }
 
@@ -697,8 +691,7 @@ __device__ __forceinline__ void load8(const RecolorFetch<kDataflow>& f, const in
 template <bool kDataflow>
 __device__ __forceinline__ void wait8(const RecolorFetch<kDataflow>& f, const int32_t (&u)[8], int32_t (&x)[8],
                                       int32_t horizon) {
-    if (!kDataflow) return;
-    for (int32_t it = 0;;) {
+    for (int32_t it = 0; kDataflow;) {
         int32_t q = -1, r = -1;
 #pragma unroll
         for (int i = 0; i < 8; ++i)

@@ -371,7 +371,7 @@ static gc_status gc_recolor_impl(const gc_graph* g, const int32_t* colors_in, gc
     } else {
         dout.d = colors_out;
     }
-    st = recolor_device(dg.g, din.d, 0, false, perm, iterations, seed, dout.d, ncolors_per_iter,
+    st = recolor_device(dg.g, din.d, 0, 0, false, perm, iterations, seed, dout.d, ncolors_per_iter,
                         stats, s);
     if (st != GC_OK) return st;
     return din.unstage(colors_out, g->n, g->mem, s);
@@ -394,10 +394,11 @@ static gc_status gc_color_recolor_impl(const gc_graph* g, gc_strategy strategy, 
     if ((st = dg.stage(g, s)) != GC_OK) return st;
     if ((st = dc.stage(colors_out, g->n, g->mem, false, s)) != GC_OK) return st;
     gc_stats cs;
-    st = color_device(dg.g, X, seed, dc.d, &cs, s);
+    int32_t max_deg = 0;
+    st = color_device(dg.g, X, seed, dc.d, &cs, s, &max_deg);
     if (st != GC_OK) return st;
     gc_stats rs;
-    st = recolor_device(dg.g, dc.d, cs.max_color, true, perm, iterations, perm_seed, dc.d,
+    st = recolor_device(dg.g, dc.d, cs.max_color, max_deg, true, perm, iterations, perm_seed, dc.d,
                         ncolors_per_iter, &rs, s);
     if (st != GC_OK) return st;
     if (stats) {

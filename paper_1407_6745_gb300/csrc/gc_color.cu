@@ -1311,32 +1311,30 @@ gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_
 // The speculative coloring; with graph_of / desc / win_round set, a batch.
 static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int32_t* graph_of,
                             const BatchDesc* desc, int32_t* win_round, const PrioRule& rule,
-                            int32_t* colors_out, gc_stats* stats, cudaStream_t s) {
+                            int32_t* colors_out, gc_stats* stats, cudaStream_t s, int32_t* max_deg = nullptr) {
+    if (max_deg) *max_deg = 0;
     if (g.n == 0) {
         if (stats) { std::memset(stats, 0, sizeof(*stats)); }
         return GC_OK;
     }
     const int64_t n = g.n;
     const bool wide = n <= kWideMax;
-    Scratch sc_prio, sc_lo, sc_hi, sc_l0, sc_l1, sc_bucket, sc_ctrl;
-    if (!sc_prio.alloc(n * (wide ? 8 : 4), s) || !sc_lo.alloc(n * 4, s) || !sc_hi.alloc(n * 4, s) ||
-        !sc_l0.alloc(n * sizeof(WorkItem), s) || !sc_l1.alloc(n * sizeof(WorkItem), s) ||
-        !sc_bucket.alloc(n, s) || !sc_ctrl.alloc(sizeof(SpecCtrl), s))
-        return GC_ERR_OOM;
     SpecArgs a;
     std::memset(&a, 0, sizeof(a));
+    ScratchSet sc;
+    sc.want(&a.ctrl, sizeof(SpecCtrl));
+    sc.want(&a.prio, n * (wide ? 8 : 4));
+    sc.want(&a.mlo, n * 4);
+    sc.want(&a.mhi, n * 4);
+    sc.want(&a.list0, n * static_cast<int64_t>(sizeof(WorkItem)));
+    sc.want(&a.list1, n * static_cast<int64_t>(sizeof(WorkItem)));
+    sc.want(&a.bucket, n);
+    if (!sc.alloc(s)) return GC_ERR_OOM;
     a.g = g;
     a.X = X;
     a.seed = seed;
     a.tune = current_tuning();
     a.color = colors_out;
-    a.prio = sc_prio.as<uint32_t>();
-    a.mlo = sc_lo.as<uint32_t>();
-    a.mhi = sc_hi.as<uint32_t>();
-    a.bucket = sc_bucket.as<uint8_t>();
-    a.list0 = sc_l0.as<WorkItem>();
-    a.list1 = sc_l1.as<WorkItem>();
-    a.ctrl = sc_ctrl.as<SpecCtrl>();
     a.graph_of = graph_of;
     a.desc = desc;
     a.win_round = win_round;
@@ -1363,47 +1361,42 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
     GC_LAUNCH(KID_SPEC_SETUP, s, setup<<<setup_grid, kBlock, 0, s>>>(a));
     SpecCtrl h;
     gc_status st = run_rounds(a, X > 1, false, &h, s);
-    Scratch sc_pbeg, sc_pcnt, sc_bref, sc_pend, sc_hbm, sc_hsums, sc_mark, sc_open, sc_orow, sc_odone, sc_olost;
+    ScratchSet sc_heavy, sc_queues;
     if (st == GC_OK && h.init_cnt[0] > 0) {
         // heavy rows: their lists and bitmaps (sizes read back), then the rounds
         const int32_t nh = h.init_cnt[0];
         const int hblocks = static_cast<int>((static_cast<int64_t>(nh) + kHeavyChunk - 1) / kHeavyChunk);
-        if (!sc_pbeg.alloc(static_cast<int64_t>(nh) * 8, s) || !sc_pcnt.alloc(static_cast<int64_t>(nh) * 4, s) ||
-            !sc_bref.alloc(n * 8, s) || !sc_hsums.alloc(static_cast<int64_t>(hblocks) * 16, s))
-            return GC_ERR_OOM;
-        GC_LAUNCH(KID_SPEC_FILL, s, k_heavy_sums<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sc_hsums.as<long long>()));
+        HeavyRows& hr = a.heavy;
+        long long* sums = nullptr;
+        sc_heavy.want(&hr.h_pbeg, static_cast<int64_t>(nh) * 8);
+        sc_heavy.want(&hr.h_pcnt, static_cast<int64_t>(nh) * 4);
+        sc_heavy.want(&hr.bref, n * 8);
+        sc_heavy.want(&sums, static_cast<int64_t>(hblocks) * 16);
+        if (!sc_heavy.alloc(s)) return GC_ERR_OOM;
+        GC_LAUNCH(KID_SPEC_FILL, s, k_heavy_sums<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sums));
         cudaError_t ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
         if (ce != cudaSuccess) return cuda_status(ce);
-        HeavyRows& hr = a.heavy;
         hr.mark_cap = h.heavy_entries / kPiece + nh;  // every piece of every row
         hr.open_rows_cap = h.heavy_entries / kLongList + 1;
         hr.open_cap = h.heavy_entries / kOpenPiece + hr.open_rows_cap;
-        if (!sc_pend.alloc(static_cast<size_t>(h.heavy_entries) * 4, s) ||
-            !sc_hbm.alloc(static_cast<size_t>(h.heavy_words) * 4, s) ||
-            !sc_mark.alloc(static_cast<size_t>(hr.mark_cap) * sizeof(WorkItem), s) ||
-            !sc_open.alloc(static_cast<size_t>(hr.open_cap) * sizeof(WorkItem), s) ||
-            !sc_orow.alloc(static_cast<size_t>(hr.open_rows_cap) * sizeof(WorkItem), s) ||
-            !sc_odone.alloc(static_cast<size_t>(hr.open_rows_cap) * 4, s) ||
-            !sc_olost.alloc(static_cast<size_t>(hr.open_rows_cap) * 4, s))
-            return GC_ERR_OOM;
-        hr.h_pbeg = sc_pbeg.as<int64_t>();
-        hr.h_pcnt = sc_pcnt.as<int32_t>();
-        hr.bref = sc_bref.as<uint64_t>();
-        hr.pend = sc_pend.as<int32_t>();
-        hr.hbm = sc_hbm.as<uint32_t>();
-        hr.mark = sc_mark.as<WorkItem>();
-        hr.open = sc_open.as<WorkItem>();
-        hr.open_row = sc_orow.as<WorkItem>();
-        hr.open_done = sc_odone.as<int32_t>();
-        hr.open_lost = sc_olost.as<int32_t>();
+        constexpr int64_t kItem = sizeof(WorkItem);
+        sc_queues.want(&hr.pend, h.heavy_entries * 4);
+        sc_queues.want(&hr.hbm, h.heavy_words * 4);
+        sc_queues.want(&hr.mark, hr.mark_cap * kItem);
+        sc_queues.want(&hr.open, hr.open_cap * kItem);
+        sc_queues.want(&hr.open_row, hr.open_rows_cap * kItem);
+        sc_queues.want(&hr.open_done, hr.open_rows_cap * 4);
+        sc_queues.want(&hr.open_lost, hr.open_rows_cap * 4);
+        if (!sc_queues.alloc(s)) return GC_ERR_OOM;
         ce = cudaMemsetAsync(hr.hbm, 0, static_cast<size_t>(h.heavy_words) * 4, s);
         if (ce != cudaSuccess) return cuda_status(ce);
         GC_LAUNCH(KID_SPEC_FILL, s,
-                  k_heavy_setup<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sc_hsums.as<long long>()));
+                  k_heavy_setup<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sums));
         st = run_rounds(a, X > 1, true, &h, s);
     }
     cudaEventRecord(ev.e1, s);
+    if (max_deg) *max_deg = h.max_deg;
     if (stats) {
         std::memset(stats, 0, sizeof(*stats));
         stats->rounds = h.round;
@@ -1419,8 +1412,8 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
 }
 
 gc_status color_device(const Graph& g, int32_t X, uint64_t seed, int32_t* colors_out,
-                       gc_stats* stats, cudaStream_t s) {
-    return color_impl(g, X, seed, nullptr, nullptr, nullptr, PrioRule{}, colors_out, stats, s);
+                       gc_stats* stats, cudaStream_t s, int32_t* max_deg) {
+    return color_impl(g, X, seed, nullptr, nullptr, nullptr, PrioRule{}, colors_out, stats, s, max_deg);
 }
 
 gc_status color_lf_device(const Graph& g, int32_t X, uint64_t seed, int32_t* colors_out,

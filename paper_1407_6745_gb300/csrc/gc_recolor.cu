@@ -77,7 +77,6 @@ struct RcCtrl {
     int32_t k;            // present classes this iteration
     int32_t total_tiles;  // warp tiles this iteration
     int32_t hub_next;     // next free split-row slot
-    int32_t max_deg;
     int32_t max_in;       // max input color (validation)
     int32_t n_heavy;      // rows in bucket 0 (split into chunks)
     uint32_t err;
@@ -152,17 +151,15 @@ __device__ __forceinline__ int32_t chunks_of(int32_t deg) { return (deg + kChunk
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBlock) k_rc_bucket(RcArgs a) {
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kBlock;
-    int32_t my_max = 0, heavy = 0;
+    int32_t heavy = 0;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * kBlock + threadIdx.x; i < a.g.n; i += stride) {
         int64_t beg;
         int32_t deg;
         row_of(a.g, static_cast<int32_t>(i), beg, deg, &a.ctrl->err);
-        my_max = max(my_max, deg);
         const int b = rc_bucket_of(deg, a.tune);
         a.bucket[i] = static_cast<uint8_t>(b);
         heavy += b == 0;
     }
-    warp_max(&a.ctrl->max_deg, my_max);
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) heavy += __shfl_xor_sync(kFull, heavy, d);
     if (lane_id() == 0 && heavy) atomicAdd(&a.ctrl->n_heavy, heavy);
@@ -188,6 +185,9 @@ constexpr int kHistSmem = 8192;
 
 constexpr int kIsoSmem = 1024;  // isolated vertices per class, colors below this counted in shared memory
 
+// kBucket: it also sets the buckets (k_rc_bucket's part, where nothing has to
+// be known of them before).
+template <bool kBucket>
 __global__ void __launch_bounds__(kBlock) k_rc_hist(RcArgs a) {
     __shared__ int32_t sh[kHistSmem];
     __shared__ int32_t s_iso[kIsoSmem];
@@ -200,11 +200,21 @@ __global__ void __launch_bounds__(kBlock) k_rc_hist(RcArgs a) {
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kBlock;
     for (int64_t v = static_cast<int64_t>(blockIdx.x) * kBlock + threadIdx.x; v < a.g.n; v += stride) {
         const int32_t c = a.old_c[v];
+        int b;
+        if (kBucket) {
+            int64_t beg;
+            int32_t deg;
+            row_of(a.g, static_cast<int32_t>(v), beg, deg, &a.ctrl->err);
+            b = rc_bucket_of(deg, a.tune);
+            a.bucket[v] = static_cast<uint8_t>(b);
+            if (b == 0 && !a.ctrl->n_heavy) atomicOr(&a.ctrl->n_heavy, 1);  // (only whether there are any is asked)
+        } else {
+            b = a.bucket[v];
+        }
         if (c < 1 || c > a.cap) {
             atomicOr(&a.ctrl->err, kErrImproper);
             continue;
         }
-        const int b = a.bucket[v];
         if (b == kIsoBucket) {
             if (c < kIsoSmem) atomicAdd(&s_iso[c], 1);
             else atomicAdd(&a.iso_cnt[c], 1);
@@ -1170,18 +1180,18 @@ gc_status class_ranks_device(const Graph& g, const int32_t* colors, bool trusted
     const Tuning tune = recolor_tuning(current_tuning());
     const int grid = persistent_grid(tune);
     const int vgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + kBlock - 1) / kBlock, grid)));
-    Scratch sc_ctrl, sc_bucket;
-    if (!sc_ctrl.alloc(sizeof(RcCtrl), s) || !sc_bucket.alloc(n + 1, s)) return GC_ERR_OOM;
     RcArgs a;
     std::memset(&a, 0, sizeof(a));
+    ScratchSet sc_rows, sc;
+    sc_rows.want(&a.ctrl, sizeof(RcCtrl));
+    sc_rows.want(&a.bucket, n);
+    if (!sc_rows.alloc(s)) return GC_ERR_OOM;
     a.g = g;
     a.tune = tune;
     a.seed = seed;
     a.perm = perm;
     a.iteration = iteration;
     a.old_c = colors;
-    a.bucket = sc_bucket.as<uint8_t>();
-    a.ctrl = sc_ctrl.as<RcCtrl>();
     cudaMemsetAsync(a.ctrl, 0, sizeof(RcCtrl), s);
     GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
     int32_t max_checked = 0;
@@ -1200,29 +1210,23 @@ gc_status class_ranks_device(const Graph& g, const int32_t* colors, bool trusted
     if (!rank_out) return GC_OK;
     const int32_t cap = std::max(h.max_in, 1);
     const int64_t ent = static_cast<int64_t>(cap + 1) * kRcNB;
-    Scratch sc_cls, sc_units, sc_present, sc_psize, sc_order, sc_jtab, sc_seg, sc_tiles, sc_fill, sc_iso;
-    if (!sc_cls.alloc(ent * 4, s) || !sc_units.alloc((cap + 1) * 4, s) || !sc_iso.alloc((cap + 1) * 4, s) ||
-        !sc_present.alloc((cap + 1) * 4, s) || !sc_psize.alloc((cap + 1) * 4, s) ||
-        !sc_order.alloc((cap + 1) * 4, s) || !sc_jtab.alloc((cap + 1) * 4, s) ||
-        !sc_seg.alloc((ent + 1) * 4, s) || !sc_tiles.alloc((ent + 1) * 4, s) || !sc_fill.alloc(ent * 4, s))
-        return GC_ERR_OOM;
+    const int64_t c4 = static_cast<int64_t>(cap + 1) * 4, hist_bytes = ent * 4 + 2 * c4;
+    sc.want(&a.cls_cnt, hist_bytes);
+    sc.want(&a.present, c4);
+    sc.want(&a.psize, c4);
+    sc.want(&a.order, c4);
+    sc.want(&a.jtab, c4);
+    sc.want(&a.seg_start, (ent + 1) * 4);
+    sc.want(&a.tile_prefix, (ent + 1) * 4);
+    sc.want(&a.fill, ent * 4);
+    if (!sc.alloc(s)) return GC_ERR_OOM;
     a.cap = cap;
-    a.cls_cnt = sc_cls.as<int32_t>();
-    a.cls_units = sc_units.as<int32_t>();
-    a.present = sc_present.as<int32_t>();
-    a.psize = sc_psize.as<int32_t>();
-    a.order = sc_order.as<int32_t>();
-    a.jtab = sc_jtab.as<int32_t>();
     a.rank_of = rank_out;
-    a.seg_start = sc_seg.as<int32_t>();
-    a.tile_prefix = sc_tiles.as<int32_t>();
-    a.fill = sc_fill.as<int32_t>();
-    a.iso_cnt = sc_iso.as<int32_t>();
-    cudaMemsetAsync(a.cls_cnt, 0, ent * 4, s);
-    cudaMemsetAsync(a.cls_units, 0, (cap + 1) * 4, s);
-    cudaMemsetAsync(a.iso_cnt, 0, (cap + 1) * 4, s);
+    a.cls_units = a.cls_cnt + ent;
+    a.iso_cnt = a.cls_units + cap + 1;
+    cudaMemsetAsync(a.cls_cnt, 0, hist_bytes, s);
     cudaMemsetAsync(rank_out, 0, (cap + 1) * 4, s);
-    GC_LAUNCH(KID_RC_HIST, s, k_rc_hist<<<vgrid, kBlock, 0, s>>>(a));
+    GC_LAUNCH(KID_RC_HIST, s, k_rc_hist<false><<<vgrid, kBlock, 0, s>>>(a));
     GC_LAUNCH(KID_RC_ORDER, s, k_rc_order<<<1, kOrderThreads, 0, s>>>(a));
     ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
@@ -1362,7 +1366,7 @@ static int scatter_launch(RcArgs& a, int32_t cap, const Tuning& tune, size_t* dy
     return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(blocks, fit)));
 }
 
-gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_in, bool trusted,
+gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_in, int32_t max_deg, bool trusted,
                          int32_t perm, int32_t iterations, uint64_t seed, int32_t* colors_out,
                          int32_t* ncolors_per_iter, gc_stats* stats, cudaStream_t s) {
     const int64_t n = g.n;
@@ -1372,37 +1376,37 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     const int vgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + kBlock - 1) / kBlock, grid)));
     cudaError_t ce;
 
-    Scratch sc_ctrl, sc_bucket;
-    if (!sc_ctrl.alloc(sizeof(RcCtrl), s) || !sc_bucket.alloc(n + 1, s)) return GC_ERR_OOM;
     RcArgs a;
     std::memset(&a, 0, sizeof(a));
+    ScratchSet sc_rows, sc;
+    const int64_t ctrl_bytes = sizeof(RcCtrl) + (static_cast<int64_t>(iterations) + 1) * 4;  // and the color counts
+    sc_rows.want(&a.ctrl, ctrl_bytes);
+    sc_rows.want(&a.bucket, n);
+    if (!sc_rows.alloc(s)) return GC_ERR_OOM;
+    a.ncolors = reinterpret_cast<int32_t*>(a.ctrl + 1);
     a.g = g;
     a.tune = tune;
     a.seed = seed;
     a.perm = perm;
     a.old_c = colors_in;
-    a.bucket = sc_bucket.as<uint8_t>();
-    a.ctrl = sc_ctrl.as<RcCtrl>();
-    cudaMemsetAsync(a.ctrl, 0, sizeof(RcCtrl), s);
+    cudaMemsetAsync(a.ctrl, 0, ctrl_bytes, s);
     RcCtrl h;
     std::memset(&h, 0, sizeof(h));
-    if (n > 0) {
-        GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
-    }
     gc_status input = GC_OK;
     if (!trusted) {
         input = check_input_device(g, colors_in, kMaxInputColor, &maxc_in, s);
         if (input != GC_OK && input != GC_ERR_IMPROPER_INPUT) return input;
     }
-    // A trusted input (our own coloring) has a known max color; the split
-    // rows are then sized by a bound (a bucket-0 row has more than
-    // max(rc_warp_max_deg, 63) entries) instead of a read-back, when the
-    // bound's scratch is small.
+    // A trusted input (our own coloring) has a known max color and longest
+    // row; the split rows are then sized by a bound (a bucket-0 row has more
+    // than max(rc_warp_max_deg, 63) entries; none if the longest row is no
+    // longer) instead of a read-back, when the bound's scratch is small.
     const int64_t heavy_min = std::max<int64_t>(tune.warp_max_deg, 63) + 1;
-    const int64_t heavy_bound = std::min<int64_t>(n, static_cast<int64_t>(g.nnz) / heavy_min);
+    const int64_t heavy_bound = max_deg < heavy_min ? 0 : std::min<int64_t>(n, static_cast<int64_t>(g.nnz) / heavy_min);
     const int64_t bound_words = (static_cast<int64_t>(std::max(maxc_in, 1)) + 1 + 31) / 32 + kRowPend;
     const bool read_back = !trusted || n == 0 || heavy_bound * bound_words * 4 > (int64_t(64) << 20);
     if (read_back) {
+        if (n > 0) GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
         ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
         if (ce != cudaSuccess) return cuda_status(ce);
@@ -1431,41 +1435,30 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     const int64_t ent = static_cast<int64_t>(cap + 1) * kRcNB;
     const int32_t hub_words = ((cap + 1 + 31) / 32 + 3) & ~3;  // 16-byte rows
     const int64_t hubs = std::max<int64_t>(1, h.n_heavy);
-    Scratch sc_cls, sc_units, sc_cls2, sc_units2, sc_present, sc_psize, sc_order, sc_jtab, sc_rank, sc_seg, sc_tiles,
-        sc_fill, sc_list, sc_alt, sc_ncol, sc_hv, sc_hn, sc_hd, sc_hb, sc_hp, sc_hl, sc_iso, sc_iso2;
     // list entries: one per vertex, one per chunk of a bucket-0 row
     const int64_t list_len = n + (static_cast<int64_t>(g.nnz) / kChunk) + h.n_heavy;
-    if (!sc_cls.alloc(ent * 4, s) || !sc_units.alloc((cap + 1) * 4, s) ||
-        !sc_cls2.alloc(ent * 4, s) || !sc_units2.alloc((cap + 1) * 4, s) ||
-        !sc_present.alloc((cap + 1) * 4, s) || !sc_psize.alloc((cap + 1) * 4, s) ||
-        !sc_order.alloc((cap + 1) * 4, s) || !sc_jtab.alloc((cap + 1) * 4, s) ||
-        !sc_rank.alloc((cap + 1) * 4, s) || !sc_seg.alloc((ent + 1) * 4, s) ||
-        !sc_tiles.alloc((ent + 1) * 4, s) || !sc_fill.alloc(ent * 4, s) ||
-        !sc_list.alloc(list_len * sizeof(WorkItem), s) || !sc_alt.alloc(n * 4, s) ||
-        !sc_ncol.alloc((iterations + 1) * 4, s) || !sc_hv.alloc(hubs * 4, s) ||
-        !sc_hn.alloc(hubs * 4, s) || !sc_hd.alloc(hubs * 4, s) ||
-        !sc_hb.alloc(hubs * hub_words * 4, s) || !sc_hp.alloc(hubs * 4, s) ||
-        !sc_hl.alloc(hubs * kRowPend * 4, s) || !sc_iso.alloc((cap + 1) * 4, s) ||
-        !sc_iso2.alloc((cap + 1) * 4, s))
-        return GC_ERR_OOM;
+    const int64_t c4 = static_cast<int64_t>(cap + 1) * 4, hist_bytes = ent * 4 + 2 * c4;
+    int32_t *hist = nullptr, *alt = nullptr;  // hist: this iteration's and the next one's class tables
+    sc.want(&hist, 2 * hist_bytes);
+    sc.want(&a.present, c4);
+    sc.want(&a.psize, c4);
+    sc.want(&a.order, c4);
+    sc.want(&a.jtab, c4);
+    sc.want(&a.rank_of, c4);
+    sc.want(&a.seg_start, (ent + 1) * 4);
+    sc.want(&a.tile_prefix, (ent + 1) * 4);
+    sc.want(&a.fill, ent * 4);
+    sc.want(&a.list, list_len * static_cast<int64_t>(sizeof(WorkItem)));
+    sc.want(&alt, n * 4);
+    sc.want(&a.hub_v, hubs * 4);
+    sc.want(&a.hub_nch, hubs * 4);
+    sc.want(&a.hub_done, hubs * 4);
+    sc.want(&a.hub_pcnt, hubs * 4);
+    sc.want(&a.hub_bm, hubs * hub_words * 4);
+    sc.want(&a.hub_pend, hubs * kRowPend * 4);
+    if (!sc.alloc(s)) return GC_ERR_OOM;
     a.cap = cap;
-    a.present = sc_present.as<int32_t>();
-    a.psize = sc_psize.as<int32_t>();
-    a.order = sc_order.as<int32_t>();
-    a.jtab = sc_jtab.as<int32_t>();
-    a.rank_of = sc_rank.as<int32_t>();
-    a.seg_start = sc_seg.as<int32_t>();
-    a.tile_prefix = sc_tiles.as<int32_t>();
-    a.fill = sc_fill.as<int32_t>();
-    a.list = sc_list.as<WorkItem>();
-    a.ncolors = sc_ncol.as<int32_t>();
-    a.hub_v = sc_hv.as<int32_t>();
-    a.hub_nch = sc_hn.as<int32_t>();
-    a.hub_done = sc_hd.as<int32_t>();
-    a.hub_bm = sc_hb.as<uint32_t>();
     a.hub_words = hub_words;
-    a.hub_pcnt = sc_hp.as<int32_t>();
-    a.hub_pend = sc_hl.as<int32_t>();
     a.fuse_hist = 1;
     const int32_t hist_entries = static_cast<int32_t>(ent);
     const size_t hist_dyn = hist_entries <= kRcHistSmem ? static_cast<size_t>(hist_entries) * 4 : 0;
@@ -1482,13 +1475,12 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     const int step_capacity =
         sm_count() * occupancy_of(reinterpret_cast<const void*>(k_rc_recolor_step), kBlock, hist_dyn);
     const int grid_step = tune.grid_blocks > 0 ? tune.grid_blocks : step_capacity;
-    cudaMemsetAsync(a.ncolors, 0, (iterations + 1) * 4, s);
+    cudaMemsetAsync(hist, 0, 2 * hist_bytes, s);
 
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
-    int32_t* alt = sc_alt.as<int32_t>();
     const int32_t* cur = colors_in;
     gc_status st = GC_OK;
     std::vector<int32_t> tp;
@@ -1499,21 +1491,20 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
         a.new_c = dst;
         // histograms: of the input (iteration 0), else filled by the previous
         // iteration's recoloring kernel
-        a.cls_cnt = (it % 2 == 0) ? sc_cls.as<int32_t>() : sc_cls2.as<int32_t>();
-        a.cls_units = (it % 2 == 0) ? sc_units.as<int32_t>() : sc_units2.as<int32_t>();
-        a.nxt_cnt = (it % 2 == 0) ? sc_cls2.as<int32_t>() : sc_cls.as<int32_t>();
-        a.nxt_units = (it % 2 == 0) ? sc_units2.as<int32_t>() : sc_units.as<int32_t>();
-        a.iso_cnt = (it % 2 == 0) ? sc_iso.as<int32_t>() : sc_iso2.as<int32_t>();
-        a.nxt_iso = (it % 2 == 0) ? sc_iso2.as<int32_t>() : sc_iso.as<int32_t>();
-        if (it == 0) {
-            cudaMemsetAsync(a.cls_cnt, 0, ent * 4, s);
-            cudaMemsetAsync(a.cls_units, 0, (cap + 1) * 4, s);
-            cudaMemsetAsync(a.iso_cnt, 0, (cap + 1) * 4, s);
-            GC_LAUNCH(KID_RC_HIST, s, k_rc_hist<<<vgrid, kBlock, 0, s>>>(a));
+        const int64_t set = hist_bytes / 4;
+        a.cls_cnt = hist + (it % 2) * set;
+        a.cls_units = a.cls_cnt + ent;
+        a.iso_cnt = a.cls_units + cap + 1;
+        a.nxt_cnt = hist + (1 - it % 2) * set;
+        a.nxt_units = a.nxt_cnt + ent;
+        a.nxt_iso = a.nxt_units + cap + 1;
+        if (it > 0) {
+            cudaMemsetAsync(a.nxt_cnt, 0, hist_bytes, s);
+        } else if (read_back) {
+            GC_LAUNCH(KID_RC_HIST, s, k_rc_hist<false><<<vgrid, kBlock, 0, s>>>(a));
+        } else {
+            GC_LAUNCH(KID_RC_HIST, s, k_rc_hist<true><<<vgrid, kBlock, 0, s>>>(a));
         }
-        cudaMemsetAsync(a.nxt_cnt, 0, ent * 4, s);
-        cudaMemsetAsync(a.nxt_units, 0, (cap + 1) * 4, s);
-        cudaMemsetAsync(a.nxt_iso, 0, (cap + 1) * 4, s);
         GC_LAUNCH(KID_RC_ORDER, s, k_rc_order<<<1, kOrderThreads, 0, s>>>(a));
         GC_LAUNCH(KID_RC_SCATTER, s, k_rc_scatter<<<grid_sc, kBlock, sc_dyn, s>>>(a));
         if (tune.recolor_mode == 0) {
@@ -1544,10 +1535,14 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     if (st == GC_OK && cur != colors_out)
         cudaMemcpyAsync(colors_out, cur, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s);
     cudaEventRecord(e1, s);
-    std::vector<int32_t> nc(iterations + 1);
-    ce = cudaMemcpyAsync(nc.data(), a.ncolors, (iterations + 1) * 4, cudaMemcpyDeviceToHost, s);
-    if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
+    std::vector<char> back(static_cast<size_t>(ctrl_bytes));
+    ce = cudaMemcpyAsync(back.data(), a.ctrl, back.size(), cudaMemcpyDeviceToHost, s);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+    std::vector<int32_t> nc(static_cast<size_t>(iterations) + 1);
+    if (ce == cudaSuccess) {
+        std::memcpy(&h, back.data(), sizeof(RcCtrl));
+        std::memcpy(nc.data(), back.data() + sizeof(RcCtrl), nc.size() * 4);
+    }
     if (ce != cudaSuccess && st == GC_OK) st = cuda_status(ce);
     if (st == GC_OK) st = status_from_err_bits(h.err);
     if (ncolors_per_iter) std::copy(nc.begin(), nc.end(), ncolors_per_iter);
@@ -1593,23 +1588,25 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
     const int grid_go = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((ng + kWarps - 1) / kWarps, grid)));
     cudaError_t ce;
 
-    Scratch sc_ctrl, sc_bucket, sc_desc, sc_gof;
-    if (!sc_ctrl.alloc(sizeof(RcCtrl), s) || !sc_bucket.alloc(n + 1, s) ||
-        !sc_desc.alloc(static_cast<size_t>(ng) * sizeof(BatchDesc), s) || !sc_gof.alloc(n * 4 + 4, s))
-        return GC_ERR_OOM;
-    ce = cudaMemcpyAsync(sc_desc.p, graphs, static_cast<size_t>(ng) * sizeof(BatchDesc), cudaMemcpyHostToDevice, s);
-    if (ce != cudaSuccess) return cuda_status(ce);
     RcArgs a;
     std::memset(&a, 0, sizeof(a));
+    ScratchSet sc_rows, sc;
+    BatchDesc* desc = nullptr;
+    int32_t* graph_of = nullptr;
+    sc_rows.want(&a.ctrl, sizeof(RcCtrl));
+    sc_rows.want(&a.bucket, n);
+    sc_rows.want(&desc, static_cast<int64_t>(ng) * static_cast<int64_t>(sizeof(BatchDesc)));
+    sc_rows.want(&graph_of, n * 4);
+    if (!sc_rows.alloc(s)) return GC_ERR_OOM;
+    ce = cudaMemcpyAsync(desc, graphs, static_cast<size_t>(ng) * sizeof(BatchDesc), cudaMemcpyHostToDevice, s);
+    if (ce != cudaSuccess) return cuda_status(ce);
     a.g = g;
     a.tune = tune;
     a.old_c = colors_in;
-    a.bucket = sc_bucket.as<uint8_t>();
-    a.ctrl = sc_ctrl.as<RcCtrl>();
-    a.desc = sc_desc.as<BatchDesc>();
-    a.graph_of = sc_gof.as<int32_t>();
+    a.desc = desc;
+    a.graph_of = graph_of;
     a.ngraphs = ng;
-    batch_graph_of(g, a.desc, ng, sc_gof.as<int32_t>(), s);
+    batch_graph_of(g, desc, ng, graph_of, s);
     cudaMemsetAsync(a.ctrl, 0, sizeof(RcCtrl), s);
     if (n > 0) {
         GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
@@ -1653,42 +1650,37 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
     const int64_t list_len = n + (static_cast<int64_t>(g.nnz) / kChunk) + h.n_heavy;
     const int grid_rc = tune.grid_blocks > 0 ? std::min(tune.grid_blocks, coop_capacity)
                                              : coop_grid(g.nnz, cap, coop_capacity);
-    Scratch sc_base, sc_cls, sc_units, sc_rank, sc_gp, sc_gs, sc_go, sc_gj, sc_segc, sc_seg, sc_tiles,
-        sc_fill, sc_list, sc_alt, sc_ncol, sc_hv, sc_hn, sc_hd, sc_hb, sc_hp, sc_hl, sc_iso;
-    if (!sc_base.alloc((ng + 1) * 8, s) || !sc_cls.alloc(T * kRcNB * 4, s) || !sc_units.alloc(T * 4, s) ||
-        !sc_rank.alloc(T * 4, s) || !sc_gp.alloc(T * 4, s) || !sc_gs.alloc(T * 4, s) ||
-        !sc_go.alloc(T * 4, s) || !sc_gj.alloc(T * 4, s) || !sc_segc.alloc(ent * 4, s) ||
-        !sc_seg.alloc((ent + 1) * 4, s) || !sc_tiles.alloc((ent + 1) * 4, s) || !sc_fill.alloc(ent * 4, s) ||
-        !sc_list.alloc(list_len * sizeof(WorkItem), s) || !sc_alt.alloc(n * 4, s) ||
-        !sc_ncol.alloc((iters + 1) * 4, s) || !sc_hv.alloc(hubs * 4, s) || !sc_hn.alloc(hubs * 4, s) ||
-        !sc_hd.alloc(hubs * 4, s) || !sc_hb.alloc(hubs * hub_words * 4, s) || !sc_hp.alloc(hubs * 4, s) ||
-        !sc_hl.alloc(hubs * kRowPend * 4, s) || !sc_iso.alloc(T * 4, s))
-        return GC_ERR_OOM;
-    ce = cudaMemcpyAsync(sc_base.p, base.data(), (ng + 1) * 8, cudaMemcpyHostToDevice, s);
+    int64_t* cls_base = nullptr;
+    int32_t *alt = nullptr;
+    const int64_t t4 = T * 4, hist_bytes = (kRcNB + 2) * t4 + ent * 4;
+    sc.want(&cls_base, (static_cast<int64_t>(ng) + 1) * 8);
+    sc.want(&a.cls_cnt, hist_bytes);
+    sc.want(&a.rank_of, t4);
+    sc.want(&a.gpresent, t4);
+    sc.want(&a.gpsize, t4);
+    sc.want(&a.gorder, t4);
+    sc.want(&a.gjtab, t4);
+    sc.want(&a.seg_start, (ent + 1) * 4);
+    sc.want(&a.tile_prefix, (ent + 1) * 4);
+    sc.want(&a.fill, ent * 4);
+    sc.want(&a.list, list_len * static_cast<int64_t>(sizeof(WorkItem)));
+    sc.want(&alt, n * 4);
+    sc.want(&a.ncolors, (static_cast<int64_t>(iters) + 1) * 4);
+    sc.want(&a.hub_v, hubs * 4);
+    sc.want(&a.hub_nch, hubs * 4);
+    sc.want(&a.hub_done, hubs * 4);
+    sc.want(&a.hub_pcnt, hubs * 4);
+    sc.want(&a.hub_bm, hubs * hub_words * 4);
+    sc.want(&a.hub_pend, hubs * kRowPend * 4);
+    if (!sc.alloc(s)) return GC_ERR_OOM;
+    ce = cudaMemcpyAsync(cls_base, base.data(), (ng + 1) * 8, cudaMemcpyHostToDevice, s);
     if (ce != cudaSuccess) return cuda_status(ce);
     a.cap = cap;
-    a.cls_base = sc_base.as<int64_t>();
-    a.cls_cnt = sc_cls.as<int32_t>();
-    a.cls_units = sc_units.as<int32_t>();
-    a.rank_of = sc_rank.as<int32_t>();
-    a.gpresent = sc_gp.as<int32_t>();
-    a.gpsize = sc_gs.as<int32_t>();
-    a.gorder = sc_go.as<int32_t>();
-    a.gjtab = sc_gj.as<int32_t>();
-    a.seg_cnt = sc_segc.as<int32_t>();
-    a.seg_start = sc_seg.as<int32_t>();
-    a.tile_prefix = sc_tiles.as<int32_t>();
-    a.fill = sc_fill.as<int32_t>();
-    a.list = sc_list.as<WorkItem>();
-    a.ncolors = sc_ncol.as<int32_t>();
-    a.hub_v = sc_hv.as<int32_t>();
-    a.hub_nch = sc_hn.as<int32_t>();
-    a.hub_done = sc_hd.as<int32_t>();
-    a.hub_bm = sc_hb.as<uint32_t>();
+    a.cls_base = cls_base;
+    a.cls_units = a.cls_cnt + T * kRcNB;
+    a.iso_cnt = a.cls_units + T;
+    a.seg_cnt = a.iso_cnt + T;
     a.hub_words = hub_words;
-    a.hub_pcnt = sc_hp.as<int32_t>();
-    a.hub_pend = sc_hl.as<int32_t>();
-    a.iso_cnt = sc_iso.as<int32_t>();
     a.fuse_hist = 0;
     size_t sc_dyn = 0;
     const int grid_sc = scatter_launch(a, cap, tune, &sc_dyn);
@@ -1698,7 +1690,6 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
-    int32_t* alt = sc_alt.as<int32_t>();
     const int32_t* cur = colors_in;
     std::vector<int32_t> tp;
     for (int32_t it = it_begin; it < iters && st == GC_OK; ++it) {
@@ -1706,10 +1697,7 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
         a.iteration = it;
         a.old_c = cur;
         a.new_c = dst;
-        cudaMemsetAsync(a.cls_cnt, 0, T * kRcNB * 4, s);
-        cudaMemsetAsync(a.cls_units, 0, T * 4, s);
-        cudaMemsetAsync(a.iso_cnt, 0, T * 4, s);
-        cudaMemsetAsync(a.seg_cnt, 0, ent * 4, s);
+        cudaMemsetAsync(a.cls_cnt, 0, hist_bytes, s);
         cudaMemsetAsync(&a.ctrl->k, 0, sizeof(int32_t), s);
         GC_LAUNCH(KID_BRC_HIST, s, k_brc_hist<<<vgrid, kBlock, 0, s>>>(a));
         GC_LAUNCH(KID_BRC_ORDER, s, k_brc_order<<<grid_go, kBlock, 0, s>>>(a));

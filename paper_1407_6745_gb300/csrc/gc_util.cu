@@ -13,7 +13,7 @@ namespace gc {
 struct ValCtrl {
     unsigned long long conflicts;
     unsigned long long uncolored;
-    long long first_bad;
+    unsigned long long bad_rank;  // n minus the first bad vertex; 0: none
     int32_t max_color;
     uint32_t err;
     unsigned long long distinct;
@@ -64,7 +64,7 @@ __device__ __forceinline__ void account(const ValArgs& a, int32_t v, int32_t cv,
                                         unsigned long long& unc, int32_t& my_max) {
     conf += static_cast<unsigned long long>(same);
     if (cv < 1) ++unc;
-    if (cv < 1 || same > 0) atomicMin(&a.c->first_bad, static_cast<long long>(v));
+    if (cv < 1 || same > 0) atomicMax(&a.c->bad_rank, static_cast<unsigned long long>(a.g.n) - static_cast<unsigned long long>(v));
     my_max = max(my_max, cv);
     if (cv >= 1 && cv < kPresColors) atomicOr(&s_pres[cv >> 5], 1u << (cv & 31));
     else if (cv >= kPresColors) atomicAdd(&a.c->big_colors, 1);
@@ -80,7 +80,7 @@ __device__ __forceinline__ void account_piece(const ValArgs& a, int32_t v, int32
         return;
     }
     conf += static_cast<unsigned long long>(same);
-    if (same > 0) atomicMin(&a.c->first_bad, static_cast<long long>(v));
+    if (same > 0) atomicMax(&a.c->bad_rank, static_cast<unsigned long long>(a.g.n) - static_cast<unsigned long long>(v));
 }
 
 __device__ __forceinline__ void flush_presence(const ValArgs& a, uint32_t* s_pres) {
@@ -203,21 +203,19 @@ __global__ void __launch_bounds__(kBlock) k_count_bits(int64_t words, const uint
 
 // The scratch of one validation and its two passes over the rows.
 struct ValRun {
-    Scratch sc, sp, shv, spc;
+    ScratchSet sc;
     ValArgs a{};
     gc_status start(const Graph& g, const int32_t* colors, int32_t max_allowed, const Tuning& t, cudaStream_t s) {
+        a = ValArgs{g, colors, nullptr, nullptr, nullptr, nullptr, 0, max_allowed};
         // pieces: at most one per kValPiece entries, plus one per row beyond kValWarpDeg
-        const int64_t piece_cap = g.nnz / kValPiece + g.nnz / kValWarpDeg + 1;
-        if (!sc.alloc(sizeof(ValCtrl), s) || !sp.alloc(kPresWords * 4, s) ||
-            !shv.alloc(static_cast<int64_t>(g.n) * 4, s) || !spc.alloc(piece_cap * sizeof(int2), s))
-            return GC_ERR_OOM;
-        a = ValArgs{g, colors, sc.as<ValCtrl>(), sp.as<uint32_t>(), shv.as<int32_t>(), spc.as<int2>(), piece_cap,
-                    max_allowed};
-        ValCtrl h;
-        std::memset(&h, 0, sizeof(h));
-        h.first_bad = LLONG_MAX;
-        cudaMemcpyAsync(a.c, &h, sizeof(h), cudaMemcpyHostToDevice, s);
-        cudaMemsetAsync(a.pres, 0, kPresWords * 4, s);
+        a.piece_cap = g.nnz / kValPiece + g.nnz / kValWarpDeg + 1;
+        static_assert(sizeof(ValCtrl) % 8 == 0, "the bitmap follows it");
+        sc.want(&a.c, sizeof(ValCtrl) + kPresWords * 4);
+        sc.want(&a.heavy, static_cast<int64_t>(g.n) * 4);
+        sc.want(&a.pieces, a.piece_cap * static_cast<int64_t>(sizeof(int2)));
+        if (!sc.alloc(s)) return GC_ERR_OOM;
+        a.pres = reinterpret_cast<uint32_t*>(a.c + 1);
+        cudaMemsetAsync(a.c, 0, sizeof(ValCtrl) + kPresWords * 4, s);
         const bool input = max_allowed != 0;
         const auto light = input ? k_validate<true> : k_validate<false>;
         GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE, s, light<<<resident_grid(light, t), kBlock, 0, s>>>(a));
@@ -287,7 +285,7 @@ gc_status validate_device(const Graph& g, const int32_t* colors, gc_validation* 
     out->n_uncolored = static_cast<int64_t>(h.uncolored);
     out->max_color = h.max_color;
     out->n_distinct = static_cast<int32_t>(distinct);
-    out->first_bad_vertex = h.first_bad == LLONG_MAX ? -1 : static_cast<int64_t>(h.first_bad);
+    out->first_bad_vertex = h.bad_rank == 0 ? -1 : static_cast<int64_t>(g.n) - static_cast<int64_t>(h.bad_rank);
     return GC_OK;
 }
 
@@ -312,13 +310,13 @@ struct NoAllocScratch {
 
 static __device__ __align__(256) NoAllocScratch g_validate_scratch;
 
-// Clears what every call must start from: counters, the first bad vertex
-// (LLONG_MAX = none yet) and the presence bitmap.
+// Clears what every call must start from: counters, the first bad vertex and
+// the presence bitmap.
 __global__ void __launch_bounds__(kBlock) k_validate_na_clear(NoAllocScratch* sc) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc->ctrl.conflicts = 0;
         sc->ctrl.uncolored = 0;
-        sc->ctrl.first_bad = LLONG_MAX;
+        sc->ctrl.bad_rank = 0;
         sc->ctrl.max_color = 0;
         sc->ctrl.err = 0;
         sc->ctrl.distinct = 0;
@@ -482,7 +480,7 @@ gc_status validate_noalloc_device(const Graph& g, const int32_t* colors, gc_vali
     out->n_uncolored = static_cast<int64_t>(h.uncolored);
     out->max_color = h.max_color;
     out->n_distinct = static_cast<int32_t>(h.distinct);
-    out->first_bad_vertex = h.first_bad == LLONG_MAX ? -1 : static_cast<int64_t>(h.first_bad);
+    out->first_bad_vertex = h.bad_rank == 0 ? -1 : static_cast<int64_t>(g.n) - static_cast<int64_t>(h.bad_rank);
     return GC_OK;
 }
 

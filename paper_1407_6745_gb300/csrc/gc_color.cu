@@ -40,13 +40,14 @@
 // their gaps (20 us a round where there is little to do), on gathers, and on
 // a block waiting through one dependent load after the other for a row that
 // then lost at once.  Coloring, set-up included, before -> after: R-MAT 24
-// First Fit 87.0 -> 51.2 ms (524 rounds), R-MAT 22 Random-4 Fit 12.1 -> 8.6,
-// RMAT-Bad 22 14.6 -> 7.9, R-MAT 20 11.4 -> 7.7, G(10^6, 24) 1.68 -> 1.12, the
+// First Fit 87.0 -> 41.2 ms (524 rounds), R-MAT 22 Random-4 Fit 12.1 -> 7.5,
+// RMAT-Bad 22 14.6 -> 7.3, R-MAT 20 11.4 -> 7.6, G(10^6, 24) 1.68 -> 1.12, the
 // 27-point stencil 128^3 with Random-8 Fit 1.12 -> 0.90, a batch of 512 graphs
 // 3.99 -> 3.73, G(10^4, 16) 0.22 -> 0.14 (kernels).
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 
 #include "gc_internal.h"
 
@@ -89,7 +90,8 @@ struct HeavyRows {
 };
 
 constexpr int32_t kPiece = 128;         // entries of a row piece (one warp, 4 per lane)
-constexpr int32_t kOpenPiece = 512;     // entries of a list piece
+constexpr int32_t kRound0Piece = 256;   // of a row piece of round 0 (8 per lane)
+constexpr int32_t kOpenPiece = 256;     // entries of a list piece (8 per lane)
 constexpr uint8_t kBucketFixed = 0xFE;  // bucket byte of a fixed vertex (pushes skip it)
 
 struct SpecArgs {
@@ -309,7 +311,7 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
         WorkItem it;
         long long e, wd;
         heavy_sizes(a, h < hi ? h : nh, nh, it, e, wd);
-        const int32_t np = (it.deg + kPiece - 1) / kPiece;
+        const int32_t np = (it.deg + kRound0Piece - 1) / kRound0Piece;
         long long ie = e, iw = wd;  // warp inclusive scans
         int32_t ip = np;
 #pragma unroll
@@ -326,7 +328,8 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
         if (l == 31 && ip) pbase = atomicAdd(&a.ctrl->mark_cnt, ip);
         pbase = __shfl_sync(kFull, pbase, 31) + ip - np;
         for (int32_t q = 0; q < np && pbase + q < hr.mark_cap; ++q)
-            store_item(hr.mark + pbase + q, it.beg + static_cast<int64_t>(q) * kPiece, h, min(kPiece, it.deg - q * kPiece));
+            store_item(hr.mark + pbase + q, it.beg + static_cast<int64_t>(q) * kRound0Piece, h,
+                       min(kRound0Piece, it.deg - q * kRound0Piece));
         if (l == 31) {
             s_e[w] = ie;
             s_w[w] = iw;
@@ -411,7 +414,7 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
 }
 
 constexpr int kHead = 128;              // list entries a warp looks at first, 4 per lane
-constexpr int kRefill = 16;             // dead ones among them that are worth replacing
+constexpr int kRefill = 8;             // dead ones among them that are worth replacing
 constexpr int32_t kLongList = 1024;     // longer lists are left open to the grid
 constexpr int32_t kPushInline = 128;    // longer winners' rows are pushed by the grid
 
@@ -574,27 +577,78 @@ __device__ __forceinline__ int32_t choose_from_bitmap(const uint32_t* bm, int32_
     return -1;
 }
 
-// A light row takes a thread (its color is among the first 64), a heavy one a
-// warp that searches its bitmap.
+// A heavy row's choice (the whole warp): the j-th clear bit of its bitmap.
+template <bool kRXF, bool kWide>
+__device__ __forceinline__ int32_t choose_heavy(Rounds& r, int32_t v, uint32_t j, uint64_t ref) {
+    const SpecArgs& a = r.a;
+    int32_t c = choose_from_bitmap(a.heavy.hbm + (ref >> 24), static_cast<int32_t>(ref & kRefWords), j);
+    if (c < 0) {  // past the bitmap's free colors (Random-X with a large X): the row in full
+        int64_t beg;
+        int32_t deg;
+        row_of(a.g, v, beg, deg, &a.ctrl->err);
+        c = choose_warp<4>(a.g, beg, deg, j, SnapshotFetch<kWide>{a}, reinterpret_cast<uint32_t*>(r.w.head), &a.ctrl->err);
+    }
+    return c;
+}
+
+// A light row takes a thread (its color is among the first 64); a heavy one's
+// bitmap is searched.
 template <bool kRXF, bool kHeavy, bool kWide>
 __device__ __forceinline__ void choose_phase(Rounds& r) {
     const SpecArgs& a = r.a;
     const WorkItem* list = this_list(r);
     if constexpr (kHeavy) {
-        const int32_t n = r.cnt(0);
-        const int32_t W = gridDim.x * kWarps;
-        for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(n); k += W) {
-            const WorkItem it = load_item_rw(list + k);
-            const uint32_t j = kRXF ? draw_index(a, it.v, r.round) : 0u;
-            const uint64_t ref = __ldg(a.heavy.bref + it.v);
-            int32_t c = choose_from_bitmap(a.heavy.hbm + (ref >> 24), static_cast<int32_t>(ref & kRefWords), j);
-            if (c < 0) {  // past the bitmap's free colors (Random-X with a large X): the row in full
-                int64_t beg;
-                int32_t deg;
-                row_of(a.g, it.v, beg, deg, &a.ctrl->err);
-                c = choose_warp<4>(a.g, beg, deg, j, SnapshotFetch<kWide>{a}, reinterpret_cast<uint32_t*>(r.w.head), &a.ctrl->err);
+        // Threads of a warp start on a row each: its first words, for First
+        // Fit from the word of its last choice on (a row's forbidden colors
+        // only grow, so its choice never gets smaller).  The rows whose color
+        // lies beyond take the whole warp.  (R-MAT 24's first choices: 300 ->
+        // 50 us and less a round.)
+        // (Fewer rows than warps take a warp each at once.)
+        const uint32_t n = r.cnt(0);
+        const uint32_t step = gridDim.x * kBlock;
+        if (n <= gridDim.x * kWarps) {
+            const uint32_t k = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+            if (k < n) {
+                const int32_t v = load_item_rw(list + k).v;
+                const int32_t c = choose_heavy<kRXF, kWide>(r, v, kRXF ? draw_index(a, v, r.round) : 0u, __ldg(a.heavy.bref + v));
+                if (lane_id() == 0) *color_word<kWide>(a, v) = c | kUnfixed;
             }
-            if (lane_id() == 0) *color_word<kWide>(a, it.v) = c | kUnfixed;
+        } else for (uint32_t k0 = blockIdx.x * kBlock + (threadIdx.x & ~31u); k0 < n; k0 += step) {
+            const uint32_t k = k0 + lane_id();
+            int32_t v = 0, c = -1;
+            uint32_t j = 0;
+            uint64_t ref = 0;
+            if (k < n) {
+                v = load_item_rw(list + k).v;
+                ref = __ldg(a.heavy.bref + v);
+                const int32_t words = static_cast<int32_t>(ref & kRefWords);
+                const uint32_t* bm = a.heavy.hbm + (ref >> 24);
+                int32_t w = 0;
+                if (kRXF) j = draw_index(a, v, r.round);
+                else w = (tent_of(__ldcg(color_word<kWide>(a, v))) - 1) >> 5;
+                uint32_t left = j;
+#pragma unroll
+                for (int q = 0; q < 2; ++q, w += 2) {
+                    const uint32_t f0 = w < words ? ~__ldcg(bm + w) : 0u;
+                    const uint32_t f1 = w + 1 < words ? ~__ldcg(bm + w + 1) : 0u;
+                    const uint64_t f = (static_cast<uint64_t>(f1) << 32) | f0;
+                    const uint32_t cnt = static_cast<uint32_t>(__popcll(f));
+                    if (left < cnt) {
+                        c = 32 * w + 1 + (left ? select_bit64(f, left) : __ffsll(static_cast<long long>(f)) - 1);
+                        break;
+                    }
+                    left -= cnt;
+                }
+            }
+            for (uint32_t m = __ballot_sync(kFull, k < n && c < 0); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const int32_t vs = __shfl_sync(kFull, v, src);
+                const uint32_t js = __shfl_sync(kFull, j, src);
+                const uint64_t rs = __shfl_sync(kFull, ref, src);
+                const int32_t cs = choose_heavy<kRXF, kWide>(r, vs, js, rs);
+                if (lane_id() == src) c = cs;
+            }
+            if (k < n) *color_word<kWide>(a, v) = c | kUnfixed;
         }
     }
     for (int b = 2; b < kNB; ++b) {
@@ -899,16 +953,16 @@ __device__ __forceinline__ void heavy_round0_piece(Rounds& r, const WorkItem& it
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t h = it.v;
-    const int32_t v = load_item(a.list0 + h).v;
+    const int32_t v = __ldg(&a.list0[h].v);
     int32_t* dst = a.heavy.pend + __ldg(a.heavy.h_pbeg + h);
     const uint32_t pv = prio_word<kWide>(a, v);
     const int32_t tv = kRXF ? tent_of(*color_word<kWide>(a, v)) : 1;
     bool lose = false, loop = false;
     {
-        int32_t u[4];
-        uint32_t p[4];
+        int32_t u[8];
+        uint32_t p[8];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 8; ++i) {
             const int32_t k = 32 * i + l;
             u[i] = k < it.deg ? load_nbr(a.g, it.beg + k, &a.ctrl->err) : -1;
             if (u[i] == v) {
@@ -917,11 +971,11 @@ __device__ __forceinline__ void heavy_round0_piece(Rounds& r, const WorkItem& it
             }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) p[i] = u[i] >= 0 ? prio_word<kWide>(a, u[i]) : 0u;
-        uint32_t keep[4];
+        for (int i = 0; i < 8; ++i) p[i] = u[i] >= 0 ? prio_word<kWide>(a, u[i]) : 0u;
+        uint32_t keep[8];
         int32_t total = 0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 8; ++i) {
             const bool up = u[i] >= 0 && above(p[i], u[i], pv, v);
             if (up && (!kRXF || tent_of(*color_word<kWide>(a, u[i])) == tv)) lose = true;
             keep[i] = __ballot_sync(kFull, up);
@@ -931,7 +985,7 @@ __device__ __forceinline__ void heavy_round0_piece(Rounds& r, const WorkItem& it
         if (l == 0 && total) pos = atomicAdd(a.heavy.h_pcnt + h, total) & INT32_MAX;
         pos = __shfl_sync(kFull, pos, 0);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 8; ++i) {
             if (keep[i] >> l & 1u) dst[pos + __popc(keep[i] & ((1u << l) - 1u))] = u[i];
             pos += __popc(keep[i]);
         }
@@ -1007,15 +1061,20 @@ __device__ __forceinline__ void leave_open(Rounds& r, const WorkItem& it) {
                    min(kOpenPiece, it.deg - q * kOpenPiece));
 }
 
-// Rounds from 1 on.  The first kHead entries of a list come first: most rows
-// of a dense core lose in every round (98 % of the visits to R-MAT 24's rows
-// beyond 1024 entries), nearly always to one of the first 32.  The items and
-// the heads of a warp's next rows are on their way while it tests one.  A
-// list of at most kHead entries is compacted in place; on a longer one the
-// entries of the head that were fixed since are replaced by the list's last
-// ones once there are kRefill, so that the head stays alive and the list
-// shrinks without a pass over it (it stays a superset of the neighbors above
-// v not fixed; its order is free).
+template <int N>
+using Int = std::integral_constant<int, N>;
+
+// Rounds from 1 on.  The first 32 entries of a list come first, then the rest
+// of the first kHead (both at once where there are fewer rows than warps, and
+// a row waits for its latency only): most rows of a dense core lose in every
+// round (98 % of the visits to R-MAT 24's rows beyond 1024 entries), nearly
+// always to one of the first 32 (R-MAT 24, all rounds, with the choice
+// above: 50.5 -> 40.5 ms).  The items and the heads of a warp's next rows are on their
+// way while it tests one.  A list seen in full is compacted in place; on a
+// longer one the entries seen that were fixed since are replaced by the
+// list's last ones once there are kRefill, so that the head stays alive and
+// the list shrinks without a pass over it (it stays a superset of the
+// neighbors above v not fixed; its order is free).
 template <bool kWide>
 __device__ __forceinline__ void heavy_rows(Rounds& r) {
     const SpecArgs& a = r.a;
@@ -1028,11 +1087,13 @@ __device__ __forceinline__ void heavy_rows(Rounds& r) {
     auto stage = [&](const WorkItem& it, int slot) {
         if (4 * l < it.deg) cp_async16(&r.w.head[slot][4 * l], a.heavy.pend + it.beg + 4 * l);
     };
+    const bool many = n > W;
     WorkItem it = load_item_rw(list + k), nx{0, 0, 0};
     if (k + W < n) nx = load_item_rw(list + k + W);
     stage(it, 0);
     cp_async_commit();
     for (int slot = 0;; slot ^= 1) {
+        int looked = 0;
         cp_async_wait<0>();
         __syncwarp();
         const bool more = n - k > W;
@@ -1043,46 +1104,57 @@ __device__ __forceinline__ void heavy_rows(Rounds& r) {
 
         const int32_t pc = it.deg;
         int32_t* lst = a.heavy.pend + it.beg;
-        const int4 q = *reinterpret_cast<const int4*>(&r.w.head[slot][4 * l]);
-        const int32_t u[4] = {q.x, q.y, q.z, q.w};
-        int32_t x[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = 4 * l + i < pc ? *color_word<kWide>(a, u[i]) : kUnfixed;
+        const int32_t* head = r.w.head[slot];
         const int32_t tv = tent_of(*color_word<kWide>(a, it.v));
-        bool mine = false;
-        uint32_t dead[4];
+        int32_t u[4] = {0, 0, 0, 0}, x[4] = {kUnfixed, kUnfixed, kUnfixed, kUnfixed};
+        uint32_t dead[4] = {0, 0, 0, 0};
         int32_t nd = 0;
+        bool lost = false;
+        auto look = [&](auto from, auto to) {  // at entries [32 from, 32 to)
+            bool mine = false;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            mine |= tent_of(x[i]) == tv;
-            dead[i] = __ballot_sync(kFull, x[i] >= 0);
-            nd += __popc(dead[i]);
+            for (int i = from; i < to; ++i)
+                if (32 * i + l < pc) {
+                    u[i] = head[32 * i + l];
+                    x[i] = *color_word<kWide>(a, u[i]);
+                }
+#pragma unroll
+            for (int i = from; i < to; ++i) {
+                mine |= tent_of(x[i]) == tv;
+                dead[i] = __ballot_sync(kFull, x[i] >= 0);
+                nd += __popc(dead[i]);
+            }
+            lost = __any_sync(kFull, mine);
+            looked = to;
+        };
+        if (many) {
+            look(Int<0>{}, Int<1>{});
+            if (!lost && pc > 32) look(Int<1>{}, Int<4>{});
+        } else {
+            look(Int<0>{}, Int<4>{});
         }
-        bool lost = __any_sync(kFull, mine);
         int32_t len = pc;
-        if (pc <= kHead) {
+        if (pc <= 32 * looked) {  // seen in full: compacted in place
             if (lost && nd) {
                 int32_t kept = 0;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const uint32_t live = __ballot_sync(kFull, 4 * l + i < pc && x[i] < 0);
+                    const uint32_t live = __ballot_sync(kFull, i < looked && 32 * i + l < pc && x[i] < 0);
                     if (live >> l & 1u) lst[kept + __popc(live & ((1u << l) - 1u))] = u[i];
                     kept += __popc(live);
                 }
                 len = kept;
             }
-        } else {
-            if (nd >= kRefill) {
-                const int32_t moved = min(nd, pc - kHead);
-                int32_t d = 0;  // rank of the entry among the dead ones
+        } else if (nd >= kRefill) {  // the dead ones seen make room for the list's last entries
+            const int32_t moved = min(nd, pc - 32 * looked);
+            int32_t d = 0;  // rank of the entry among the dead ones
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int32_t rank = d + __popc(dead[i] & ((1u << l) - 1u));
-                    if ((dead[i] >> l & 1u) && rank < moved) lst[4 * l + i] = __ldcg(lst + pc - 1 - rank);
-                    d += __popc(dead[i]);
-                }
-                len = pc - moved;
+            for (int i = 0; i < 4; ++i) {
+                const int32_t rank = d + __popc(dead[i] & ((1u << l) - 1u));
+                if ((dead[i] >> l & 1u) && rank < moved) lst[32 * i + l] = __ldcg(lst + pc - 1 - rank);
+                d += __popc(dead[i]);
             }
+            len = pc - moved;
         }
         bool open = false;
         if (!lost && pc > kHead) {
@@ -1120,14 +1192,21 @@ __device__ __forceinline__ void open_phase(Rounds& r) {
     const int32_t W = gridDim.x * kWarps;
     for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(n); k += W) {
         const WorkItem it = load_item_rw(a.heavy.open + k);
-        const WorkItem row = load_item_rw(a.heavy.open_row + it.v);
-        if (!__ldcg(a.heavy.open_lost + it.v)) {
-            const int32_t tv = tent_of(*color_word<kWide>(a, row.v));
-            const int32_t* lst = a.heavy.pend + it.beg;
-            bool lost = false;
-            for (int32_t k0 = 0; k0 < it.deg && !lost; k0 += 256) lost = __any_sync(kFull, list_hit<kWide>(a, lst, k0, it.deg, tv));
-            if (lost && l == 0) atomicExch(a.heavy.open_lost + it.v, 1);
-        }
+        const WorkItem row = load_item_rw(a.heavy.open_row + it.v);  // beside the piece's entries
+        const int32_t* lst = a.heavy.pend + it.beg;
+        int32_t u[8], x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) u[i] = 32 * i + l < it.deg ? __ldcg(lst + 32 * i + l) : -1;
+        const int32_t tv = tent_of(*color_word<kWide>(a, row.v));  // and the row beside their colors
+        int64_t beg;
+        int32_t deg;
+        row_of(a.g, row.v, beg, deg, &a.ctrl->err);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = u[i] >= 0 ? *color_word<kWide>(a, u[i]) : 0;
+        bool hit = false;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) hit |= tent_of(x[i]) == tv;
+        if (__any_sync(kFull, hit) && l == 0) atomicExch(a.heavy.open_lost + it.v, 1);
         __syncwarp();
         int last = 0;
         if (l == 0) last = add_acq_rel(a.heavy.open_done + it.v) == -1;
@@ -1139,10 +1218,7 @@ __device__ __forceinline__ void open_phase(Rounds& r) {
                 store_item(next_list(r) + pos, row.beg, row.v, row.deg);
             }
         } else {
-            int64_t beg;
-            int32_t deg;
-            row_of(a.g, row.v, beg, deg, &a.ctrl->err);
-            heavy_win<kWide>(r, row.v, tent_of(*color_word<kWide>(a, row.v)), beg, deg);
+            heavy_win<kWide>(r, row.v, tv, beg, deg);
         }
     }
 }
@@ -1165,8 +1241,15 @@ __device__ __forceinline__ void test_phase(Rounds& r) {
         if constexpr (kHeavy) {
             const int32_t np = static_cast<int32_t>(min(static_cast<int64_t>(a.ctrl->mark_cnt), a.heavy.mark_cap));
             const int32_t W = gridDim.x * kWarps;
-            for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(np); k += W)
-                heavy_round0_piece<kRXF, kWide>(r, load_item(a.heavy.mark + k));
+            uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5);
+            WorkItem it{0, 0, 0};
+            if (k < static_cast<uint32_t>(np)) it = load_item(a.heavy.mark + k);
+            for (; k < static_cast<uint32_t>(np); k += W) {
+                WorkItem nx{0, 0, 0};
+                if (k + W < static_cast<uint32_t>(np)) nx = load_item(a.heavy.mark + k + W);
+                heavy_round0_piece<kRXF, kWide>(r, it);
+                it = nx;
+            }
         }
         light_rows<2, kRXF, kHeavy, kWide, true>(r, 0);
         return;

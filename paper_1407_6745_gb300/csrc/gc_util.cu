@@ -1,6 +1,6 @@
 // gc_util.cu -- validation of a coloring (the definition of Sec. 1:
 // C(u) != C(v) on every edge, #colors = max_u C(u)) and the CSR structure
-// check.  Both are one pass over the adjacency, warp per vertex.
+// check, each one pass over the adjacency.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -17,22 +17,19 @@ struct ValCtrl {
     int32_t max_color;
     uint32_t err;
     unsigned long long distinct;
-    int32_t heavy;          // rows deferred to the block-per-row pass (gc_validate: to the warp-per-row one)
     int32_t big_colors;     // vertices with a color >= kPresColors
-    int32_t big;            // gc_validate: pieces of the rows beyond kValWarpDeg
+    int32_t pad;
 };
 
 constexpr int kValG = 4;                 // lanes per light row (measured: 8 -> 4 saves 30 us on the stencil)
 constexpr int32_t kHeavyDeg = 256;       // heavier rows: one block each (gc_validate_noalloc)
-// gc_validate: rows of up to kValLightDeg entries take kValG lanes (one
-// pass of loads), up to kValWarpDeg a warp, longer ones a block.  (R-MAT
-// scale 24: 2.77 + 1.60 ms with the noalloc form's split at 256 entries.)
-constexpr int32_t kValLightDeg = 64;
-constexpr int32_t kValWarpDeg = 4096;
-// Rows beyond kValWarpDeg are cut into pieces of kValPiece entries, a block
-// each (the largest R-MAT rows hold hundreds of thousands of entries; one
-// block per row left a single block walking the largest).
-constexpr int32_t kValPiece = 4096;
+// gc_validate: rows and entries of one warp's step together (8 entries a
+// lane, less what the 16-byte boundary before the first one can take), and
+// the blocks of an SM the registers are limited for (R-MAT 24 / 22 with 3:
+// 1.73 / 0.38 ms, with 4: 2.03 / 0.37, with 5: 2.06 / 0.39).
+constexpr int kValSlots = 8 * 32;
+constexpr int kValChunk = kValSlots - 4;
+constexpr int kValBlocks = 3;
 constexpr int kPresWords = 2048;         // presence bitmap of colors < 65536
 constexpr int32_t kPresColors = kPresWords * 32;
 
@@ -41,9 +38,9 @@ struct ValArgs {
     const int32_t* colors;
     ValCtrl* c;
     uint32_t* pres;    // kPresWords
-    int32_t* heavy;    // n
-    int2* pieces;      // gc_validate: (row, piece index) of the rows beyond kValWarpDeg
-    int64_t piece_cap;
+    uint8_t* low;      // gc_validate: the low byte of every color
+    int32_t* first;    // gc_validate: the row each step of kValChunk begins in
+    int64_t steps;     // length of `first`
     int32_t max_allowed;  // a recoloring input: the row of a vertex whose color is outside [1, max_allowed]
                           // is not read; 0: a validation, which reads every row
 };
@@ -66,21 +63,13 @@ __device__ __forceinline__ void account(const ValArgs& a, int32_t v, int32_t cv,
     if (cv < 1) ++unc;
     if (cv < 1 || same > 0) atomicMax(&a.c->bad_rank, static_cast<unsigned long long>(a.g.n) - static_cast<unsigned long long>(v));
     my_max = max(my_max, cv);
-    if (cv >= 1 && cv < kPresColors) atomicOr(&s_pres[cv >> 5], 1u << (cv & 31));
-    else if (cv >= kPresColors) atomicAdd(&a.c->big_colors, 1);
-}
-
-// One piece of a row: its same-colored neighbors; the row's own accounting
-// (uncolored, max color, presence) with its first piece only.
-__device__ __forceinline__ void account_piece(const ValArgs& a, int32_t v, int32_t cv, int32_t same, bool first,
-                                              uint32_t* s_pres, unsigned long long& conf,
-                                              unsigned long long& unc, int32_t& my_max) {
-    if (first) {
-        account(a, v, cv, same, s_pres, conf, unc, my_max);
-        return;
+    if (cv >= 1 && cv < kPresColors) {
+        // (a read first: atomics of a warp on one word take turns; R-MAT 24 112 -> 97 us)
+        if (!(*reinterpret_cast<volatile uint32_t*>(&s_pres[cv >> 5]) >> (cv & 31) & 1u))
+            atomicOr(&s_pres[cv >> 5], 1u << (cv & 31));
+    } else if (cv >= kPresColors) {
+        atomicAdd(&a.c->big_colors, 1);
     }
-    conf += static_cast<unsigned long long>(same);
-    if (same > 0) atomicMax(&a.c->bad_rank, static_cast<unsigned long long>(a.g.n) - static_cast<unsigned long long>(v));
 }
 
 __device__ __forceinline__ void flush_presence(const ValArgs& a, uint32_t* s_pres) {
@@ -89,98 +78,202 @@ __device__ __forceinline__ void flush_presence(const ValArgs& a, uint32_t* s_pre
         if (s_pres[i]) atomicOr(&a.pres[i], s_pres[i]);
 }
 
-// Light rows: kValG lanes per vertex; longer rows are listed for the next
-// pass, from the front of `heavy` up to kValWarpDeg entries, from the back
-// beyond.  kInput: a recoloring input, with max_allowed.
-template <bool kInput>
-__global__ void __launch_bounds__(kBlock) k_validate(ValArgs a) {
+// One pass over the vertices: a vertex's own accounting, the low byte of its
+// color, and which row each step of the pass over the entries begins in.
+// Steps are cut on the count of rows plus entries (row v covers
+// [v + off[v], v + 1 + off[v + 1]) of it, less off[0]), so that neither a
+// long row nor a long run of empty rows falls to one block.
+__global__ void __launch_bounds__(kBlock) k_validate_rows(ValArgs a) {
     __shared__ uint32_t s_pres[kPresWords];
     for (int i = threadIdx.x; i < kPresWords; i += kBlock) s_pres[i] = 0u;
     __syncthreads();
-    const int gi = threadIdx.x / kValG, gl = threadIdx.x % kValG;
-    const int64_t groups = static_cast<int64_t>(gridDim.x) * (kBlock / kValG);
     int32_t my_max = 0;
     unsigned long long conf = 0, unc = 0;
-    const int64_t n_pad = (a.g.n + groups - 1) / groups * groups;
-    for (int64_t v = static_cast<int64_t>(blockIdx.x) * (kBlock / kValG) + gi; v < n_pad; v += groups) {
-        const bool valid = v < a.g.n;
-        int64_t beg = 0;
-        int32_t deg = 0, cv = 0;
-        bool heavy = false;
-        if (valid) {
-            row_of(a.g, static_cast<int32_t>(v), beg, deg, &a.c->err);
-            cv = a.colors[v];
-            if (kInput && (cv < 1 || cv > a.max_allowed)) deg = 0;
-            heavy = deg > kValLightDeg;
-        }
-        int32_t same = same_color<1>(a, beg, heavy ? 0 : deg, cv, gl, kValG);
+    const int64_t off0 = __ldg(a.g.off);
+    const bool narrow = a.g.n + a.g.nnz < int64_t(1) << 31;
+    constexpr int U = 4;  // vertices of a thread whose loads are in flight together
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * (U * kBlock);
+    for (int64_t b = static_cast<int64_t>(blockIdx.x) * (U * kBlock) + threadIdx.x; b < a.g.n; b += stride) {
+        int64_t beg[U];
+        int32_t deg[U], cv[U];
 #pragma unroll
-        for (int d = kValG / 2; d >= 1; d >>= 1) same += __shfl_xor_sync(kFull, same, d);
-        if (valid && gl == 0) {
-            if (!heavy) account(a, static_cast<int32_t>(v), cv, same, s_pres, conf, unc, my_max);
-            else if (deg <= kValWarpDeg) a.heavy[atomicAdd(&a.c->heavy, 1)] = static_cast<int32_t>(v);
-            else {
-                const int32_t np = (deg + kValPiece - 1) / kValPiece;
-                const int32_t p0 = atomicAdd(&a.c->big, np);
-                for (int32_t i = 0; i < np && p0 + i < a.piece_cap; ++i)
-                    a.pieces[p0 + i] = make_int2(static_cast<int32_t>(v), i);
+        for (int i = 0; i < U; ++i) {
+            const int64_t v = min(b + i * kBlock, static_cast<int64_t>(a.g.n) - 1);
+            row_of(a.g, static_cast<int32_t>(v), beg[i], deg[i], &a.c->err);
+            cv[i] = __ldg(a.colors + v);
+        }
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int64_t v = b + i * kBlock;
+            if (v >= a.g.n) break;
+            account(a, static_cast<int32_t>(v), cv[i], 0, s_pres, conf, unc, my_max);
+            a.low[v] = static_cast<uint8_t>(cv[i]);
+            const int64_t d = v + beg[i] - off0;  // (negative only where the offsets are malformed)
+            const int64_t d1 = d + deg[i];
+            int64_t k0, k1;
+            if (narrow) {  // (a 64-bit division takes a third of the pass)
+                k0 = (static_cast<uint32_t>(d) + (kValChunk - 1u)) / kValChunk;
+                k1 = static_cast<uint32_t>(d1) / kValChunk;
+            } else {
+                k0 = (max(d, int64_t(0)) + kValChunk - 1) / kValChunk;
+                k1 = d1 / kValChunk;
             }
+            for (k1 = min(k1, a.steps - 1); k0 <= k1; ++k0) a.first[k0] = static_cast<int32_t>(v);
         }
     }
-    warp_add(&a.c->conflicts, conf);
     warp_add(&a.c->uncolored, unc);
     warp_max(&a.c->max_color, my_max);
     flush_presence(a, s_pres);
 }
 
-// The rows k_validate listed: a warp each up to kValWarpDeg entries, then a
-// block per piece of kValPiece entries beyond.
-__global__ void __launch_bounds__(kBlock) k_validate_heavy(ValArgs a) {
-    __shared__ uint32_t s_pres[kPresWords];
-    __shared__ int32_t s_sum[kWarps];
-    for (int i = threadIdx.x; i < kPresWords; i += kBlock) s_pres[i] = 0u;
-    __syncthreads();
-    int32_t my_max = 0;
-    unsigned long long conf = 0, unc = 0;
-    const int32_t nmid = a.c->heavy, nbig = a.c->big;
-    const int w = threadIdx.x >> 5, l = lane_id();
-    for (int32_t h = blockIdx.x * kWarps + w; h < nmid; h += gridDim.x * kWarps) {
-        const int32_t v = a.heavy[h];
-        int64_t beg;
-        int32_t deg;
-        row_of(a.g, v, beg, deg, &a.c->err);
-        const int32_t cv = a.colors[v];
-        int32_t same = same_color<2>(a, beg, deg, cv, l, 32);
+// The ids of a step in the lane's 8 slots (a0: 16-byte aligned), those of
+// slots outside [e0, e1) unspecified.
+__device__ __forceinline__ void step_ids(const Graph& g, int64_t a0, int64_t e1, int32_t (&u)[8]) {
 #pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) same += __shfl_xor_sync(kFull, same, d);
-        if (l == 0) account(a, v, cv, same, s_pres, conf, unc, my_max);
-    }
-    const int64_t npieces = nbig < a.piece_cap ? nbig : a.piece_cap;
-    for (int64_t k = blockIdx.x; k < npieces; k += gridDim.x) {
-        const int2 pc = a.pieces[k];
-        const int32_t v = pc.x;
-        int64_t beg;
-        int32_t deg;
-        row_of(a.g, v, beg, deg, &a.c->err);
-        const int64_t off = static_cast<int64_t>(pc.y) * kValPiece;
-        const int32_t len = static_cast<int32_t>(min(static_cast<int64_t>(kValPiece), deg - off));
-        const int32_t cv = a.colors[v];
-        int32_t same = same_color<1>(a, beg + off, len, cv, threadIdx.x, kBlock);
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) same += __shfl_xor_sync(kFull, same, d);
-        if (lane_id() == 0) s_sum[threadIdx.x >> 5] = same;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int32_t tot = 0;
-            for (int q = 0; q < kWarps; ++q) tot += s_sum[q];
-            account_piece(a, v, cv, tot, pc.y == 0, s_pres, conf, unc, my_max);
+    for (int h = 0; h < 2; ++h) {
+        const int64_t e = a0 + 4 * (h * 32 + lane_id());
+        int4 q = make_int4(0, 0, 0, 0);
+        if (g.vec && e + 4 <= g.nnz) {
+            if (e < e1) q = ld_stream4(g.idx + e);
+        } else {
+            if (e < e1) q.x = ld_stream(g.idx + e);
+            if (e + 1 < e1) q.y = ld_stream(g.idx + e + 1);
+            if (e + 2 < e1) q.z = ld_stream(g.idx + e + 2);
+            if (e + 3 < e1) q.w = ld_stream(g.idx + e + 3);
         }
-        __syncthreads();
+        u[4 * h] = q.x, u[4 * h + 1] = q.y, u[4 * h + 2] = q.z, u[4 * h + 3] = q.w;
     }
-    warp_add(&a.c->conflicts, conf);
-    warp_add(&a.c->uncolored, unc);
-    warp_max(&a.c->max_color, my_max);
-    flush_presence(a, s_pres);
+}
+
+// One pass over the entries, flat: every lane takes 8 entries of a warp's
+// step whatever rows they belong to, so none waits for a longer row; the
+// next step's ids are read meanwhile.  Whose an entry is: a bit where a row
+// begins, the row's color beside it; an entry's row is the last bit at or
+// before it.  The low bytes are gathered, and a color only where its byte
+// equals the row's: four times as many vertices stay in L1, where a random
+// gather takes a third of the time it takes from L2 (800 against 280 G/s
+// measured).  Bound by the gathers: both passes take 0.41 ms on R-MAT 22
+// (128 M entries) and 1.83 ms on R-MAT 24 (522 M), where 4 lanes a short
+// row, a warp or blocks a longer one, and 4-byte gathers took 0.69 and 2.63;
+// bytes alone 0.69 and 2.62; this with a block's steps and its barriers 0.52
+// and 2.23.  On a stencil of shuffled vertices, where nothing stays in L1,
+// 241 us for 230.  kInput: a recoloring input, with max_allowed.
+template <bool kInput>
+__global__ void __launch_bounds__(kBlock, kValBlocks) k_validate(ValArgs a) {
+    constexpr int kWords = kValSlots / 32;
+    __shared__ uint32_t s_bits_[kWarps][kWords];
+    __shared__ int32_t s_color_[kWarps][kValSlots];  // of the row that begins at the slot
+    const int w = threadIdx.x >> 5, l = lane_id();
+    uint32_t* s_bits = s_bits_[w];
+    int32_t* s_color = s_color_[w];
+    if (*reinterpret_cast<volatile uint32_t*>(&a.c->err)) return;  // malformed offsets: the steps mean nothing
+    const int32_t n = a.g.n;
+    const int64_t off0 = __ldg(a.g.off);
+    const int64_t total = n + __ldg(a.g.off + n) - off0;
+    const int64_t nsteps = (total + kValChunk - 1) / kValChunk;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * kWarps;
+    uint32_t conf = 0;
+    int64_t k = static_cast<int64_t>(blockIdx.x) * kWarps + w;
+    // rows [v0, v1], entries [e0, e1)
+    int32_t v0 = 0, v1 = 0;
+    int64_t e0 = 0, e1 = 0;
+    int32_t u[8];
+    const auto stage = [&](int64_t step) {
+        v0 = __ldg(a.first + step);
+        v1 = step + 1 < nsteps ? __ldg(a.first + step + 1) : n;
+        e0 = step * kValChunk - v0 + off0;
+        e1 = min((step + 1) * kValChunk, total) - v1 + off0;
+        step_ids(a.g, e0 & ~int64_t(3), e1, u);
+    };
+    if (k < nsteps) stage(k);
+    for (; k < nsteps; k += stride) {
+        const int64_t a0 = e0 & ~int64_t(3);
+        const int32_t first_row = v0, last_row = min(v1, n - 1);
+        const int32_t lo = static_cast<int32_t>(e0 - a0), hi = static_cast<int32_t>(e1 - a0);  // slots
+        if (l < kWords) s_bits[l] = 0u;
+        __syncwarp();
+        for (int32_t r = first_row; r <= last_row; r += 32) {
+            const int32_t v = r + l;
+            if (v <= last_row) {
+                const int64_t b = max(__ldg(a.g.off + v), e0), e = min(__ldg(a.g.off + v + 1), e1);
+                if (b < e) {
+                    const int32_t at = static_cast<int32_t>(b - a0);
+                    s_color[at] = __ldg(a.colors + v);
+                    atomicOr(&s_bits[at >> 5], 1u << (at & 31));
+                }
+            }
+        }
+        uint32_t invalid = 0;  // slots of the lane with an id outside [0, n)
+        uint32_t low[8];
+        int32_t x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int32_t at = 4 * ((i >> 2) * 32 + l) + (i & 3);
+            x[i] = u[i];
+            low[i] = 256u;  // no entry: equals no byte
+            if (at >= lo && at < hi) {
+                if (static_cast<uint32_t>(x[i]) < static_cast<uint32_t>(n)) low[i] = __ldg(a.low + x[i]);
+                else invalid |= 1u << i;
+            }
+        }
+        if (k + stride < nsteps) stage(k + stride);
+        __syncwarp();
+        // the last row start before each word
+        const uint32_t wb = l < kWords ? s_bits[l] : 0u;
+        int32_t m = wb ? 32 * l + 31 - __clz(wb) : -1;
+#pragma unroll
+        for (int d = 1; d < kWords; d <<= 1) {
+            const int32_t o = __shfl_up_sync(kFull, m, d);
+            if (l >= d) m = max(m, o);
+        }
+        int32_t bad = INT_MAX;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int wi = 4 * h + (l >> 3);
+            const int at = 4 * (h * 32 + l);
+            const int32_t before = __shfl_sync(kFull, m, wi ? wi - 1 : 0);
+            const uint32_t word = __shfl_sync(kFull, wb, wi);
+            const uint32_t upto = word & (0xffffffffu >> (31 - (at & 31)));
+            int32_t row = upto ? (at & ~31) + 31 - __clz(upto) : wi ? before : -1;
+            const uint32_t begins = word >> (at & 31);
+            int32_t cv = row >= 0 ? s_color[row] : 0;
+            int32_t cvs[4];
+            uint32_t look = invalid >> (4 * h) & 15u;  // entries to look at again
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (j && (begins >> j & 1u)) cv = s_color[at + j];
+                cvs[j] = cv;
+                look |= static_cast<uint32_t>(low[4 * h + j] == (static_cast<uint32_t>(cv) & 255u)) << j;
+            }
+            if (look == 0) continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (j && (begins >> j & 1u)) row = at + j;
+                if (!(look >> j & 1u) || (kInput && (cvs[j] < 1 || cvs[j] > a.max_allowed))) continue;
+                if (invalid >> (4 * h + j) & 1u) {
+                    atomicOr(&a.c->err, kErrBadGraph);
+                } else if (__ldg(a.colors + x[4 * h + j]) == cvs[j]) {
+                    ++conf;
+                    bad = min(bad, row);
+                }
+            }
+        }
+        bad = __reduce_min_sync(kFull, bad);
+        if (bad != INT_MAX && l == 0) {
+            // the row that begins at the slot: the last one at or before that entry
+            const int64_t e = a0 + bad;
+            int32_t p = first_row, q = last_row;
+            while (p < q) {
+                const int32_t mid = p + (q - p + 1) / 2;
+                if (__ldg(a.g.off + mid) <= e) p = mid;
+                else q = mid - 1;
+            }
+            const unsigned long long rank = static_cast<unsigned long long>(n) - static_cast<unsigned long long>(p);
+            if (rank > *reinterpret_cast<volatile unsigned long long*>(&a.c->bad_rank)) atomicMax(&a.c->bad_rank, rank);
+        }
+        __syncwarp();
+    }
+    warp_add(&a.c->conflicts, static_cast<unsigned long long>(conf));
 }
 
 __global__ void __launch_bounds__(kBlock) k_mark_present(int64_t n, const int32_t* colors,
@@ -201,35 +294,34 @@ __global__ void __launch_bounds__(kBlock) k_count_bits(int64_t words, const uint
     warp_add(&c->distinct, s);
 }
 
-// The scratch of one validation and its two passes over the rows.
+// The scratch of one validation, its pass over the rows and that over the entries.
 struct ValRun {
     ScratchSet sc;
     ValArgs a{};
     gc_status start(const Graph& g, const int32_t* colors, int32_t max_allowed, const Tuning& t, cudaStream_t s) {
         a = ValArgs{g, colors, nullptr, nullptr, nullptr, nullptr, 0, max_allowed};
-        // pieces: at most one per kValPiece entries, plus one per row beyond kValWarpDeg
-        a.piece_cap = g.nnz / kValPiece + g.nnz / kValWarpDeg + 1;
+        a.steps = (static_cast<int64_t>(g.n) + g.nnz) / kValChunk + 1;
         static_assert(sizeof(ValCtrl) % 8 == 0, "the bitmap follows it");
         sc.want(&a.c, sizeof(ValCtrl) + kPresWords * 4);
-        sc.want(&a.heavy, static_cast<int64_t>(g.n) * 4);
-        sc.want(&a.pieces, a.piece_cap * static_cast<int64_t>(sizeof(int2)));
+        sc.want(&a.low, static_cast<int64_t>(g.n));
+        sc.want(&a.first, a.steps * 4);
         if (!sc.alloc(s)) return GC_ERR_OOM;
         a.pres = reinterpret_cast<uint32_t*>(a.c + 1);
         cudaMemsetAsync(a.c, 0, sizeof(ValCtrl) + kPresWords * 4, s);
         const bool input = max_allowed != 0;
-        const auto light = input ? k_validate<true> : k_validate<false>;
-        GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE, s, light<<<resident_grid(light, t), kBlock, 0, s>>>(a));
-        GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE_HEAVY, s,
-                  k_validate_heavy<<<resident_grid(k_validate_heavy, t), kBlock, 0, s>>>(a));
+        const int64_t row_blocks = (static_cast<int64_t>(g.n) + 4 * kBlock - 1) / (4 * kBlock);
+        const int rows = static_cast<int>(std::min<int64_t>(row_blocks, resident_grid(k_validate_rows, t)));
+        GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE_ROWS, s, k_validate_rows<<<rows, kBlock, 0, s>>>(a));
+        const auto entries = input ? k_validate<true> : k_validate<false>;
+        const int grid = static_cast<int>(std::min<int64_t>((a.steps + kWarps - 1) / kWarps, resident_grid(entries, t)));
+        GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE, s, entries<<<grid, kBlock, 0, s>>>(a));
         return GC_OK;
     }
 };
 
 // The input of a recoloring call: proper (Sec. 1), colors in [1,
-// max_allowed].  The validation's passes (4 lanes a light row, longer rows
-// listed and cut into pieces) instead of a warp per row, which left one warp
-// walking each hub row: R-MAT 18 742 -> 70 us (of 4.75 ms -> 3.98 ms for
-// the call with 5 iterations).
+// max_allowed].  The validation's passes instead of a warp per row, which
+// left one warp walking each hub row: R-MAT 18 742 -> 41 us.
 gc_status check_input_device(const Graph& g, const int32_t* colors, int32_t max_allowed, int32_t* max_color,
                              cudaStream_t s) {
     *max_color = 0;
@@ -320,7 +412,6 @@ __global__ void __launch_bounds__(kBlock) k_validate_na_clear(NoAllocScratch* sc
         sc->ctrl.max_color = 0;
         sc->ctrl.err = 0;
         sc->ctrl.distinct = 0;
-        sc->ctrl.heavy = 0;
         sc->ctrl.big_colors = 0;
     }
     for (int i = blockIdx.x * kBlock + threadIdx.x; i < kPresWords; i += gridDim.x * kBlock)
@@ -453,7 +544,7 @@ gc_status validate_noalloc_device(const Graph& g, const int32_t* colors, gc_vali
     NoAllocScratch* sc = nullptr;
     gc_status st = noalloc_scratch(&sc);
     if (st != GC_OK) return st;
-    ValArgs a{g, colors, &sc->ctrl, sc->pres, nullptr};
+    ValArgs a{g, colors, &sc->ctrl, sc->pres, nullptr, nullptr, 0, 0};
     // Each launch is checked before the next is enqueued: a clear that failed
     // to launch must not let the read-back return the previous call's counts.
     // (Not bracketed by the profiling events, which would create events.)

@@ -1233,34 +1233,73 @@ gc_status class_ranks_device(const Graph& g, const int32_t* colors, bool trusted
 // rank, and ranks are global segment keys, so the cooperative launch above
 // serves the whole batch unchanged.
 // ---------------------------------------------------------------------------
+// A block's slice of consecutive vertices belongs to few graphs, and these
+// own consecutive class tables, so the slice is counted in shared memory where
+// the tables it spans fit (small graphs' in any case spread over many
+// counters).  A batch of 512 graphs (11 M vertices): 47 us instead of 79 with
+// a global atomic per warp and key, nearly all on the few counters of the
+// graph at hand; 69 while a vertex's reads were not issued together.
+constexpr int32_t kBrcSlice = 2048;
+constexpr int32_t kBrcClasses = 512;
 __global__ void __launch_bounds__(kBlock) k_brc_hist(RcArgs a) {
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * kBlock;
-    for (int64_t v = static_cast<int64_t>(blockIdx.x) * kBlock + threadIdx.x; v < a.g.n; v += stride) {
-        const int32_t gi = a.graph_of[v];
-        if (a.iteration >= a.desc[gi].iterations) continue;
-        const int64_t base = a.cls_base[gi];
-        const int32_t maxc = static_cast<int32_t>(a.cls_base[gi + 1] - base - 1);
-        const int32_t c = a.old_c[v];
-        if (c < 1 || c > maxc) {
-            atomicOr(&a.ctrl->err, kErrImproper);
-            continue;
+    __shared__ int32_t s_cnt[kBrcClasses * kRcNB];
+    __shared__ int32_t s_iso[kBrcClasses];
+    for (int64_t c0 = static_cast<int64_t>(blockIdx.x) * kBrcSlice; c0 < a.g.n;
+         c0 += static_cast<int64_t>(gridDim.x) * kBrcSlice) {
+        const int64_t c1 = min(c0 + kBrcSlice, static_cast<int64_t>(a.g.n));
+        const int64_t k0 = a.cls_base[a.graph_of[c0]];
+        const int64_t classes = a.cls_base[a.graph_of[c1 - 1] + 1] - k0;
+        const bool local = classes <= kBrcClasses;
+        if (local) {
+            for (int i = threadIdx.x; i < classes * kRcNB; i += kBlock) s_cnt[i] = 0;
+            for (int i = threadIdx.x; i < classes; i += kBlock) s_iso[i] = 0;
         }
-        const int b = a.bucket[v];
-        const int64_t key = base + c;
-        if (b == kIsoBucket) {
-            const unsigned act = __activemask();
-            const unsigned peers = __match_any_sync(act, static_cast<uint32_t>(key));
-            if (lane_id() == __ffs(peers) - 1) atomicAdd(&a.iso_cnt[key], __popc(peers));
-            continue;
+        __syncthreads();
+        constexpr int U = kBrcSlice / kBlock;
+        int32_t gv[U], cv[U];
+        uint8_t bv[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int64_t v = min(c0 + i * kBlock + threadIdx.x, c1 - 1);
+            gv[i] = __ldg(a.graph_of + v);
+            cv[i] = __ldg(a.old_c + v);
+            bv[i] = __ldg(a.bucket + v);
         }
-        const unsigned act = __activemask();
-        const unsigned peers = __match_any_sync(act, static_cast<uint32_t>(key * kRcNB + b));
-        if (lane_id() == __ffs(peers) - 1) atomicAdd(&a.cls_cnt[key * kRcNB + b], __popc(peers));
-        if (b == 0) {
-            int64_t rb;
-            int32_t deg;
-            row_of(a.g, static_cast<int32_t>(v), rb, deg, &a.ctrl->err);
-            atomicAdd(&a.cls_units[key], chunks_of(deg));
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int64_t v = c0 + i * kBlock + threadIdx.x;
+            if (v >= c1) break;
+            const int32_t gi = gv[i], c = cv[i], b = bv[i];
+            if (a.iteration >= a.desc[gi].iterations) continue;
+            const int64_t base = a.cls_base[gi];
+            const int32_t maxc = static_cast<int32_t>(a.cls_base[gi + 1] - base - 1);
+            if (c < 1 || c > maxc) {
+                atomicOr(&a.ctrl->err, kErrImproper);
+                continue;
+            }
+            const int64_t key = base + c;
+            if (local) {
+                if (b == kIsoBucket) atomicAdd(&s_iso[key - k0], 1);
+                else atomicAdd(&s_cnt[(key - k0) * kRcNB + b], 1);
+            } else {
+                int32_t* at = b == kIsoBucket ? &a.iso_cnt[key] : &a.cls_cnt[key * kRcNB + b];
+                const unsigned peers = __match_any_sync(__activemask(), reinterpret_cast<unsigned long long>(at));
+                if (lane_id() == __ffs(peers) - 1) atomicAdd(at, __popc(peers));
+            }
+            if (b == 0) {
+                int64_t rb;
+                int32_t deg;
+                row_of(a.g, static_cast<int32_t>(v), rb, deg, &a.ctrl->err);
+                atomicAdd(&a.cls_units[key], chunks_of(deg));
+            }
+        }
+        __syncthreads();
+        if (local) {
+            for (int i = threadIdx.x; i < classes * kRcNB; i += kBlock)
+                if (s_cnt[i]) atomicAdd(&a.cls_cnt[k0 * kRcNB + i], s_cnt[i]);
+            for (int i = threadIdx.x; i < classes; i += kBlock)
+                if (s_iso[i]) atomicAdd(&a.iso_cnt[k0 + i], s_iso[i]);
+            __syncthreads();
         }
     }
 }

@@ -515,18 +515,24 @@ __device__ __forceinline__ int32_t hot_or_own(int32_t* s_cnt, int32_t sg, int32_
 // keeps slices (a block then looks up few graphs' class ranks).  Per iteration,
 // before / with the loads ahead / and strided: R-MAT 24 0.445 / 0.399 / 0.207
 // ms, R-MAT 22 0.104 / 0.097 / 0.060, stencil 128^3 27 / 25 / 23 us, a batch
-// of 512 graphs 0.18 / 0.109 / 0.126 ms.
+// of 512 graphs 0.18 / 0.109 / 0.126 ms.  A graph without split rows keeps
+// slices too once its colors outgrow what L2 serves at full rate: the lists
+// are then in the order of the ids, and a graph whose ids are local gathers
+// locally (2048 graphs as one of 304 M vertices: 48 / 29 instead of 61 / 61 ms
+// of cooperative / stepwise recoloring; the shuffled stencil, whose 8 MB of
+// colors need no order, would lose 3 %).
+constexpr int64_t kSliceMin = int64_t(16) << 20;
 template <bool kBatch>
 __global__ void __launch_bounds__(kBlock) k_rc_scatter(RcArgs a) {
     extern __shared__ int32_t s_cnt[];  // a.scatter_segs counts, then as many bases
     int32_t* const s_base = s_cnt + a.scatter_segs;
     if (a.ctrl->err & (kErrImproper | kErrBadGraph)) return;
     const int32_t nseg = a.ctrl->k * kRcNB;
-    // one graph: every grid-th group of kBlock vertices; a batch: a slice
+    const bool slices = kBatch || (a.g.n > kSliceMin && a.ctrl->n_heavy == 0);
     const int64_t slice = (static_cast<int64_t>(a.g.n) + gridDim.x - 1) / gridDim.x;
-    const int64_t first = static_cast<int64_t>(blockIdx.x) * (kBatch ? slice : kBlock) + threadIdx.x;
-    const int64_t hi = kBatch ? min(static_cast<int64_t>(a.g.n), (blockIdx.x + 1) * slice) : a.g.n;
-    const int64_t stride = kBatch ? kBlock : static_cast<int64_t>(gridDim.x) * kBlock;
+    const int64_t first = static_cast<int64_t>(blockIdx.x) * (slices ? slice : kBlock) + threadIdx.x;
+    const int64_t hi = slices ? min(static_cast<int64_t>(a.g.n), (blockIdx.x + 1) * slice) : a.g.n;
+    const int64_t stride = slices ? kBlock : static_cast<int64_t>(gridDim.x) * kBlock;
     const bool many = nseg > a.scatter_segs;  // many classes: global atomics
     const int32_t hot = a.ctrl->hot_sg;
     if (!many) {

@@ -166,7 +166,8 @@ __global__ void __launch_bounds__(kBlock, kValBlocks) k_validate(ValArgs a) {
     const int w = threadIdx.x >> 5, l = lane_id();
     uint32_t* s_bits = s_bits_[w];
     int32_t* s_color = s_color_[w];
-    if (*reinterpret_cast<volatile uint32_t*>(&a.c->err)) return;  // malformed offsets: the steps mean nothing
+    // malformed offsets: the steps mean nothing (a vote: an id found bad meanwhile stops whole warps)
+    if (__any_sync(kFull, *reinterpret_cast<volatile uint32_t*>(&a.c->err) != 0u)) return;
     const int32_t n = a.g.n;
     const int64_t off0 = __ldg(a.g.off);
     const int64_t total = n + __ldg(a.g.off + n) - off0;

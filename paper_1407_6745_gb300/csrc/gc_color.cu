@@ -61,6 +61,7 @@ struct SpecCtrl {
     int32_t max_color;
     int32_t max_deg;
     uint32_t err;
+    uint32_t setup_err;     // malformed offsets (written by the set-up only: see k_spec_rounds)
     uint32_t barrier;       // arrivals at the grid barrier
     int32_t mark_cnt;       // row pieces to be pushed (round 0: to be tested) by the whole grid
     int32_t open_cnt;       // list pieces left open
@@ -196,7 +197,7 @@ __global__ void __launch_bounds__(kBlock) k_spec_setup(SpecArgs a) {
         int64_t beg = 0;
         int32_t deg = 0, b = kNB;
         if (valid) {
-            row_of(a.g, v, beg, deg, &a.ctrl->err);
+            row_of(a.g, v, beg, deg, &a.ctrl->setup_err);
             my_max_deg = max(my_max_deg, deg);
             int32_t X = a.X, vl = v;
             uint64_t seed = a.seed;
@@ -1273,12 +1274,18 @@ __device__ __forceinline__ void test_phase(Rounds& r) {
 
 // kHeavy: the graph has heavy rows (the form without them returns at once on
 // such a graph, and is launched before the host knows).
+//
+// The grid barriers need every block, so whether a launch runs is decided on
+// words that no launch writes: the set-up's errors and bucket counts.  `err`
+// is not among them -- a block of round 0 may have flagged an id in it before
+// another has started, and one that left on it would be waited for by the
+// others until their polls run out.
 template <bool kRXF, bool kHeavy, bool kWide>
 __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant__ SpecArgs a) {
     __shared__ WarpRounds s_w[kWarps];
     static_assert(sizeof(WarpRounds::head) >= kWarpBitmapWords * 4, "the full-row fallback's bitmap");
     SpecCtrl* const c = a.ctrl;
-    if (c->err || (!kHeavy && c->init_cnt[0] > 0)) return;
+    if (c->setup_err || (!kHeavy && c->init_cnt[0] > 0)) return;
     const int warp = threadIdx.x >> 5;
     const int l = lane_id();
     const int32_t mine = l < kNB && l != 1 ? c->init_cnt[l] : 0;
@@ -1387,7 +1394,7 @@ gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_
         if (e == cudaSuccess) e = cudaMemcpyAsync(h, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_status(e);
-        if (h->err) return status_from_err_bits(h->err);
+        if (h->err | h->setup_err) return status_from_err_bits(h->err | h->setup_err);
         if ((!heavy && h->init_cnt[0] > 0) || h->active == 0) return GC_OK;
         e = cudaMemsetAsync(&a.ctrl->barrier, 0, sizeof(uint32_t), s);
         if (e != cudaSuccess) return cuda_status(e);

@@ -55,22 +55,35 @@ static_assert(kRowPend == 256, "8 entries per lane of the warp that takes them")
 // 5.07 to 4.91 ms per iteration.)
 constexpr int kIsoBucket = 8;
 
-// The recoloring phase's buckets: those of bucket_of, and 7: rows of up to
+// The recoloring phase's buckets: 0 split rows, 1 a warp per row (bucket_of's 1
+// and 2, which the row's length tells apart: see kBitsDeg), 2..5 groups of
+// 16/8/4/2 lanes, and 6: rows of up to
 // kOneLaneDeg entries, a lane each (its gathers are one batch), where the
 // 2-lane threshold allows it.  Such rows are most of a skewed graph's and all
 // of a 7-point mesh's; with 2 lanes a warp tile held 16 of them (recoloring
 // launch, 2 lanes -> 1: 7-point mesh of 1 M vertices 53 -> 40 us, a batch of
 // 512 graphs 0.74 -> 0.66 ms, RMAT-Bad 22 0.56 -> 0.53, R-MAT 24 within 3 %).
-constexpr int kRcNB = 8;
+// No more than 7: the (class, bucket) tables of the largest input color are
+// then within 32-bit indices (an eighth bucket's were not).
+constexpr int kRcNB = 7;
 constexpr int32_t kOneLaneDeg = 8;
+constexpr int32_t kBitsDeg = 63;  // rows of up to this many entries: their color is among the first 64
+static_assert((static_cast<int64_t>(kMaxInputColor) + 1) * kRcNB <= INT32_MAX, "32-bit (class, bucket) indices");
+// Entries of the (class, bucket) tables for the colors [1, cap] (0: beyond 32-bit indices).
+inline int64_t class_entries(int32_t cap) {
+    const int64_t ent = (static_cast<int64_t>(cap) + 1) * kRcNB;
+    return ent <= INT32_MAX ? ent : 0;
+}
 __device__ __forceinline__ int rc_bucket_of(int32_t deg, const Tuning& t) {
     if (deg == 0) return kIsoBucket;
-    return deg <= min(kOneLaneDeg, t.g2_max_deg) ? 7 : bucket_of(deg, 1, t);
+    if (deg <= min(kOneLaneDeg, t.g2_max_deg)) return 6;
+    const int b = bucket_of(deg, 1, t);
+    return b < 2 ? b : b - 1;
 }
 
 // Lanes per row (log2) of a bucket's warp tiles, and rows (bucket 0: row
 // chunks) per tile.
-__host__ __device__ constexpr int lanes_log2(int b) { return b < 2 ? 5 : 7 - b; }
+__host__ __device__ constexpr int lanes_log2(int b) { return b < 2 ? 5 : 6 - b; }
 __host__ __device__ constexpr int warp_tile(int b) { return 32 >> lanes_log2(b); }
 
 struct RcCtrl {
@@ -404,6 +417,8 @@ __global__ void __launch_bounds__(kOrderThreads) k_rc_order(RcArgs a) {
 constexpr int kScatterSegs = 6144;  // segments counted in (dynamic) shared memory: 48 KB
 
 struct ScatterInfo {
+    int32_t rank;
+    int32_t b;
     int32_t sg;
     int32_t units;
     int64_t beg;
@@ -425,23 +440,23 @@ struct ScatterRow {
             end = __ldg(a.g.off + v + 1);
         }
     }
-    // Its segment, or -1: a batch's finished graph (keeps its colors), -2: isolated.
-    __device__ __forceinline__ int32_t segment(const RcArgs& a) const {
+    // The rank of its class, or -1: a batch's finished graph (keeps its colors), -2: isolated.
+    __device__ __forceinline__ int32_t rank(const RcArgs& a) const {
         int64_t key = c;
         if (kBatch) {  // the graph's own class ranks
             if (a.iteration >= a.desc[gi].iterations) return -1;
             key += a.cls_base[gi];
         }
-        return b == kIsoBucket ? -2 : a.rank_of[key] * kRcNB + b;
+        return b == kIsoBucket ? -2 : a.rank_of[key];
     }
     __device__ __forceinline__ int32_t deg() const { return static_cast<int32_t>(end - beg); }
     __device__ __forceinline__ int32_t units() const { return b == 0 ? chunks_of(deg()) : 1; }
 };
 
-// A vertex without a list entry: a finished graph's (segment -1) keeps its color,
+// A vertex without a list entry: a finished graph's (rank -1) keeps its color,
 // an isolated one (-2) takes color 1 and is counted in `iso`.
-__device__ __forceinline__ void place_unlisted(const RcArgs& a, int32_t v, int32_t sg, int32_t& iso) {
-    if (sg == -2) {
+__device__ __forceinline__ void place_unlisted(const RcArgs& a, int32_t v, int32_t rank, int32_t& iso) {
+    if (rank == -2) {
         a.new_c[v] = 1;
         ++iso;
     } else {
@@ -463,8 +478,8 @@ __device__ __forceinline__ void flush_placed(const RcArgs& a, int32_t iso, unsig
 }
 
 __device__ __forceinline__ void place(const RcArgs& a, int32_t v, const ScatterInfo& si, int32_t pos) {
-    a.new_c[v] = -(si.sg / kRcNB + 1);
-    if (si.sg % kRcNB != 0) {
+    a.new_c[v] = -(si.rank + 1);
+    if (si.b != 0) {
         store_item(a.list + pos, si.beg, v, si.deg);
         return;
     }
@@ -548,11 +563,11 @@ __global__ void __launch_bounds__(kBlock) k_rc_scatter(RcArgs a) {
         for (int64_t i = first; i < hi; i += stride) {
             row = next;
             if (i + stride < hi) next.load(a, i + stride, false);
-            const int32_t sg = row.segment(a);
-            if (sg < 0) continue;
+            const int32_t rank = row.rank(a);
+            if (rank < 0) continue;
             int32_t units = 1;
             if (row.b == 0) units = chunks_of(static_cast<int32_t>(__ldg(a.g.off + i + 1) - __ldg(a.g.off + i)));
-            hot_or_own(s_cnt, sg, units, hot);
+            hot_or_own(s_cnt, rank * kRcNB + row.b, units, hot);
         }
         __syncthreads();
         for (int i = threadIdx.x; i < nseg; i += kBlock) {
@@ -571,11 +586,13 @@ __global__ void __launch_bounds__(kBlock) k_rc_scatter(RcArgs a) {
         if (i + stride < hi) next.load(a, i + stride, true);
         const int32_t v = static_cast<int32_t>(i);
         ScatterInfo si;
-        si.sg = row.segment(a);
-        if (si.sg < 0) {
-            place_unlisted(a, v, si.sg, iso);
+        si.rank = row.rank(a);
+        if (si.rank < 0) {
+            place_unlisted(a, v, si.rank, iso);
             continue;
         }
+        si.b = row.b;
+        si.sg = si.rank * kRcNB + si.b;
         si.units = row.units();
         si.beg = row.beg;
         si.deg = row.deg();
@@ -641,7 +658,7 @@ struct RecolorFetch {
 };
 
 // Histogram of the new colors for the next iteration: counts in dynamic
-// shared memory sized to the colors (up to 1023 colors), flushed once per
+// shared memory sized to the colors (up to 1169 colors), flushed once per
 // block; beyond that, global counts, where the lanes of a warp that add to
 // the same (color, bucket) are merged into one atomic (most vertices of a
 // skewed graph take the same few colors, and unmerged adds to one global
@@ -822,8 +839,8 @@ __device__ __forceinline__ void defer_near(const RcArgs&, const RecolorFetch<fal
                                            int32_t (&)[8]) {}
 
 // One warp tile whose items and ids are staged: its rows' lanes gather the
-// neighbors' colors 8 at a time.  A row of the lane buckets (2..6) keeps its
-// forbidden colors in 64 register bits; a warp row or a chunk of a split row
+// neighbors' colors 8 at a time.  A row of up to kBitsDeg entries keeps its
+// forbidden colors in 64 register bits; a longer warp row or a chunk of a split row
 // keeps colors 1..32 in a register (most neighbors of a hub carry one of the
 // lowest colors, and as shared atomics they would all hit one word) and the
 // others in a shared bitmap.
@@ -869,8 +886,9 @@ __device__ __forceinline__ void recolor_tile(const RcArgs& a, const NextHist& nh
     __syncwarp();   // the slot and the staged ids are read: the next tiles' may land there
     stage_ahead();
 
+    const bool bits = b >= 2 || (b == 1 && it.deg <= kBitsDeg);  // (the same for the whole warp)
     uint32_t lo = 0, hi = 0;
-    if (b < 2) {
+    if (!bits) {
         w.bm[l] = 0u;
         w.bm[l + 32] = 0u;
         if (b == 0) {
@@ -886,7 +904,7 @@ __device__ __forceinline__ void recolor_tile(const RcArgs& a, const NextHist& nh
         load8<kDataflow>(f, u, x);
         wait8<kDataflow>(f, u, x, b == 0 ? max(p - kNearClasses, 0) : p);
         if (b == 0 && kDataflow) defer_near(a, f, -it.v - 1, u, x);
-        if (b >= 2) {
+        if (bits) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 lo |= bit_or_none(x[i] - 1);
@@ -909,7 +927,7 @@ __device__ __forceinline__ void recolor_tile(const RcArgs& a, const NextHist& nh
     }
     if (bad) atomicOr(&a.ctrl->err, kErrBadGraph);
 
-    if (b >= 2) {
+    if (bits) {
         for (int d = G >> 1; d >= 1; d >>= 1) {
             lo |= __shfl_xor_sync(kFull, lo, d);
             hi |= __shfl_xor_sync(kFull, hi, d);
@@ -1208,7 +1226,8 @@ gc_status class_ranks_device(const Graph& g, const int32_t* colors, bool trusted
     *maxc_out = h.max_in;
     if (!rank_out) return GC_OK;
     const int32_t cap = std::max(h.max_in, 1);
-    const int64_t ent = static_cast<int64_t>(cap + 1) * kRcNB;
+    const int64_t ent = class_entries(cap);
+    if (ent == 0) return GC_ERR_OOM;
     const int64_t c4 = static_cast<int64_t>(cap + 1) * 4, hist_bytes = ent * 4 + 2 * c4;
     sc.want(&a.cls_cnt, hist_bytes);
     sc.want(&a.present, c4);
@@ -1470,7 +1489,8 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     // Colors stay within [1, maxc_in]: a vertex of the class of rank p takes
     // at most color p + 1 <= k <= maxc_in.
     const int32_t cap = std::max(maxc_in, 1);
-    const int64_t ent = static_cast<int64_t>(cap + 1) * kRcNB;
+    const int64_t ent = class_entries(cap);
+    if (ent == 0) return GC_ERR_OOM;
     const int32_t hub_words = ((cap + 1 + 31) / 32 + 3) & ~3;  // 16-byte rows
     const int64_t hubs = std::max<int64_t>(1, h.n_heavy);
     // list entries: one per vertex, one per chunk of a bucket-0 row
@@ -1682,7 +1702,8 @@ static gc_status recolor_batch_impl(const Graph& g, const gc_batch_graph* graphs
         if (max_color_out) std::copy(gmax.begin(), gmax.end(), max_color_out);
         return cuda_status(cudaStreamSynchronize(s));
     }
-    const int64_t ent = static_cast<int64_t>(cap + 1) * kRcNB;
+    const int64_t ent = class_entries(cap);
+    if (ent == 0) return GC_ERR_OOM;
     const int32_t hub_words = ((cap + 1 + 31) / 32 + 3) & ~3;  // 16-byte rows
     const int64_t hubs = std::max<int64_t>(1, h.n_heavy);
     const int64_t list_len = n + (static_cast<int64_t>(g.nnz) / kChunk) + h.n_heavy;

@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "gc_internal.h"
+#include "gc_steps.h"
 
 namespace gc {
 
@@ -23,12 +24,8 @@ struct ValCtrl {
 
 constexpr int kValG = 4;                 // lanes per light row (measured: 8 -> 4 saves 30 us on the stencil)
 constexpr int32_t kHeavyDeg = 256;       // heavier rows: one block each (gc_validate_noalloc)
-// gc_validate: rows and entries of one warp's step together (8 entries a
-// lane, less what the 16-byte boundary before the first one can take), and
-// the blocks of an SM the registers are limited for (R-MAT 24 / 22 with 3:
-// 1.73 / 0.38 ms, with 4: 2.03 / 0.37, with 5: 2.06 / 0.39).
-constexpr int kValSlots = 8 * 32;
-constexpr int kValChunk = kValSlots - 4;
+// The blocks of an SM that the pass over the entries is limited for (R-MAT 24 /
+// 22 with 3: 1.73 / 0.38 ms, with 4: 2.03 / 0.37, with 5: 2.06 / 0.39).
 constexpr int kValBlocks = 3;
 constexpr int kPresWords = 2048;         // presence bitmap of colors < 65536
 constexpr int32_t kPresColors = kPresWords * 32;
@@ -78,11 +75,14 @@ __device__ __forceinline__ void flush_presence(const ValArgs& a, uint32_t* s_pre
         if (s_pres[i]) atomicOr(&a.pres[i], s_pres[i]);
 }
 
+constexpr int32_t kOwnSteps = 4;
+
 // One pass over the vertices: a vertex's own accounting, the low byte of its
 // color, and which row each step of the pass over the entries begins in.
 // Steps are cut on the count of rows plus entries (row v covers
 // [v + off[v], v + 1 + off[v + 1]) of it, less off[0]), so that neither a
-// long row nor a long run of empty rows falls to one block.
+// long row nor a long run of empty rows falls to one block (and the step
+// starts inside a long row are written by a warp, not by a thread).
 __global__ void __launch_bounds__(kBlock) k_validate_rows(ValArgs a) {
     __shared__ uint32_t s_pres[kPresWords];
     for (int i = threadIdx.x; i < kPresWords; i += kBlock) s_pres[i] = 0u;
@@ -92,33 +92,36 @@ __global__ void __launch_bounds__(kBlock) k_validate_rows(ValArgs a) {
     const int64_t off0 = __ldg(a.g.off);
     const bool narrow = a.g.n + a.g.nnz < int64_t(1) << 31;
     constexpr int U = 4;  // vertices of a thread whose loads are in flight together
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * (U * kBlock);
-    for (int64_t b = static_cast<int64_t>(blockIdx.x) * (U * kBlock) + threadIdx.x; b < a.g.n; b += stride) {
+    const int64_t all = static_cast<int64_t>(gridDim.x) * kBlock;
+    for (int64_t b0 = static_cast<int64_t>(blockIdx.x) * kBlock; b0 < a.g.n; b0 += U * all) {
+        const int64_t b = b0 + threadIdx.x;
         int64_t beg[U];
         int32_t deg[U], cv[U];
 #pragma unroll
         for (int i = 0; i < U; ++i) {
-            const int64_t v = min(b + i * kBlock, static_cast<int64_t>(a.g.n) - 1);
+            const int64_t v = min(b + i * all, static_cast<int64_t>(a.g.n) - 1);
             row_of(a.g, static_cast<int32_t>(v), beg[i], deg[i], &a.c->err);
             cv[i] = __ldg(a.colors + v);
         }
 #pragma unroll
         for (int i = 0; i < U; ++i) {
-            const int64_t v = b + i * kBlock;
-            if (v >= a.g.n) break;
-            account(a, static_cast<int32_t>(v), cv[i], 0, s_pres, conf, unc, my_max);
-            a.low[v] = static_cast<uint8_t>(cv[i]);
-            const int64_t d = v + beg[i] - off0;  // (negative only where the offsets are malformed)
-            const int64_t d1 = d + deg[i];
-            int64_t k0, k1;
-            if (narrow) {  // (a 64-bit division takes a third of the pass)
-                k0 = (static_cast<uint32_t>(d) + (kValChunk - 1u)) / kValChunk;
-                k1 = static_cast<uint32_t>(d1) / kValChunk;
-            } else {
-                k0 = (max(d, int64_t(0)) + kValChunk - 1) / kValChunk;
-                k1 = d1 / kValChunk;
+            const int64_t v = b + i * all;
+            int64_t k0 = 0, k1 = -1;
+            if (v < a.g.n) {
+                account(a, static_cast<int32_t>(v), cv[i], 0, s_pres, conf, unc, my_max);
+                a.low[v] = static_cast<uint8_t>(cv[i]);
+                row_steps(v + beg[i] - off0, deg[i], a.steps, narrow, k0, k1);
             }
-            for (k1 = min(k1, a.steps - 1); k0 <= k1; ++k0) a.first[k0] = static_cast<int32_t>(v);
+            // a row's steps: its own thread writes a few, its warp those of a longer row
+            const bool own = k1 - k0 < kOwnSteps;
+            if (own)
+                for (; k0 <= k1; ++k0) a.first[k0] = static_cast<int32_t>(v);
+            for (uint32_t m = __ballot_sync(kFull, !own); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const int64_t last = __shfl_sync(kFull, k1, src);
+                const int32_t row = static_cast<int32_t>(__shfl_sync(kFull, v, src));
+                for (int64_t k = __shfl_sync(kFull, k0, src) + lane_id(); k <= last; k += 32) a.first[k] = row;
+            }
         }
     }
     warp_add(&a.c->uncolored, unc);
@@ -157,7 +160,10 @@ __device__ __forceinline__ void step_ids(const Graph& g, int64_t a0, int64_t e1,
 // row, a warp or blocks a longer one, and 4-byte gathers took 0.69 and 2.63;
 // bytes alone 0.69 and 2.62; this with a block's steps and its barriers 0.52
 // and 2.23.  On a stencil of shuffled vertices, where nothing stays in L1,
-// 241 us for 230.  kInput: a recoloring input, with max_allowed.
+// 241 us for 230.  A step inside one row skips the bits, and a step's row is
+// read a step before its ids, which wait for it (both passes: R-MAT 22 416 ->
+// 367 us, K_4000 67 -> 43, its rows' steps written by warps included: 28 -> 9).
+// kInput: a recoloring input, with max_allowed.
 template <bool kInput>
 __global__ void __launch_bounds__(kBlock, kValBlocks) k_validate(ValArgs a) {
     constexpr int kWords = kValSlots / 32;
@@ -179,28 +185,40 @@ __global__ void __launch_bounds__(kBlock, kValBlocks) k_validate(ValArgs a) {
     int32_t v0 = 0, v1 = 0;
     int64_t e0 = 0, e1 = 0;
     int32_t u[8];
+    int32_t f0 = 0, f1 = 0;  // v0, v1 of the step staged next, read a step before its ids
+    const auto rows_of = [&](int64_t step) {
+        if (step >= nsteps) return;
+        f0 = __ldg(a.first + step);
+        f1 = step + 1 < nsteps ? __ldg(a.first + step + 1) : n;
+    };
+    rows_of(k);
     const auto stage = [&](int64_t step) {
-        v0 = __ldg(a.first + step);
-        v1 = step + 1 < nsteps ? __ldg(a.first + step + 1) : n;
+        v0 = f0;
+        v1 = f1;
         e0 = step * kValChunk - v0 + off0;
         e1 = min((step + 1) * kValChunk, total) - v1 + off0;
         step_ids(a.g, e0 & ~int64_t(3), e1, u);
+        rows_of(step + stride);
     };
     if (k < nsteps) stage(k);
     for (; k < nsteps; k += stride) {
         const int64_t a0 = e0 & ~int64_t(3);
         const int32_t first_row = v0, last_row = min(v1, n - 1);
         const int32_t lo = static_cast<int32_t>(e0 - a0), hi = static_cast<int32_t>(e1 - a0);  // slots
-        if (l < kWords) s_bits[l] = 0u;
-        __syncwarp();
-        for (int32_t r = first_row; r <= last_row; r += 32) {
-            const int32_t v = r + l;
-            if (v <= last_row) {
-                const int64_t b = max(__ldg(a.g.off + v), e0), e = min(__ldg(a.g.off + v + 1), e1);
-                if (b < e) {
-                    const int32_t at = static_cast<int32_t>(b - a0);
-                    s_color[at] = __ldg(a.colors + v);
-                    atomicOr(&s_bits[at >> 5], 1u << (at & 31));
+        const bool inside = first_row == last_row;  // of a long row: its entries have one color
+        const int32_t row_color = inside ? __ldg(a.colors + first_row) : 0;
+        if (!inside) {
+            if (l < kWords) s_bits[l] = 0u;
+            __syncwarp();
+            for (int32_t r = first_row; r <= last_row; r += 32) {
+                const int32_t v = r + l;
+                if (v <= last_row) {
+                    const int64_t b = max(__ldg(a.g.off + v), e0), e = min(__ldg(a.g.off + v + 1), e1);
+                    if (b < e) {
+                        const int32_t at = static_cast<int32_t>(b - a0);
+                        s_color[at] = __ldg(a.colors + v);
+                        atomicOr(&s_bits[at >> 5], 1u << (at & 31));
+                    }
                 }
             }
         }
@@ -218,44 +236,54 @@ __global__ void __launch_bounds__(kBlock, kValBlocks) k_validate(ValArgs a) {
             }
         }
         if (k + stride < nsteps) stage(k + stride);
-        __syncwarp();
-        // the last row start before each word
-        const uint32_t wb = l < kWords ? s_bits[l] : 0u;
-        int32_t m = wb ? 32 * l + 31 - __clz(wb) : -1;
-#pragma unroll
-        for (int d = 1; d < kWords; d <<= 1) {
-            const int32_t o = __shfl_up_sync(kFull, m, d);
-            if (l >= d) m = max(m, o);
-        }
         int32_t bad = INT_MAX;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int wi = 4 * h + (l >> 3);
-            const int at = 4 * (h * 32 + l);
-            const int32_t before = __shfl_sync(kFull, m, wi ? wi - 1 : 0);
-            const uint32_t word = __shfl_sync(kFull, wb, wi);
-            const uint32_t upto = word & (0xffffffffu >> (31 - (at & 31)));
-            int32_t row = upto ? (at & ~31) + 31 - __clz(upto) : wi ? before : -1;
-            const uint32_t begins = word >> (at & 31);
-            int32_t cv = row >= 0 ? s_color[row] : 0;
-            int32_t cvs[4];
-            uint32_t look = invalid >> (4 * h) & 15u;  // entries to look at again
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (j && (begins >> j & 1u)) cv = s_color[at + j];
-                cvs[j] = cv;
-                look |= static_cast<uint32_t>(low[4 * h + j] == (static_cast<uint32_t>(cv) & 255u)) << j;
+        // entry i of the lane, of the row that begins at slot `row` and has color cv
+        const auto look_at = [&](int i, int32_t cv, int32_t row) {
+            if (kInput && (cv < 1 || cv > a.max_allowed)) return;
+            if (invalid >> i & 1u) {
+                atomicOr(&a.c->err, kErrBadGraph);
+            } else if (__ldg(a.colors + x[i]) == cv) {
+                ++conf;
+                bad = min(bad, row);
             }
-            if (look == 0) continue;
+        };
+        if (inside) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (j && (begins >> j & 1u)) row = at + j;
-                if (!(look >> j & 1u) || (kInput && (cvs[j] < 1 || cvs[j] > a.max_allowed))) continue;
-                if (invalid >> (4 * h + j) & 1u) {
-                    atomicOr(&a.c->err, kErrBadGraph);
-                } else if (__ldg(a.colors + x[4 * h + j]) == cvs[j]) {
-                    ++conf;
-                    bad = min(bad, row);
+            for (int i = 0; i < 8; ++i)
+                if ((invalid >> i & 1u) || low[i] == (static_cast<uint32_t>(row_color) & 255u)) look_at(i, row_color, lo);
+        } else {
+            __syncwarp();
+            // the last row start before each word
+            const uint32_t wb = l < kWords ? s_bits[l] : 0u;
+            int32_t m = wb ? 32 * l + 31 - __clz(wb) : -1;
+#pragma unroll
+            for (int d = 1; d < kWords; d <<= 1) {
+                const int32_t o = __shfl_up_sync(kFull, m, d);
+                if (l >= d) m = max(m, o);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int wi = 4 * h + (l >> 3);
+                const int at = 4 * (h * 32 + l);
+                const int32_t before = __shfl_sync(kFull, m, wi ? wi - 1 : 0);
+                const uint32_t word = __shfl_sync(kFull, wb, wi);
+                const uint32_t upto = word & (0xffffffffu >> (31 - (at & 31)));
+                int32_t row = upto ? (at & ~31) + 31 - __clz(upto) : wi ? before : -1;
+                const uint32_t begins = word >> (at & 31);
+                int32_t cv = row >= 0 ? s_color[row] : 0;
+                int32_t cvs[4];
+                uint32_t look = invalid >> (4 * h) & 15u;  // entries to look at again
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (j && (begins >> j & 1u)) cv = s_color[at + j];
+                    cvs[j] = cv;
+                    look |= static_cast<uint32_t>(low[4 * h + j] == (static_cast<uint32_t>(cv) & 255u)) << j;
+                }
+                if (look == 0) continue;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (j && (begins >> j & 1u)) row = at + j;
+                    if (look >> j & 1u) look_at(4 * h + j, cvs[j], row);
                 }
             }
         }
@@ -310,7 +338,7 @@ struct ValRun {
         a.pres = reinterpret_cast<uint32_t*>(a.c + 1);
         cudaMemsetAsync(a.c, 0, sizeof(ValCtrl) + kPresWords * 4, s);
         const bool input = max_allowed != 0;
-        const int64_t row_blocks = (static_cast<int64_t>(g.n) + 4 * kBlock - 1) / (4 * kBlock);
+        const int64_t row_blocks = (static_cast<int64_t>(g.n) + kBlock - 1) / kBlock;
         const int rows = static_cast<int>(std::min<int64_t>(row_blocks, resident_grid(k_validate_rows, t)));
         GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE_ROWS, s, k_validate_rows<<<rows, kBlock, 0, s>>>(a));
         const auto entries = input ? k_validate<true> : k_validate<false>;

@@ -75,7 +75,10 @@ __device__ __forceinline__ void flush_presence(const ValArgs& a, uint32_t* s_pre
         if (s_pres[i]) atomicOr(&a.pres[i], s_pres[i]);
 }
 
-constexpr int32_t kOwnSteps = 4;
+// Steps of a row that its own thread writes (more: its warp).  Both ways are a
+// few stores; the warp's turns cost where many rows have some (R-MAT 22 with 4,
+// 32, 128: 42, 33, 31 us of row pass; a star of 10^7 vertices 187 -> 52 us).
+constexpr int32_t kOwnSteps = 128;
 
 // One pass over the vertices: a vertex's own accounting, the low byte of its
 // color, and which row each step of the pass over the entries begins in.
@@ -161,8 +164,8 @@ __device__ __forceinline__ void step_ids(const Graph& g, int64_t a0, int64_t e1,
 // bytes alone 0.69 and 2.62; this with a block's steps and its barriers 0.52
 // and 2.23.  On a stencil of shuffled vertices, where nothing stays in L1,
 // 241 us for 230.  A step inside one row skips the bits, and a step's row is
-// read a step before its ids, which wait for it (both passes: R-MAT 22 416 ->
-// 367 us, K_4000 67 -> 43, its rows' steps written by warps included: 28 -> 9).
+// read a step before its ids, which wait for it (this pass: R-MAT 22 376 ->
+// 327 us, K_4000 39 -> 34).
 // kInput: a recoloring input, with max_allowed.
 template <bool kInput>
 __global__ void __launch_bounds__(kBlock, kValBlocks) k_validate(ValArgs a) {
@@ -338,7 +341,9 @@ struct ValRun {
         a.pres = reinterpret_cast<uint32_t*>(a.c + 1);
         cudaMemsetAsync(a.c, 0, sizeof(ValCtrl) + kPresWords * 4, s);
         const bool input = max_allowed != 0;
-        const int64_t row_blocks = (static_cast<int64_t>(g.n) + kBlock - 1) / kBlock;
+        // (four vertices a thread, but a block per SM first: K_4000 10.6 -> 5.2 us)
+        const int64_t row_blocks = std::max<int64_t>((static_cast<int64_t>(g.n) + 4 * kBlock - 1) / (4 * kBlock),
+                                                     std::min<int64_t>((static_cast<int64_t>(g.n) + kBlock - 1) / kBlock, sm_count()));
         const int rows = static_cast<int>(std::min<int64_t>(row_blocks, resident_grid(k_validate_rows, t)));
         GC_LAUNCH(input ? KID_RC_VALIDATE : KID_VALIDATE_ROWS, s, k_validate_rows<<<rows, kBlock, 0, s>>>(a));
         const auto entries = input ? k_validate<true> : k_validate<false>;

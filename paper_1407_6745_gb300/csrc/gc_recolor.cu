@@ -759,7 +759,7 @@ constexpr int kStageIds = 384;
 struct __align__(16) WarpStage {
     WorkItem item[2][32];
     int32_t ids[kStageIds];
-    int4 meta[2];  // segment, entries
+    int4 meta[2];  // class rank, bucket, entries
     uint32_t bm[kWarpBitmapWords];
     uint32_t have[kWarpBitmapWords];  // a chunk's row: its merged bits, as read with the chunk
     int32_t win_t[32], win_s[32];     // tile prefix and start of the segments sought next
@@ -783,9 +783,9 @@ __device__ __forceinline__ void stage_copy4(void* smem, const void* gmem) {
 __device__ __forceinline__ void stage_ids(const RcArgs& a, WarpStage& w, int slot) {
     if (!a.g.vec) return;
     const int4 m = w.meta[slot];
-    const int lg = lanes_log2(m.x % kRcNB), G = 1 << lg;
+    const int lg = lanes_log2(m.y), G = 1 << lg;
     const int gi = lane_id() >> lg, gl = lane_id() & (G - 1);
-    if (gi >= m.y) return;
+    if (gi >= m.z) return;
     const WorkItem it = w.item[slot][gi];
     int32_t* dst = w.ids + gi * (kStageIds >> (5 - lg));
     const int64_t e0 = it.beg & ~static_cast<int64_t>(3);
@@ -857,11 +857,11 @@ __device__ __forceinline__ void recolor_tile(const RcArgs& a, const NextHist& nh
                                              int32_t& my_max, Ahead&& stage_ahead) {
     const int l = lane_id();
     const int4 m = w.meta[slot];
-    const int32_t p = m.x / kRcNB;
-    const int b = m.x % kRcNB;
+    const int32_t p = m.x;
+    const int b = m.y;
     const int lg = lanes_log2(b), G = 1 << lg;
     const int gi = l >> lg, gl = l & (G - 1);
-    const bool valid = gi < m.y;
+    const bool valid = gi < m.z;
     WorkItem it{0, 0, 0};
     if (valid) it = w.item[slot][gi];
     const RecolorFetch<kDataflow> f{a.new_c, p, a.tune.spin_limit, &a.ctrl->err, cached};
@@ -1083,11 +1083,12 @@ __device__ __forceinline__ void recolor_tiles(const RcArgs& a, const NextHist& n
         sg += n - 1;
         const int32_t seg_t = __shfl_sync(kFull, win_t, n - 1), seg_s = __shfl_sync(kFull, win_s, n - 1);
         const int32_t seg_e = __shfl_sync(kFull, win_s, n);
-        const int tile = warp_tile(sg % kRcNB);
+        const int32_t rank = sg / kRcNB, bucket = sg - rank * kRcNB;
+        const int tile = warp_tile(bucket);
         const int32_t first = seg_s + static_cast<int32_t>(tt - static_cast<uint32_t>(seg_t)) * tile;
         const int32_t cnt = min(tile, seg_e - first);
         if (l < cnt) stage_copy16(&w.item[slot][l], a.list + first + l, 16);
-        if (l == 0) w.meta[slot] = make_int4(sg, cnt, 0, 0);
+        if (l == 0) w.meta[slot] = make_int4(rank, bucket, cnt, 0);
     };
     sg = find_segment(a.tile_prefix, nseg, static_cast<int32_t>(t));
     load_window();

@@ -128,11 +128,14 @@ __device__ __forceinline__ int32_t tent_of(int32_t x) { return x & INT32_MAX; }
 
 // A vertex's color word (tentative color | kUnfixed, or the fixed color) and
 // priority.  Up to kWideMax vertices they share an 8-byte word, so that the
-// test of a light row takes one gather; beyond, 8-byte words would not stay
-// in L2 (gathers measured: 280 G/s up to 67 MB, 266 G/s at 80 MB, 119 G/s at 134 MB), and the
+// test of a light row takes one gather; beyond, the words, the masks and the
+// streamed rows would crowd each other out of L2, and the
 // color words (the output array) and the priorities are arrays of their own,
-// the priorities gathered only where a color matches.
-constexpr int64_t kWideMax = 10 << 20;
+// the priorities gathered only where a color matches.  (Coloring with shared /
+// separate words: G(3 10^6, 6) First Fit 0.80 / 0.82 ms, G(10^7, 6) 3.8 / 3.4,
+// G(10^7, 24) Random-8 Fit 7.4 / 6.0, RMAT-ER 23 First Fit 6.4 / 6.0, R-MAT 22
+// First Fit 16.6 / 16.0.)
+constexpr int64_t kWideMax = 15 << 18;
 template <bool kWide>
 __device__ __forceinline__ int32_t* color_word(const SpecArgs& a, int32_t v) {
     return kWide ? reinterpret_cast<int32_t*>(a.prio) + 2 * static_cast<int64_t>(v) + 1 : a.color + v;
@@ -409,9 +412,19 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
 }
 
+// The same for what a pass reads once (ids, offsets): first out of L2.
+__device__ __forceinline__ void cp_async16_stream(void* smem, const void* gmem) {
+    const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(sa), "l"(gmem),
+                 "l"(policy_evict_first())
+                 : "memory");
+}
+
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
     const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 8, %2;" ::"r"(sa), "l"(gmem),
+                 "l"(policy_evict_first())
+                 : "memory");
 }
 
 constexpr int kHead = 128;              // list entries a warp looks at first, 4 per lane
@@ -421,64 +434,83 @@ constexpr int32_t kPushInline = 128;    // longer winners' rows are pushed by th
 
 // What a warp keeps in shared memory: the heads of its current and next heavy
 // row's lists, or the items and ids of its current and next tile of light
-// rows; and the losers it has not yet written to the next list (one counter
-// update and one coalesced write per 16 or more of them).
-constexpr int kLightIds = 576;  // 36 per row with 2 lanes, 72 with 4
+// rows; and the losers it has not yet written to the next list.  kOut of them:
+// a counter update by all warps of the grid goes to one word, and pushes wait
+// behind it (G(10^7, 6) First Fit with 32: round 0 1.94 ms, 0.86 with no
+// update at all); large graphs (separate words) trade staged ids for more.
+template <bool kWide>
 struct __align__(16) WarpRounds {
+    static constexpr int kIds = kWide ? 512 : 448;  // per row with 2 lanes: 32, 28
+    static constexpr int kOut = kWide ? 64 : 96;
     union {
         int32_t head[2][kHead];
         struct {
             WorkItem item[2][16];
-            int32_t ids[2][kLightIds];
+            int32_t ids[2][kIds];
         } light;
     };
-    WorkItem out[32];
+    WorkItem out[kOut];
 };
 
 // State of a warp over the launch.  Lane b keeps the count of bucket b's work
 // list and the start of its region.
+template <bool kWide>
 struct Rounds {
     const SpecArgs& a;
-    WarpRounds& w;
+    WarpRounds<kWide>& w;
     int32_t lane_start, lane_cnt;
     int32_t round;
     int32_t par;
     int32_t out_n;         // buffered losers
+    int32_t out_at;        // lane 0: their places in the next list, once asked for
     int32_t my_max;
     unsigned long long edges;
     __device__ __forceinline__ int32_t start(int b) const { return __shfl_sync(kFull, lane_start, b); }
     __device__ __forceinline__ int32_t cnt(int b) const { return __shfl_sync(kFull, lane_cnt, b); }
 };
 
-__device__ __forceinline__ WorkItem* next_list(const Rounds& r) { return r.par ? r.a.list0 : r.a.list1; }
-__device__ __forceinline__ const WorkItem* this_list(const Rounds& r) { return r.par ? r.a.list1 : r.a.list0; }
+template <bool kWide>
+__device__ __forceinline__ WorkItem* next_list(const Rounds<kWide>& r) { return r.par ? r.a.list0 : r.a.list1; }
+template <bool kWide>
+__device__ __forceinline__ const WorkItem* this_list(const Rounds<kWide>& r) { return r.par ? r.a.list1 : r.a.list0; }
 
-// Writes the buffered losers of bucket b to the next list (in one go: fewer
-// than 16 were there before the last lanes', at most 32, came in).
-__device__ __forceinline__ void flush_losers(Rounds& r, int b) {
-    const int l = lane_id();
-    const int32_t n = r.out_n;
-    if (n == 0) return;
-    int32_t base = 0;
-    if (l == 0) base = atomicAdd(&r.a.ctrl->cnt[r.par ^ 1][b], n);
-    base = __shfl_sync(kFull, base, 0) + r.start(b);
-    for (int32_t i = l; i < n; i += 32) {
+// The buffered losers of bucket b ask for their places in the next list once
+// the next 16 may not fit any more, and are written there when these come (the
+// answer takes its time).
+template <bool kWide>
+__device__ __forceinline__ bool losers_asked(const Rounds<kWide>& r) { return r.out_n > WarpRounds<kWide>::kOut - 16; }
+template <bool kWide>
+__device__ __forceinline__ void ask_places(Rounds<kWide>& r, int b) {
+    if (lane_id() == 0) r.out_at = atomicAdd(&r.a.ctrl->cnt[r.par ^ 1][b], r.out_n);
+}
+template <bool kWide>
+__device__ __forceinline__ void write_losers(Rounds<kWide>& r, int b) {
+    const int32_t base = __shfl_sync(kFull, r.out_at, 0) + r.start(b);
+    for (int32_t i = lane_id(); i < r.out_n; i += 32) {
         const WorkItem x = r.w.out[i];
         store_item(next_list(r) + base + i, x.beg, x.v, x.deg);
     }
     __syncwarp();
     r.out_n = 0;
 }
+template <bool kWide>
+__device__ __forceinline__ void flush_losers(Rounds<kWide>& r, int b) {
+    if (r.out_n == 0) return;
+    if (!losers_asked(r)) ask_places(r, b);
+    write_losers(r, b);
+}
 
-// The lanes with `want` add their row to the losers of bucket b (one bucket
-// at a time is buffered).  The whole warp calls it.
-__device__ __forceinline__ void add_losers(Rounds& r, int b, bool want, int64_t beg, int32_t v, int32_t deg) {
+// The lanes with `want` (16 at most) add their row to the losers of bucket b
+// (one bucket at a time is buffered).  The whole warp calls it.
+template <bool kWide>
+__device__ __forceinline__ void add_losers(Rounds<kWide>& r, int b, bool want, int64_t beg, int32_t v, int32_t deg) {
     const uint32_t m = __ballot_sync(kFull, want);
     if (m == 0) return;
+    if (losers_asked(r)) write_losers(r, b);
     if (want) r.w.out[r.out_n + __popc(m & ((1u << lane_id()) - 1u))] = WorkItem{beg, v, deg};
     r.out_n += __popc(m);
     __syncwarp();
-    if (r.out_n >= 16) flush_losers(r, b);
+    if (losers_asked(r)) ask_places(r, b);
 }
 
 // A vertex fixed at color c sets its bit in the mask of each neighbor not yet
@@ -536,7 +568,7 @@ __device__ __forceinline__ void push_row(const SpecArgs& a, int64_t beg, int32_t
 // round that its vertex is in the work set (the method's choice and test;
 // the choice of round 0 is counted for all rows by the host).
 template <bool kHeavy, bool kWide>
-__device__ __forceinline__ void fix_color(Rounds& r, int32_t v, int32_t c, int32_t deg) {
+__device__ __forceinline__ void fix_color(Rounds<kWide>& r, int32_t v, int32_t c, int32_t deg) {
     r.a.color[v] = c;
     if (kWide) *color_word<true>(r.a, v) = c;
     if (kHeavy) r.a.bucket[v] = kBucketFixed;
@@ -580,7 +612,7 @@ __device__ __forceinline__ int32_t choose_from_bitmap(const uint32_t* bm, int32_
 
 // A heavy row's choice (the whole warp): the j-th clear bit of its bitmap.
 template <bool kRXF, bool kWide>
-__device__ __forceinline__ int32_t choose_heavy(Rounds& r, int32_t v, uint32_t j, uint64_t ref) {
+__device__ __forceinline__ int32_t choose_heavy(Rounds<kWide>& r, int32_t v, uint32_t j, uint64_t ref) {
     const SpecArgs& a = r.a;
     int32_t c = choose_from_bitmap(a.heavy.hbm + (ref >> 24), static_cast<int32_t>(ref & kRefWords), j);
     if (c < 0) {  // past the bitmap's free colors (Random-X with a large X): the row in full
@@ -595,7 +627,7 @@ __device__ __forceinline__ int32_t choose_heavy(Rounds& r, int32_t v, uint32_t j
 // A light row takes a thread (its color is among the first 64); a heavy one's
 // bitmap is searched.
 template <bool kRXF, bool kHeavy, bool kWide>
-__device__ __forceinline__ void choose_phase(Rounds& r) {
+__device__ __forceinline__ void choose_phase(Rounds<kWide>& r) {
     const SpecArgs& a = r.a;
     const WorkItem* list = this_list(r);
     if constexpr (kHeavy) {
@@ -758,8 +790,8 @@ __device__ __forceinline__ bool beaten(const SpecArgs& a, const int32_t (&u)[4],
 
 // The lanes with `want` add their light row to the losers (of bucket b;
 // round 0: of its own).
-template <bool kRound0>
-__device__ __forceinline__ void light_losers(Rounds& r, int b, bool want, const WorkItem& it) {
+template <bool kRound0, bool kWide>
+__device__ __forceinline__ void light_losers(Rounds<kWide>& r, int b, bool want, const WorkItem& it) {
     if (!kRound0) {
         add_losers(r, b, want, it.beg, it.v, it.deg);
         return;
@@ -780,10 +812,10 @@ __device__ __forceinline__ void light_losers(Rounds& r, int b, bool want, const 
 // checks of the adjacency; colors and priorities are gathered until the row
 // has lost.
 template <int G, bool kRXF, bool kHeavy, bool kWide, bool kRound0>
-__device__ __forceinline__ void light_rows(Rounds& r, int b) {
+__device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
     const SpecArgs& a = r.a;
     constexpr int R = 32 / G;
-    constexpr int kRow = kLightIds / R;  // ids of a row in the stage
+    constexpr int kRow = WarpRounds<kWide>::kIds / R;  // ids of a row in the stage
     static_assert(R <= 16 && kRow % 4 == 0, "16-byte rows");
     const int l = lane_id(), gi = l / G, gl = l % G;
     const int32_t cnt = kRound0 ? a.g.n : r.cnt(b);
@@ -798,7 +830,7 @@ __device__ __forceinline__ void light_rows(Rounds& r, int b) {
             int64_t* off = reinterpret_cast<int64_t*>(st.item[slot]);
             if (l <= min(R, cnt - tt * R)) cp_async8(off + l, a.g.off + tt * R + l);
         } else if (l < min(R, cnt - tt * R)) {
-            cp_async16(&st.item[slot][l], lst + tt * R + l);
+            cp_async16_stream(&st.item[slot][l], lst + tt * R + l);
         }
     };
     auto item = [&](int32_t tt, int slot) {
@@ -820,7 +852,7 @@ __device__ __forceinline__ void light_rows(Rounds& r, int b) {
         const int32_t np = min(row_pieces(a.g, it.beg, it.deg), kRow / 4);
         for (int32_t c = gl; c < np; c += G) {
             const int64_t e = (it.beg & ~static_cast<int64_t>(3)) + 4 * static_cast<int64_t>(c);
-            if (e + 4 <= a.g.nnz) cp_async16(&st.ids[slot][gi * kRow + 4 * c], a.g.idx + e);
+            if (e + 4 <= a.g.nnz) cp_async16_stream(&st.ids[slot][gi * kRow + 4 * c], a.g.idx + e);
         }
     };
     stage_items(t, 0);
@@ -904,6 +936,7 @@ __device__ __forceinline__ void light_rows(Rounds& r, int b) {
             lost |= group_any<G>(lose);
         }
         if (kRound0 && loop) atomicOr(&a.ctrl->err, kErrBadGraph);
+        light_losers<kRound0>(r, b, valid && lost && gl == 0, it);
         if (valid && !lost) {
             if (gl == 0) fix_color<kHeavy, kWide>(r, it.v, tv, it.deg);
             for (int32_t c = gl, q = 0; c < np; c += G, ++q) {
@@ -915,7 +948,6 @@ __device__ __forceinline__ void light_rows(Rounds& r, int b) {
                 push4<kHeavy>(a, u, tv);
             }
         }
-        light_losers<kRound0>(r, b, valid && lost && gl == 0, it);
         if (left <= W) break;
         t += W;
     }
@@ -933,7 +965,7 @@ __device__ __forceinline__ void light_rows(Rounds& r, int b) {
 // A heavy winner (the whole warp): fixed, and its row pushed or queued for
 // the whole grid.
 template <bool kWide>
-__device__ __forceinline__ void heavy_win(Rounds& r, int32_t v, int32_t c, int64_t beg, int32_t deg) {
+__device__ __forceinline__ void heavy_win(Rounds<kWide>& r, int32_t v, int32_t c, int64_t beg, int32_t deg) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     if (l == 0) fix_color<true, kWide>(r, v, c, deg);
@@ -954,7 +986,7 @@ __device__ __forceinline__ void heavy_win(Rounds& r, int32_t v, int32_t c, int64
 // ones that can beat it in a later round (their order is free, so the pieces
 // of a row just take places).
 template <bool kRXF, bool kWide>
-__device__ __forceinline__ void heavy_round0_piece(Rounds& r, const WorkItem& it) {
+__device__ __forceinline__ void heavy_round0_piece(Rounds<kWide>& r, const WorkItem& it) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t h = it.v;
@@ -1001,7 +1033,7 @@ __device__ __forceinline__ void heavy_round0_piece(Rounds& r, const WorkItem& it
 
 // Round 0, once every piece is done: winners and losers (32 rows per warp).
 template <bool kWide>
-__device__ __forceinline__ void heavy_round0_close(Rounds& r) {
+__device__ __forceinline__ void heavy_round0_close(Rounds<kWide>& r) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t nh = a.ctrl->init_cnt[0];
@@ -1047,7 +1079,8 @@ __device__ __forceinline__ bool list_hit(const SpecArgs& a, const int32_t* lst, 
 
 // A long list none of whose first entries beat its row is left to the whole
 // grid, in pieces.
-__device__ __forceinline__ void leave_open(Rounds& r, const WorkItem& it) {
+template <bool kWide>
+__device__ __forceinline__ void leave_open(const Rounds<kWide>& r, const WorkItem& it) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t np = (it.deg + kOpenPiece - 1) / kOpenPiece;
@@ -1081,7 +1114,7 @@ using Int = std::integral_constant<int, N>;
 // the list shrinks without a pass over it (it stays a superset of the
 // neighbors above v not fixed; its order is free).
 template <bool kWide>
-__device__ __forceinline__ void heavy_rows(Rounds& r) {
+__device__ __forceinline__ void heavy_rows(Rounds<kWide>& r) {
     const SpecArgs& a = r.a;
     const WorkItem* list = this_list(r);
     const int l = lane_id();
@@ -1190,7 +1223,7 @@ __device__ __forceinline__ void heavy_rows(Rounds& r) {
 // the row (acquire-release on the row's counter orders the other pieces'
 // findings before it).
 template <bool kWide>
-__device__ __forceinline__ void open_phase(Rounds& r) {
+__device__ __forceinline__ void open_phase(Rounds<kWide>& r) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t n = __ldcg(&a.ctrl->open_cnt);
@@ -1229,8 +1262,7 @@ __device__ __forceinline__ void open_phase(Rounds& r) {
 }
 
 // The long winners' rows, in pieces.
-__device__ __forceinline__ void push_phase(Rounds& r) {
-    const SpecArgs& a = r.a;
+__device__ __forceinline__ void push_phase(const SpecArgs& a) {
     const int32_t n = static_cast<int32_t>(min(static_cast<int64_t>(__ldcg(&a.ctrl->mark_cnt)), a.heavy.mark_cap));
     const int32_t W = gridDim.x * kWarps;
     for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(n); k += W) {
@@ -1240,7 +1272,7 @@ __device__ __forceinline__ void push_phase(Rounds& r) {
 }
 
 template <bool kRXF, bool kHeavy, bool kWide>
-__device__ __forceinline__ void test_phase(Rounds& r) {
+__device__ __forceinline__ void test_phase(Rounds<kWide>& r) {
     const SpecArgs& a = r.a;
     if (r.round == 0) {
         if constexpr (kHeavy) {
@@ -1282,16 +1314,16 @@ __device__ __forceinline__ void test_phase(Rounds& r) {
 // others until their polls run out.
 template <bool kRXF, bool kHeavy, bool kWide>
 __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant__ SpecArgs a) {
-    __shared__ WarpRounds s_w[kWarps];
-    static_assert(sizeof(WarpRounds::head) >= kWarpBitmapWords * 4, "the full-row fallback's bitmap");
+    __shared__ WarpRounds<kWide> s_w[kWarps];
+    static_assert(sizeof(WarpRounds<kWide>::head) >= kWarpBitmapWords * 4, "the full-row fallback's bitmap");
     SpecCtrl* const c = a.ctrl;
     if (c->setup_err || (!kHeavy && c->init_cnt[0] > 0)) return;
     const int warp = threadIdx.x >> 5;
     const int l = lane_id();
     const int32_t mine = l < kNB && l != 1 ? c->init_cnt[l] : 0;
-    Rounds r{a, s_w[warp],
+    Rounds<kWide> r{a, s_w[warp],
              static_cast<int32_t>(warp_inclusive_scan(static_cast<uint32_t>(mine))) - mine,
-             l < kNB ? c->cnt[c->round & 1][l] : 0, c->round, 0, 0, 0, 0ull};
+             l < kNB ? c->cnt[c->round & 1][l] : 0, c->round, 0, 0, 0, 0, 0ull};
     GridBarrier bar;
     unsigned long long conflicts = 0;
     int32_t total = 0;
@@ -1322,7 +1354,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant
                 if (!(ok = bar.sync(c))) break;
             }
             if (__ldcg(&c->mark_cnt) > 0) {
-                push_phase(r);
+                push_phase(a);
                 if (!(ok = bar.sync(c))) break;
             }
         }

@@ -259,11 +259,12 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_sums(SpecArgs a, int32_
     __shared__ long long s_e[kHeavyThreads / 32], s_w[kHeavyThreads / 32];
     const int l = lane_id(), w = threadIdx.x >> 5;
     long long te = 0, tw = 0;
-    const int32_t lo = blockIdx.x * kHeavyChunk;
-    for (int32_t h = lo + static_cast<int32_t>(threadIdx.x); h < min(nh, lo + kHeavyChunk); h += kHeavyThreads) {
+    const int64_t lo = static_cast<int64_t>(blockIdx.x) * kHeavyChunk;
+    const int64_t hi = min(static_cast<int64_t>(nh), lo + kHeavyChunk);
+    for (int64_t h = lo + threadIdx.x; h < hi; h += kHeavyThreads) {
         WorkItem it;
         long long e, wd;
-        heavy_sizes(a, h, nh, it, e, wd);
+        heavy_sizes(a, static_cast<int32_t>(h), nh, it, e, wd);
         te += e;
         tw += wd;
     }
@@ -307,14 +308,14 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
         s_base_w = bw;
     }
     __syncthreads();
-    const int32_t lo = blockIdx.x * kHeavyChunk;
-    const int32_t hi = min(nh, lo + kHeavyChunk);
+    const int64_t lo = static_cast<int64_t>(blockIdx.x) * kHeavyChunk;
+    const int64_t hi = min(static_cast<int64_t>(nh), lo + kHeavyChunk);
     const HeavyRows& hr = a.heavy;
-    for (int32_t h0 = lo; h0 < hi; h0 += kHeavyThreads) {
-        const int32_t h = h0 + static_cast<int32_t>(threadIdx.x);
+    for (int64_t h0 = lo; h0 < hi; h0 += kHeavyThreads) {
+        const int64_t h = h0 + threadIdx.x;
         WorkItem it;
         long long e, wd;
-        heavy_sizes(a, h < hi ? h : nh, nh, it, e, wd);
+        heavy_sizes(a, h < hi ? static_cast<int32_t>(h) : nh, nh, it, e, wd);
         const int32_t np = (it.deg + kRound0Piece - 1) / kRound0Piece;
         long long ie = e, iw = wd;  // warp inclusive scans
         int32_t ip = np;
@@ -332,7 +333,7 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
         if (l == 31 && ip) pbase = atomicAdd(&a.ctrl->mark_cnt, ip);
         pbase = __shfl_sync(kFull, pbase, 31) + ip - np;
         for (int32_t q = 0; q < np && pbase + q < hr.mark_cap; ++q)
-            store_item(hr.mark + pbase + q, it.beg + static_cast<int64_t>(q) * kRound0Piece, h,
+            store_item(hr.mark + pbase + q, it.beg + static_cast<int64_t>(q) * kRound0Piece, static_cast<int32_t>(h),
                        min(kRound0Piece, it.deg - q * kRound0Piece));
         if (l == 31) {
             s_e[w] = ie;
@@ -611,7 +612,7 @@ __device__ __forceinline__ int32_t choose_from_bitmap(const uint32_t* bm, int32_
 }
 
 // A heavy row's choice (the whole warp): the j-th clear bit of its bitmap.
-template <bool kRXF, bool kWide>
+template <bool kWide>
 __device__ __forceinline__ int32_t choose_heavy(Rounds<kWide>& r, int32_t v, uint32_t j, uint64_t ref) {
     const SpecArgs& a = r.a;
     int32_t c = choose_from_bitmap(a.heavy.hbm + (ref >> 24), static_cast<int32_t>(ref & kRefWords), j);
@@ -643,7 +644,7 @@ __device__ __forceinline__ void choose_phase(Rounds<kWide>& r) {
             const uint32_t k = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
             if (k < n) {
                 const int32_t v = load_item_rw(list + k).v;
-                const int32_t c = choose_heavy<kRXF, kWide>(r, v, kRXF ? draw_index(a, v, r.round) : 0u, __ldg(a.heavy.bref + v));
+                const int32_t c = choose_heavy<kWide>(r, v, kRXF ? draw_index(a, v, r.round) : 0u, __ldg(a.heavy.bref + v));
                 if (lane_id() == 0) *color_word<kWide>(a, v) = c | kUnfixed;
             }
         } else for (uint32_t k0 = blockIdx.x * kBlock + (threadIdx.x & ~31u); k0 < n; k0 += step) {
@@ -678,7 +679,7 @@ __device__ __forceinline__ void choose_phase(Rounds<kWide>& r) {
                 const int32_t vs = __shfl_sync(kFull, v, src);
                 const uint32_t js = __shfl_sync(kFull, j, src);
                 const uint64_t rs = __shfl_sync(kFull, ref, src);
-                const int32_t cs = choose_heavy<kRXF, kWide>(r, vs, js, rs);
+                const int32_t cs = choose_heavy<kWide>(r, vs, js, rs);
                 if (lane_id() == src) c = cs;
             }
             if (k < n) *color_word<kWide>(a, v) = c | kUnfixed;
@@ -990,7 +991,7 @@ __device__ __forceinline__ void heavy_round0_piece(Rounds<kWide>& r, const WorkI
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t h = it.v;
-    const int32_t v = __ldg(&a.list0[h].v);
+    const int32_t v = __ldcg(&a.list0[h].v);
     int32_t* dst = a.heavy.pend + __ldg(a.heavy.h_pbeg + h);
     const uint32_t pv = prio_word<kWide>(a, v);
     const int32_t tv = kRXF ? tent_of(*color_word<kWide>(a, v)) : 1;
@@ -1037,14 +1038,14 @@ __device__ __forceinline__ void heavy_round0_close(Rounds<kWide>& r) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t nh = a.ctrl->init_cnt[0];
-    const int32_t W = gridDim.x * kWarps;
-    for (int32_t h0 = (blockIdx.x * kWarps + (threadIdx.x >> 5)) * 32; h0 < nh; h0 += W * 32) {
-        const int32_t h = h0 + l;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * kBlock;
+    for (int64_t h0 = (static_cast<int64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5)) * 32; h0 < nh; h0 += step) {
+        const int64_t h = h0 + l;
         WorkItem it{0, 0, 0};
         int32_t pc = 0, c = 0;
         int64_t pb = 0;
         if (h < nh) {
-            it = load_item(a.list0 + h);
+            it = load_item_rw(a.list0 + h);
             pc = __ldcg(a.heavy.h_pcnt + h);
             pb = __ldg(a.heavy.h_pbeg + h);
             c = tent_of(*color_word<kWide>(a, it.v));
@@ -1280,10 +1281,10 @@ __device__ __forceinline__ void test_phase(Rounds<kWide>& r) {
             const int32_t W = gridDim.x * kWarps;
             uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5);
             WorkItem it{0, 0, 0};
-            if (k < static_cast<uint32_t>(np)) it = load_item(a.heavy.mark + k);
+            if (k < static_cast<uint32_t>(np)) it = load_item_rw(a.heavy.mark + k);
             for (; k < static_cast<uint32_t>(np); k += W) {
                 WorkItem nx{0, 0, 0};
-                if (k + W < static_cast<uint32_t>(np)) nx = load_item(a.heavy.mark + k + W);
+                if (k + W < static_cast<uint32_t>(np)) nx = load_item_rw(a.heavy.mark + k + W);
                 heavy_round0_piece<kRXF, kWide>(r, it);
                 it = nx;
             }
@@ -1485,7 +1486,7 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
     const auto setup = wide ? k_spec_setup<true> : k_spec_setup<false>;
     const int setup_grid = static_cast<int>(std::min<int64_t>((n + kBlock - 1) / kBlock, resident_grid(setup, a.tune)));
     GC_LAUNCH(KID_SPEC_SETUP, s, setup<<<setup_grid, kBlock, 0, s>>>(a));
-    SpecCtrl h;
+    SpecCtrl h{};
     gc_status st = run_rounds(a, X > 1, false, &h, s);
     ScratchSet sc_heavy, sc_queues;
     if (st == GC_OK && h.init_cnt[0] > 0) {

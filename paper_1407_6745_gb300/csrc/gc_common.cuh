@@ -182,6 +182,13 @@ __device__ __forceinline__ int select_bit64(uint64_t x, uint32_t j) {
     return 32 + select_bit32(static_cast<uint32_t>(x >> 32), j - pl);
 }
 
+// 1 << d, 0 for d outside [0, 32) (the shift clamps).
+__device__ __forceinline__ uint32_t bit_or_none(int32_t d) {
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(d));
+    return r;
+}
+
 // Streamed data (adjacency, work items) is read once per pass: it is loaded
 // with an L2 evict-first policy and without L1 allocation, so it does not
 // push the gathered color arrays out of L2.

@@ -94,6 +94,7 @@ struct RcCtrl {
     int32_t n_heavy;      // rows in bucket 0 (split into chunks)
     uint32_t err;
     int32_t hot_sg;       // the largest segment of single-entry vertices (scatter)
+    uint32_t over;        // a vertex took a color above cap (only where the CSR is not symmetric)
     unsigned long long edges;
 };
 
@@ -336,6 +337,8 @@ __device__ __forceinline__ void build_segments(const RcArgs& a, int32_t k, Order
 __global__ void __launch_bounds__(kOrderThreads) k_rc_order(RcArgs a) {
     __shared__ OrderShared s;
     const int t = threadIdx.x;
+    // the tables hold the colors up to cap: no iteration on others
+    if (t == 0 && a.ctrl->over) atomicOr(&a.ctrl->err, kErrImproper);
     // present classes in ascending color, with their sizes
     int32_t k = 0;
     for (int32_t c0 = 1; c0 <= a.cap; c0 += kOrderThreads) {
@@ -670,8 +673,12 @@ struct NextHist {
     int32_t* glob;
     int32_t* units;
     int32_t cap;
+    uint32_t* over;
     __device__ __forceinline__ void add(int32_t c, int b, int32_t chunks) const {
-        if (c < 1 || c > cap) return;
+        if (c < 1 || c > cap) {
+            if (over) atomicOr(over, 1u);
+            return;
+        }
         const int32_t key = c * kRcNB + b;
         if (sh) {
             atomicAdd(&sh[key], 1);
@@ -743,13 +750,6 @@ __device__ __forceinline__ void wait8(const RecolorFetch<kDataflow>& f, const in
         for (int i = 0; i < 8; ++i)
             if (in_flight(x[i], f.p)) x[i] = ld_relaxed(f.new_c + u[i]);
     }
-}
-
-// 1 << d, 0 for d outside [0, 32) (the shift clamps).
-__device__ __forceinline__ uint32_t bit_or_none(int32_t d) {
-    uint32_t r;
-    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(d));
-    return r;
 }
 
 // What a warp keeps in shared memory: the work items of its current and next
@@ -1041,6 +1041,14 @@ __device__ __forceinline__ void recolor_tile(const RcArgs& a, const NextHist& nh
             return;
         }
     }
+    // every color of the bitmap is taken (not on a symmetric CSR): a color
+    // all the same, above cap, since others wait for the row
+    if (l == 0) {
+        const int32_t c = 32 * a.hub_words + 1;
+        st_relaxed(a.new_c + hv, c);
+        my_max = max(my_max, c);
+        nh.add(c, 0, 0);
+    }
 }
 
 // A warp's tiles t, t + step, ... below `end`, in order.  A tile is reached
@@ -1141,11 +1149,11 @@ inline int coop_grid(int64_t nnz, int32_t classes, int capacity) {
 // unfinished tile has finished all its earlier tiles, so it is working on
 // that tile: the waits always end.
 __device__ __forceinline__ NextHist setup_next_hist(const RcArgs& a, int32_t* s_hist) {
-    if (!a.fuse_hist) return NextHist{nullptr, nullptr, nullptr, 0};  // cap 0: add() is a no-op
+    if (!a.fuse_hist) return NextHist{nullptr, nullptr, nullptr, 0, nullptr};  // cap 0: add() is a no-op
     const bool local = a.hist_smem > 0;  // (cap + 1) * kRcNB entries of dynamic shared memory
     if (local)
         for (int i = threadIdx.x; i < a.hist_smem; i += kBlock) s_hist[i] = 0;
-    return NextHist{local ? s_hist : nullptr, a.nxt_cnt, a.nxt_units, a.cap};
+    return NextHist{local ? s_hist : nullptr, a.nxt_cnt, a.nxt_units, a.cap, &a.ctrl->over};
 }
 
 __device__ __forceinline__ void flush_next_hist(const RcArgs& a, const NextHist& nh) {

@@ -63,6 +63,7 @@ struct SpecCtrl {
     uint32_t err;
     uint32_t setup_err;     // malformed offsets (written by the set-up only: see k_spec_rounds)
     uint32_t barrier;       // arrivals at the grid barrier
+    int32_t stuck;          // a round had no winner (see k_pull_choose)
     int32_t mark_cnt;       // row pieces to be pushed (round 0: to be tested) by the whole grid
     int32_t open_cnt;       // list pieces left open
     int32_t open_rows;
@@ -110,6 +111,7 @@ struct SpecArgs {
     SpecCtrl* ctrl;
     int32_t round_limit;
     int32_t max_rounds;   // rounds of this launch
+    int32_t chosen;       // the first round's choice has been made (k_pull_choose)
     // batches: graph of every vertex and the graphs' descriptors (nullptr for
     // one graph), and the round in which every vertex kept its color
     const int32_t* graph_of;
@@ -1332,7 +1334,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant
     for (int32_t done = 0; done < a.max_rounds; ++done) {
         r.par = r.round & 1;
         if (r.round > 0) {
-            choose_phase<kRXF, kHeavy, kWide>(r);
+            if (done > 0 || !a.chosen) choose_phase<kRXF, kHeavy, kWide>(r);
             if (blockIdx.x == 0 && threadIdx.x < kNB) c->cnt[r.par ^ 1][threadIdx.x] = 0;
             if (blockIdx.x == 0 && threadIdx.x == 0) {
                 c->mark_cnt = 0;
@@ -1359,11 +1361,16 @@ __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant
                 if (!(ok = bar.sync(c))) break;
             }
         }
+        const int32_t before = __reduce_add_sync(kFull, r.lane_cnt);  // (0 in round 0)
         r.lane_cnt = l < kNB ? __ldcg(&c->cnt[r.par ^ 1][l]) : 0;
         total = __reduce_add_sync(kFull, r.lane_cnt);
         conflicts += static_cast<unsigned long long>(total);
         ++r.round;
         if (total == 0) break;
+        if (total == before) {  // no winner: see k_pull_choose
+            if (blockIdx.x == 0 && threadIdx.x == 0) c->stuck = 1;
+            break;
+        }
         if (r.round >= a.round_limit) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&c->err, kErrRoundLimit);
             break;
@@ -1376,6 +1383,40 @@ __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant
     }
     warp_add(&c->edges, r.edges);
     warp_max(&c->max_color, r.my_max);
+}
+
+// Start of bucket b's region of the work lists.
+__device__ __forceinline__ int32_t region_start(const SpecCtrl* c, int b) {
+    int32_t s = 0;
+    for (int q = 0; q < b; ++q) s += q != 1 ? c->init_cnt[q] : 0;
+    return s;
+}
+
+// The choice of a whole round from the rows, a warp each.  The row of the
+// work set above all others wins a round unless a neighbor fixed before has
+// its color, so a round without a winner means that a neighbor did not push
+// it: the CSR is not symmetric, or a bad id was dropped.  The launch then
+// ends, and the rounds left are run one by one with this choice.
+template <bool kWide>
+__global__ void __launch_bounds__(kBlock) k_pull_choose(const __grid_constant__ SpecArgs a) {
+    __shared__ uint32_t s_bm[kWarps][kWarpBitmapWords];
+    SpecCtrl* const c = a.ctrl;
+    if (blockIdx.x == 0 && threadIdx.x == 0) c->barrier = 0;  // of the next launch
+    const int par = c->round & 1;
+    const WorkItem* list = par ? a.list1 : a.list0;
+    for (int b = 0; b < kNB; ++b) {
+        const uint32_t n = b != 1 ? c->cnt[par][b] : 0;
+        const WorkItem* lst = list + region_start(c, b);
+        for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < n; k += gridDim.x * kWarps) {
+            const int32_t v = load_item(lst + k).v;
+            int64_t beg;
+            int32_t deg;
+            row_of(a.g, v, beg, deg, &c->err);
+            const uint32_t j = a.graph_of || a.X > 1 ? draw_index(a, v, c->round) : 0u;
+            const int32_t color = choose_warp<4>(a.g, beg, deg, j, SnapshotFetch<kWide>{a}, s_bm[threadIdx.x >> 5], &c->err);
+            if (lane_id() == 0) *color_word<kWide>(a, v) = color | kUnfixed;
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kBlock) k_priorities(uint64_t seed, int64_t n, uint32_t* out) {
@@ -1413,13 +1454,16 @@ const void* rounds_kernel_of(bool rxf, bool heavy) {
 // The rounds: one cooperative launch (spec_graph 1), or one per round.  h
 // receives the final control block.
 gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_t s) {
-    const void* k = a.g.n <= kWideMax ? rounds_kernel_of<true>(rxf, heavy) : rounds_kernel_of<false>(rxf, heavy);
+    const bool wide = a.g.n <= kWideMax;
+    const void* k = wide ? rounds_kernel_of<true>(rxf, heavy) : rounds_kernel_of<false>(rxf, heavy);
+    const auto pull = wide ? k_pull_choose<true> : k_pull_choose<false>;
     const int fit = sm_count() * occupancy_of(k, kBlock);
     // a block per tile of round 0 at most: on small graphs more blocks would only lengthen the barriers
     const int64_t tiles = heavy ? fit : (static_cast<int64_t>(a.g.n) * 2 + kBlock - 1) / kBlock;
     const int64_t want = a.tune.grid_blocks > 0 ? a.tune.grid_blocks : std::max<int64_t>(1, tiles);
     const int grid = static_cast<int>(std::min<int64_t>(fit, want));
     a.max_rounds = a.tune.spec_graph ? INT32_MAX : 1;
+    a.chosen = 0;
     for (;;) {
         void* args[] = {&a};
         cudaError_t e;
@@ -1429,6 +1473,12 @@ gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_
         if (e != cudaSuccess) return cuda_status(e);
         if (h->err | h->setup_err) return status_from_err_bits(h->err | h->setup_err);
         if ((!heavy && h->init_cnt[0] > 0) || h->active == 0) return GC_OK;
+        if (h->stuck) {
+            a.chosen = 1;
+            a.max_rounds = 1;
+            GC_LAUNCH(KID_SPEC_PULL, s, pull<<<resident_grid(pull, a.tune), kBlock, 0, s>>>(a));
+            continue;
+        }
         e = cudaMemsetAsync(&a.ctrl->barrier, 0, sizeof(uint32_t), s);
         if (e != cudaSuccess) return cuda_status(e);
     }

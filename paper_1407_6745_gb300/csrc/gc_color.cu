@@ -849,8 +849,26 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
         }
         return it;
     };
+    // Round 0: the rows of a tile are consecutive in the adjacency, and are
+    // staged as one run where that fits (else, and later, a part for each row:
+    // most rows of a skewed graph are short, and the few longer than their
+    // part were read id by id).  First place of the run, -1: it does not fit.
+    auto run_of = [&](int32_t tt, int slot, int64_t& end) -> int64_t {
+        if (!kRound0) return -1;
+        const int64_t* off = reinterpret_cast<const int64_t*>(st.item[slot]);
+        const int64_t base = off[0] & ~static_cast<int64_t>(3);
+        end = off[min(R, cnt - tt * R)];
+        return end - base <= WarpRounds<kWide>::kIds ? base : -1;
+    };
     auto stage_ids = [&](int32_t tt, int slot) {
         if (!a.g.vec) return;
+        int64_t end = 0;
+        const int64_t base = run_of(tt, slot, end);
+        if (kRound0 && base >= 0) {
+            for (int64_t e = base + 4 * l; e < end; e += 128)
+                if (e + 4 <= a.g.nnz) cp_async16_stream(&st.ids[slot][e - base], a.g.idx + e);
+            return;
+        }
         const WorkItem it = item(tt, slot);
         const int32_t np = min(row_pieces(a.g, it.beg, it.deg), kRow / 4);
         for (int32_t c = gl; c < np; c += G) {
@@ -873,6 +891,13 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
         cp_async_wait<0>();
         __syncwarp();
         const WorkItem it = item(t, slot);
+        const int32_t shift = static_cast<int32_t>(it.beg & 3);
+        int64_t run_end = 0;
+        const int64_t run = run_of(t, slot, run_end);
+        // where the row's pieces are staged, and how many of them
+        const int32_t at0 = run >= 0 ? static_cast<int32_t>(it.beg - shift - run) : gi * kRow;
+        const int32_t staged = a.g.vec ? static_cast<int32_t>(min(static_cast<int64_t>(run >= 0 ? INT32_MAX : kRow / 4),
+                                                                  (a.g.nnz - it.beg + shift) >> 2)) : 0;
         __syncwarp();  // the slot's items are read: the ones after the next tile's may land there
         const bool valid = gi < cnt - t * R && (!kRound0 || !kHeavy || bucket != 0);
         const int32_t left = tiles - t;
@@ -882,11 +907,9 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
         }
         cp_async_commit();
 
-        const int32_t shift = static_cast<int32_t>(it.beg & 3);
-        const int32_t staged = a.g.vec ? static_cast<int32_t>(min(static_cast<int64_t>(kRow / 4), (a.g.nnz - it.beg + shift) >> 2)) : 0;
         auto piece = [&](int32_t c, int32_t (&u)[4]) {
             if (c < staged) {
-                const int4 q = *reinterpret_cast<const int4*>(&st.ids[slot][gi * kRow + 4 * c]);
+                const int4 q = *reinterpret_cast<const int4*>(&st.ids[slot][at0 + 4 * c]);
                 u[0] = q.x;
                 u[1] = q.y;
                 u[2] = q.z;

@@ -135,7 +135,7 @@ void note_launches(int64_t k) { g_launches.fetch_add(k, std::memory_order_relaxe
 // ---------------------------------------------------------------------------
 namespace {
 const char* const kKernelNames[] = {
-    "k_spec_setup", "k_heavy_setup", "k_spec_rounds", "k_pull_choose", "k_priorities",
+    "k_spec_setup", "k_heavy_setup", "k_spec_rounds", "k_pull_choose", "k_late_marks", "k_priorities",
     "k_rc_bucket", "k_rc_validate", "k_rc_hist", "k_rc_order", "k_rc_scatter",
     "k_rc_recolor_coop", "k_rc_recolor_step", "k_validate", "k_validate_rows",
     "k_mark_present", "k_count_bits", "k_check_graph", "k_batch", "k_brc_hist",

@@ -63,12 +63,13 @@ struct SpecCtrl {
     uint32_t err;
     uint32_t setup_err;     // malformed offsets (written by the set-up only: see k_spec_rounds)
     uint32_t barrier;       // arrivals at the grid barrier
-    int32_t stuck;          // a round had no winner (see k_pull_choose)
     int32_t mark_cnt;       // row pieces to be pushed (round 0: to be tested) by the whole grid
     int32_t open_cnt;       // list pieces left open
     int32_t open_rows;
+    int32_t stuck;          // a round had no winner (see k_pull_choose)
     unsigned long long edges;
     unsigned long long conflicts;
+    unsigned long long lose16;  // Random-X: 16 x the entries of the rows expected to lose round 0 (set-up)
     long long heavy_entries;  // list entries over all heavy rows
     long long heavy_words;    // bitmap words over all heavy rows
 };
@@ -111,6 +112,7 @@ struct SpecArgs {
     SpecCtrl* ctrl;
     int32_t round_limit;
     int32_t max_rounds;   // rounds of this launch
+    float late_share;     // round 0 leaves its marks to k_late_marks below this share of losers (see late_of)
     int32_t chosen;       // the first round's choice has been made (k_pull_choose)
     // batches: graph of every vertex and the graphs' descriptors (nullptr for
     // one graph), and the round in which every vertex kept its color
@@ -188,6 +190,14 @@ __device__ __forceinline__ uint32_t draw_index(const SpecArgs& a, int32_t v, int
 // the heavy rows' region of the round-0 list.  (The light rows of round 0
 // are taken in id order and need no list.)
 // ---------------------------------------------------------------------------
+// Chance that a row of deg entries loses round 0: about Poisson(deg / X)
+// neighbors draw its color, and it wins over k of them with chance 1 / (k + 1).
+__device__ __forceinline__ float lose_chance(float deg, int32_t X) {
+    if (X <= 1) return deg / (deg + 1.0f);
+    const float m = deg / static_cast<float>(X);
+    return m < 0.01f ? 0.5f * m : 1.0f - (1.0f - expf(-m)) / m;
+}
+
 template <bool kWide>
 __global__ void __launch_bounds__(kBlock) k_spec_setup(SpecArgs a) {
     __shared__ int32_t s_cnt[kNB];
@@ -195,6 +205,7 @@ __global__ void __launch_bounds__(kBlock) k_spec_setup(SpecArgs a) {
     __syncthreads();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kBlock;
     int32_t my_max_deg = 0;
+    unsigned long long lose16 = 0;
     for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * kBlock; i0 < a.g.n; i0 += stride) {
         const int64_t i = i0 + threadIdx.x;
         const bool valid = i < a.g.n;
@@ -219,6 +230,7 @@ __global__ void __launch_bounds__(kBlock) k_spec_setup(SpecArgs a) {
             if (a.prio_kind == 1) p = ordered_prio(deg, p);
             else if (a.prio_kind == 2) p = ordered_prio(65535 - static_cast<int64_t>(a.prio_rank[a.prio_old[v]]), p);
             const uint32_t j0 = (a.graph_of || a.X > 1) ? draw_index(a, v, 0) : 0u;
+            if (a.X > 1) lose16 += static_cast<unsigned long long>(16.0f * static_cast<float>(deg) * lose_chance(static_cast<float>(deg), X));
             const int32_t c0 = static_cast<int32_t>(j0 + 1u) | kUnfixed;
             if (kWide) {
                 reinterpret_cast<uint2*>(a.prio)[v] = make_uint2(p, static_cast<uint32_t>(c0));
@@ -236,6 +248,7 @@ __global__ void __launch_bounds__(kBlock) k_spec_setup(SpecArgs a) {
         }
     }
     warp_max(&a.ctrl->max_deg, my_max_deg);
+    warp_add(&a.ctrl->lose16, lose16);
     __syncthreads();
     if (threadIdx.x >= 2 && threadIdx.x < kNB && s_cnt[threadIdx.x])
         atomicAdd(&a.ctrl->init_cnt[threadIdx.x], s_cnt[threadIdx.x]);
@@ -363,6 +376,31 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
         }
         __syncthreads();
     }
+}
+
+// Random-X with few losers in round 0 (a large X, a sparse graph): most rows
+// would push their whole row for few that still read their masks.  Round 0
+// then pushes nothing and ends its launch, the losers gather the colors fixed
+// in it from their own rows (k_late_marks), and the rounds go on as ever.
+// A gather for each of the losers' entries takes the place of a push for each
+// of the winners', so late_share, the share of the entries that the losers are
+// expected to hold (the set-up sums it) up to which this is done, is larger the
+// more a push costs against a gather: with heavy rows (it looks up the kind of
+// the neighbor and its bitmap) and beyond what L2 holds; on light graphs that
+// L2 holds a push costs no more.  Coloring with the pushes / without:
+// G(10^6, 40) Random-32 Fit (heavy) 1.87 / 1.55 ms, RMAT-Good 23 Random-8 5.8 /
+// 4.7, G(10^7, 24) Random-5 7.3 / 6.4, Random-32 7.5 / 3.6; light: the 27-point
+// mesh 100^3 Random-32 0.32 / 0.35, G(6 10^6, 24) Random-8 2.6 / 2.8.
+// kLateMin: below, the read-back and launches more cost what is saved.
+constexpr int64_t kLateMin = 11 << 18;
+inline float late_share_limit(int64_t n, int64_t nnz, bool heavy) {
+    if (nnz < kLateMin) return 0.f;
+    if (n <= kWideMax) return heavy ? 0.7f : 0.f;
+    return heavy || n > (int64_t(9) << 20) ? 0.92f : 0.6f;
+}
+__device__ __forceinline__ bool late_of(const SpecArgs& a) {
+    return a.late_share > 0.f &&
+           static_cast<float>(a.ctrl->lose16) < a.late_share * 16.0f * static_cast<float>(a.g.nnz);
 }
 
 // ---------------------------------------------------------------------------
@@ -827,6 +865,7 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
     int32_t t = blockIdx.x * kWarps + (threadIdx.x >> 5);
     if (t >= tiles) return;
     const WorkItem* lst = kRound0 ? nullptr : this_list(r) + r.start(b);
+    const bool late = kRXF && kRound0 && late_of(a);
     auto& st = r.w.light;
     auto stage_items = [&](int32_t tt, int slot) {
         if (kRound0) {  // the R + 1 offsets
@@ -965,7 +1004,7 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
         light_losers<kRound0>(r, b, valid && lost && gl == 0, it);
         if (valid && !lost) {
             if (gl == 0) fix_color<kHeavy, kWide>(r, it.v, tv, it.deg);
-            for (int32_t c = gl, q = 0; c < np; c += G, ++q) {
+            for (int32_t c = gl, q = 0; c < np && !late; c += G, ++q) {
                 int32_t u[4];
                 piece(c, u);
 #pragma unroll
@@ -1005,6 +1044,24 @@ __device__ __forceinline__ void heavy_win(Rounds<kWide>& r, int32_t v, int32_t c
     pos = __shfl_sync(kFull, pos, 0);
     for (int32_t q = l; q < np && pos + q < a.heavy.mark_cap; q += 32)  // (the capacity holds every piece of every row)
         store_item(a.heavy.mark + pos + q, beg + static_cast<int64_t>(q) * kPiece, c, min(kPiece, deg - q * kPiece));
+}
+
+// The lanes with `want` queue the pieces of their row for the whole grid.
+__device__ __forceinline__ void queue_losers(const SpecArgs& a, bool want, const WorkItem& it) {
+    const int l = lane_id();
+    const uint32_t np = want ? (static_cast<uint32_t>(it.deg) + kPiece - 1) / kPiece : 0u;
+    const uint32_t incl = warp_inclusive_scan(np);
+    int32_t base = 0;
+    if (l == 31 && incl) base = atomicAdd(&a.ctrl->mark_cnt, static_cast<int32_t>(incl));
+    base = __shfl_sync(kFull, base, 31) + static_cast<int32_t>(incl - np);
+    for (uint32_t m = __ballot_sync(kFull, np != 0); m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        const int64_t beg = __shfl_sync(kFull, it.beg, src);
+        const int32_t deg = __shfl_sync(kFull, it.deg, src), v = __shfl_sync(kFull, it.v, src);
+        const int32_t pos = __shfl_sync(kFull, base, src), n = static_cast<int32_t>(__shfl_sync(kFull, np, src));
+        for (int32_t q = l; q < n && pos + q < a.heavy.mark_cap; q += 32)  // (the capacity holds every piece of every row)
+            store_item(a.heavy.mark + pos + q, beg + static_cast<int64_t>(q) * kPiece, v, min(kPiece, deg - q * kPiece));
+    }
 }
 
 // Round 0, a piece of a heavy row (the whole warp): its share of the test,
@@ -1058,12 +1115,13 @@ __device__ __forceinline__ void heavy_round0_piece(Rounds<kWide>& r, const WorkI
 }
 
 // Round 0, once every piece is done: winners and losers (32 rows per warp).
-template <bool kWide>
+template <bool kRXF, bool kWide>
 __device__ __forceinline__ void heavy_round0_close(Rounds<kWide>& r) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t nh = a.ctrl->init_cnt[0];
     const int64_t step = static_cast<int64_t>(gridDim.x) * kBlock;
+    const bool late = kRXF && late_of(a);
     for (int64_t h0 = (static_cast<int64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5)) * 32; h0 < nh; h0 += step) {
         const int64_t h = h0 + l;
         WorkItem it{0, 0, 0};
@@ -1075,10 +1133,16 @@ __device__ __forceinline__ void heavy_round0_close(Rounds<kWide>& r) {
             pb = __ldg(a.heavy.h_pbeg + h);
             c = tent_of(*color_word<kWide>(a, it.v));
         }
-        warp_append(h < nh && pc < 0, pb, it.v, pc & INT32_MAX, &a.ctrl->cnt[1][0], a.list1, 0);
-        for (uint32_t m = __ballot_sync(kFull, h < nh && pc >= 0); m; m &= m - 1) {
+        const bool lost = h < nh && pc < 0, won = h < nh && pc >= 0;
+        warp_append(lost, pb, it.v, pc & INT32_MAX, &a.ctrl->cnt[1][0], a.list1, 0);
+        if (late) {
+            if (won) fix_color<true>(r, it.v, c, it.deg);
+            queue_losers(a, lost, it);
+            continue;
+        }
+        for (uint32_t m = __ballot_sync(kFull, won); m; m &= m - 1) {
             const int src = __ffs(m) - 1;
-            heavy_win<kWide>(r, __shfl_sync(kFull, it.v, src), __shfl_sync(kFull, c, src), __shfl_sync(kFull, it.beg, src),
+            heavy_win(r, __shfl_sync(kFull, it.v, src), __shfl_sync(kFull, c, src), __shfl_sync(kFull, it.beg, src),
                       __shfl_sync(kFull, it.deg, src));
         }
     }
@@ -1235,7 +1299,7 @@ __device__ __forceinline__ void heavy_rows(Rounds<kWide>& r) {
             int64_t beg;
             int32_t deg;
             row_of(a.g, it.v, beg, deg, &a.ctrl->err);
-            heavy_win<kWide>(r, it.v, tv, beg, deg);
+            heavy_win(r, it.v, tv, beg, deg);
         }
         if (!more) break;
         it = nx;
@@ -1282,7 +1346,7 @@ __device__ __forceinline__ void open_phase(Rounds<kWide>& r) {
                 store_item(next_list(r) + pos, row.beg, row.v, row.deg);
             }
         } else {
-            heavy_win<kWide>(r, row.v, tv, beg, deg);
+            heavy_win(r, row.v, tv, beg, deg);
         }
     }
 }
@@ -1372,14 +1436,14 @@ __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant
             if (r.round == 0) {
                 if (blockIdx.x == 0 && threadIdx.x == 0) c->mark_cnt = 0;
                 if (!(ok = bar.sync(c))) break;
-                heavy_round0_close<kWide>(r);
+                heavy_round0_close<kRXF>(r);
                 if (!(ok = bar.sync(c))) break;
             }
             if (__ldcg(&c->open_cnt) > 0) {
                 open_phase<kWide>(r);
                 if (!(ok = bar.sync(c))) break;
             }
-            if (__ldcg(&c->mark_cnt) > 0) {
+            if (!(kRXF && r.round == 0 && late_of(a)) && __ldcg(&c->mark_cnt) > 0) {
                 push_phase(a);
                 if (!(ok = bar.sync(c))) break;
             }
@@ -1394,6 +1458,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant
             if (blockIdx.x == 0 && threadIdx.x == 0) c->stuck = 1;
             break;
         }
+        if (kRXF && r.round == 1 && late_of(a)) break;  // k_late_marks comes next
         if (r.round >= a.round_limit) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&c->err, kErrRoundLimit);
             break;
@@ -1413,6 +1478,92 @@ __device__ __forceinline__ int32_t region_start(const SpecCtrl* c, int b) {
     int32_t s = 0;
     for (int q = 0; q < b; ++q) s += q != 1 ? c->init_cnt[q] : 0;
     return s;
+}
+
+// The marks that a late round 0 left out (see late_of): of every light loser
+// by 2 or 8 lanes, of the heavy ones by queued pieces.  (A kernel of its own:
+// with this code in theirs the rounds ran up to 7 % slower.)
+template <int G, bool kWide>
+__device__ __forceinline__ void late_light(const SpecArgs& a, const WorkItem* lst, int32_t cnt) {
+    constexpr int R = 32 / G;
+    const int l = lane_id(), gi = l / G, gl = l % G;
+    const uint32_t step = gridDim.x * kWarps * R;
+    uint32_t k = (blockIdx.x * kWarps + (threadIdx.x >> 5)) * R + gi;
+    WorkItem nx{0, 0, 0};
+    if (k < static_cast<uint32_t>(cnt)) nx = load_item(lst + k);
+    while (__any_sync(kFull, k < static_cast<uint32_t>(cnt))) {
+        const WorkItem it = nx;
+        const bool valid = k < static_cast<uint32_t>(cnt);
+        k += step;
+        nx = WorkItem{0, 0, 0};
+        if (k < static_cast<uint32_t>(cnt)) nx = load_item(lst + k);
+        const int32_t np = valid ? row_pieces(a.g, it.beg, it.deg) : 0;
+        uint32_t lo = 0, hi = 0;
+        for (int32_t c0 = gl; c0 < np; c0 += 2 * G) {
+            int32_t u[2][4], x[2][4];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) u[q][i] = -1;
+                if (c0 + q * G < np) row_piece(a.g, it.beg, it.deg, c0 + q * G, u[q], &a.ctrl->err);
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) x[q][i] = u[q][i] >= 0 ? *color_word<kWide>(a, u[q][i]) : kUnfixed;
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {  // (a word with kUnfixed set: no bit)
+                    lo |= bit_or_none(x[q][i] - 1);
+                    hi |= bit_or_none(x[q][i] - 33);
+                }
+        }
+#pragma unroll
+        for (int d = G / 2; d >= 1; d >>= 1) {
+            lo |= __shfl_xor_sync(kFull, lo, d);
+            hi |= __shfl_xor_sync(kFull, hi, d);
+        }
+        if (valid && gl == 0) {
+            a.mlo[it.v] = lo;
+            a.mhi[it.v] = hi;
+        }
+    }
+}
+
+template <bool kWide>
+__global__ void __launch_bounds__(kBlock) k_late_marks(const __grid_constant__ SpecArgs a) {
+    SpecCtrl* const c = a.ctrl;
+    if (blockIdx.x == 0 && threadIdx.x == 0) c->barrier = 0;  // of the next launch
+    if (c->round != 1 || c->active == 0 || !late_of(a)) return;
+    for (int b = 2; b < kNB; ++b) {
+        const int32_t n = c->cnt[1][b];
+        if (n == 0) continue;
+        const WorkItem* lst = a.list1 + region_start(c, b);
+        if (b <= 4) late_light<8, kWide>(a, lst, n);
+        else late_light<2, kWide>(a, lst, n);
+    }
+    if (c->init_cnt[0] == 0) return;
+    const int32_t n = static_cast<int32_t>(min(static_cast<int64_t>(c->mark_cnt), a.heavy.mark_cap));
+    for (uint32_t k = blockIdx.x * kWarps + (threadIdx.x >> 5); k < static_cast<uint32_t>(n); k += gridDim.x * kWarps) {
+        const WorkItem it = load_item(a.heavy.mark + k);
+        const uint64_t ref = __ldg(a.heavy.bref + it.v);
+        int32_t u[4], x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int32_t e = lane_id() + 32 * i;
+            u[i] = e < it.deg ? load_nbr(a.g, it.beg + e, &c->err) : -1;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = u[i] >= 0 ? *color_word<kWide>(a, u[i]) : kUnfixed;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t bit = static_cast<uint32_t>(x[i] - 1);
+            if (x[i] <= 0 || bit >= 32u * static_cast<uint32_t>(ref & kRefWords)) continue;
+            uint32_t* const w = a.heavy.hbm + (ref >> 24) + (bit >> 5);
+            if (!(__ldcg(w) >> (bit & 31u) & 1u)) atomicOr(w, 1u << (bit & 31u));
+        }
+    }
 }
 
 // The choice of a whole round from the rows, a warp each.  The row of the
@@ -1474,23 +1625,30 @@ const void* rounds_kernel_of(bool rxf, bool heavy) {
                  : reinterpret_cast<const void*>(k_spec_rounds<false, false, kWide>);
 }
 
-// The rounds: one cooperative launch (spec_graph 1), or one per round.  h
+// The rounds: one cooperative launch (spec_graph 1), or one per round; two
+// with the marks of round 0 in between where it pushed nothing (late_of).  h
 // receives the final control block.
 gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_t s) {
     const bool wide = a.g.n <= kWideMax;
     const void* k = wide ? rounds_kernel_of<true>(rxf, heavy) : rounds_kernel_of<false>(rxf, heavy);
+    const auto late = wide ? k_late_marks<true> : k_late_marks<false>;
     const auto pull = wide ? k_pull_choose<true> : k_pull_choose<false>;
     const int fit = sm_count() * occupancy_of(k, kBlock);
     // a block per tile of round 0 at most: on small graphs more blocks would only lengthen the barriers
     const int64_t tiles = heavy ? fit : (static_cast<int64_t>(a.g.n) * 2 + kBlock - 1) / kBlock;
     const int64_t want = a.tune.grid_blocks > 0 ? a.tune.grid_blocks : std::max<int64_t>(1, tiles);
     const int grid = static_cast<int>(std::min<int64_t>(fit, want));
+    a.late_share = rxf ? late_share_limit(a.g.n, a.g.nnz, heavy) : 0.f;
     a.max_rounds = a.tune.spec_graph ? INT32_MAX : 1;
     a.chosen = 0;
-    for (;;) {
+    const auto launch = [&]() {
         void* args[] = {&a};
         cudaError_t e;
         GC_LAUNCH(KID_SPEC_ROUNDS, s, e = cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kBlock), args, 0, s));
+        return e;
+    };
+    for (;;) {
+        cudaError_t e = launch();
         if (e == cudaSuccess) e = cudaMemcpyAsync(h, a.ctrl, sizeof(SpecCtrl), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_status(e);
@@ -1500,10 +1658,12 @@ gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_
             a.chosen = 1;
             a.max_rounds = 1;
             GC_LAUNCH(KID_SPEC_PULL, s, pull<<<resident_grid(pull, a.tune), kBlock, 0, s>>>(a));
-            continue;
+        } else if (a.late_share > 0.f && h->round == 1) {
+            GC_LAUNCH(KID_SPEC_LATE, s, late<<<resident_grid(late, a.tune), kBlock, 0, s>>>(a));
+        } else {
+            e = cudaMemsetAsync(&a.ctrl->barrier, 0, sizeof(uint32_t), s);
+            if (e != cudaSuccess) return cuda_status(e);
         }
-        e = cudaMemsetAsync(&a.ctrl->barrier, 0, sizeof(uint32_t), s);
-        if (e != cudaSuccess) return cuda_status(e);
     }
 }
 }  // namespace

@@ -38,7 +38,7 @@ void note_launches(int64_t k);
 
 // Kernel timing (gc_profile_enable): events around each launch.
 enum KernelId {
-    KID_SPEC_SETUP, KID_SPEC_FILL, KID_SPEC_ROUNDS, KID_SPEC_PULL, KID_PRIORITIES,
+    KID_SPEC_SETUP, KID_SPEC_FILL, KID_SPEC_ROUNDS, KID_SPEC_PULL, KID_SPEC_LATE, KID_PRIORITIES,
     KID_RC_BUCKET, KID_RC_VALIDATE, KID_RC_HIST, KID_RC_ORDER, KID_RC_SCATTER,
     KID_RC_RECOLOR, KID_RC_STEP, KID_VALIDATE, KID_VALIDATE_ROWS, KID_MARK_PRESENT,
     KID_COUNT_BITS, KID_CHECK_GRAPH, KID_BATCH, KID_BRC_HIST, KID_BRC_ORDER,

@@ -132,14 +132,33 @@ struct Request {
     gc_request_result res{};
 };
 
-// Device bytes one request holds while its cohort runs: its CSR and colors,
-// the coloring scratch (priority keys, two work lists, buckets, per-vertex
-// graph index and win round) or the recoloring scratch (work list, alternate
-// colors, per-class tables over at most min(n, max degree + X) + 1 classes),
-// whichever is larger, with room to spare.
-int64_t request_bytes(int64_t n, int64_t nnz, int64_t max_deg, int32_t X) {
-    const int64_t classes = std::min<int64_t>(n, max_deg + X) + 2;
-    return 16 * (n + 1) + 4 * nnz + 4 * n + 64 * n + 16 * (nnz / 256 + 1) + 256 * classes + 1024;
+// What a request's memory depends on (its offsets' check fills it in).
+struct Shape {
+    int64_t n = 0, nnz = 0;
+    int64_t max_deg = 0;
+    int64_t heavy_rows = 0, heavy_entries = 0;  // degree + X > 64 (coloring)
+    int64_t split_rows = 0;                     // bucket 0 of the recoloring
+};
+
+// Device bytes one request holds while its cohort runs: its CSR (its staged
+// offsets too) and colors, and the scratch of the coloring or the recoloring,
+// whichever is larger, rounded up.
+//   Coloring: per vertex 57 (words or priorities 8, masks 8, two lists 32,
+// bucket 1, graph index and win round 8) and, as soon as the cohort has a heavy
+// row, 8 (bitmap reference); per heavy entry 4 (list) and 0.35 (bitmap, row
+// and list pieces); per heavy row 57 (bounds, roundings, its first piece).
+//   Recoloring: per vertex 25, 16 per row chunk, and per split row 16 and its
+// list (1 KB) and bitmap (a bit per class).
+//   Classes: no more than the longest row and X allow, nor than the entries:
+// a vertex of color c has neighbors of c - X smaller colors at least, and so
+// have these, so k colors take k - 2 X <= sqrt(nnz) + 1.
+int64_t request_bytes(const Shape& g, int32_t X) {
+    const int64_t by_edges = static_cast<int64_t>(std::sqrt(static_cast<double>(g.nnz))) + 2 * static_cast<int64_t>(X) + 2;
+    const int64_t classes = std::min({g.n, g.max_deg + X, by_edges}) + 2;
+    const int64_t csr = 16 * (g.n + 1) + 4 * g.nnz + 4 * g.n;
+    const int64_t color = 66 * g.n + 4 * g.heavy_entries + g.heavy_entries / 2 + 64 * g.heavy_rows;
+    const int64_t recolor = 25 * g.n + 16 * (g.nnz / 256 + 1) + g.split_rows * (1024 + 96 + classes / 8);
+    return csr + std::max(color, recolor) + 256 * classes + 2048;
 }
 // The part of it that stays with the cohort until compaction: offsets, ids, colors.
 int64_t resident_bytes(int64_t n, int64_t nnz) { return 8 * (n + 1) + 4 * nnz + 4 * n; }
@@ -575,16 +594,24 @@ void gc_server::compact(Cohort* c, cudaStream_t s) {
 namespace {
 
 // Host check of a request's offsets (the ids are checked on the device when
-// its batch is staged); *max_deg receives the largest row.
-gc_status check_offsets(const int64_t* off, int64_t n, int64_t nnz, int64_t* max_deg) {
+// its batch is staged); *shape receives what its memory depends on.
+gc_status check_offsets(const int64_t* off, int64_t n, int64_t nnz, int32_t X, const Tuning& t, Shape* shape) {
     if (off[0] != 0 || off[n] != nnz) return GC_ERR_BAD_GRAPH;
-    int64_t md = 0;
+    const int64_t split = std::max<int64_t>(t.rc_warp_max_deg, 63);
+    Shape g;
+    g.n = n;
+    g.nnz = nnz;
     for (int64_t v = 0; v < n; ++v) {
         const int64_t d = off[v + 1] - off[v];
         if (d < 0) return GC_ERR_BAD_GRAPH;
-        md = std::max(md, d);
+        g.max_deg = std::max(g.max_deg, d);
+        if (d + X > 64) {
+            ++g.heavy_rows;
+            g.heavy_entries += d;
+        }
+        g.split_rows += d > split;
     }
-    *max_deg = md;
+    *shape = g;
     return GC_OK;
 }
 
@@ -636,19 +663,19 @@ gc_status gc_server_submit(gc_server* s, const gc_request* q, uint64_t* ticket) 
     r->nnz = g.nnz;
     r->off = g.offsets;
     r->idx = g.idx;
-    int64_t max_deg = 0;
+    const int32_t X = q->strategy == GC_FIRST_FIT ? 1 : q->X;
+    Shape shape;
     gc_status st = GC_OK;
     if (g.mem == GC_MEM_HOST) {
-        st = check_offsets(g.offsets, g.n, g.nnz, &max_deg);
+        st = check_offsets(g.offsets, g.n, g.nnz, X, s->tune, &shape);
     } else {
         std::vector<int64_t> off(static_cast<size_t>(g.n) + 1);
         cudaSetDevice(s->device);
         const cudaError_t e =
             cudaMemcpy(off.data(), g.offsets, off.size() * sizeof(int64_t), cudaMemcpyDeviceToHost);
-        st = e == cudaSuccess ? check_offsets(off.data(), g.n, g.nnz, &max_deg) : cuda_status(e);
+        st = e == cudaSuccess ? check_offsets(off.data(), g.n, g.nnz, X, s->tune, &shape) : cuda_status(e);
     }
-    const int32_t X = q->strategy == GC_FIRST_FIT ? 1 : q->X;
-    r->bytes = request_bytes(g.n, g.nnz, max_deg, X);
+    r->bytes = request_bytes(shape, X);
     r->resident = resident_bytes(g.n, g.nnz);
     if (st == GC_OK && r->bytes > s->budget) st = GC_ERR_BUDGET;
     if (st != GC_OK) {

@@ -1458,10 +1458,11 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     cudaMemsetAsync(a.ctrl, 0, ctrl_bytes, s);
     RcCtrl h;
     std::memset(&h, 0, sizeof(h));
-    gc_status input = GC_OK;
     if (!trusted) {
-        input = check_input_device(g, colors_in, kMaxInputColor, &maxc_in, s);
-        if (input != GC_OK && input != GC_ERR_IMPROPER_INPUT) return input;
+        // (the bucket pass first: its result is there when the check has been waited for)
+        if (n > 0 && iterations > 0) GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
+        const gc_status input = check_input_device(g, colors_in, kMaxInputColor, &maxc_in, s);
+        if (input != GC_OK) return input;
     }
     // A trusted input (our own coloring) has a known max color and longest
     // row; the split rows are then sized by a bound (a bucket-0 row has more
@@ -1470,14 +1471,14 @@ gc_status recolor_device(const Graph& g, const int32_t* colors_in, int32_t maxc_
     const int64_t heavy_min = std::max<int64_t>(tune.warp_max_deg, 63) + 1;
     const int64_t heavy_bound = max_deg < heavy_min ? 0 : std::min<int64_t>(n, static_cast<int64_t>(g.nnz) / heavy_min);
     const int64_t bound_words = (static_cast<int64_t>(std::max(maxc_in, 1)) + 1 + 31) / 32 + kRowPend;
-    const bool read_back = !trusted || n == 0 || heavy_bound * bound_words * 4 > (int64_t(64) << 20);
+    const bool read_back = n > 0 && iterations > 0 &&
+                           (!trusted || heavy_bound * bound_words * 4 > (int64_t(64) << 20));
     if (read_back) {
-        if (n > 0) GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
+        if (trusted) GC_LAUNCH(KID_RC_BUCKET, s, k_rc_bucket<<<vgrid, kBlock, 0, s>>>(a));
         ce = cudaMemcpyAsync(&h, a.ctrl, sizeof(RcCtrl), cudaMemcpyDeviceToHost, s);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
         if (ce != cudaSuccess) return cuda_status(ce);
         if (h.err & kErrBadGraph) return GC_ERR_BAD_GRAPH;
-        if (input != GC_OK) return input;
     } else {
         h.n_heavy = static_cast<int32_t>(heavy_bound);
     }

@@ -391,12 +391,14 @@ __global__ void __launch_bounds__(kHeavyThreads) k_heavy_setup(SpecArgs a, int32
 // G(10^6, 40) Random-32 Fit (heavy) 1.87 / 1.55 ms, RMAT-Good 23 Random-8 5.8 /
 // 4.7, G(10^7, 24) Random-5 7.3 / 6.4, Random-32 7.5 / 3.6; light: the 27-point
 // mesh 100^3 Random-32 0.32 / 0.35, G(6 10^6, 24) Random-8 2.6 / 2.8.
-// kLateMin: below, the read-back and launches more cost what is saved.
+// Below kLateMin entries the read-back and launches more cost what is saved
+// (200,000 x 12 with 5 % of the rows heavy, Random-32: 0.25 / 0.27 ms), below
+// half of it also where most rows are heavy (Random-70: 0.45 / 0.36).
 constexpr int64_t kLateMin = 11 << 18;
-inline float late_share_limit(int64_t n, int64_t nnz, bool heavy) {
-    if (nnz < kLateMin) return 0.f;
-    if (n <= kWideMax) return heavy ? 0.7f : 0.f;
-    return heavy || n > (int64_t(9) << 20) ? 0.92f : 0.6f;
+inline float late_share_limit(int64_t n, int64_t nnz, int64_t heavy_rows) {
+    if (nnz < (2 * heavy_rows > n ? kLateMin / 2 : kLateMin)) return 0.f;
+    if (n <= kWideMax) return heavy_rows ? 0.7f : 0.f;
+    return heavy_rows || n > (int64_t(9) << 20) ? 0.92f : 0.6f;
 }
 __device__ __forceinline__ bool late_of(const SpecArgs& a) {
     return a.late_share > 0.f &&
@@ -1067,51 +1069,72 @@ __device__ __forceinline__ void queue_losers(const SpecArgs& a, bool want, const
 // Round 0, a piece of a heavy row (the whole warp): its share of the test,
 // and the row's list -- the neighbors above it in the total order, the only
 // ones that can beat it in a later round (their order is free, so the pieces
-// of a row just take places).
+// of a row just take places; a row of one piece needs none).  Bound by the
+// latency of its dependent reads: a shared word gives priority and color at
+// once (separate ones: the color of those above only; with all R-MAT 24
+// Random-8 Fit took 24.6 ms, 22.8 without).  Random-70 Fit, round 0, with the
+// places of all rows counted and the words read one after the other / now:
+// G(20,000, 1500) 234 / 198 us, G(2 10^6, 60) 1.45 / 1.23 ms, G(3 10^7, 6) 20.4 /
+// 16.8.
 template <bool kRXF, bool kWide>
 __device__ __forceinline__ void heavy_round0_piece(Rounds<kWide>& r, const WorkItem& it) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t h = it.v;
-    const int32_t v = __ldcg(&a.list0[h].v);
+    const WorkItem row = load_item_rw(a.list0 + h);
     int32_t* dst = a.heavy.pend + __ldg(a.heavy.h_pbeg + h);
-    const uint32_t pv = prio_word<kWide>(a, v);
-    const int32_t tv = kRXF ? tent_of(*color_word<kWide>(a, v)) : 1;
-    bool lose = false, loop = false;
-    {
-        int32_t u[8];
-        uint32_t p[8];
+    int32_t u[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int32_t k = 32 * i + l;
-            u[i] = k < it.deg ? load_nbr(a.g, it.beg + k, &a.ctrl->err) : -1;
-            if (u[i] == v) {
-                loop = true;
-                u[i] = -1;
-            }
-        }
+    for (int i = 0; i < 8; ++i) {
+        const int32_t k = 32 * i + l;
+        u[i] = k < it.deg ? load_nbr(a.g, it.beg + k, &a.ctrl->err) : -1;
+    }
+    uint32_t p[8];
+    int32_t x[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) p[i] = u[i] >= 0 ? prio_word<kWide>(a, u[i]) : 0u;
-        uint32_t keep[8];
-        int32_t total = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const bool up = u[i] >= 0 && above(p[i], u[i], pv, v);
-            if (up && (!kRXF || tent_of(*color_word<kWide>(a, u[i])) == tv)) lose = true;
-            keep[i] = __ballot_sync(kFull, up);
-            total += __popc(keep[i]);
-        }
-        int32_t pos = 0;
-        if (l == 0 && total) pos = atomicAdd(a.heavy.h_pcnt + h, total) & INT32_MAX;
-        pos = __shfl_sync(kFull, pos, 0);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            if (keep[i] >> l & 1u) dst[pos + __popc(keep[i] & ((1u << l) - 1u))] = u[i];
-            pos += __popc(keep[i]);
+    for (int i = 0; i < 8; ++i) {
+        p[i] = 0u;
+        x[i] = 0;
+        if (u[i] < 0) continue;
+        if (kRXF && kWide) {
+            const uint2 w = reinterpret_cast<const uint2*>(a.prio)[u[i]];
+            p[i] = w.x;
+            x[i] = static_cast<int32_t>(w.y);
+        } else {
+            p[i] = prio_word<kWide>(a, u[i]);
         }
     }
+    const uint32_t pv = prio_word<kWide>(a, row.v);
+    const int32_t tv = kRXF ? tent_of(*color_word<kWide>(a, row.v)) : 1;
+    bool lose = false, loop = false;
+    uint32_t keep[8];
+    int32_t total = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        loop |= u[i] == row.v;
+        const bool up = u[i] >= 0 && u[i] != row.v && above(p[i], u[i], pv, row.v);
+        if (kRXF && !kWide && up) x[i] = *color_word<kWide>(a, u[i]);
+        lose |= up && (!kRXF || tent_of(x[i]) == tv);
+        keep[i] = __ballot_sync(kFull, up);
+        total += __popc(keep[i]);
+    }
+    const bool single = row.deg <= kRound0Piece;
+    int32_t pos = 0;
+    if (!single) {
+        if (l == 0 && total) pos = atomicAdd(a.heavy.h_pcnt + h, total) & INT32_MAX;
+        pos = __shfl_sync(kFull, pos, 0);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if (keep[i] >> l & 1u) dst[pos + __popc(keep[i] & ((1u << l) - 1u))] = u[i];
+        pos += __popc(keep[i]);
+    }
     if (loop) atomicOr(&a.ctrl->err, kErrBadGraph);
-    if (__any_sync(kFull, lose) && l == 0) atomicOr(a.heavy.h_pcnt + h, INT32_MIN);
+    lose = __any_sync(kFull, lose);
+    if (l == 0) {
+        if (single) a.heavy.h_pcnt[h] = total | (lose ? INT32_MIN : 0);
+        else if (lose) atomicOr(a.heavy.h_pcnt + h, INT32_MIN);
+    }
 }
 
 // Round 0, once every piece is done: winners and losers (32 rows per warp).
@@ -1627,8 +1650,9 @@ const void* rounds_kernel_of(bool rxf, bool heavy) {
 
 // The rounds: one cooperative launch (spec_graph 1), or one per round; two
 // with the marks of round 0 in between where it pushed nothing (late_of).  h
-// receives the final control block.
-gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_t s) {
+// receives the final control block.  heavy_rows: 0 for the form without them.
+gc_status run_rounds(SpecArgs& a, bool rxf, int32_t heavy_rows, SpecCtrl* h, cudaStream_t s) {
+    const bool heavy = heavy_rows > 0;
     const bool wide = a.g.n <= kWideMax;
     const void* k = wide ? rounds_kernel_of<true>(rxf, heavy) : rounds_kernel_of<false>(rxf, heavy);
     const auto late = wide ? k_late_marks<true> : k_late_marks<false>;
@@ -1638,7 +1662,7 @@ gc_status run_rounds(SpecArgs& a, bool rxf, bool heavy, SpecCtrl* h, cudaStream_
     const int64_t tiles = heavy ? fit : (static_cast<int64_t>(a.g.n) * 2 + kBlock - 1) / kBlock;
     const int64_t want = a.tune.grid_blocks > 0 ? a.tune.grid_blocks : std::max<int64_t>(1, tiles);
     const int grid = static_cast<int>(std::min<int64_t>(fit, want));
-    a.late_share = rxf ? late_share_limit(a.g.n, a.g.nnz, heavy) : 0.f;
+    a.late_share = rxf ? late_share_limit(a.g.n, a.g.nnz, heavy_rows) : 0.f;
     a.max_rounds = a.tune.spec_graph ? INT32_MAX : 1;
     a.chosen = 0;
     const auto launch = [&]() {
@@ -1720,7 +1744,7 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
     const int setup_grid = static_cast<int>(std::min<int64_t>((n + kBlock - 1) / kBlock, resident_grid(setup, a.tune)));
     GC_LAUNCH(KID_SPEC_SETUP, s, setup<<<setup_grid, kBlock, 0, s>>>(a));
     SpecCtrl h{};
-    gc_status st = run_rounds(a, X > 1, false, &h, s);
+    gc_status st = run_rounds(a, X > 1, 0, &h, s);
     ScratchSet sc_heavy, sc_queues;
     if (st == GC_OK && h.init_cnt[0] > 0) {
         // heavy rows: their lists and bitmaps (sizes read back), then the rounds
@@ -1753,7 +1777,7 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
         if (ce != cudaSuccess) return cuda_status(ce);
         GC_LAUNCH(KID_SPEC_FILL, s,
                   k_heavy_setup<<<hblocks, kHeavyThreads, 0, s>>>(a, nh, sums));
-        st = run_rounds(a, X > 1, true, &h, s);
+        st = run_rounds(a, X > 1, nh, &h, s);
     }
     cudaEventRecord(ev.e1, s);
     if (max_deg) *max_deg = h.max_deg;

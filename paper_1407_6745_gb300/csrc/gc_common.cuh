@@ -31,7 +31,8 @@ struct Tuning {
     int32_t g4_max_deg;    // deg <= this -> 4 lanes
     int32_t g8_max_deg;    // -> 8 lanes
     int32_t g16_max_deg;   // -> 16 lanes
-    int32_t warp_max_deg;  // deg + X > 64 and deg <= this -> warp + smem bitmap
+    int32_t warp_max_deg;  // recoloring (rc_warp_max_deg): deg > 63 and deg <= this -> a warp, beyond: split;
+                           // no effect on the coloring
     int32_t grid_blocks;   // persistent grid size (0 = 8 per SM)
     int32_t recolor_mode;  // 0 = dataflow (one launch), 1 = one launch per class
     int32_t spin_limit;    // bounded wait iterations in the dataflow recolor
@@ -408,7 +409,7 @@ __device__ __forceinline__ int32_t choose_warp(const Graph& g, int64_t beg, int3
 
 // ---------------------------------------------------------------------------
 // Tiles: a list is cut into segments (one bucket each); segment s holds
-// tiles tile_prefix[s] .. tile_prefix[s+1]-1 of bucket_tile(bucket) vertices.
+// tiles tile_prefix[s] .. tile_prefix[s+1]-1.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int find_segment(const int32_t* prefix, int nseg, int32_t t) {
     int lo = 0, hi = nseg - 1;  // largest s with prefix[s] <= t

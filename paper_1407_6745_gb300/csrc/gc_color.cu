@@ -455,12 +455,20 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
 }
 
-// The same for what a pass reads once (ids, offsets): first out of L2.
+// The same for what a pass reads once (ids, items): first out of L2.  (Light
+// forms only: large light graphs run 3 to 6 % faster, R-MAT 24 with Random-8 1 %
+// slower.)
 __device__ __forceinline__ void cp_async16_stream(void* smem, const void* gmem) {
     const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
     asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(sa), "l"(gmem),
                  "l"(policy_evict_first())
                  : "memory");
+}
+
+template <bool kHeavy>
+__device__ __forceinline__ void cp_async16_rows(void* smem, const void* gmem) {
+    if constexpr (kHeavy) cp_async16(smem, gmem);
+    else cp_async16_stream(smem, gmem);
 }
 
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
@@ -480,11 +488,12 @@ constexpr int32_t kPushInline = 128;    // longer winners' rows are pushed by th
 // rows; and the losers it has not yet written to the next list.  kOut of them:
 // a counter update by all warps of the grid goes to one word, and pushes wait
 // behind it (G(10^7, 6) First Fit with 32: round 0 1.94 ms, 0.86 with no
-// update at all); large graphs (separate words) trade staged ids for more.
-template <bool kWide>
+// update at all); large graphs of light rows trade staged ids for more (G(2 10^7,
+// 6) First Fit 8.7 -> 8.1 ms; with heavy rows too, RMAT-Good 24 lost 1 to 2 %).
+template <bool kHeavy, bool kWide>
 struct __align__(16) WarpRounds {
-    static constexpr int kIds = kWide ? 512 : 448;  // per row with 2 lanes: 32, 28
-    static constexpr int kOut = kWide ? 64 : 96;
+    static constexpr int kIds = kHeavy || kWide ? 512 : 448;  // per row with 2 lanes: 32, 28
+    static constexpr int kOut = kHeavy || kWide ? 64 : 96;
     union {
         int32_t head[2][kHead];
         struct {
@@ -497,10 +506,10 @@ struct __align__(16) WarpRounds {
 
 // State of a warp over the launch.  Lane b keeps the count of bucket b's work
 // list and the start of its region.
-template <bool kWide>
+template <bool kHeavy, bool kWide>
 struct Rounds {
     const SpecArgs& a;
-    WarpRounds<kWide>& w;
+    WarpRounds<kHeavy, kWide>& w;
     int32_t lane_start, lane_cnt;
     int32_t round;
     int32_t par;
@@ -512,22 +521,22 @@ struct Rounds {
     __device__ __forceinline__ int32_t cnt(int b) const { return __shfl_sync(kFull, lane_cnt, b); }
 };
 
-template <bool kWide>
-__device__ __forceinline__ WorkItem* next_list(const Rounds<kWide>& r) { return r.par ? r.a.list0 : r.a.list1; }
-template <bool kWide>
-__device__ __forceinline__ const WorkItem* this_list(const Rounds<kWide>& r) { return r.par ? r.a.list1 : r.a.list0; }
+template <bool kHeavy, bool kWide>
+__device__ __forceinline__ WorkItem* next_list(const Rounds<kHeavy, kWide>& r) { return r.par ? r.a.list0 : r.a.list1; }
+template <bool kHeavy, bool kWide>
+__device__ __forceinline__ const WorkItem* this_list(const Rounds<kHeavy, kWide>& r) { return r.par ? r.a.list1 : r.a.list0; }
 
 // The buffered losers of bucket b ask for their places in the next list once
 // the next 16 may not fit any more, and are written there when these come (the
 // answer takes its time).
-template <bool kWide>
-__device__ __forceinline__ bool losers_asked(const Rounds<kWide>& r) { return r.out_n > WarpRounds<kWide>::kOut - 16; }
-template <bool kWide>
-__device__ __forceinline__ void ask_places(Rounds<kWide>& r, int b) {
+template <bool kHeavy, bool kWide>
+__device__ __forceinline__ bool losers_asked(const Rounds<kHeavy, kWide>& r) { return r.out_n > WarpRounds<kHeavy, kWide>::kOut - 16; }
+template <bool kHeavy, bool kWide>
+__device__ __forceinline__ void ask_places(Rounds<kHeavy, kWide>& r, int b) {
     if (lane_id() == 0) r.out_at = atomicAdd(&r.a.ctrl->cnt[r.par ^ 1][b], r.out_n);
 }
-template <bool kWide>
-__device__ __forceinline__ void write_losers(Rounds<kWide>& r, int b) {
+template <bool kHeavy, bool kWide>
+__device__ __forceinline__ void write_losers(Rounds<kHeavy, kWide>& r, int b) {
     const int32_t base = __shfl_sync(kFull, r.out_at, 0) + r.start(b);
     for (int32_t i = lane_id(); i < r.out_n; i += 32) {
         const WorkItem x = r.w.out[i];
@@ -536,8 +545,8 @@ __device__ __forceinline__ void write_losers(Rounds<kWide>& r, int b) {
     __syncwarp();
     r.out_n = 0;
 }
-template <bool kWide>
-__device__ __forceinline__ void flush_losers(Rounds<kWide>& r, int b) {
+template <bool kHeavy, bool kWide>
+__device__ __forceinline__ void flush_losers(Rounds<kHeavy, kWide>& r, int b) {
     if (r.out_n == 0) return;
     if (!losers_asked(r)) ask_places(r, b);
     write_losers(r, b);
@@ -545,8 +554,8 @@ __device__ __forceinline__ void flush_losers(Rounds<kWide>& r, int b) {
 
 // The lanes with `want` (16 at most) add their row to the losers of bucket b
 // (one bucket at a time is buffered).  The whole warp calls it.
-template <bool kWide>
-__device__ __forceinline__ void add_losers(Rounds<kWide>& r, int b, bool want, int64_t beg, int32_t v, int32_t deg) {
+template <bool kHeavy, bool kWide>
+__device__ __forceinline__ void add_losers(Rounds<kHeavy, kWide>& r, int b, bool want, int64_t beg, int32_t v, int32_t deg) {
     const uint32_t m = __ballot_sync(kFull, want);
     if (m == 0) return;
     if (losers_asked(r)) write_losers(r, b);
@@ -611,7 +620,7 @@ __device__ __forceinline__ void push_row(const SpecArgs& a, int64_t beg, int32_t
 // round that its vertex is in the work set (the method's choice and test;
 // the choice of round 0 is counted for all rows by the host).
 template <bool kHeavy, bool kWide>
-__device__ __forceinline__ void fix_color(Rounds<kWide>& r, int32_t v, int32_t c, int32_t deg) {
+__device__ __forceinline__ void fix_color(Rounds<kHeavy, kWide>& r, int32_t v, int32_t c, int32_t deg) {
     r.a.color[v] = c;
     if (kWide) *color_word<true>(r.a, v) = c;
     if (kHeavy) r.a.bucket[v] = kBucketFixed;
@@ -655,7 +664,7 @@ __device__ __forceinline__ int32_t choose_from_bitmap(const uint32_t* bm, int32_
 
 // A heavy row's choice (the whole warp): the j-th clear bit of its bitmap.
 template <bool kWide>
-__device__ __forceinline__ int32_t choose_heavy(Rounds<kWide>& r, int32_t v, uint32_t j, uint64_t ref) {
+__device__ __forceinline__ int32_t choose_heavy(Rounds<true, kWide>& r, int32_t v, uint32_t j, uint64_t ref) {
     const SpecArgs& a = r.a;
     int32_t c = choose_from_bitmap(a.heavy.hbm + (ref >> 24), static_cast<int32_t>(ref & kRefWords), j);
     if (c < 0) {  // past the bitmap's free colors (Random-X with a large X): the row in full
@@ -670,7 +679,7 @@ __device__ __forceinline__ int32_t choose_heavy(Rounds<kWide>& r, int32_t v, uin
 // A light row takes a thread (its color is among the first 64); a heavy one's
 // bitmap is searched.
 template <bool kRXF, bool kHeavy, bool kWide>
-__device__ __forceinline__ void choose_phase(Rounds<kWide>& r) {
+__device__ __forceinline__ void choose_phase(Rounds<kHeavy, kWide>& r) {
     const SpecArgs& a = r.a;
     const WorkItem* list = this_list(r);
     if constexpr (kHeavy) {
@@ -833,8 +842,8 @@ __device__ __forceinline__ bool beaten(const SpecArgs& a, const int32_t (&u)[4],
 
 // The lanes with `want` add their light row to the losers (of bucket b;
 // round 0: of its own).
-template <bool kRound0, bool kWide>
-__device__ __forceinline__ void light_losers(Rounds<kWide>& r, int b, bool want, const WorkItem& it) {
+template <bool kRound0, bool kHeavy, bool kWide>
+__device__ __forceinline__ void light_losers(Rounds<kHeavy, kWide>& r, int b, bool want, const WorkItem& it) {
     if (!kRound0) {
         add_losers(r, b, want, it.beg, it.v, it.deg);
         return;
@@ -855,10 +864,10 @@ __device__ __forceinline__ void light_losers(Rounds<kWide>& r, int b, bool want,
 // checks of the adjacency; colors and priorities are gathered until the row
 // has lost.
 template <int G, bool kRXF, bool kHeavy, bool kWide, bool kRound0>
-__device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
+__device__ __forceinline__ void light_rows(Rounds<kHeavy, kWide>& r, int b) {
     const SpecArgs& a = r.a;
     constexpr int R = 32 / G;
-    constexpr int kRow = WarpRounds<kWide>::kIds / R;  // ids of a row in the stage
+    constexpr int kRow = WarpRounds<kHeavy, kWide>::kIds / R;  // ids of a row in the stage
     static_assert(R <= 16 && kRow % 4 == 0, "16-byte rows");
     const int l = lane_id(), gi = l / G, gl = l % G;
     const int32_t cnt = kRound0 ? a.g.n : r.cnt(b);
@@ -874,7 +883,7 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
             int64_t* off = reinterpret_cast<int64_t*>(st.item[slot]);
             if (l <= min(R, cnt - tt * R)) cp_async8(off + l, a.g.off + tt * R + l);
         } else if (l < min(R, cnt - tt * R)) {
-            cp_async16_stream(&st.item[slot][l], lst + tt * R + l);
+            cp_async16_rows<kHeavy>(&st.item[slot][l], lst + tt * R + l);
         }
     };
     auto item = [&](int32_t tt, int slot) {
@@ -899,7 +908,7 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
         const int64_t* off = reinterpret_cast<const int64_t*>(st.item[slot]);
         const int64_t base = off[0] & ~static_cast<int64_t>(3);
         end = off[min(R, cnt - tt * R)];
-        return end - base <= WarpRounds<kWide>::kIds ? base : -1;
+        return end - base <= WarpRounds<kHeavy, kWide>::kIds ? base : -1;
     };
     auto stage_ids = [&](int32_t tt, int slot) {
         if (!a.g.vec) return;
@@ -907,14 +916,14 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
         const int64_t base = run_of(tt, slot, end);
         if (kRound0 && base >= 0) {
             for (int64_t e = base + 4 * l; e < end; e += 128)
-                if (e + 4 <= a.g.nnz) cp_async16_stream(&st.ids[slot][e - base], a.g.idx + e);
+                if (e + 4 <= a.g.nnz) cp_async16_rows<kHeavy>(&st.ids[slot][e - base], a.g.idx + e);
             return;
         }
         const WorkItem it = item(tt, slot);
         const int32_t np = min(row_pieces(a.g, it.beg, it.deg), kRow / 4);
         for (int32_t c = gl; c < np; c += G) {
             const int64_t e = (it.beg & ~static_cast<int64_t>(3)) + 4 * static_cast<int64_t>(c);
-            if (e + 4 <= a.g.nnz) cp_async16_stream(&st.ids[slot][gi * kRow + 4 * c], a.g.idx + e);
+            if (e + 4 <= a.g.nnz) cp_async16_rows<kHeavy>(&st.ids[slot][gi * kRow + 4 * c], a.g.idx + e);
         }
     };
     stage_items(t, 0);
@@ -1032,7 +1041,7 @@ __device__ __forceinline__ void light_rows(Rounds<kWide>& r, int b) {
 // A heavy winner (the whole warp): fixed, and its row pushed or queued for
 // the whole grid.
 template <bool kWide>
-__device__ __forceinline__ void heavy_win(Rounds<kWide>& r, int32_t v, int32_t c, int64_t beg, int32_t deg) {
+__device__ __forceinline__ void heavy_win(Rounds<true, kWide>& r, int32_t v, int32_t c, int64_t beg, int32_t deg) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     if (l == 0) fix_color<true, kWide>(r, v, c, deg);
@@ -1077,7 +1086,7 @@ __device__ __forceinline__ void queue_losers(const SpecArgs& a, bool want, const
 // G(20,000, 1500) 234 / 198 us, G(2 10^6, 60) 1.45 / 1.23 ms, G(3 10^7, 6) 20.4 /
 // 16.8.
 template <bool kRXF, bool kWide>
-__device__ __forceinline__ void heavy_round0_piece(Rounds<kWide>& r, const WorkItem& it) {
+__device__ __forceinline__ void heavy_round0_piece(Rounds<true, kWide>& r, const WorkItem& it) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t h = it.v;
@@ -1139,7 +1148,7 @@ __device__ __forceinline__ void heavy_round0_piece(Rounds<kWide>& r, const WorkI
 
 // Round 0, once every piece is done: winners and losers (32 rows per warp).
 template <bool kRXF, bool kWide>
-__device__ __forceinline__ void heavy_round0_close(Rounds<kWide>& r) {
+__device__ __forceinline__ void heavy_round0_close(Rounds<true, kWide>& r) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t nh = a.ctrl->init_cnt[0];
@@ -1193,7 +1202,7 @@ __device__ __forceinline__ bool list_hit(const SpecArgs& a, const int32_t* lst, 
 // A long list none of whose first entries beat its row is left to the whole
 // grid, in pieces.
 template <bool kWide>
-__device__ __forceinline__ void leave_open(const Rounds<kWide>& r, const WorkItem& it) {
+__device__ __forceinline__ void leave_open(const Rounds<true, kWide>& r, const WorkItem& it) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t np = (it.deg + kOpenPiece - 1) / kOpenPiece;
@@ -1227,7 +1236,7 @@ using Int = std::integral_constant<int, N>;
 // the list shrinks without a pass over it (it stays a superset of the
 // neighbors above v not fixed; its order is free).
 template <bool kWide>
-__device__ __forceinline__ void heavy_rows(Rounds<kWide>& r) {
+__device__ __forceinline__ void heavy_rows(Rounds<true, kWide>& r) {
     const SpecArgs& a = r.a;
     const WorkItem* list = this_list(r);
     const int l = lane_id();
@@ -1336,7 +1345,7 @@ __device__ __forceinline__ void heavy_rows(Rounds<kWide>& r) {
 // the row (acquire-release on the row's counter orders the other pieces'
 // findings before it).
 template <bool kWide>
-__device__ __forceinline__ void open_phase(Rounds<kWide>& r) {
+__device__ __forceinline__ void open_phase(Rounds<true, kWide>& r) {
     const SpecArgs& a = r.a;
     const int l = lane_id();
     const int32_t n = __ldcg(&a.ctrl->open_cnt);
@@ -1385,7 +1394,7 @@ __device__ __forceinline__ void push_phase(const SpecArgs& a) {
 }
 
 template <bool kRXF, bool kHeavy, bool kWide>
-__device__ __forceinline__ void test_phase(Rounds<kWide>& r) {
+__device__ __forceinline__ void test_phase(Rounds<kHeavy, kWide>& r) {
     const SpecArgs& a = r.a;
     if (r.round == 0) {
         if constexpr (kHeavy) {
@@ -1427,14 +1436,14 @@ __device__ __forceinline__ void test_phase(Rounds<kWide>& r) {
 // others until their polls run out.
 template <bool kRXF, bool kHeavy, bool kWide>
 __global__ void __launch_bounds__(kBlock, 4) k_spec_rounds(const __grid_constant__ SpecArgs a) {
-    __shared__ WarpRounds<kWide> s_w[kWarps];
-    static_assert(sizeof(WarpRounds<kWide>::head) >= kWarpBitmapWords * 4, "the full-row fallback's bitmap");
+    __shared__ WarpRounds<kHeavy, kWide> s_w[kWarps];
+    static_assert(sizeof(WarpRounds<kHeavy, kWide>::head) >= kWarpBitmapWords * 4, "the full-row fallback's bitmap");
     SpecCtrl* const c = a.ctrl;
     if (c->setup_err || (!kHeavy && c->init_cnt[0] > 0)) return;
     const int warp = threadIdx.x >> 5;
     const int l = lane_id();
     const int32_t mine = l < kNB && l != 1 ? c->init_cnt[l] : 0;
-    Rounds<kWide> r{a, s_w[warp],
+    Rounds<kHeavy, kWide> r{a, s_w[warp],
              static_cast<int32_t>(warp_inclusive_scan(static_cast<uint32_t>(mine))) - mine,
              l < kNB ? c->cnt[c->round & 1][l] : 0, c->round, 0, 0, 0, 0, 0ull};
     GridBarrier bar;

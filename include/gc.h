@@ -30,7 +30,8 @@
  *
  * Graph layout: symmetric CSR, offsets int64[n+1] with offsets[0] = 0,
  * non-decreasing, offsets[n] = nnz; idx int32[nnz] neighbor ids in [0, n).
- * Every undirected edge appears in both rows; duplicates are tolerated.  A
+ * Every undirected edge appears in both rows (a call on a CSR where one does not
+ * ends, with colors that may conflict there); duplicates are tolerated.  A
  * self-loop makes a graph uncolorable: the coloring calls report it as
  * GC_ERR_BAD_GRAPH, and a coloring given to gc_recolor / gc_validate counts
  * it as a conflict.
@@ -393,9 +394,9 @@ gc_status gc_check_graph(const gc_graph* g, int64_t* first_bad_vertex, void* str
  * launch (vertices wait, with a bounded spin of spin_limit polls, for their
  * earlier-class neighbors); 1 launches one grid per color class.
  * spec_graph 1 (default) runs the speculative rounds in one cooperative
- * launch with grid barriers (no host round trip per round); 0 launches them
- * one by one from the
- * host.  gc_set_tuning sets the process-wide knobs (change them only while
+ * launch with grid barriers (no host round trip per round; two launches where
+ * Random-X Fit's losers gather the colors of round 0); 0 launches them
+ * one by one from the host.  gc_set_tuning sets the process-wide knobs (change them only while
  * no call is running); a plan's knobs apply to its own calls only.
  */
 typedef struct {

@@ -22,7 +22,10 @@
 // a light row (degree + X <= 64: its color is among the first 64), a bitmap
 // for a heavy one -- so the choice is the j-th clear bit of the mask.  Each
 // row is pushed once in a run instead of being gathered in every round
-// (G(10^6, 24) First Fit: 24 M pushes instead of 128 M gathers).
+// (G(10^6, 24) First Fit: 24 M pushes instead of 128 M gathers).  Where
+// Random-X Fit has few losers in round 0, these gather its colors instead
+// (late_of).  Pushes need a symmetric CSR; the rounds of another one end by
+// k_pull_choose.
 //
 // The conflict test of a light row reads the row a few neighbors at a time and
 // ends at the first one it loses to (most vertices of an early round lose to
@@ -30,8 +33,8 @@
 // the total order that were not fixed at its last look, built from the row
 // in round 0; only those can beat it.
 //
-// All rounds run in one cooperative launch with a grid barrier between the
-// phases of a round (choice, test, and where there are any the long lists left
+// All rounds (after such a round 0: the others) run in one cooperative launch
+// with a grid barrier between the phases of a round (choice, test, and where there are any the long lists left
 // open and the long rows' pushes); a barrier takes about 1.2 us.
 //
 // What it replaced -- three launches a round in a CUDA graph, every light row
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__(kBlock) k_spec_setup(SpecArgs a) {
             if (a.prio_kind == 1) p = ordered_prio(deg, p);
             else if (a.prio_kind == 2) p = ordered_prio(65535 - static_cast<int64_t>(a.prio_rank[a.prio_old[v]]), p);
             const uint32_t j0 = (a.graph_of || a.X > 1) ? draw_index(a, v, 0) : 0u;
-            if (a.X > 1) lose16 += static_cast<unsigned long long>(16.0f * static_cast<float>(deg) * lose_chance(static_cast<float>(deg), X));
+            if (a.late_share > 0.f) lose16 += static_cast<unsigned long long>(16.0f * static_cast<float>(deg) * lose_chance(static_cast<float>(deg), X));
             const int32_t c0 = static_cast<int32_t>(j0 + 1u) | kUnfixed;
             if (kWide) {
                 reinterpret_cast<uint2*>(a.prio)[v] = make_uint2(p, static_cast<uint32_t>(c0));
@@ -1749,6 +1752,7 @@ static gc_status color_impl(const Graph& g, int32_t X, uint64_t seed, const int3
     } ev;
     cudaEventRecord(ev.e0, s);
     cudaMemsetAsync(a.ctrl, 0, sizeof(SpecCtrl), s);
+    a.late_share = X > 1 && g.nnz >= kLateMin / 2 ? 1.f : 0.f;  // (the set-up counts; the rounds take their own limit)
     const auto setup = wide ? k_spec_setup<true> : k_spec_setup<false>;
     const int setup_grid = static_cast<int>(std::min<int64_t>((n + kBlock - 1) / kBlock, resident_grid(setup, a.tune)));
     GC_LAUNCH(KID_SPEC_SETUP, s, setup<<<setup_grid, kBlock, 0, s>>>(a));

@@ -337,8 +337,7 @@ __device__ __forceinline__ void build_segments(const RcArgs& a, int32_t k, Order
 __global__ void __launch_bounds__(kOrderThreads) k_rc_order(RcArgs a) {
     __shared__ OrderShared s;
     const int t = threadIdx.x;
-    // the tables hold the colors up to cap: no iteration on others
-    if (t == 0 && a.ctrl->over) atomicOr(&a.ctrl->err, kErrImproper);
+    const uint32_t over = t == 0 ? __ldcg(&a.ctrl->over) : 0u;  // (used last: its latency is in no one's way)
     // present classes in ascending color, with their sizes
     int32_t k = 0;
     for (int32_t c0 = 1; c0 <= a.cap; c0 += kOrderThreads) {
@@ -408,6 +407,7 @@ __global__ void __launch_bounds__(kOrderThreads) k_rc_order(RcArgs a) {
         const int32_t c = a.order[sg / kRcNB];
         return b == 0 ? a.cls_units[c] : a.cls_cnt[c * kRcNB + b];
     });
+    if (over) atomicOr(&a.ctrl->err, kErrImproper);  // the tables hold the colors up to cap: no iteration on others
 }
 
 // ---------------------------------------------------------------------------
